@@ -407,7 +407,7 @@ struct Builder {
         op.type = L.kind == KIND_DW ? OP_DW : OP_CONV;
         op.layer = li; op.in = in; op.out = out; op.res = res;
         ConvArgs &a = op.conv;
-        a.w = L.w; a.scale = L.scale; a.shift = L.shift;
+        a.w = L.w; a.scale = L.scale; a.shift = L.shift; a.early_weights = 1;
         a.N = N; a.H = H; a.W = W; a.C = L.kind == KIND_DW ? s.K : s.C; a.K = s.K;
         a.k = s.k; a.stride = stride; a.act = act;
         int p = (s.k - 1) / 2;

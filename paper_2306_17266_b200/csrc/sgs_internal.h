@@ -73,6 +73,8 @@ struct ConvArgs {
     int layer = 0;
     int throughput = 0;  // 0: tiles for the latency of this launch; 1: for aggregate throughput (many launches in flight);
                          // 2: member of a grouped launch (128-filter tiles, reduction never split)
+    int early_weights = 0;  // 1: the weights belong to a loaded SuperNet, so a kernel may read them before the previous kernel of
+                            // the stream has finished; 0: they are the caller's and may come from that kernel
     // split-K scratch of the tensor-core kernel: fp32 partial tiles [splits][M][K]
     float *ws = nullptr;
     size_t ws_elems = 0;
@@ -162,7 +164,7 @@ struct Plan {
     std::vector<PqOp> pq;  // the plan as an op list of the persistent SubNet kernel (built on first use)
 };
 
-// ---- launchers implemented in sgs_kernels.cu (T = float or __nv_bfloat16) -------------------
+// ---- launchers implemented in sgs_kernels.cu (the convolution: sgs_conv_simt.cu), T = float or __nv_bfloat16
 template <typename T> cudaError_t launch_conv_plain(const ConvArgs &a, cudaStream_t st);
 template <typename T> cudaError_t launch_dw(const ConvArgs &a, cudaStream_t st);
 template <typename T> cudaError_t launch_maxpool3s2(const T *x, T *y, int N, int H, int W, int C, cudaStream_t st);

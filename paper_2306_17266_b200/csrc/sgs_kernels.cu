@@ -25,117 +25,6 @@ __device__ __forceinline__ float apply_act(float v, int act) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// Sliced convolution as an implicit GEMM on CUDA cores.
-//   D[m][f] = sum_kk A[m][kk] * B[f][kk],  m = output pixel, f < K', kk = (r*k + s)*C' + c
-//   A[m][kk] = x[n][ho*st + r - p][wo*st + s - p][c]   (zero outside the image)
-//   B[f][kk] = w[f][o + r][o + s][c]                   (stored [Kmax][R][R][Cmax], o = (R-k)/2)
-// 64 x 64 output tile per block, 16-wide k chunks, 4 x 4 outputs per thread.
-// ---------------------------------------------------------------------------------------------
-constexpr int PT_M = 64, PT_N = 64, PT_K = 16;
-
-template <typename T>
-__global__ void __launch_bounds__(256) conv_plain_kernel(ConvArgs a) {
-    __shared__ float As[PT_K][PT_M + 4];
-    __shared__ float Bs[PT_K][PT_N + 4];
-    const T *__restrict__ x = static_cast<const T *>(a.x);
-    const T *__restrict__ w = static_cast<const T *>(a.w);
-    const int M = a.N * a.Ho * a.Wo;
-    const int KK = a.k * a.k * a.C;
-    const int p = (a.k - 1) / 2, o = (a.R - a.k) / 2;
-    const int m0 = blockIdx.x * PT_M, f0 = blockIdx.y * PT_N;
-    const int t = threadIdx.x;
-    const int lk = t % PT_K, lrow = t / PT_K;  // loader coordinates
-    const int tx = t % 16, ty = t / 16;        // compute coordinates
-
-    // decode the four pixels this thread loads
-    int pn[4], ph[4], pw[4];
-    bool pv[4];
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-        int m = m0 + lrow + 16 * j;
-        pv[j] = m < M;
-        int mm = pv[j] ? m : 0;
-        pw[j] = mm % a.Wo;
-        ph[j] = (mm / a.Wo) % a.Ho;
-        pn[j] = mm / (a.Wo * a.Ho);
-    }
-    float acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; i++)
-#pragma unroll
-        for (int j = 0; j < 4; j++) acc[i][j] = 0.f;
-
-    for (int kk0 = 0; kk0 < KK; kk0 += PT_K) {
-        const int kk = kk0 + lk;
-        const bool kv = kk < KK;
-        int c = 0, r = 0, s = 0;
-        if (kv) {
-            c = kk % a.C;
-            int rs = kk / a.C;
-            s = rs % a.k;
-            r = rs / a.k;
-        }
-#pragma unroll
-        for (int j = 0; j < 4; j++) {
-            float v = 0.f;
-            if (kv && pv[j]) {
-                int hi = ph[j] * a.stride + r - p, wi = pw[j] * a.stride + s - p;
-                if (hi >= 0 && hi < a.H && wi >= 0 && wi < a.W)
-                    v = to_f<T>(x[(((size_t)pn[j] * a.H + hi) * a.W + wi) * a.C + c]);
-            }
-            As[lk][lrow + 16 * j] = v;
-        }
-#pragma unroll
-        for (int j = 0; j < 4; j++) {
-            int f = f0 + lrow + 16 * j;
-            float v = 0.f;
-            if (kv && f < a.K) v = to_f<T>(w[(((size_t)f * a.R + (o + r)) * a.R + (o + s)) * a.Cmax + c]);
-            Bs[lk][lrow + 16 * j] = v;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < PT_K; q++) {
-            float av[4], bv[4];
-#pragma unroll
-            for (int i = 0; i < 4; i++) av[i] = As[q][ty * 4 + i];
-#pragma unroll
-            for (int j = 0; j < 4; j++) bv[j] = Bs[q][tx * 4 + j];
-#pragma unroll
-            for (int i = 0; i < 4; i++)
-#pragma unroll
-                for (int j = 0; j < 4; j++) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-    const T *__restrict__ res = static_cast<const T *>(a.res);
-    T *__restrict__ y = static_cast<T *>(a.y);
-#pragma unroll
-    for (int i = 0; i < 4; i++) {
-        int m = m0 + ty * 4 + i;
-        if (m >= M) continue;
-#pragma unroll
-        for (int j = 0; j < 4; j++) {
-            int f = f0 + tx * 4 + j;
-            if (f >= a.K) continue;
-            float v = acc[i][j] * a.scale[f] + a.shift[f];
-            size_t oi = (size_t)m * a.K + f;
-            if (res) v += to_f<T>(res[oi]);
-            y[oi] = from_f<T>(apply_act(v, a.act));
-        }
-    }
-}
-
-template <typename T> cudaError_t launch_conv_plain(const ConvArgs &a, cudaStream_t st) {
-    int M = a.N * a.Ho * a.Wo;
-    if (M <= 0 || a.K <= 0) return cudaSuccess;
-    dim3 grid((M + PT_M - 1) / PT_M, (a.K + PT_N - 1) / PT_N);
-    conv_plain_kernel<T><<<grid, 256, 0, st>>>(a);
-    return cudaGetLastError();
-}
-template cudaError_t launch_conv_plain<float>(const ConvArgs &, cudaStream_t);
-template cudaError_t launch_conv_plain<__nv_bfloat16>(const ConvArgs &, cudaStream_t);
-
-// ---------------------------------------------------------------------------------------------
 // Depthwise k x k convolution, kernel = centre window of the stored R x R kernel, weights
 // [R][R][Kmax].  One thread per (pixel, channel), channels fastest (coalesced NHWC).
 // ---------------------------------------------------------------------------------------------

@@ -4,6 +4,7 @@
 #pragma once
 
 #include "sgs_internal.h"
+#include "sgs_pdl.cuh"
 
 namespace sgs {
 
@@ -125,11 +126,6 @@ __device__ __forceinline__ bool elect_one() {
         : "=r"(pred));
     return pred != 0;
 }
-// Programmatic dependent launch: wait() returns once the grids this one depends on have completed and
-// their writes are visible; launch_dependents() lets the next grid in the stream start its own prologue
-// early.  Both are no-ops for a grid that was launched without the attribute.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void tmem_alloc(uint32_t *dst_smem, uint32_t cols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)), "r"(cols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
