@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
 #pragma unroll
                     for (int g = 0; g < 4; g++) {
                         const int c = c0 + 8 * g;
-                        rv[g] = (res && m >= 0 && c < cend) ? __ldg(reinterpret_cast<const uint4 *>(res + obase + c)) : make_uint4(0u, 0u, 0u, 0u);
+                        rv[g] = (res && m >= 0 && c < cend) ? ld_act(reinterpret_cast<const uint4 *>(res + obase + c)) : make_uint4(0u, 0u, 0u, 0u);
                     }
                 };
                 uint4 rv[4], rn[4];
@@ -398,8 +398,8 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
                     for (int q = 0; q < 16; q++) {
                         const int p0 = c0 + 2 * q;
                         uint32_t lo = 0, hi = 0;
-                        if (res && fvalid && p0 < cend) lo = __ldg(resu + (size_t)p0 * ldk + f);
-                        if (res && fvalid && p0 + 1 < cend) hi = __ldg(resu + (size_t)(p0 + 1) * ldk + f);
+                        if (res && fvalid && p0 < cend) lo = ld_act(resu + (size_t)p0 * ldk + f);
+                        if (res && fvalid && p0 + 1 < cend) hi = ld_act(resu + (size_t)(p0 + 1) * ldk + f);
                         rv[q] = lo | (hi << 16);
                     }
                 };

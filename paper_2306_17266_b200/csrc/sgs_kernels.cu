@@ -1,15 +1,20 @@
-// Plain CUDA-core kernels: sliced convolution (shared-memory implicit GEMM in fp32), depthwise
-// convolution with centre-cropped kernels, pooling, squeeze-excite, linear layers, and the
-// load-time re-layout / batch-norm folding kernels.
-//
-// These are the complete path in fp32 mode and, in bf16 mode, serve the layers the tensor-core
-// kernel does not take (3-channel stems, channel counts that are not multiples of 8).
+// CUDA-core kernels other than the convolution (sgs_conv_simt.cu): depthwise convolution with centre-cropped
+// kernels, pooling, squeeze-excite, linear layers, and the load-time re-layout / batch-norm folding kernels.
 #include "sgs_internal.h"
+#include "sgs_pdl.cuh"
 
 #include <algorithm>
 #include <cooperative_groups.h>
 
 namespace sgs {
+
+// Launch that may overlap the tail of the previous kernel of the stream: most kernels here last 2 to 5 us, of which the
+// launch gap was 1 to 2.  The kernels wait (pdl_wait) before they touch what earlier kernels write.
+#define SGS_LAUNCH(kernel, grid, block, smem, st, ...)                                    \
+    do {                                                                                  \
+        const cudaError_t e_ = launch_pdl(kernel, grid, block, smem, st, 1u, __VA_ARGS__); \
+        if (e_ != cudaSuccess) return e_;                                                 \
+    } while (0)
 
 template <typename T> __device__ __forceinline__ float to_f(T v);
 template <> __device__ __forceinline__ float to_f<float>(float v) { return v; }
@@ -30,9 +35,11 @@ __device__ __forceinline__ float apply_act(float v, int act) {
 // ---------------------------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(256) dw_plain_kernel(ConvArgs a) {
-    const T *__restrict__ x = static_cast<const T *>(a.x);
-    const T *__restrict__ w = static_cast<const T *>(a.w);
-    T *__restrict__ y = static_cast<T *>(a.y);
+    pdl_launch_dependents();
+    pdl_wait();
+    const T *x = static_cast<const T *>(a.x);
+    const T *w = static_cast<const T *>(a.w);
+    T *y = static_cast<T *>(a.y);
     const size_t total = (size_t)a.N * a.Ho * a.Wo * a.K;
     const int p = (a.k - 1) / 2, o = (a.R - a.k) / 2;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
@@ -46,7 +53,7 @@ __global__ void __launch_bounds__(256) dw_plain_kernel(ConvArgs a) {
             for (int s = 0; s < a.k; s++) {
                 int wi = wo * a.stride + s - p;
                 if (wi < 0 || wi >= a.W) continue;
-                acc = fmaf(to_f<T>(x[(((size_t)n * a.H + hi) * a.W + wi) * a.K + c]),
+                acc = fmaf(to_f<T>(ld_act(x + (((size_t)n * a.H + hi) * a.W + wi) * a.K + c)),
                            to_f<T>(w[((size_t)(o + r) * a.R + (o + s)) * a.Kmax + c]), acc);
             }
         }
@@ -73,6 +80,7 @@ __device__ __forceinline__ float2 bf2_lo(uint32_t u) { return make_float2(__uint
         __syncthreads();                                                                                       \
     }                                                                                                          \
     const ConvArgs &a = GROUP ? *reinterpret_cast<const ConvArgs *>(a_raw_) : a1;                              \
+    if (!a.early_weights) pdl_wait();                                                                          \
     const int n = GROUP ? (int)(blockIdx.z % n_img) : (int)blockIdx.z;
 static_assert(sizeof(ConvArgs) % 4 == 0 && sizeof(ConvArgs) <= DW_ENTRY_BYTES, "depthwise table record");
 
@@ -87,7 +95,7 @@ __device__ __forceinline__ void dw_vec_body(const ConvArgs &a, const int n) {
     const int cg = idx % groups, wb = idx / groups;
     const int ho = blockIdx.y;
     const int c0 = cg * 8, wo0 = wb * TW, o = (a.R - K) / 2;
-    const __nv_bfloat16 *__restrict__ x = static_cast<const __nv_bfloat16 *>(a.x);
+    const __nv_bfloat16 *x = static_cast<const __nv_bfloat16 *>(a.x);
     const __nv_bfloat16 *__restrict__ w = static_cast<const __nv_bfloat16 *>(a.w);
 
     float2 acc[TW][4];
@@ -97,6 +105,7 @@ __device__ __forceinline__ void dw_vec_body(const ConvArgs &a, const int n) {
         for (int j = 0; j < 4; j++) acc[t][j] = make_float2(0.f, 0.f);
 
     const __nv_bfloat16 *ximg = x + ((size_t)n * a.H) * a.W * a.K + c0;
+    pdl_wait();
 #pragma unroll
     for (int r = 0; r < K; r++) {
         const int hi = ho * ST + r - P;
@@ -106,7 +115,7 @@ __device__ __forceinline__ void dw_vec_body(const ConvArgs &a, const int n) {
 #pragma unroll
         for (int j = 0; j < NCOL; j++) {
             const int wi = wo0 * ST + j - P;
-            col[j] = (wi >= 0 && wi < a.W) ? __ldg(reinterpret_cast<const uint4 *>(xrow + wi * a.K)) : make_uint4(0u, 0u, 0u, 0u);
+            col[j] = (wi >= 0 && wi < a.W) ? ld_act(reinterpret_cast<const uint4 *>(xrow + wi * a.K)) : make_uint4(0u, 0u, 0u, 0u);
         }
         const __nv_bfloat16 *wrow = w + ((o + r) * a.R + o) * a.Kmax + c0;
 #pragma unroll
@@ -141,6 +150,7 @@ __device__ __forceinline__ void dw_vec_body(const ConvArgs &a, const int n) {
 }
 template <int K, int ST, bool GROUP>
 __global__ void __launch_bounds__(256) dw_vec_kernel(const ConvArgs a1, const char *__restrict__ tbl, int n_img) {
+    pdl_launch_dependents();
     SGS_DW_ARGS()
     dw_vec_body<K, ST>(a, n);
 }
@@ -162,7 +172,7 @@ __device__ __forceinline__ void dw_tile_body(const ConvArgs &a, const int n) {
     const int cg = idx % groups, wb = idx / groups;
     const int ho0 = blockIdx.y * TH;
     const int c0 = cg * 8, wo0 = wb * TW, o = (a.R - K) / 2;
-    const __nv_bfloat16 *__restrict__ x = static_cast<const __nv_bfloat16 *>(a.x);
+    const __nv_bfloat16 *x = static_cast<const __nv_bfloat16 *>(a.x);
     const __nv_bfloat16 *__restrict__ w = static_cast<const __nv_bfloat16 *>(a.w);
 
     // weights stay packed in registers and are unpacked at use
@@ -194,6 +204,7 @@ __device__ __forceinline__ void dw_tile_body(const ConvArgs &a, const int n) {
     const int wi0 = wo0 * ST - P, hi0 = ho0 * ST - P;
     const bool interior = hi0 >= 0 && hi0 + NROW <= a.H && wi0 >= 0 && wi0 + NCOL <= a.W;
     uint4 raw[PRELOAD ? NROW : 1][NCOL];
+    pdl_wait();  // (the filters above do not depend on the previous layer)
     if (PRELOAD) {
 #pragma unroll
         for (int ir = 0; ir < NROW; ir++) {
@@ -203,7 +214,7 @@ __device__ __forceinline__ void dw_tile_body(const ConvArgs &a, const int n) {
 #pragma unroll
             for (int j = 0; j < NCOL; j++) {
                 const int wi = wi0 + j;
-                raw[PRELOAD ? ir : 0][j] = (rok && wi >= 0 && wi < a.W) ? __ldg(reinterpret_cast<const uint4 *>(xrow + wi * a.K)) : make_uint4(0u, 0u, 0u, 0u);
+                raw[PRELOAD ? ir : 0][j] = (rok && wi >= 0 && wi < a.W) ? ld_act(reinterpret_cast<const uint4 *>(xrow + wi * a.K)) : make_uint4(0u, 0u, 0u, 0u);
             }
         }
     }
@@ -218,8 +229,8 @@ __device__ __forceinline__ void dw_tile_body(const ConvArgs &a, const int n) {
             const int wi = wi0 + j;
             uint4 v;
             if (PRELOAD) v = raw[PRELOAD ? ir : 0][j];
-            else if (interior) v = __ldg(reinterpret_cast<const uint4 *>(xrow + wi * a.K));
-            else v = (wi >= 0 && wi < a.W) ? __ldg(reinterpret_cast<const uint4 *>(xrow + wi * a.K)) : make_uint4(0u, 0u, 0u, 0u);
+            else if (interior) v = ld_act(reinterpret_cast<const uint4 *>(xrow + wi * a.K));
+            else v = (wi >= 0 && wi < a.W) ? ld_act(reinterpret_cast<const uint4 *>(xrow + wi * a.K)) : make_uint4(0u, 0u, 0u, 0u);
             xc[j][0] = bf2_lo(v.x); xc[j][1] = bf2_lo(v.y); xc[j][2] = bf2_lo(v.z); xc[j][3] = bf2_lo(v.w);
         }
 #pragma unroll
@@ -277,6 +288,7 @@ __device__ __forceinline__ void dw_tile_body(const ConvArgs &a, const int n) {
 }
 template <int K, int ST, int TH, int TW, bool PRELOAD, int ACT, bool GROUP>
 __global__ void __launch_bounds__(128) dw_tile_kernel(const ConvArgs a1, const char *__restrict__ tbl, int n_img) {
+    pdl_launch_dependents();
     SGS_DW_ARGS()
     if (GROUP) { const ConvArgs al = a; dw_tile_body<K, ST, TH, TW, PRELOAD, ACT>(al, n); }  // (register copy, see dw_mixed_kernel)
     else dw_tile_body<K, ST, TH, TW, PRELOAD, ACT>(a, n);
@@ -377,6 +389,7 @@ __device__ __forceinline__ void dw_walk_body(const ConvArgs &a, const int n, uns
         }
         cp_async_commit();  // (a group per row, also when it is empty: the wait below counts groups)
     };
+    pdl_wait();  // (the filters above do not depend on the previous layer)
 #pragma unroll 1
     for (int d = 0; d < RING - 1; d++) copy_row(hi_first + d);
 
@@ -448,6 +461,7 @@ __device__ __forceinline__ void dw_walk_body(const ConvArgs &a, const int n, uns
 }
 template <int K, int ACT, bool GROUP>
 __global__ void __launch_bounds__(128, K == 7 ? 3 : 4) dw_walk_kernel(const ConvArgs a1, const char *__restrict__ tbl, int n_img, int chblocks) {
+    pdl_launch_dependents();
     __shared__ __align__(16) unsigned char smem[DwWalkShape<K>::SMEM];
     SGS_DW_ARGS()
     if (GROUP) { const ConvArgs al = a; dw_walk_body<K, ACT>(al, n, smem, chblocks); }
@@ -467,6 +481,7 @@ static dim3 dw_walk_grid(const ConvArgs &a, int kmax, int TW, int images) {
 template <int ST, int ACT, bool WALK> __device__ __forceinline__ void dw_mixed_dispatch(const ConvArgs &a, const int n, unsigned char *wsm, int chblocks);
 template <int ST, int ACT, bool WALK>
 __global__ void __launch_bounds__(128, 3) dw_mixed_kernel(const char *__restrict__ tbl, int n_img, int chblocks) {
+    pdl_launch_dependents();
     constexpr bool GROUP = true;
     __shared__ __align__(16) unsigned char wsm[WALK ? DwWalkShape<7>::SMEM : 16];  // (7x7 needs the most; 5x5: 37376, 3x3: 41472 bytes)
     static_assert(DwWalkShape<7>::SMEM >= DwWalkShape<5>::SMEM && DwWalkShape<7>::SMEM >= DwWalkShape<3>::SMEM && DwWalkShape<7>::SMEM <= 48 * 1024, "ring sizes");
@@ -497,9 +512,9 @@ template <int K, int ST, int TH, int TW, bool PRELOAD, bool GROUP>
 static cudaError_t launch_dw_tile(const ConvArgs &a, int kmax, const char *tbl, int members, cudaStream_t st) {
     const int per_row = ((a.Wo + TW - 1) / TW) * (kmax / 8);
     dim3 grid((per_row + 127) / 128, (a.Ho + TH - 1) / TH, a.N * (GROUP ? members : 1));
-    if (a.act == ACT_RELU) dw_tile_kernel<K, ST, TH, TW, PRELOAD, ACT_RELU, GROUP><<<grid, 128, 0, st>>>(a, tbl, a.N);
-    else if (a.act == ACT_HSWISH) dw_tile_kernel<K, ST, TH, TW, PRELOAD, ACT_HSWISH, GROUP><<<grid, 128, 0, st>>>(a, tbl, a.N);
-    else dw_tile_kernel<K, ST, TH, TW, PRELOAD, ACT_NONE, GROUP><<<grid, 128, 0, st>>>(a, tbl, a.N);
+    if (a.act == ACT_RELU) SGS_LAUNCH((dw_tile_kernel<K, ST, TH, TW, PRELOAD, ACT_RELU, GROUP>), grid, dim3(128), 0, st, a, tbl, a.N);
+    else if (a.act == ACT_HSWISH) SGS_LAUNCH((dw_tile_kernel<K, ST, TH, TW, PRELOAD, ACT_HSWISH, GROUP>), grid, dim3(128), 0, st, a, tbl, a.N);
+    else SGS_LAUNCH((dw_tile_kernel<K, ST, TH, TW, PRELOAD, ACT_NONE, GROUP>), grid, dim3(128), 0, st, a, tbl, a.N);
     return cudaGetLastError();
 }
 
@@ -507,9 +522,9 @@ template <int K, bool GROUP>
 static cudaError_t launch_dw_walk(const ConvArgs &a, int kmax, const char *tbl, int members, cudaStream_t st) {
     const dim3 grid = dw_walk_grid(a, kmax, DwWalkShape<K>::TW, a.N * (GROUP ? members : 1));
     const int chblocks = (kmax / 4 + 31) / 32;
-    if (a.act == ACT_RELU) dw_walk_kernel<K, ACT_RELU, GROUP><<<grid, 128, 0, st>>>(a, tbl, a.N, chblocks);
-    else if (a.act == ACT_HSWISH) dw_walk_kernel<K, ACT_HSWISH, GROUP><<<grid, 128, 0, st>>>(a, tbl, a.N, chblocks);
-    else dw_walk_kernel<K, ACT_NONE, GROUP><<<grid, 128, 0, st>>>(a, tbl, a.N, chblocks);
+    if (a.act == ACT_RELU) SGS_LAUNCH((dw_walk_kernel<K, ACT_RELU, GROUP>), grid, dim3(128), 0, st, a, tbl, a.N, chblocks);
+    else if (a.act == ACT_HSWISH) SGS_LAUNCH((dw_walk_kernel<K, ACT_HSWISH, GROUP>), grid, dim3(128), 0, st, a, tbl, a.N, chblocks);
+    else SGS_LAUNCH((dw_walk_kernel<K, ACT_NONE, GROUP>), grid, dim3(128), 0, st, a, tbl, a.N, chblocks);
     return cudaGetLastError();
 }
 
@@ -518,7 +533,7 @@ static cudaError_t launch_dw_vec(const ConvArgs &a, int kmax, const char *tbl, i
     const int per_row = ((a.Wo + 3) / 4) * (kmax / 8);
     const int block = per_row >= 256 ? 256 : per_row >= 128 ? 128 : 64;
     dim3 grid((per_row + block - 1) / block, a.Ho, a.N * (GROUP ? members : 1));
-    dw_vec_kernel<K, ST, GROUP><<<grid, block, 0, st>>>(a, tbl, a.N);
+    SGS_LAUNCH((dw_vec_kernel<K, ST, GROUP>), grid, block, 0, st, a, tbl, a.N);
     return cudaGetLastError();
 }
 
@@ -577,21 +592,21 @@ cudaError_t launch_dw_group(const char *h_tbl, const char *d_tbl, int members, c
     const int chblocks = (kmax / 4 + 31) / 32;
     if (a0.stride == 1 && dw_walks(a0, kmax, members)) {
         const dim3 grid = dw_walk_grid(a0, kmax, 2, a0.N * members);
-        if (a0.act == ACT_RELU) dw_mixed_kernel<1, ACT_RELU, true><<<grid, 128, 0, st>>>(d_tbl, a0.N, chblocks);
-        else if (a0.act == ACT_HSWISH) dw_mixed_kernel<1, ACT_HSWISH, true><<<grid, 128, 0, st>>>(d_tbl, a0.N, chblocks);
-        else dw_mixed_kernel<1, ACT_NONE, true><<<grid, 128, 0, st>>>(d_tbl, a0.N, chblocks);
+        if (a0.act == ACT_RELU) SGS_LAUNCH((dw_mixed_kernel<1, ACT_RELU, true>), grid, dim3(128), 0, st, d_tbl, a0.N, chblocks);
+        else if (a0.act == ACT_HSWISH) SGS_LAUNCH((dw_mixed_kernel<1, ACT_HSWISH, true>), grid, dim3(128), 0, st, d_tbl, a0.N, chblocks);
+        else SGS_LAUNCH((dw_mixed_kernel<1, ACT_NONE, true>), grid, dim3(128), 0, st, d_tbl, a0.N, chblocks);
     } else if (a0.stride == 1) {
         // (the patch bodies of 3x3 and 5x5 own 2 resp. 1 output rows per block row: the grid covers single rows,
         // blocks beyond a member's own extent leave at once)
         dim3 grid((per_row + 127) / 128, a0.Ho, a0.N * members);
-        if (a0.act == ACT_RELU) dw_mixed_kernel<1, ACT_RELU, false><<<grid, 128, 0, st>>>(d_tbl, a0.N, chblocks);
-        else if (a0.act == ACT_HSWISH) dw_mixed_kernel<1, ACT_HSWISH, false><<<grid, 128, 0, st>>>(d_tbl, a0.N, chblocks);
-        else dw_mixed_kernel<1, ACT_NONE, false><<<grid, 128, 0, st>>>(d_tbl, a0.N, chblocks);
+        if (a0.act == ACT_RELU) SGS_LAUNCH((dw_mixed_kernel<1, ACT_RELU, false>), grid, dim3(128), 0, st, d_tbl, a0.N, chblocks);
+        else if (a0.act == ACT_HSWISH) SGS_LAUNCH((dw_mixed_kernel<1, ACT_HSWISH, false>), grid, dim3(128), 0, st, d_tbl, a0.N, chblocks);
+        else SGS_LAUNCH((dw_mixed_kernel<1, ACT_NONE, false>), grid, dim3(128), 0, st, d_tbl, a0.N, chblocks);
     } else {
         dim3 grid((per_row + 127) / 128, a0.Ho, a0.N * members);
-        if (a0.act == ACT_RELU) dw_mixed_kernel<2, ACT_RELU, false><<<grid, 128, 0, st>>>(d_tbl, a0.N, chblocks);
-        else if (a0.act == ACT_HSWISH) dw_mixed_kernel<2, ACT_HSWISH, false><<<grid, 128, 0, st>>>(d_tbl, a0.N, chblocks);
-        else dw_mixed_kernel<2, ACT_NONE, false><<<grid, 128, 0, st>>>(d_tbl, a0.N, chblocks);
+        if (a0.act == ACT_RELU) SGS_LAUNCH((dw_mixed_kernel<2, ACT_RELU, false>), grid, dim3(128), 0, st, d_tbl, a0.N, chblocks);
+        else if (a0.act == ACT_HSWISH) SGS_LAUNCH((dw_mixed_kernel<2, ACT_HSWISH, false>), grid, dim3(128), 0, st, d_tbl, a0.N, chblocks);
+        else SGS_LAUNCH((dw_mixed_kernel<2, ACT_NONE, false>), grid, dim3(128), 0, st, d_tbl, a0.N, chblocks);
     }
     return cudaGetLastError();
 }
@@ -604,7 +619,7 @@ template <typename T> cudaError_t launch_dw(const ConvArgs &a, cudaStream_t st) 
         if (e != cudaErrorNotSupported) return e;
     }
     int blocks = (int)std::min<size_t>((total + 255) / 256, 148 * 16);
-    dw_plain_kernel<T><<<blocks, 256, 0, st>>>(a);
+    SGS_LAUNCH((dw_plain_kernel<T>), dim3(blocks), dim3(256), 0, st, a);
     return cudaGetLastError();
 }
 template cudaError_t launch_dw<float>(const ConvArgs &, cudaStream_t);
@@ -614,7 +629,9 @@ template cudaError_t launch_dw<__nv_bfloat16>(const ConvArgs &, cudaStream_t);
 // 3x3 stride-2 max pool, padding 1 (only in-image taps compared)
 // ---------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void maxpool_kernel(const T *__restrict__ x, T *__restrict__ y, int N, int H, int W, int C, int Ho, int Wo) {
+__global__ void maxpool_kernel(const T *x, T *y, int N, int H, int W, int C, int Ho, int Wo) {
+    pdl_launch_dependents();
+    pdl_wait();
     size_t total = (size_t)N * Ho * Wo * C;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         int c = (int)(i % C);
@@ -627,7 +644,7 @@ __global__ void maxpool_kernel(const T *__restrict__ x, T *__restrict__ y, int N
             for (int s = 0; s < 3; s++) {
                 int wi = 2 * wo + s - 1;
                 if (wi < 0 || wi >= W) continue;
-                best = fmaxf(best, to_f<T>(x[(((size_t)n * H + hi) * W + wi) * C + c]));
+                best = fmaxf(best, to_f<T>(ld_act(x + (((size_t)n * H + hi) * W + wi) * C + c)));
             }
         }
         y[i] = from_f<T>(best);
@@ -638,7 +655,7 @@ template <typename T> cudaError_t launch_maxpool3s2(const T *x, T *y, int N, int
     size_t total = (size_t)N * Ho * Wo * C;
     if (!total) return cudaSuccess;
     int blocks = (int)std::min<size_t>((total + 255) / 256, 148 * 16);
-    maxpool_kernel<T><<<blocks, 256, 0, st>>>(x, y, N, H, W, C, Ho, Wo);
+    SGS_LAUNCH((maxpool_kernel<T>), dim3(blocks), dim3(256), 0, st, x, y, N, H, W, C, Ho, Wo);
     return cudaGetLastError();
 }
 template cudaError_t launch_maxpool3s2<float>(const float *, float *, int, int, int, int, cudaStream_t);
@@ -649,12 +666,14 @@ template cudaError_t launch_maxpool3s2<__nv_bfloat16>(const __nv_bfloat16 *, __n
 // grid (ceil(C/32), N), block (32, 8): 8 pixel lanes per channel, reduced through shared memory.
 // ---------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void gap_kernel(const T *__restrict__ x, float *__restrict__ g, int HW, int C) {
+__global__ void gap_kernel(const T *x, float *g, int HW, int C) {
+    pdl_launch_dependents();
+    pdl_wait();
     __shared__ float part[8][33];
     int c = blockIdx.x * 32 + threadIdx.x, n = blockIdx.y;
     float s = 0.f;
     if (c < C)
-        for (int i = threadIdx.y; i < HW; i += 8) s += to_f<T>(x[((size_t)n * HW + i) * C + c]);
+        for (int i = threadIdx.y; i < HW; i += 8) s += to_f<T>(ld_act(x + ((size_t)n * HW + i) * C + c));
     part[threadIdx.y][threadIdx.x] = s;
     __syncthreads();
     if (threadIdx.y == 0 && c < C) {
@@ -668,7 +687,9 @@ __global__ void gap_kernel(const T *__restrict__ x, float *__restrict__ g, int H
 // loads and the lane sums are combined by a fixed shuffle tree (same result every run).
 __device__ __forceinline__ float2 bf2f(uint32_t u) { return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u)); }
 
-__global__ void __launch_bounds__(256) gap_vec_kernel(const __nv_bfloat16 *__restrict__ x, float *__restrict__ g, int N, int HW, int C) {
+__global__ void __launch_bounds__(256) gap_vec_kernel(const __nv_bfloat16 *x, float *g, int N, int HW, int C) {
+    pdl_launch_dependents();
+    pdl_wait();
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     const int cvecs = C >> 3;
     if (warp >= N * cvecs) return;
@@ -676,7 +697,7 @@ __global__ void __launch_bounds__(256) gap_vec_kernel(const __nv_bfloat16 *__res
     const __nv_bfloat16 *base = x + (size_t)n * HW * C + cv * 8;
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     for (int i = lane; i < HW; i += 32) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(base + (size_t)i * C));
+        const uint4 v = ld_act(reinterpret_cast<const uint4 *>(base + (size_t)i * C));
         const float2 a = bf2f(v.x), b = bf2f(v.y), c = bf2f(v.z), d = bf2f(v.w);
         acc[0] += a.x; acc[1] += a.y; acc[2] += b.x; acc[3] += b.y; acc[4] += c.x; acc[5] += c.y; acc[6] += d.x; acc[7] += d.y;
     }
@@ -696,11 +717,11 @@ template <typename T> cudaError_t launch_gap(const T *x, float *g, int N, int HW
     if (N <= 0 || C <= 0) return cudaSuccess;
     if (sizeof(T) == 2 && C % 8 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0 && (reinterpret_cast<uintptr_t>(g) & 15) == 0) {
         const int warps = N * (C / 8);
-        gap_vec_kernel<<<(warps * 32 + 255) / 256, 256, 0, st>>>(reinterpret_cast<const __nv_bfloat16 *>(x), g, N, HW, C);
+        SGS_LAUNCH(gap_vec_kernel, dim3((warps * 32 + 255) / 256), dim3(256), 0, st, reinterpret_cast<const __nv_bfloat16 *>(x), g, N, HW, C);
         return cudaGetLastError();
     }
     dim3 grid((C + 31) / 32, N), block(32, 8);
-    gap_kernel<T><<<grid, block, 0, st>>>(x, g, HW, C);
+    SGS_LAUNCH((gap_kernel<T>), grid, block, 0, st, x, g, HW, C);
     return cudaGetLastError();
 }
 template cudaError_t launch_gap<float>(const float *, float *, int, int, int, cudaStream_t);
@@ -711,14 +732,16 @@ template cudaError_t launch_gap<__nv_bfloat16>(const __nv_bfloat16 *, float *, i
 // One block per image; warps stride over outputs and reduce with shuffles.
 // ---------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(1024) se_gate_kernel(const float *__restrict__ g, const T *__restrict__ w1,
+__global__ void __launch_bounds__(1024) se_gate_kernel(const float *g, const T *__restrict__ w1,
                                                       const float *__restrict__ b1, const T *__restrict__ w2,
-                                                      const float *__restrict__ b2, float *__restrict__ gate, int mid,
+                                                      const float *__restrict__ b2, float *gate, int mid,
                                                       int sq, int w1_ld, int w2_ld) {
+    pdl_launch_dependents();
+    pdl_wait();
     extern __shared__ float sm[];
     float *gs = sm, *zs = sm + mid;
     int n = blockIdx.x, lane = threadIdx.x % 32, warp = threadIdx.x / 32, nw = blockDim.x / 32;
-    for (int c = threadIdx.x; c < mid; c += blockDim.x) gs[c] = g[(size_t)n * mid + c];
+    for (int c = threadIdx.x; c < mid; c += blockDim.x) gs[c] = ld_act(g + (size_t)n * mid + c);
     __syncthreads();
     for (int j = warp; j < sq; j += nw) {
         float s = 0.f;
@@ -740,7 +763,7 @@ template <typename T>
 cudaError_t launch_se_gate(const float *g, const T *w1, const float *b1, const T *w2, const float *b2, float *gate,
                            int N, int mid, int sq, int w1_ld, int w2_ld, cudaStream_t st) {
     if (N <= 0) return cudaSuccess;
-    se_gate_kernel<T><<<N, 1024, (size_t)(mid + sq) * sizeof(float), st>>>(g, w1, b1, w2, b2, gate, mid, sq, w1_ld, w2_ld);
+    SGS_LAUNCH((se_gate_kernel<T>), dim3(N), dim3(1024), (size_t)(mid + sq) * sizeof(float), st, g, w1, b1, w2, b2, gate, mid, sq, w1_ld, w2_ld);
     return cudaGetLastError();
 }
 template cudaError_t launch_se_gate<float>(const float *, const float *, const float *, const float *, const float *, float *, int, int, int, int, int, cudaStream_t);
@@ -748,22 +771,26 @@ template cudaError_t launch_se_gate<__nv_bfloat16>(const float *, const __nv_bfl
 
 // y[n][hw][c] = x[n][hw][c] * gate[n][c]
 template <typename T>
-__global__ void scale_kernel(const T *__restrict__ x, const float *__restrict__ gate, T *__restrict__ y, size_t total,
+__global__ void scale_kernel(const T *x, const float *gate, T *y, size_t total,
                              int HW, int C) {
+    pdl_launch_dependents();
+    pdl_wait();
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         int c = (int)(i % C);
         size_t n = i / ((size_t)HW * C);
-        y[i] = from_f<T>(to_f<T>(x[i]) * gate[n * C + c]);
+        y[i] = from_f<T>(to_f<T>(ld_act(x + i)) * ld_act(gate + n * C + c));
     }
 }
-__global__ void __launch_bounds__(256) scale_vec_kernel(const __nv_bfloat16 *__restrict__ x, const float *__restrict__ gate,
-                                                        __nv_bfloat16 *__restrict__ y, int vecs_per_image, int cvecs, int C, int total) {
+__global__ void __launch_bounds__(256) scale_vec_kernel(const __nv_bfloat16 *x, const float *gate,
+                                                        __nv_bfloat16 *y, int vecs_per_image, int cvecs, int C, int total) {
+    pdl_launch_dependents();
+    pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;  // one 8-channel vector
     if (i >= total) return;
     const int n = i / vecs_per_image, cv = i % cvecs;
-    const uint4 v = *reinterpret_cast<const uint4 *>(x + (size_t)i * 8);
-    const float4 g0 = __ldg(reinterpret_cast<const float4 *>(gate + (size_t)n * C + cv * 8));
-    const float4 g1 = __ldg(reinterpret_cast<const float4 *>(gate + (size_t)n * C + cv * 8 + 4));
+    const uint4 v = ld_act(reinterpret_cast<const uint4 *>(x + (size_t)i * 8));
+    const float4 g0 = ld_act(reinterpret_cast<const float4 *>(gate + (size_t)n * C + cv * 8));
+    const float4 g1 = ld_act(reinterpret_cast<const float4 *>(gate + (size_t)n * C + cv * 8 + 4));
     const float2 a = bf2f(v.x), b = bf2f(v.y), c = bf2f(v.z), d = bf2f(v.w);
     uint4 o;
     __nv_bfloat162 *ob = reinterpret_cast<__nv_bfloat162 *>(&o);
@@ -780,12 +807,11 @@ template <typename T> cudaError_t launch_scale(const T *x, const float *gate, T 
     if (sizeof(T) == 2 && C % 8 == 0 && total / 8 < (1u << 30) &&
         ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y) | reinterpret_cast<uintptr_t>(gate)) & 15) == 0) {
         const int tv = (int)(total / 8);
-        scale_vec_kernel<<<(tv + 255) / 256, 256, 0, st>>>(reinterpret_cast<const __nv_bfloat16 *>(x), gate,
-                                                          reinterpret_cast<__nv_bfloat16 *>(y), HW * (C / 8), C / 8, C, tv);
+        SGS_LAUNCH(scale_vec_kernel, dim3((tv + 255) / 256), dim3(256), 0, st, reinterpret_cast<const __nv_bfloat16 *>(x), gate, reinterpret_cast<__nv_bfloat16 *>(y), HW * (C / 8), C / 8, C, tv);
         return cudaGetLastError();
     }
     int blocks = (int)std::min<size_t>((total + 255) / 256, 148 * 16);
-    scale_kernel<T><<<blocks, 256, 0, st>>>(x, gate, y, total, HW, C);
+    SGS_LAUNCH((scale_kernel<T>), dim3(blocks), dim3(256), 0, st, x, gate, y, total, HW, C);
     return cudaGetLastError();
 }
 template cudaError_t launch_scale<float>(const float *, const float *, float *, int, int, int, cudaStream_t);
@@ -796,22 +822,26 @@ template cudaError_t launch_scale<__nv_bfloat16>(const __nv_bfloat16 *, const fl
 // One warp per (n, j).
 // ---------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(256) linear_kernel(const float *__restrict__ v, const T *__restrict__ w,
-                                                     const float *__restrict__ bias, float *__restrict__ y, int N,
+__global__ void __launch_bounds__(256) linear_kernel(const float *v, const T *__restrict__ w,
+                                                     const float *__restrict__ bias, float *y, int N,
                                                      int C, int K, int ld, int act) {
+    pdl_launch_dependents();
+    pdl_wait();
     int warp = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x % 32;
     if (warp >= N * K) return;
     int n = warp / K, j = warp % K;
     float s = 0.f;
-    for (int c = lane; c < C; c += 32) s = fmaf(to_f<T>(w[(size_t)j * ld + c]), v[(size_t)n * C + c], s);
+    for (int c = lane; c < C; c += 32) s = fmaf(to_f<T>(w[(size_t)j * ld + c]), ld_act(v + (size_t)n * C + c), s);
 #pragma unroll
     for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) y[(size_t)n * K + j] = apply_act(s + bias[j], act);
 }
 // bf16 weights, C % 8 == 0, ld % 8 == 0: each lane takes 8 weights (16 bytes) and 8 inputs per step
-__global__ void __launch_bounds__(256) linear_vec_kernel(const float *__restrict__ v, const __nv_bfloat16 *__restrict__ w,
-                                                         const float *__restrict__ bias, float *__restrict__ y, int N, int C,
+__global__ void __launch_bounds__(256) linear_vec_kernel(const float *v, const __nv_bfloat16 *__restrict__ w,
+                                                         const float *__restrict__ bias, float *y, int N, int C,
                                                          int K, int ld, int act) {
+    pdl_launch_dependents();
+    pdl_wait();
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (warp >= N * K) return;
     const int n = warp / K, j = warp % K;
@@ -820,7 +850,7 @@ __global__ void __launch_bounds__(256) linear_vec_kernel(const float *__restrict
     float s = 0.f;
     for (int c = lane * 8; c < C; c += 256) {
         const uint4 wv = __ldg(reinterpret_cast<const uint4 *>(wr + c));
-        const float4 x0 = *reinterpret_cast<const float4 *>(vr + c), x1 = *reinterpret_cast<const float4 *>(vr + c + 4);
+        const float4 x0 = ld_act(reinterpret_cast<const float4 *>(vr + c)), x1 = ld_act(reinterpret_cast<const float4 *>(vr + c + 4));
         const float2 a = bf2f(wv.x), b = bf2f(wv.y), cc = bf2f(wv.z), d = bf2f(wv.w);
         s = fmaf(a.x, x0.x, s); s = fmaf(a.y, x0.y, s); s = fmaf(b.x, x0.z, s); s = fmaf(b.y, x0.w, s);
         s = fmaf(cc.x, x1.x, s); s = fmaf(cc.y, x1.y, s); s = fmaf(d.x, x1.z, s); s = fmaf(d.y, x1.w, s);
@@ -836,12 +866,11 @@ cudaError_t launch_linear(const float *v, const T *w, const float *bias, float *
     long long warps = (long long)N * K;
     if (warps <= 0) return cudaSuccess;
     if (sizeof(T) == 2 && C % 8 == 0 && ld % 8 == 0 && ((reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(v)) & 15) == 0) {
-        linear_vec_kernel<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, st>>>(v, reinterpret_cast<const __nv_bfloat16 *>(w), bias, y, N,
-                                                                               C, K, ld, act);
+        SGS_LAUNCH(linear_vec_kernel, dim3((unsigned)((warps * 32 + 255) / 256)), dim3(256), 0, st, v, reinterpret_cast<const __nv_bfloat16 *>(w), bias, y, N, C, K, ld, act);
         return cudaGetLastError();
     }
     int blocks = (int)((warps * 32 + 255) / 256);
-    linear_kernel<T><<<blocks, 256, 0, st>>>(v, w, bias, y, N, C, K, ld, act);
+    SGS_LAUNCH((linear_kernel<T>), dim3(blocks), dim3(256), 0, st, v, w, bias, y, N, C, K, ld, act);
     return cudaGetLastError();
 }
 template cudaError_t launch_linear<float>(const float *, const float *, const float *, float *, int, int, int, int, int, cudaStream_t);
@@ -874,7 +903,7 @@ __device__ __forceinline__ void maxpool_body(const SmallEntry &e, int bx, int nb
             for (int s = 0; s < 3; s++) {
                 const int wi = 2 * wo + s - 1;
                 if (wi < 0 || wi >= e.W) continue;
-                const uint4 v = __ldg(reinterpret_cast<const uint4 *>(x + (((size_t)n * e.H + hi) * e.W + wi) * e.C) + c);
+                const uint4 v = ld_act(reinterpret_cast<const uint4 *>(x + (((size_t)n * e.H + hi) * e.W + wi) * e.C) + c);
                 best.x = bf2_max(best.x, v.x); best.y = bf2_max(best.y, v.y); best.z = bf2_max(best.z, v.z); best.w = bf2_max(best.w, v.w);
             }
         }
@@ -891,7 +920,7 @@ __device__ __forceinline__ void gap_body(const SmallEntry &e, int bx) {
     const __nv_bfloat16 *base = static_cast<const __nv_bfloat16 *>(e.x) + (size_t)n * HW * e.C + cv * 8;
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     for (int i = lane; i < HW; i += 32) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(base + (size_t)i * e.C));
+        const uint4 v = ld_act(reinterpret_cast<const uint4 *>(base + (size_t)i * e.C));
         const float2 a = bf2f(v.x), b = bf2f(v.y), c = bf2f(v.z), d = bf2f(v.w);
         acc[0] += a.x; acc[1] += a.y; acc[2] += b.x; acc[3] += b.y; acc[4] += c.x; acc[5] += c.y; acc[6] += d.x; acc[7] += d.y;
     }
@@ -915,9 +944,9 @@ __device__ __forceinline__ void scale_body(const SmallEntry &e, int bx, int nbx)
     __nv_bfloat16 *y = static_cast<__nv_bfloat16 *>(e.y);
     for (int i = bx * blockDim.x + threadIdx.x; i < total; i += nbx * blockDim.x) {
         const int n = i / per_image, cv = i % cvecs;
-        const uint4 v = *reinterpret_cast<const uint4 *>(x + (size_t)i * 8);
-        const float4 g0 = __ldg(reinterpret_cast<const float4 *>(gate + (size_t)n * e.C + cv * 8));
-        const float4 g1 = __ldg(reinterpret_cast<const float4 *>(gate + (size_t)n * e.C + cv * 8 + 4));
+        const uint4 v = ld_act(reinterpret_cast<const uint4 *>(x + (size_t)i * 8));
+        const float4 g0 = ld_act(reinterpret_cast<const float4 *>(gate + (size_t)n * e.C + cv * 8));
+        const float4 g1 = ld_act(reinterpret_cast<const float4 *>(gate + (size_t)n * e.C + cv * 8 + 4));
         const float2 a = bf2f(v.x), b = bf2f(v.y), c = bf2f(v.z), d = bf2f(v.w);
         uint4 o;
         __nv_bfloat162 *ob = reinterpret_cast<__nv_bfloat162 *>(&o);
@@ -947,6 +976,8 @@ __device__ __forceinline__ float dot8(uint4 wv, float4 x0, float4 x1, float s) {
 // after the cluster barrier a share of the second FC's.
 constexpr int SE_SPLIT = 4, SE_THREADS = 512;
 __global__ void __cluster_dims__(SE_SPLIT, 1, 1) __launch_bounds__(SE_THREADS) se_gate_group_kernel(const SmallEntry *__restrict__ tbl) {
+    pdl_launch_dependents();
+    pdl_wait();
     extern __shared__ __align__(16) float sm[];
     __shared__ SmallEntry e;
     cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
@@ -962,8 +993,8 @@ __global__ void __cluster_dims__(SE_SPLIT, 1, 1) __launch_bounds__(SE_THREADS) s
     const float *g = static_cast<const float *>(e.x);
     const __nv_bfloat16 *w1 = static_cast<const __nv_bfloat16 *>(e.w), *w2 = static_cast<const __nv_bfloat16 *>(e.w2);
     float *gate = static_cast<float *>(e.y);
-    for (int c = threadIdx.x; c < mid; c += blockDim.x) gs[c] = g[(size_t)n * mid + c];
-    __syncthreads();
+    for (int c = threadIdx.x; c < mid; c += blockDim.x) gs[c] = ld_act(g + (size_t)n * mid + c);
+    cluster.sync();  // (also: every block of the cluster is running before the others write into its shared memory)
     const bool vec = ((mid | sq | e.ld | e.ld2) & 7) == 0 && ((reinterpret_cast<uintptr_t>(w1) | reinterpret_cast<uintptr_t>(w2)) & 15) == 0;
     if (vec) {
         constexpr int JB = 4;
@@ -1040,7 +1071,7 @@ __device__ __forceinline__ void linear_body(const SmallEntry &e, int bx) {
     float s = 0.f;
     for (int c = lane * 8; c < e.C; c += 256) {
         const uint4 wv = __ldg(reinterpret_cast<const uint4 *>(wr + c));
-        const float4 x0 = *reinterpret_cast<const float4 *>(vr + c), x1 = *reinterpret_cast<const float4 *>(vr + c + 4);
+        const float4 x0 = ld_act(reinterpret_cast<const float4 *>(vr + c)), x1 = ld_act(reinterpret_cast<const float4 *>(vr + c + 4));
         const float2 a = bf2f(wv.x), b = bf2f(wv.y), cc = bf2f(wv.z), d = bf2f(wv.w);
         s = fmaf(a.x, x0.x, s); s = fmaf(a.y, x0.y, s); s = fmaf(b.x, x0.z, s); s = fmaf(b.y, x0.w, s);
         s = fmaf(cc.x, x1.x, s); s = fmaf(cc.y, x1.y, s); s = fmaf(d.x, x1.z, s); s = fmaf(d.y, x1.w, s);
@@ -1076,7 +1107,7 @@ __device__ __forceinline__ void im2col_body(const SmallEntry &e, int bx) {
         const unsigned short *src = ximg + (size_t)(rok ? hi : 0) * rowlen;
         for (int i = threadIdx.x; i < padded; i += blockDim.x) {
             const int j = i - P * 3;
-            rows[r][i] = (rok && j >= 0 && j < rowlen) ? __ldg(src + j) : (unsigned short)0;
+            rows[r][i] = (rok && j >= 0 && j < rowlen) ? ld_act(src + j) : (unsigned short)0;
         }
     }
     __syncthreads();
@@ -1116,8 +1147,8 @@ __device__ __forceinline__ void pad8_body(const SmallEntry &e, int bx, int nbx) 
         uint4 v = make_uint4(0u, 0u, 0u, 0u);
         if (h >= 0 && h < e.H && w >= 0 && w < e.W) {
             const unsigned short *p = x + (((size_t)n * e.H + h) * e.W + w) * 3;
-            v.x = __ldg(p) | ((uint32_t)__ldg(p + 1) << 16);
-            v.y = __ldg(p + 2);
+            v.x = ld_act(p) | ((uint32_t)ld_act(p + 1) << 16);
+            v.y = ld_act(p + 2);
         }
         y[i] = v;
     }
@@ -1132,9 +1163,13 @@ template <int KIND, int K, int ST> __device__ __forceinline__ void small_body(co
     else im2col_body<K, ST>(e, bx);
 }
 template <int KIND, int K, int ST> __global__ void __launch_bounds__(256) small_single_kernel(const SmallEntry e) {
+    pdl_launch_dependents();
+    pdl_wait();
     small_body<KIND, K, ST>(e, blockIdx.x, gridDim.x);
 }
 template <int KIND, int K, int ST> __global__ void __launch_bounds__(256) small_group_kernel(const SmallEntry *__restrict__ tbl) {
+    pdl_launch_dependents();
+    pdl_wait();
     __shared__ SmallEntry e;
     if (threadIdx.x < 8) reinterpret_cast<uint4 *>(&e)[threadIdx.x] = __ldg(reinterpret_cast<const uint4 *>(tbl + blockIdx.y) + threadIdx.x);
     __syncthreads();
@@ -1147,6 +1182,8 @@ template <int KIND, int K, int ST> __global__ void __launch_bounds__(256) small_
 // order are those of linear_body.
 constexpr int LIN_CHUNK = 8;
 __global__ void __launch_bounds__(256) linear_multi_kernel(const SmallEntry *__restrict__ tbl, int n_members) {
+    pdl_launch_dependents();
+    pdl_wait();
     __shared__ SmallEntry es[LIN_CHUNK];
     const int m0 = blockIdx.y * LIN_CHUNK, nm = min(LIN_CHUNK, n_members - m0);
     if ((int)threadIdx.x < nm * 8) reinterpret_cast<uint4 *>(es)[threadIdx.x] = __ldg(reinterpret_cast<const uint4 *>(tbl + m0) + threadIdx.x);
@@ -1168,7 +1205,7 @@ __global__ void __launch_bounds__(256) linear_multi_kernel(const SmallEntry *__r
         for (int m = 0; m < LIN_CHUNK; m++) {
             if (m < nm && c < es[m].C) {
                 const float *vr = static_cast<const float *>(es[m].x) + (size_t)n * es[m].C + c;
-                const float4 x0 = *reinterpret_cast<const float4 *>(vr), x1 = *reinterpret_cast<const float4 *>(vr + 4);
+                const float4 x0 = ld_act(reinterpret_cast<const float4 *>(vr)), x1 = ld_act(reinterpret_cast<const float4 *>(vr + 4));
                 float t = s[m];
                 t = fmaf(a.x, x0.x, t); t = fmaf(a.y, x0.y, t); t = fmaf(b.x, x0.z, t); t = fmaf(b.y, x0.w, t);
                 t = fmaf(cc.x, x1.x, t); t = fmaf(cc.y, x1.y, t); t = fmaf(d.x, x1.z, t); t = fmaf(d.y, x1.w, t);
@@ -1216,8 +1253,8 @@ static long long small_blocks(int kind, const SmallEntry &e) {
 
 template <int KIND, int K, int ST>
 static cudaError_t launch_small_t(const SmallEntry *h, const SmallEntry *d, int n, unsigned bx, cudaStream_t st) {
-    if (d) small_group_kernel<KIND, K, ST><<<dim3(bx, (unsigned)n), 256, 0, st>>>(d);
-    else small_single_kernel<KIND, K, ST><<<bx, 256, 0, st>>>(*h);
+    if (d) SGS_LAUNCH((small_group_kernel<KIND, K, ST>), dim3(bx, (unsigned)n), dim3(256), 0, st, d);
+    else SGS_LAUNCH((small_single_kernel<KIND, K, ST>), dim3(bx), dim3(256), 0, st, *h);
     return cudaGetLastError();
 }
 
@@ -1238,7 +1275,7 @@ cudaError_t launch_small(int kind, const SmallEntry *h, const SmallEntry *d, int
         if (!d) return cudaErrorInvalidValue;
         int nimg = 0, fl = 0;
         for (int i = 0; i < n; i++) { nimg = std::max(nimg, h[i].N); fl = std::max(fl, h[i].C + h[i].K); }
-        se_gate_group_kernel<<<dim3((unsigned)nimg * SE_SPLIT, (unsigned)n), SE_THREADS, (size_t)fl * sizeof(float), st>>>(d);
+        SGS_LAUNCH(se_gate_group_kernel, dim3((unsigned)nimg * SE_SPLIT, (unsigned)n), dim3(SE_THREADS), (size_t)fl * sizeof(float), st, d);
         return cudaGetLastError();
     }
     case OP_LINEAR: {
@@ -1246,7 +1283,7 @@ cudaError_t launch_small(int kind, const SmallEntry *h, const SmallEntry *d, int
         for (int i = 1; i < n && same; i++)
             same = h[i].w == h[0].w && h[i].K == h[0].K && h[i].ld == h[0].ld && h[i].N == h[0].N && h[i].act == h[0].act && h[i].bias == h[0].bias;
         if (same) {  // one stored layer for all members: share its weight rows
-            linear_multi_kernel<<<dim3(bx, (unsigned)((n + LIN_CHUNK - 1) / LIN_CHUNK)), 256, 0, st>>>(d, n);
+            SGS_LAUNCH(linear_multi_kernel, dim3(bx, (unsigned)((n + LIN_CHUNK - 1) / LIN_CHUNK)), dim3(256), 0, st, d, n);
             return cudaGetLastError();
         }
         return launch_small_t<OP_LINEAR, 0, 0>(h, d, n, bx, st);
