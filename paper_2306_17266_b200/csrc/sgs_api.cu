@@ -486,6 +486,29 @@ struct Builder {
         plan->weight_bytes += (double)s.K * s.C * net->elem();
         plan->ops.push_back(op);
     }
+    // Squeeze-excite block on the map `buf` (in place): one op, or pool + gate + scale where the map is too large for it.
+    void squeeze_excite(const std::string &fc1, const std::string &fc2, int buf, int h, int w, int mid) {
+        Op g;
+        g.layer = net->idx(fc1); g.layer2 = net->idx(fc2);
+        g.N = N; g.C = mid; g.K = plan->slices[g.layer].K;
+        g.flops = 4.0 * N * mid * g.K;
+        g.alg_bytes = 2.0 * mid * g.K * net->elem();
+        plan->flops += g.flops;
+        plan->weight_bytes += g.alg_bytes;
+        if (se_supported(N, h * w, mid, g.K, net->layers[g.layer].C, net->layers[g.layer2].C, net->dtype == SGS_BF16)) {
+            g.type = OP_SE; g.in = g.out = buf; g.H = h; g.W = w;
+            g.alg_bytes += 2.0 * N * h * w * mid * net->elem();
+            plan->ops.push_back(g);
+            return;
+        }
+        gap(buf, 0, h, w, mid);
+        g.type = OP_SE_GATE; g.vin = 0; g.vout = 1;
+        plan->ops.push_back(g);
+        Op sc;
+        sc.type = OP_SCALE; sc.in = buf; sc.out = buf; sc.vin = 1; sc.N = N; sc.H = h; sc.W = w; sc.C = mid;
+        sc.alg_bytes = 2.0 * N * h * w * mid * net->elem();
+        plan->ops.push_back(sc);
+    }
     void gap(int in, int vout, int H, int W, int C) {
         Op op;
         op.type = OP_GAP; op.in = in; op.vout = vout; op.N = N; op.H = H; op.W = W; op.C = phys(C);
@@ -559,21 +582,7 @@ sgs_status_t build_plan(sgs_supernet *net, const sgs_subnet_cfg_t *cfg, int batc
                 int h = H, w = W;
                 B.conv(bname(s, b, "expand"), X, T1, -1, h, w, 1, d.act[s]);
                 B.conv(bname(s, b, "dw"), T1, T2, -1, h, w, st, d.act[s]);
-                if (d.se[s]) {
-                    B.gap(T2, 0, h, w, mid);
-                    Op g;
-                    g.type = OP_SE_GATE; g.layer = net->idx(bname(s, b, "se1")); g.layer2 = net->idx(bname(s, b, "se2"));
-                    g.vin = 0; g.vout = 1; g.N = batch; g.C = mid; g.K = plan->slices[g.layer].K;
-                    g.flops = 4.0 * batch * mid * g.K;
-                    g.alg_bytes = 2.0 * mid * g.K * net->elem();
-                    plan->flops += g.flops;
-                    plan->weight_bytes += 2.0 * mid * g.K * net->elem();
-                    plan->ops.push_back(g);
-                    Op sc;
-                    sc.type = OP_SCALE; sc.in = T2; sc.out = T2; sc.vin = 1; sc.N = batch; sc.H = h; sc.W = w; sc.C = mid;
-                    sc.alg_bytes = 2.0 * batch * h * w * mid * net->elem();
-                    plan->ops.push_back(sc);
-                }
+                if (d.se[s]) B.squeeze_excite(bname(s, b, "se1"), bname(s, b, "se2"), T2, h, w, mid);
                 int resid = (st == 1 && C == out) ? X : -1;
                 B.conv(bname(s, b, "project"), T2, T1, resid, h, w, 1, ACT_NONE);
                 std::swap(X, T1); H = h; W = w; C = out;
@@ -817,6 +826,13 @@ SmallEntry small_entry(const sgs_supernet *net, const Plan *plan, const Op &op, 
         e.N = op.N; e.C = op.C; e.K = op.K;
         break;
     }
+    case OP_SE: {
+        const StoredLayer &L1 = net->layers[op.layer], &L2 = net->layers[op.layer2];
+        e.x = sl.act[op.in]; e.y = sl.act[op.out];
+        e.w = L1.w; e.bias = L1.shift; e.ld = L1.C; e.w2 = L2.w; e.bias2 = L2.shift; e.ld2 = L2.C;
+        e.N = op.N; e.H = op.H; e.W = op.W; e.C = op.C; e.K = op.K;
+        break;
+    }
     case OP_PAD8:
         e.x = d_input; e.y = sl.act[op.out];
         e.N = op.N; e.H = op.H; e.W = op.W; e.C = 3; e.k = op.K; e.Ho = op.conv.Ho; e.Wo = op.conv.Wo;
@@ -847,6 +863,12 @@ sgs_status_t launch_op(sgs_supernet *net, Plan *plan, Op &op, const void *d_inpu
         if (op.type == OP_DW) { CU(launch_dw<T>(a, st)); net->kernel_launches++; }
         else if (op.impl == 1) { int n = 0; CU(tc_conv_launch(*op.tc, a, st, &n)); net->kernel_launches += n; }
         else { CU(launch_conv_plain<T>(a, st)); net->kernel_launches++; }
+        break;
+    }
+    case OP_SE: {
+        SmallEntry e = small_entry(net, plan, op, d_input, d_logits);
+        CU(launch_se(&e, nullptr, 1, net->dtype == SGS_BF16, st));
+        net->kernel_launches++;
         break;
     }
     case OP_PAD8:
@@ -1640,7 +1662,7 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
             // member's op has the vectorised form; the remaining ops run member by member
             const Op &op0 = plans[b[0].first]->ops[(size_t)b[0].second];
             const int kind = op0.type;
-            bool grouped = kind == OP_MAXPOOL || kind == OP_GAP || kind == OP_LINEAR || kind == OP_IM2COL || kind == OP_SCALE || kind == OP_SE_GATE || kind == OP_PAD8;
+            bool grouped = kind == OP_MAXPOOL || kind == OP_GAP || kind == OP_LINEAR || kind == OP_IM2COL || kind == OP_SCALE || kind == OP_SE_GATE || kind == OP_PAD8 || kind == OP_SE;
             if (grouped) {
                 const size_t off0 = off;
                 for (const auto &mo : b) {
@@ -1902,11 +1924,26 @@ static sgs_status_t build_pq_ops(sgs_supernet *net, Plan *plan) {
             if (!mult8(op.C) || op.C > 1280) return fail(net, SGS_EUNSUPPORTED, "persistent kernel: pooled width");
             q.type = PQ_GAP; q.in = op.in; q.vout = op.vout; q.H = op.H; q.W = op.W; q.C = op.C;
             break;
+        case OP_SE:
         case OP_SE_GATE: {
+            // (a fused block of the layer-by-layer paths is three ops here: pool, gate, scale)
             const StoredLayer &L1 = net->layers[op.layer], &L2 = net->layers[op.layer2];
             if (!mult8(op.C) || !mult8(op.K) || !mult8(L1.C) || !mult8(L2.C) || op.C > 1280 || op.K > 1280) return fail(net, SGS_EUNSUPPORTED, "persistent kernel: squeeze-excite shape");
-            q.type = PQ_SE_GATE; q.vin = op.vin; q.vout = op.vout; q.C = op.C; q.K = op.K;
+            const bool fused = op.type == OP_SE;
+            if (fused && op.in > 3) return fail(net, SGS_EUNSUPPORTED, "persistent kernel: buffer id");
+            if (fused) {
+                PqOp g = q;
+                g.type = PQ_GAP; g.in = op.in; g.vout = 0; g.H = op.H; g.W = op.W; g.C = op.C;
+                plan->pq.push_back(g);
+            }
+            q.type = PQ_SE_GATE; q.vin = fused ? 0 : op.vin; q.vout = fused ? 1 : op.vout; q.C = op.C; q.K = op.K;
             q.w = L1.w; q.ld = L1.C; q.shift = L1.shift; q.w2 = L2.w; q.ld2 = L2.C; q.bias2 = L2.shift;
+            if (fused) {
+                plan->pq.push_back(q);
+                std::memset(&q, 0, sizeof q);
+                q.res = q.vout = -1; q.cache_off = -1;
+                q.type = PQ_SCALE; q.in = op.in; q.out = op.out; q.vin = 1; q.H = op.H; q.W = op.W; q.C = op.C;
+            }
             break;
         }
         case OP_SCALE:

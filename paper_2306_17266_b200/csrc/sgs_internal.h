@@ -130,7 +130,7 @@ struct PqParams {
     int *status;             // device status word: nonzero after a bounded wait ran out
 };
 
-enum OpType { OP_CONV, OP_DW, OP_MAXPOOL, OP_GAP, OP_SE_GATE, OP_SCALE, OP_LINEAR, OP_IM2COL, OP_PAD8 };
+enum OpType { OP_CONV, OP_DW, OP_MAXPOOL, OP_GAP, OP_SE_GATE, OP_SCALE, OP_LINEAR, OP_IM2COL, OP_PAD8, OP_SE };
 
 struct TcConvPlan;  // tensor-core launch description (sgs_conv_tc.cu)
 
@@ -208,6 +208,10 @@ static_assert(sizeof(SmallEntry) == 128, "record size");
 // at device address `d` (it sizes the grid); with d == nullptr, n must be 1 and the record is passed by value.
 bool small_supported(int kind, const SmallEntry &e);
 cudaError_t launch_small(int kind, const SmallEntry *h, const SmallEntry *d, int n, cudaStream_t st);
+// Squeeze-excite block (pool, gate, in-place scale) in one launch (sgs_se.cu): x = y = the map [N][H][W][C], w / bias / ld =
+// first layer (K = squeeze width), w2 / bias2 / ld2 = second.  d == nullptr: one record, fp32 or bf16; else n bf16 members.
+bool se_supported(int N, int HW, int C, int sq, int ld, int ld2, int bf16);
+cudaError_t launch_se(const SmallEntry *h, const SmallEntry *d, int n, int bf16, cudaStream_t st);
 // Depthwise convolution of several members in one launch: h_tbl / d_tbl = host image and device copy of
 // `members` ConvArgs records, DW_ENTRY_BYTES apart.  All members must share stride, activation and image dims
 // and take the vectorised bf16 kernels (kernel sizes 3, 5, 7 may be mixed); otherwise cudaErrorNotSupported and

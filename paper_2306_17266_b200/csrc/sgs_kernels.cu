@@ -1231,6 +1231,7 @@ bool small_supported(int kind, const SmallEntry &e) {
     case OP_GAP: return e.C % 8 == 0;
     case OP_SCALE: return e.C % 8 == 0 && al(e.w) && (long long)e.N * e.H * e.W * (e.C / 8) < (1ll << 31);
     case OP_SE_GATE: return e.w2 != nullptr;
+    case OP_SE: return e.w2 != nullptr && al(e.w) && al(e.w2) && se_supported(e.N, e.H * e.W, e.C, e.K, e.ld, e.ld2, 1);
     case OP_PAD8: return (long long)e.N * e.Ho * e.Wo < (1ll << 31);
     case OP_LINEAR: return e.C % 8 == 0 && e.ld % 8 == 0 && al(e.w);
     case OP_IM2COL: return (e.k == 3 || e.k == 7) && (e.stride == 1 || e.stride == 2) && e.KKp % 8 == 0 && e.KKp >= e.k * e.k * 3 &&
@@ -1271,6 +1272,7 @@ cudaError_t launch_small(int kind, const SmallEntry *h, const SmallEntry *d, int
     case OP_GAP: return launch_small_t<OP_GAP, 0, 0>(h, d, n, bx, st);
     case OP_SCALE: return launch_small_t<OP_SCALE, 0, 0>(h, d, n, bx, st);
     case OP_PAD8: return launch_small_t<OP_PAD8, 0, 0>(h, d, n, bx, st);
+    case OP_SE: return launch_se(h, d, n, 1, st);
     case OP_SE_GATE: {
         if (!d) return cudaErrorInvalidValue;
         int nimg = 0, fl = 0;
