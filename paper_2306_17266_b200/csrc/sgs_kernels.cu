@@ -654,6 +654,11 @@ template <typename T> cudaError_t launch_maxpool3s2(const T *x, T *y, int N, int
     int Ho = (H - 1) / 2 + 1, Wo = (W - 1) / 2 + 1;
     size_t total = (size_t)N * Ho * Wo * C;
     if (!total) return cudaSuccess;
+    if (sizeof(T) == 2) {
+        SmallEntry e = {};
+        e.x = x; e.y = y; e.N = N; e.H = H; e.W = W; e.C = C; e.Ho = Ho; e.Wo = Wo;
+        if (small_supported(OP_MAXPOOL, e)) return launch_small(OP_MAXPOOL, &e, nullptr, 1, st);
+    }
     int blocks = (int)std::min<size_t>((total + 255) / 256, 148 * 16);
     SGS_LAUNCH((maxpool_kernel<T>), dim3(blocks), dim3(256), 0, st, x, y, N, H, W, C, Ho, Wo);
     return cudaGetLastError();
@@ -836,46 +841,6 @@ __global__ void __launch_bounds__(256) linear_kernel(const float *v, const T *__
     for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) y[(size_t)n * K + j] = apply_act(s + bias[j], act);
 }
-// bf16 weights, C % 8 == 0, ld % 8 == 0: each lane takes 8 weights (16 bytes) and 8 inputs per step
-__global__ void __launch_bounds__(256) linear_vec_kernel(const float *v, const __nv_bfloat16 *__restrict__ w,
-                                                         const float *__restrict__ bias, float *y, int N, int C,
-                                                         int K, int ld, int act) {
-    pdl_launch_dependents();
-    pdl_wait();
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (warp >= N * K) return;
-    const int n = warp / K, j = warp % K;
-    const __nv_bfloat16 *wr = w + (size_t)j * ld;
-    const float *vr = v + (size_t)n * C;
-    float s = 0.f;
-    for (int c = lane * 8; c < C; c += 256) {
-        const uint4 wv = __ldg(reinterpret_cast<const uint4 *>(wr + c));
-        const float4 x0 = ld_act(reinterpret_cast<const float4 *>(vr + c)), x1 = ld_act(reinterpret_cast<const float4 *>(vr + c + 4));
-        const float2 a = bf2f(wv.x), b = bf2f(wv.y), cc = bf2f(wv.z), d = bf2f(wv.w);
-        s = fmaf(a.x, x0.x, s); s = fmaf(a.y, x0.y, s); s = fmaf(b.x, x0.z, s); s = fmaf(b.y, x0.w, s);
-        s = fmaf(cc.x, x1.x, s); s = fmaf(cc.y, x1.y, s); s = fmaf(d.x, x1.z, s); s = fmaf(d.y, x1.w, s);
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) y[(size_t)n * K + j] = apply_act(s + bias[j], act);
-}
-
-template <typename T>
-cudaError_t launch_linear(const float *v, const T *w, const float *bias, float *y, int N, int C, int K, int ld, int act,
-                          cudaStream_t st) {
-    long long warps = (long long)N * K;
-    if (warps <= 0) return cudaSuccess;
-    if (sizeof(T) == 2 && C % 8 == 0 && ld % 8 == 0 && ((reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(v)) & 15) == 0) {
-        SGS_LAUNCH(linear_vec_kernel, dim3((unsigned)((warps * 32 + 255) / 256)), dim3(256), 0, st, v, reinterpret_cast<const __nv_bfloat16 *>(w), bias, y, N, C, K, ld, act);
-        return cudaGetLastError();
-    }
-    int blocks = (int)((warps * 32 + 255) / 256);
-    SGS_LAUNCH((linear_kernel<T>), dim3(blocks), dim3(256), 0, st, v, w, bias, y, N, C, K, ld, act);
-    return cudaGetLastError();
-}
-template cudaError_t launch_linear<float>(const float *, const float *, const float *, float *, int, int, int, int, int, cudaStream_t);
-template cudaError_t launch_linear<__nv_bfloat16>(const float *, const __nv_bfloat16 *, const float *, float *, int, int, int, int, int, cudaStream_t);
-
 // ---------------------------------------------------------------------------------------------
 // Record-driven bf16 kernels (see SmallEntry): each body works on one member; the `single` kernels get
 // the record by value, the `group` kernels pick it from a device table with blockIdx.y.
@@ -1061,26 +1026,6 @@ __global__ void __cluster_dims__(SE_SPLIT, 1, 1) __launch_bounds__(SE_THREADS) s
     }
 }
 
-// Sliced linear layer on fp32 vectors: one warp per (image, output), 16-byte weight loads.
-__device__ __forceinline__ void linear_body(const SmallEntry &e, int bx) {
-    const int warp = (bx * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (warp >= e.N * e.K) return;
-    const int n = warp / e.K, j = warp % e.K;
-    const __nv_bfloat16 *wr = static_cast<const __nv_bfloat16 *>(e.w) + (size_t)j * e.ld;
-    const float *vr = static_cast<const float *>(e.x) + (size_t)n * e.C;
-    float s = 0.f;
-    for (int c = lane * 8; c < e.C; c += 256) {
-        const uint4 wv = __ldg(reinterpret_cast<const uint4 *>(wr + c));
-        const float4 x0 = ld_act(reinterpret_cast<const float4 *>(vr + c)), x1 = ld_act(reinterpret_cast<const float4 *>(vr + c + 4));
-        const float2 a = bf2f(wv.x), b = bf2f(wv.y), cc = bf2f(wv.z), d = bf2f(wv.w);
-        s = fmaf(a.x, x0.x, s); s = fmaf(a.y, x0.y, s); s = fmaf(b.x, x0.z, s); s = fmaf(b.y, x0.w, s);
-        s = fmaf(cc.x, x1.x, s); s = fmaf(cc.y, x1.y, s); s = fmaf(d.x, x1.z, s); s = fmaf(d.y, x1.w, s);
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) static_cast<float *>(e.y)[(size_t)n * e.K + j] = apply_act(s + e.bias[j], e.act);
-}
-
 // Patch matrix of a convolution with 3 input channels (the stems): row m = output pixel, column
 // kk = (r * k + s) * 3 + c holds x[n][ho*st + r - p][wo*st + s - p][c] (0 outside the image and for the
 // padding columns kk >= k*k*3).  With it the stem is a GEMM on the tensor cores like every other layer.
@@ -1157,7 +1102,6 @@ __device__ __forceinline__ void pad8_body(const SmallEntry &e, int bx, int nbx) 
 template <int KIND, int K, int ST> __device__ __forceinline__ void small_body(const SmallEntry &e, int bx, int nbx) {
     if constexpr (KIND == OP_MAXPOOL) maxpool_body(e, bx, nbx);
     else if constexpr (KIND == OP_GAP) gap_body(e, bx);
-    else if constexpr (KIND == OP_LINEAR) linear_body(e, bx);
     else if constexpr (KIND == OP_SCALE) scale_body(e, bx, nbx);
     else if constexpr (KIND == OP_PAD8) pad8_body(e, bx, nbx);
     else im2col_body<K, ST>(e, bx);
@@ -1176,52 +1120,118 @@ template <int KIND, int K, int ST> __global__ void __launch_bounds__(256) small_
     small_body<KIND, K, ST>(e, blockIdx.x, gridDim.x);
 }
 
-// Linear layer for several members that use the SAME stored layer (same weights, outputs, batch): a warp
-// owns one (image, output) pair for up to LIN_CHUNK members, loads every 16-byte piece of the weight row
-// once and uses it for each member whose (sliced) input is that long.  Per member the arithmetic and its
-// order are those of linear_body.
-constexpr int LIN_CHUNK = 8;
-__global__ void __launch_bounds__(256) linear_multi_kernel(const SmallEntry *__restrict__ tbl, int n_members) {
+// Sliced linear layer on fp32 vectors, bf16 weights, for the images of one query or of all members of a wave that use the
+// SAME stored layer.  A row is one image of one member; a warp owns JB outputs of up to LIN_ROWS rows: every 16-byte piece
+// of a weight row is loaded once for all of them, every piece of an input vector once for JB outputs.  What bounds it is
+// the latency of a chain of such loads (the weights of a classifier, 2 to 4 MB, lie in L2) and, with many rows, the loads of
+// the input vectors from L1: with JB = 1 a wave of 32 spent 22 - 27 us here, every warp reading 64 KB of inputs for one
+// weight row.  The first two pieces of the weight rows are requested before the wait for the previous layer.
+// Per output the arithmetic and its order do not depend on JB or on the rows that share the warp.
+constexpr int LIN_ROWS = 8;
+template <int JB, bool GROUP>
+__global__ void __launch_bounds__(256) linear_rows_kernel(const SmallEntry e1, const SmallEntry *__restrict__ tbl, int n_members) {
+    __shared__ SmallEntry first;
+    __shared__ const float *xr[LIN_ROWS];
+    __shared__ float *yr[LIN_ROWS];
+    __shared__ int cr[LIN_ROWS];
     pdl_launch_dependents();
-    pdl_wait();
-    __shared__ SmallEntry es[LIN_CHUNK];
-    const int m0 = blockIdx.y * LIN_CHUNK, nm = min(LIN_CHUNK, n_members - m0);
-    if ((int)threadIdx.x < nm * 8) reinterpret_cast<uint4 *>(es)[threadIdx.x] = __ldg(reinterpret_cast<const uint4 *>(tbl + m0) + threadIdx.x);
+    if (GROUP) {
+        if (threadIdx.x < 8) reinterpret_cast<uint4 *>(&first)[threadIdx.x] = __ldg(reinterpret_cast<const uint4 *>(tbl) + threadIdx.x);
+        __syncthreads();
+    }
+    const SmallEntry &e0 = GROUP ? first : e1;
+    const int N = e0.N, K = e0.K, ld = e0.ld;
+    const int r0 = blockIdx.y * LIN_ROWS, nr = min(LIN_ROWS, (GROUP ? n_members : 1) * N - r0);
+    if ((int)threadIdx.x < LIN_ROWS) {
+        const int r = min(r0 + (int)threadIdx.x, r0 + nr - 1), m = r / N, n = r % N;
+        const SmallEntry *e = GROUP ? tbl + m : nullptr;
+        const int C = GROUP ? e->C : e1.C;
+        xr[threadIdx.x] = static_cast<const float *>(GROUP ? e->x : e1.x) + (size_t)n * C;
+        yr[threadIdx.x] = static_cast<float *>(GROUP ? e->y : e1.y) + (size_t)n * K;
+        cr[threadIdx.x] = (int)threadIdx.x < nr ? C : 0;
+    }
     __syncthreads();
-    const SmallEntry &e0 = es[0];
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (warp >= e0.N * e0.K) return;
-    const int n = warp / e0.K, j = warp % e0.K;
-    const __nv_bfloat16 *wr = static_cast<const __nv_bfloat16 *>(e0.w) + (size_t)j * e0.ld;
-    int Cmax = 0;
-    for (int m = 0; m < nm; m++) Cmax = max(Cmax, es[m].C);
-    float s[LIN_CHUNK];
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31, j0 = warp * JB;
+    if (j0 >= K) return;
+    int cmax = 0;
 #pragma unroll
-    for (int m = 0; m < LIN_CHUNK; m++) s[m] = 0.f;
-    for (int c = lane * 8; c < Cmax; c += 256) {
-        const uint4 wv = __ldg(reinterpret_cast<const uint4 *>(wr + c));
-        const float2 a = bf2f(wv.x), b = bf2f(wv.y), cc = bf2f(wv.z), d = bf2f(wv.w);
+    for (int r = 0; r < LIN_ROWS; r++) cmax = max(cmax, cr[r]);
+    const __nv_bfloat16 *w = static_cast<const __nv_bfloat16 *>(e0.w);
+    auto load_w = [&](int c, uint4 *q) {
 #pragma unroll
-        for (int m = 0; m < LIN_CHUNK; m++) {
-            if (m < nm && c < es[m].C) {
-                const float *vr = static_cast<const float *>(es[m].x) + (size_t)n * es[m].C + c;
-                const float4 x0 = ld_act(reinterpret_cast<const float4 *>(vr)), x1 = ld_act(reinterpret_cast<const float4 *>(vr + 4));
-                float t = s[m];
-                t = fmaf(a.x, x0.x, t); t = fmaf(a.y, x0.y, t); t = fmaf(b.x, x0.z, t); t = fmaf(b.y, x0.w, t);
-                t = fmaf(cc.x, x1.x, t); t = fmaf(cc.y, x1.y, t); t = fmaf(d.x, x1.z, t); t = fmaf(d.y, x1.w, t);
-                s[m] = t;
+        for (int u = 0; u < JB; u++)
+            q[u] = c < cmax ? __ldg(reinterpret_cast<const uint4 *>(w + (size_t)min(j0 + u, K - 1) * ld + c)) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    uint4 wa[JB], wb[JB];
+    load_w(lane * 8, wa);
+    load_w(lane * 8 + 256, wb);
+    pdl_wait();
+    float s[JB][LIN_ROWS];
+#pragma unroll
+    for (int u = 0; u < JB; u++)
+#pragma unroll
+        for (int r = 0; r < LIN_ROWS; r++) s[u][r] = 0.f;
+    for (int c = lane * 8; c < cmax; c += 256) {
+        uint4 wc[JB];
+        load_w(c + 512, wc);
+#pragma unroll
+        for (int r = 0; r < LIN_ROWS; r++) {
+            if (c < cr[r]) {
+                const float4 x0 = ld_act(reinterpret_cast<const float4 *>(xr[r] + c)), x1 = ld_act(reinterpret_cast<const float4 *>(xr[r] + c + 4));
+#pragma unroll
+                for (int u = 0; u < JB; u++) s[u][r] = dot8(wa[u], x0, x1, s[u][r]);
             }
         }
+#pragma unroll
+        for (int u = 0; u < JB; u++) { wa[u] = wb[u]; wb[u] = wc[u]; }
     }
-    const float bias = e0.bias[j];
 #pragma unroll
-    for (int m = 0; m < LIN_CHUNK; m++) {
-        float t = s[m];
+    for (int u = 0; u < JB; u++) {
+        if (j0 + u >= K) break;
+        const float bias = __ldg(e0.bias + j0 + u);
 #pragma unroll
-        for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (lane == 0 && m < nm) static_cast<float *>(es[m].y)[(size_t)n * e0.K + j] = apply_act(t + bias, e0.act);
+        for (int r = 0; r < LIN_ROWS; r++) {
+            if (r >= nr) break;
+            float t = s[u][r];
+#pragma unroll
+            for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (lane == 0) yr[r][j0 + u] = apply_act(t + bias, e0.act);
+        }
     }
 }
+// rows = images over all members.  One or two rows: a warp per output (a classifier then fills the GPU); more: 4 outputs.
+static cudaError_t launch_linear_rows(const SmallEntry *h, const SmallEntry *d, int n, cudaStream_t st) {
+    const long long rows = (long long)n * h[0].N;
+    const unsigned gy = (unsigned)((rows + LIN_ROWS - 1) / LIN_ROWS);
+    const int jb = rows <= 2 ? 1 : 4;
+    const unsigned gx = (unsigned)(((h[0].K + jb - 1) / jb * 32ll + 255) / 256);
+    if (gy > 65535) return cudaErrorInvalidValue;
+    if (d) {
+        if (jb == 1) SGS_LAUNCH((linear_rows_kernel<1, true>), dim3(gx, gy), dim3(256), 0, st, h[0], d, n);
+        else SGS_LAUNCH((linear_rows_kernel<4, true>), dim3(gx, gy), dim3(256), 0, st, h[0], d, n);
+    } else {
+        if (jb == 1) SGS_LAUNCH((linear_rows_kernel<1, false>), dim3(gx, gy), dim3(256), 0, st, h[0], d, n);
+        else SGS_LAUNCH((linear_rows_kernel<4, false>), dim3(gx, gy), dim3(256), 0, st, h[0], d, n);
+    }
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_linear(const float *v, const T *w, const float *bias, float *y, int N, int C, int K, int ld, int act,
+                          cudaStream_t st) {
+    long long warps = (long long)N * K;
+    if (warps <= 0) return cudaSuccess;
+    if (sizeof(T) == 2 && C % 8 == 0 && ld % 8 == 0 && ((reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(v)) & 15) == 0 && N <= 65535) {
+        SmallEntry e = {};
+        e.x = v; e.y = y; e.w = w; e.bias = bias; e.N = N; e.C = C; e.K = K; e.ld = ld; e.act = act;
+        return launch_linear_rows(&e, nullptr, 1, st);
+    }
+    int blocks = (int)((warps * 32 + 255) / 256);
+    SGS_LAUNCH((linear_kernel<T>), dim3(blocks), dim3(256), 0, st, v, w, bias, y, N, C, K, ld, act);
+    return cudaGetLastError();
+}
+template cudaError_t launch_linear<float>(const float *, const float *, const float *, float *, int, int, int, int, int, cudaStream_t);
+template cudaError_t launch_linear<__nv_bfloat16>(const float *, const __nv_bfloat16 *, const float *, float *, int, int, int, int, int, cudaStream_t);
 
 bool small_supported(int kind, const SmallEntry &e) {
     auto al = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
@@ -1247,7 +1257,6 @@ static long long small_blocks(int kind, const SmallEntry &e) {
     case OP_GAP: return ((long long)e.N * (e.C / 8) * 32 + 255) / 256;
     case OP_SCALE: return ((long long)e.N * e.H * e.W * (e.C / 8) + 255) / 256;
     case OP_PAD8: return ((long long)e.N * e.Ho * e.Wo + 255) / 256;
-    case OP_LINEAR: return ((long long)e.N * e.K * 32 + 255) / 256;
     default: return (long long)e.N * e.Ho;  // patch matrix: one block per output row
     }
 }
@@ -1281,14 +1290,16 @@ cudaError_t launch_small(int kind, const SmallEntry *h, const SmallEntry *d, int
         return cudaGetLastError();
     }
     case OP_LINEAR: {
-        bool same = d != nullptr && n > 1;
-        for (int i = 1; i < n && same; i++)
-            same = h[i].w == h[0].w && h[i].K == h[0].K && h[i].ld == h[0].ld && h[i].N == h[0].N && h[i].act == h[0].act && h[i].bias == h[0].bias;
-        if (same) {  // one stored layer for all members: share its weight rows
-            SGS_LAUNCH(linear_multi_kernel, dim3(bx, (unsigned)((n + LIN_CHUNK - 1) / LIN_CHUNK)), dim3(256), 0, st, d, n);
-            return cudaGetLastError();
+        // members with one stored layer and batch (every wave: the classifier, the mixing layer) share a launch
+        int i = 0;
+        while (i < n) {
+            int k = i + 1;
+            while (k < n && h[k].w == h[i].w && h[k].K == h[i].K && h[k].ld == h[i].ld && h[k].N == h[i].N && h[k].act == h[i].act && h[k].bias == h[i].bias) k++;
+            const cudaError_t e = launch_linear_rows(h + i, d ? d + i : nullptr, k - i, st);
+            if (e != cudaSuccess) return e;
+            i = k;
         }
-        return launch_small_t<OP_LINEAR, 0, 0>(h, d, n, bx, st);
+        return cudaSuccess;
     }
     case OP_IM2COL: {
         const int key = h[0].k * 10 + h[0].stride;
