@@ -310,8 +310,8 @@ sgs_status_t sgs_subnet_cost(const sgs_supernet_t *net, const sgs_subnet_cfg_t *
  *   d_x     [N][H][W][C] NHWC, dtype elements            d_y, d_res  [N][Ho][Wo][K] (d_res may be NULL)
  *   d_w     stored weights, [Kmax][R][R][Cmax] (depthwise: [R][R][Kmax]), dtype elements
  *   d_scale, d_shift  [>= K] fp32
- * impl 0 = automatic (tensor cores when dtype is bf16, C, K, Cmax are multiples of 8, pointers are
- * 16-byte aligned and stride-2 inputs have even sizes), 1 = CUDA-core kernel, 2 = tensor cores or
+ * impl 0 = automatic (tensor cores when dtype is bf16, C, K, Cmax are multiples of 8 and pointers are
+ * 16-byte aligned; kernels larger than 1x1 at stride 2 need at least 2x2 pixels), 1 = CUDA-core kernel, 2 = tensor cores or
  * SGS_EUNSUPPORTED.  weight_policy 0 = no L2 hint, 1 = evict-last for weight tiles with filter <
  * cache_k and channel < cache_c (default replacement for the rest), 2 = all weights evict-first.
  * Asynchronous on `cuda_stream`.  The tensor-core path may split the reduction over several CTAs
@@ -378,8 +378,8 @@ sgs_status_t sgs_conv2d_sliced_static(const sgs_conv_desc_t *desc, const void *d
  *   d_x    [N][H][W][C] bytes (unsigned, or signed if x_signed)     d_y, d_res  [N][Ho][Wo][K] bytes
  *   d_w    stored weights [Kmax][R][R][Cmax] signed bytes            d_mult, d_shift, d_bias  [>= K] int32
  * Limits of this entry point: pixels of x in multiples of 16 bytes (C a multiple of 16, or of 8 with ldx), Cmax a
- * multiple of 16, K a multiple of 8, 16-byte aligned pointers, stride-2
- * inputs of even size, 0 <= shift[f] <= 31, and zx == 0 (an input zero point other than 0 would need the sum of the
+ * multiple of 16, K a multiple of 8, 16-byte aligned pointers, at least
+ * 2x2 pixels at stride 2, 0 <= shift[f] <= 31, and zx == 0 (an input zero point other than 0 would need the sum of the
  * sliced weights under every window position, which changes with the slice and at image borders; post-ReLU tensors
  * and symmetric signed tensors have zx = 0).  Other values: SGS_EUNSUPPORTED.  Asynchronous on `cuda_stream`.
  */

@@ -523,10 +523,10 @@ sgs_status_t build_plan(sgs_supernet *net, const sgs_subnet_cfg_t *cfg, int batc
     plan->slices = slices_for(net, cfg);
     Builder B{net, plan, batch};
     // Waves of the ResNet-shaped family on bf16 handles: every convolution runs in the grouped tensor-core kernel
-    // (all channel counts are multiples of 8, and with res % 32 == 0 every stride-2 layer sees even sizes), so the
-    // activation tensors can be padded to 16-channel pixels.  choose_impls refuses a padded plan otherwise.
+    // (all channel counts are multiples of 8, and every stride-2 layer sees at least 2x2 pixels), so the activation
+    // tensors can be padded to 16-channel pixels.  choose_impls refuses a padded plan otherwise.
     B.padded = net->family == SGS_RESNET && net->throughput_mode == 2 && net->dtype == SGS_BF16 && !net->force_plain &&
-               tc_available() && res % 32 == 0 && net->stem_win_w != nullptr && net->pad_channels;
+               tc_available() && (res >= 64 || res % 32 == 0) && net->stem_win_w != nullptr && net->pad_channels;
     plan->padded = B.padded;
     int H = res, W = res;
     // activation buffers: X current tensor, T1/T2 temporaries, SC shortcut

@@ -524,7 +524,7 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
     if (a.C < 8 || a.K < 8) return no("too few channels");
     if (a.k % 2 == 0 || a.k > a.R) return no("kernel size");
     if (a.stride != 1 && a.stride != 2) return no("stride");
-    if (a.stride == 2 && ((a.H | a.W) & 1)) return no("stride 2 needs even input sizes");
+    if (a.stride == 2 && a.k > 1 && (a.H < 2 || a.W < 2)) return no("a parity view of a one-pixel side would be empty");
     if ((reinterpret_cast<uintptr_t>(a.x) | reinterpret_cast<uintptr_t>(a.w) | reinterpret_cast<uintptr_t>(a.y) |
          reinterpret_cast<uintptr_t>(a.res)) & 15)
         return no("pointers must be 16-byte aligned");
@@ -591,10 +591,12 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
             uint64_t str[3] = {C * eb, (uint64_t)a.W * C * eb, (uint64_t)a.H * a.W * C * eb};
             if (!encode_map(&p.tmA[0], a.x, 4, dims, str, box, b8)) return no("activation tensor map");
         } else {
-            for (int ph = 0; ph < 2; ph++)
-                for (int pw = 0; pw < 2; pw++) {
+            // (odd sizes: the views of odd rows / columns are one shorter; what lies beyond is zero fill like any border)
+            const int views = a.k > 1 ? 2 : 1;  // a 1x1 kernel reads even rows and columns only
+            for (int ph = 0; ph < views; ph++)
+                for (int pw = 0; pw < views; pw++) {
                     const char *base = static_cast<const char *>(a.x) + ((size_t)ph * a.W + pw) * C * eb;
-                    uint64_t dims[4] = {C, (uint64_t)a.W / 2, (uint64_t)a.H / 2, (uint64_t)a.N};
+                    uint64_t dims[4] = {C, (uint64_t)(a.W - pw + 1) / 2, (uint64_t)(a.H - ph + 1) / 2, (uint64_t)a.N};
                     uint64_t str[3] = {2 * C * eb, 2 * (uint64_t)a.W * C * eb, (uint64_t)a.H * a.W * C * eb};
                     if (!encode_map(&p.tmA[ph * 2 + pw], base, 4, dims, str, box, b8)) return no("activation tensor map");
                 }
