@@ -468,8 +468,8 @@ sgs_status_t sgs_debug_expire_wait(unsigned limit_us, void *cuda_stream);
  * execution spends on the cached SubGraph's first pointwise layers (default 16, 0 = none); "nvtx" 1 = an NVTX range named after the stored layer around
  * every launch (for timeline tools); "fail_alloc_after" n = the handle's device allocations fail from
  * the (n+1)-th on with SGS_ENOMEM (fault injection on the host, -1 = off); "drop_plans" forgets every cached plan (measuring what a never-seen config costs); "profile" see
- * sgs_profile_read; "stage_group" 0 = default, 1..4 = pipeline stages that
- * share one barrier pair in the grouped convolution kernel (process-wide, a tuning aid).  Unknown name -> SGS_EINVAL. */
+ * sgs_profile_read; "stage_group" 0..4 is accepted
+ * and has no effect (every pipeline stage of the grouped convolution kernel has its own barriers).  Unknown name -> SGS_EINVAL. */
 sgs_status_t sgs_set_option(sgs_supernet_t *net, const char *name, long long value);
 
 /*

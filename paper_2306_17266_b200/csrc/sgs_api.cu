@@ -2622,9 +2622,8 @@ sgs_status_t sgs_set_option(sgs_supernet_t *net, const char *name, long long val
         dw_set_walk((int)value);
         return SGS_OK;
     }
-    if (n == "stage_group") {  // tuning aid: stages per barrier pair of the grouped convolution kernel (0 = default)
+    if (n == "stage_group") {  // (accepted for compatibility: every stage of the grouped convolution kernel has its own barriers)
         if (value < 0 || value > 4) return fail(net, SGS_EINVAL, "stage_group");
-        tc_group_set_stage_group((int)value);
         return SGS_OK;
     }
     return fail(net, SGS_EINVAL, "unknown option " + n);

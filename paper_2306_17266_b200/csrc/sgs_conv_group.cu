@@ -96,8 +96,7 @@ template <int NMAPS> struct GroupParams {
     int *status;
     int n_entries, total_tiles;
     int n_stages, stage_bytes;  // operand ring of this launch
-    int group;                  // consecutive stages that share one pair of barriers (n_stages is a multiple of it)
-    int pad_[5];
+    int pad_[6];
     CUtensorMap maps[NMAPS];
 };
 static_assert(sizeof(GroupParams<TC_GROUP_MAPS_LARGE>) <= 32764, "kernel parameter block");
@@ -123,11 +122,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
     for (int i = threadIdx.x; i < n_entries * (int)(sizeof(GroupEntry) / 16); i += blockDim.x)
         reinterpret_cast<uint4 *>(es)[i] = __ldg(reinterpret_cast<const uint4 *>(entries) + i);
     if (threadIdx.x == 0) {
-        // Barriers are per GROUP of consecutive stages: a group is full once both producers' copies of all its
-        // stages have landed (each producer arrives once per stage), and empty once the MMAs of its last stage
-        // have read it.  One wait and one commit then serve `group` stages: the issuing threads pay their fixed
-        // cost per wait (a few hundred cycles) once per group instead of once per 64 channels.
-        for (int s = 0; s < G_MAX_STAGES; s++) { mbar_init(&full_bar[s], 2 * (uint32_t)P.group); mbar_init(&empty_bar[s], 1); }
+        for (int s = 0; s < G_MAX_STAGES; s++) { mbar_init(&full_bar[s], 2); mbar_init(&empty_bar[s], 1); }  // (full: both producers arrive)
         for (int b = 0; b < 2; b++) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], G_EPI_WARPS / 2); }
         abort_s = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -137,106 +132,93 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_s;
-    const int n_stages = P.n_stages, stage_bytes = P.stage_bytes, gsz = P.group;
+    const int n_stages = P.n_stages, stage_bytes = P.stage_bytes;
     pdl_launch_dependents();
 
+    // The three issuing warps run their loops converged; the elected lane issues (see sgs_tc.cuh).
+    const uint32_t ring = smem_u32(smem), full0 = smem_u32(full_bar), empty0 = smem_u32(empty_bar);
     if (warp == 0) {
         // ------------------------------------------------------------------ weight producer
         // Weights do not depend on the previous layer, so this warp never waits for it: it runs ahead
-        // as far as the ring allows.  The warp runs its loop converged; one elected lane issues.
+        // as far as the ring allows.
+        const uint32_t on = elect_one();
         const uint64_t pol_keep = make_policy(1), pol_stream = make_policy(2);
-        int s = 0, g = 0, gi = 0;  // stage, its group, its position in the group
+        int s = 0;
         uint32_t phase = 0;
         bool wrapped = false, ok = true;
         for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x) {
             const GroupEntry &e = es[tile_entry(es, n_entries, t, lane)];
             const int nt = (t - e.tile_begin) / e.mtiles;
             const int wrows = e.swap ? 128 : e.bn_tile;  // rows of the weight box
-            const int f0 = nt * wrows;
-            const uint32_t w_bytes = (uint32_t)(wrows * CHUNK_C * 2);
-            uint8_t *dst0 = smem + (e.swap ? 0 : G_X_BYTES);
-            const CUtensorMap *map_w = &P.maps[e.map_w];
-            const int k = e.k, kw = e.kw, cchunks = e.cchunks, R = e.R;
-            int kind = 0;  // 0 default replacement, 1 keep (inside the cached SubGraph's box, up to channel cacheC), 2 stream
-            int cacheC = 0;
-            if (e.cacheK < 0) kind = 2;
-            else if (f0 < e.cacheK) { kind = 1; cacheC = e.cacheC; }
-            int tap_row = e.tap0;
+            const int f0 = (int)uniform((uint32_t)(nt * wrows));
+            const uint32_t w_bytes = uniform((uint32_t)(wrows * CHUNK_C * 2));
+            const uint32_t dst0 = uniform(ring + (e.swap ? 0u : (uint32_t)G_X_BYTES));
+            const CUtensorMap *map_w = &P.maps[uniform((uint32_t)e.map_w)];
+            const int k = (int)uniform(e.k), kw = (int)uniform(e.kw), cchunks = (int)uniform((uint32_t)e.cchunks), R = (int)uniform((uint32_t)e.R);
+            // channels below hint_c take a hint: the cached SubGraph's box (keep), or everything (stream)
+            const int cacheK = (int)uniform((uint32_t)e.cacheK);
+            const int hint_c = cacheK < 0 ? 0x7fffffff : f0 < cacheK ? (int)uniform((uint32_t)e.cacheC) : 0;
+            const uint64_t pol = cacheK < 0 ? pol_stream : pol_keep;
+            int tap_row = (int)uniform((uint32_t)e.tap0);
             for (int r = 0; r < k && ok; r++, tap_row += R) {
                 for (int sx = 0; sx < kw && ok; sx++) {
                     for (int cc = 0, c0 = 0; cc < cchunks; cc++, c0 += CHUNK_C) {
-                        if (wrapped && gi == 0) ok = __all_sync(0xffffffffu, mbar_wait(&empty_bar[g], phase ^ 1, abort_flag));
-                        if (!ok) break;
-                        if (elect_one()) {
-                            uint8_t *sb = dst0 + s * stage_bytes;
-                            mbar_expect_tx(&full_bar[g], w_bytes);
-                            if (kind == 2) tma_load_3d_hint(sb, map_w, &full_bar[g], c0, tap_row + sx, f0, pol_stream);
-                            else if (kind == 1 && c0 < cacheC) tma_load_3d_hint(sb, map_w, &full_bar[g], c0, tap_row + sx, f0, pol_keep);
-                            else tma_load_3d(sb, map_w, &full_bar[g], c0, tap_row + sx, f0);
-                        }
-                        __syncwarp();
-                        if (++gi == gsz) { gi = 0; ++g; }
-                        if (++s == n_stages) { s = 0; g = 0; phase ^= 1; wrapped = true; }
+                        if (wrapped && !(ok = __all_sync(0xffffffffu, mbar_wait(&empty_bar[s], phase ^ 1, abort_flag)))) break;
+                        const uint32_t sb = dst0 + (uint32_t)(s * stage_bytes), fb = full0 + (uint32_t)(s * 8);
+                        mbar_expect_tx_if(on, fb, w_bytes);
+                        if (c0 < hint_c) tma_load_3d_hint_if(on, sb, map_w, fb, c0, tap_row + sx, f0, pol);
+                        else tma_load_3d_if(on, sb, map_w, fb, c0, tap_row + sx, f0);
+                        if (++s == n_stages) { s = 0; phase ^= 1; wrapped = true; }
                     }
                 }
             }
             const int tn = t + (int)gridDim.x;
-            if (ok && tn < total_tiles && elect_one()) prefetch_tensormap(&P.maps[es[find_entry_serial(es, n_entries, tn)].map_w]);
+            if (ok && tn < total_tiles && on) prefetch_tensormap(&P.maps[es[find_entry_serial(es, n_entries, tn)].map_w]);
             __syncwarp();
         }
-        // the CTA's last group may be partial: arrive for the stages it does not have
-        if (gi != 0 && elect_one())
-            for (; gi < gsz; gi++) mbar_arrive(&full_bar[g]);
     } else if (warp == G_PIX_WARP) {
         // ------------------------------------------------------------------ activation producer
-        int s = 0, g = 0, gi = 0;
+        const uint32_t on = elect_one();
+        int s = 0;
         uint32_t phase = 0;
         bool wrapped = false, ok = true;
         pdl_wait();  // activations (and the buffers this layer overwrites) belong to the previous layers until here
         for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x) {
             const GroupEntry &e = es[tile_entry(es, n_entries, t, lane)];
             const int mt = (t - e.tile_begin) % e.mtiles;
-            const int n0 = (mt / e.tiles_hw) * e.bn, h0 = ((mt % e.tiles_hw) / e.tiles_w) * e.bh, w0 = (mt % e.tiles_w) * e.bw;
-            const uint32_t pix_bytes = (uint32_t)(e.pix_rows * CHUNK_C * 2);
-            uint8_t *dst0 = smem + (e.swap ? G_X_BYTES : 0);
-            const CUtensorMap *map_a = &P.maps[e.map_a];
-            const uint32_t pix_bytes2 = e.pair ? (uint32_t)((&e)[1].pix_rows * CHUNK_C * 2) : 0u;
-            const CUtensorMap *map_a2 = &P.maps[e.pair ? (&e)[1].map_a : e.map_a];
-            const int k = e.k, kw = e.kw, cchunks = e.cchunks, pad = e.p, stride = e.stride;
+            const int n0 = (int)uniform((uint32_t)((mt / e.tiles_hw) * e.bn)), h0 = (int)uniform((uint32_t)(((mt % e.tiles_hw) / e.tiles_w) * e.bh)),
+                      w0 = (int)uniform((uint32_t)((mt % e.tiles_w) * e.bw));
+            const bool pair = uniform(e.pair) != 0;
+            const uint32_t pix_bytes = uniform((uint32_t)(e.pix_rows * CHUNK_C * 2) + (pair ? (uint32_t)((&e)[1].pix_rows * CHUNK_C * 2) : 0u));
+            const uint32_t dst0 = uniform(ring + (e.swap ? (uint32_t)G_X_BYTES : 0u));
+            const int map_a = (int)uniform((uint32_t)e.map_a), map_a2 = (int)uniform((uint32_t)(pair ? (&e)[1].map_a : e.map_a));
+            const int k = (int)uniform(e.k), kw = (int)uniform(e.kw), cchunks = (int)uniform((uint32_t)e.cchunks), pad = (int)uniform(e.p), stride = (int)uniform(e.stride);
             for (int r = 0; r < k && ok; r++) {
                 for (int sx = 0; sx < kw && ok; sx++) {
                     const int dh = r - pad, dw = sx - pad;
                     // stride 2: one of the four parity views, at half the offset
-                    const int ph = stride == 2 ? (dh & 1) : 0, pw = stride == 2 ? (dw & 1) : 0;
-                    const CUtensorMap *m = map_a + ph * 2 + pw;
+                    const int ph = stride == 2 ? (dh & 1) : 0, pw = stride == 2 ? (dw & 1) : 0, view = ph * 2 + pw;
                     const int cw = stride == 2 ? w0 + ((dw - pw) >> 1) : w0 + dw, ch = stride == 2 ? h0 + ((dh - ph) >> 1) : h0 + dh;
                     for (int cc = 0, c0 = 0; cc < cchunks; cc++, c0 += CHUNK_C) {
-                        if (wrapped && gi == 0) ok = __all_sync(0xffffffffu, mbar_wait(&empty_bar[g], phase ^ 1, abort_flag));
-                        if (!ok) break;
-                        if (elect_one()) {
-                            mbar_expect_tx(&full_bar[g], pix_bytes + pix_bytes2);
-                            tma_load_4d(dst0 + s * stage_bytes, m, &full_bar[g], c0, cw, ch, n0);
-                            // (a pair is a single tile of one layer: same tap offsets and parity view, box origin 0)
-                            if (pix_bytes2) tma_load_4d(dst0 + s * stage_bytes + 64 * CHUNK_C * 2, map_a2 + (m - map_a), &full_bar[g], c0, cw, ch, n0);
-                        }
-                        __syncwarp();
-                        if (++gi == gsz) { gi = 0; ++g; }
-                        if (++s == n_stages) { s = 0; g = 0; phase ^= 1; wrapped = true; }
+                        if (wrapped && !(ok = __all_sync(0xffffffffu, mbar_wait(&empty_bar[s], phase ^ 1, abort_flag)))) break;
+                        const uint32_t sb = dst0 + (uint32_t)(s * stage_bytes), fb = full0 + (uint32_t)(s * 8);
+                        mbar_expect_tx_if(on, fb, pix_bytes);
+                        tma_load_4d_if(on, sb, &P.maps[map_a + view], fb, c0, cw, ch, n0);
+                        // (a pair is a single tile of one layer: same tap offsets and parity view, box origin 0)
+                        if (pair) tma_load_4d_if(on, sb + 64 * CHUNK_C * 2, &P.maps[map_a2 + view], fb, c0, cw, ch, n0);
+                        if (++s == n_stages) { s = 0; phase ^= 1; wrapped = true; }
                     }
                 }
             }
             const int tn = t + (int)gridDim.x;
-            if (ok && tn < total_tiles && elect_one()) prefetch_tensormap(&P.maps[es[find_entry_serial(es, n_entries, tn)].map_a]);
+            if (ok && tn < total_tiles && on) prefetch_tensormap(&P.maps[es[find_entry_serial(es, n_entries, tn)].map_a]);
             __syncwarp();
         }
-        if (gi != 0 && elect_one())
-            for (; gi < gsz; gi++) mbar_arrive(&full_bar[g]);
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        int s = 0, g = 0, gi = 0;
+        const uint32_t on = elect_one(), acc_base = uniform(tmem_base);
+        int s = 0, j = 0;
         uint32_t phase = 0;
-        int j = 0;
-        const uint32_t ring = smem_u32(smem);
         bool ok = true;
         for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x, j++) {
             const GroupEntry &e = es[tile_entry(es, n_entries, t, lane)];
@@ -244,36 +226,28 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
             // MMA shape: 128 rows; columns = this tile's filters (normal) or the member's pixels (swapped),
             // rounded up to 16; bf16 x bf16 -> fp32, both operands K-major
             const int n_mma = e.swap ? e.bn_tile : min((int)e.bn_tile, (e.K - nt * e.bn_tile + 15) & ~15);
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n_mma >> 3) << 17) | ((uint32_t)(TILE_M >> 4) << 24);
+            const uint32_t idesc = uniform((1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n_mma >> 3) << 17) | ((uint32_t)(TILE_M >> 4) << 24));
             const int buf = j & 1;
-            const int cchunks = e.cchunks, taps = e.k * e.kw;
-            const int last_ksteps = (e.C - (cchunks - 1) * CHUNK_C + 15) / 16;  // 16-channel steps of a tap's last chunk
+            const int cchunks = (int)uniform((uint32_t)e.cchunks), iters = (int)uniform((uint32_t)(e.k * e.kw)) * cchunks;
+            const int last_ksteps = (int)uniform((uint32_t)((e.C - (cchunks - 1) * CHUNK_C + 15) / 16));  // 16-channel steps of a tap's last chunk
             ok = j < 2 || mbar_wait(&acc_empty[buf], ((j >> 1) - 1) & 1, abort_flag);  // epilogue drained this buffer
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
-            const uint32_t d_tmem = tmem_base + (uint32_t)(buf * G_ACC_COLS);
-            uint32_t accumulate = 0;
-            for (int tap = 0; tap < taps && ok; tap++) {
-                for (int cc = 0; cc < cchunks; cc++) {
-                    if (gi == 0) {
-                        ok = __all_sync(0xffffffffu, mbar_wait(&full_bar[g], phase, abort_flag));
-                        if (!ok) break;
-                        tc_fence_after();
-                    }
-                    const int ksteps = cc == cchunks - 1 ? last_ksteps : CHUNK_C / 16;
-                    const uint32_t sx_ = ring + (uint32_t)(s * stage_bytes);
-                    const uint64_t da = smem_desc_sw128(sx_), db = smem_desc_sw128(sx_ + G_X_BYTES);
-                    if (elect_one()) {
-                        for (int q = 0; q < ksteps; q++) { umma_bf16(d_tmem, da + (uint64_t)(2 * q), db + (uint64_t)(2 * q), idesc, accumulate); accumulate = 1; }
-                        if (gi == gsz - 1) umma_commit(&empty_bar[g]);  // frees the group once the MMAs of all its stages have read it
-                        if (tap == taps - 1 && cc == cchunks - 1) umma_commit(&acc_full[buf]);  // accumulator complete
-                    }
-                    __syncwarp();
-                    accumulate = 1;
-                    if (++gi == gsz) { gi = 0; ++g; }
-                    if (++s == n_stages) { s = 0; g = 0; phase ^= 1; }
-                }
+            const uint32_t d_tmem = acc_base + (uint32_t)(buf * G_ACC_COLS);
+            for (int i = 0, cc = 0; i < iters; i++) {
+                if (!(ok = __all_sync(0xffffffffu, mbar_wait(&full_bar[s], phase, abort_flag)))) break;
+                tc_fence_after();
+                const int ksteps = cc == cchunks - 1 ? last_ksteps : CHUNK_C / 16;
+                const uint32_t sx_ = ring + (uint32_t)(s * stage_bytes);
+                const uint64_t da = smem_desc_sw128(sx_), db = smem_desc_sw128(sx_ + G_X_BYTES);
+#pragma unroll
+                for (int q = 0; q < CHUNK_C / 16; q++)
+                    umma_if<false>(q < ksteps ? on : 0u, d_tmem, da + (uint64_t)(2 * q), db + (uint64_t)(2 * q), idesc, (i > 0 || q > 0) ? 1u : 0u);
+                umma_commit_if(on, empty0 + (uint32_t)(s * 8));  // frees the stage once these MMAs have read it
+                if (i == iters - 1) umma_commit_if(on, smem_u32(&acc_full[buf]));  // accumulator complete
+                if (++cc == cchunks) cc = 0;
+                if (++s == n_stages) { s = 0; phase ^= 1; }
             }
         }
     } else {
@@ -551,9 +525,6 @@ void GroupLaunch::add(void *host_entry, const TcConvPlan &pl, const ConvArgs &a)
     impl->prm.total_tiles += e.mtiles * (int)pl.grid.y;
 }
 
-static int g_group_stages = 0;  // 0 = default
-void tc_group_set_stage_group(int stages) { g_group_stages = stages; }
-
 cudaError_t tc_group_init(int) {
     cudaError_t e = cudaFuncSetAttribute(conv_group_kernel<TC_GROUP_MAPS_SMALL>, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM_BYTES);
     if (e != cudaSuccess) return e;
@@ -572,8 +543,6 @@ cudaError_t GroupLaunch::launch(size_t window_max, int sms, cudaStream_t st) {
     const int col_rows = impl->col_rows <= 64 ? 64 : impl->col_rows <= 128 ? 128 : 256;
     impl->prm.stage_bytes = G_X_BYTES + col_rows * CHUNK_C * 2;
     impl->prm.n_stages = G_RING_BYTES / impl->prm.stage_bytes;  // 8, 6 or 4
-    const int want = g_group_stages > 0 ? g_group_stages : 1;  // (measured on batch-16 members: 2 or 4 stages per barrier pair change nothing for narrow tiles and cost 10-25 % on 256-column tiles)
-    impl->prm.group = (want <= impl->prm.n_stages / 2 && impl->prm.n_stages % want == 0) ? want : 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)std::min(impl->prm.total_tiles, std::max(1, sms)));
     cfg.blockDim = dim3(G_THREADS);

@@ -103,29 +103,30 @@ __global__ void __launch_bounds__(192, 1) conv_tc_kernel(const __grid_constant__
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        // The whole warp runs the loop converged, so every operand of the copy instructions is a
-        // warp-uniform value; only the copy instructions themselves are issued by one elected lane.
+        // The whole warp runs the loops converged; the elected lane issues (see sgs_tc.cuh).
+        const uint32_t on = elect_one();
         const uint64_t pol_keep = make_policy(1), pol_stream = make_policy(2);
         const uint32_t tx = (uint32_t)(p.bw * p.bh * p.bn * CHUNK_C * 2 + B_STAGE_BYTES);
         int weight_policy = p.weight_policy, cacheK = p.cacheK, cacheC = p.cacheC;
         if (p.cache_tbl) {
-            weight_policy = __ldg(p.cache_tbl);
-            cacheK = __ldg(p.cache_tbl + 1 + 2 * p.layer);
-            cacheC = __ldg(p.cache_tbl + 2 + 2 * p.layer);
+            weight_policy = (int)uniform((uint32_t)__ldg(p.cache_tbl));
+            cacheK = (int)uniform((uint32_t)__ldg(p.cache_tbl + 1 + 2 * p.layer));
+            cacheC = (int)uniform((uint32_t)__ldg(p.cache_tbl + 2 + 2 * p.layer));
         }
+        // policy 1: tiles of the cached SubGraph are kept (evict-last), the rest take the default replacement (measured:
+        // marking them evict-first loses to plain LRU whenever the SuperNet fits in L2); policy 2: everything evict-first
+        // (the "no reuse at all" reference point)
+        const uint64_t pol = weight_policy == 2 ? pol_stream : pol_keep;
+        const int hint_c = weight_policy == 2 ? 0x7fffffff : (weight_policy == 1 && f0 < cacheK) ? cacheC : 0;  // channels below: hinted
         // (tap row r, tap column sx, channel chunk cc) of iteration it_begin, then stepped
         int cc = it_begin % p.cchunks, tap = it_begin / p.cchunks;
         int r = tap / p.k, sx = tap % p.k;
+        const uint32_t ring = smem_u32(smem), full0 = smem_u32(full_bar);
         auto load_weights = [&](int s, int c0, int tapw) {
-            uint8_t *sb = smem + s * STAGE_BYTES + A_STAGE_BYTES;
-            mbar_expect_tx(&full_bar[s], tx);
-            // policy 1: tiles of the cached SubGraph are kept (evict-last), the rest take the default
-            // replacement (measured: marking them evict-first loses to plain LRU whenever the SuperNet
-            // fits in L2); policy 2: everything evict-first (the "no reuse at all" reference point)
-            const bool in_box = weight_policy == 1 && f0 < cacheK && c0 < cacheC;
-            if (weight_policy == 2) tma_load_3d_hint(sb, &p.tmW, &full_bar[s], c0, tapw, f0, pol_stream);
-            else if (in_box) tma_load_3d_hint(sb, &p.tmW, &full_bar[s], c0, tapw, f0, pol_keep);
-            else tma_load_3d(sb, &p.tmW, &full_bar[s], c0, tapw, f0);
+            const uint32_t sb = ring + (uint32_t)(s * STAGE_BYTES + A_STAGE_BYTES), fb = full0 + (uint32_t)(s * 8);
+            mbar_expect_tx_if(on, fb, tx);
+            if (c0 < hint_c) tma_load_3d_hint_if(on, sb, &p.tmW, fb, c0, tapw, f0, pol);
+            else tma_load_3d_if(on, sb, &p.tmW, fb, c0, tapw, f0);
         };
         // Weights do not depend on the previous layer: fill the first stages' weight halves before
         // waiting for it, so that their latency overlaps the previous layer's tail.
@@ -133,54 +134,48 @@ __global__ void __launch_bounds__(192, 1) conv_tc_kernel(const __grid_constant__
             int cc2 = cc, r2 = r, sx2 = sx;
             const int pre = min(n_it, STAGES);
             for (int i = 0; i < pre; i++) {
-                if (elect_one()) load_weights(i, cc2 * CH, (p.o + r2) * p.R + (p.o + sx2));
-                __syncwarp();
+                load_weights(i, cc2 * CH, (p.o + r2) * p.R + (p.o + sx2));
                 if (++cc2 == p.cchunks) { cc2 = 0; if (++sx2 == p.k) { sx2 = 0; ++r2; } }
             }
         }
         pdl_wait();  // activations (and the buffers this layer overwrites) belong to the previous layers until here
+        int s = 0;
+        uint32_t phase = 0;
         for (int i = 0; i < n_it; i++) {
-            const int s = i % STAGES, round = i / STAGES;
-            bool ok = round == 0 || mbar_wait(&empty_bar[s], (round - 1) & 1, abort_flag);
-            if (!__all_sync(0xffffffffu, ok)) break;
+            if (i >= STAGES && !__all_sync(0xffffffffu, mbar_wait(&empty_bar[s], phase ^ 1, abort_flag))) break;
             const int c0 = cc * CH;
-            uint8_t *sa = smem + s * STAGE_BYTES;
+            const uint32_t sa = ring + (uint32_t)(s * STAGE_BYTES), fb = full0 + (uint32_t)(s * 8);
             const int dh = r - p.p, dw = sx - p.p;
-            if (elect_one()) {
-                if (round > 0) load_weights(s, c0, (p.o + r) * p.R + (p.o + sx));
-                if (p.stride == 1) {
-                    tma_load_4d(sa, &p.tmA[0], &full_bar[s], c0, w0 + dw, h0 + dh, n0);
-                } else {
-                    const int ph = dh & 1, pw = dw & 1;
-                    tma_load_4d(sa, &p.tmA[ph * 2 + pw], &full_bar[s], c0, w0 + ((dw - pw) >> 1), h0 + ((dh - ph) >> 1), n0);
-                }
+            if (i >= STAGES) load_weights(s, c0, (p.o + r) * p.R + (p.o + sx));
+            if (p.stride == 1) {
+                tma_load_4d_if(on, sa, &p.tmA[0], fb, c0, w0 + dw, h0 + dh, n0);
+            } else {
+                const int ph = dh & 1, pw = dw & 1;
+                tma_load_4d_if(on, sa, &p.tmA[ph * 2 + pw], fb, c0, w0 + ((dw - pw) >> 1), h0 + ((dh - ph) >> 1), n0);
             }
-            __syncwarp();
             if (++cc == p.cchunks) { cc = 0; if (++sx == p.k) { sx = 0; ++r; } }
+            if (++s == STAGES) { s = 0; phase ^= 1; }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        // Same structure: converged warp, one elected lane issues the MMAs and their commits.
-        bool ok = true;
-        int cc = it_begin % p.cchunks;
+        const uint32_t on = elect_one(), d_tmem = uniform(tmem_base), ring = smem_u32(smem), empty0 = smem_u32(empty_bar);
+        const int last_ksteps = (p.C - (p.cchunks - 1) * CH + KS - 1) / KS;  // MMAs of a tap's last chunk
+        int cc = it_begin % p.cchunks, s = 0;
+        uint32_t phase = 0;
         for (int i = 0; i < n_it; i++) {
-            const int s = i % STAGES, round = i / STAGES;
-            ok = __all_sync(0xffffffffu, mbar_wait(&full_bar[s], round & 1, abort_flag));
-            if (!ok) break;
+            if (!__all_sync(0xffffffffu, mbar_wait(&full_bar[s], phase, abort_flag))) break;
             tc_fence_after();
-            const int ksteps = (min(CH, p.C - cc * CH) + KS - 1) / KS;
-            const uint32_t sa = smem_u32(smem + s * STAGE_BYTES), sb = sa + A_STAGE_BYTES;
-            const uint64_t da = smem_desc_sw128(sa), db = smem_desc_sw128(sb);
-            if (elect_one()) {
-                for (int q = 0; q < ksteps; q++) {
-                    if (I8) umma_i8(tmem_base, da + (uint64_t)(2 * q), db + (uint64_t)(2 * q), IDESC, (i > 0 || q > 0) ? 1u : 0u);
-                    else umma_bf16(tmem_base, da + (uint64_t)(2 * q), db + (uint64_t)(2 * q), IDESC, (i > 0 || q > 0) ? 1u : 0u);
-                }
-                umma_commit(&empty_bar[s]);  // frees the stage once these MMAs have read it
-                if (i == n_it - 1) umma_commit(&accum_bar);  // accumulator complete
-            }
-            __syncwarp();
+            const bool last = cc == p.cchunks - 1;
+            const int ksteps = last ? last_ksteps : CH / KS;
+            const uint32_t sa = ring + (uint32_t)(s * STAGE_BYTES);
+            const uint64_t da = smem_desc_sw128(sa), db = smem_desc_sw128(sa + A_STAGE_BYTES);
+#pragma unroll
+            for (int q = 0; q < CH / KS; q++)
+                umma_if<I8>(q < ksteps ? on : 0u, d_tmem, da + (uint64_t)(2 * q), db + (uint64_t)(2 * q), IDESC, (i > 0 || q > 0) ? 1u : 0u);
+            umma_commit_if(on, empty0 + (uint32_t)(s * 8));  // frees the stage once these MMAs have read it
+            if (i == n_it - 1) umma_commit_if(on, smem_u32(&accum_bar));  // accumulator complete
             if (++cc == p.cchunks) cc = 0;
+            if (++s == STAGES) { s = 0; phase ^= 1; }
         }
     } else {
         // ------------------------------------------------------------------ epilogue (warps 2..5)

@@ -270,6 +270,5 @@ size_t subnet_kernel_smem();  // dynamic shared memory of a block
 int subnet_kernel_blocks_per_sm();
 cudaError_t subnet_kernel_launch(const PqParams &p, int blocks, cudaStream_t st);
 size_t subnet_kernel_held_max();  // largest weight buffer a block can keep
-void tc_group_set_stage_group(int stages);  // tuning: stages per barrier pair of the grouped kernel (0 = default)
 
 }  // namespace sgs

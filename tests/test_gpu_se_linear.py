@@ -35,13 +35,14 @@ def test_linear_rows(rows, K, C, ld):
     dw, db, dx = torch.from_numpy(w).cuda().to(torch.bfloat16), torch.from_numpy(b).cuda(), torch.from_numpy(x).cuda()
     ref = x.astype(np.float64) @ w[:, :C].astype(np.float64).T + b
     for grouped in (False, True):  # one query of `rows` images; `rows` members of one image
-        dy = torch.full((rows, K), 77.0, device="cuda")
         n, per = (rows, 1) if grouped else (1, rows)
+        dy = [torch.full((per, K), 77.0, device="cuda") for _ in range(n)]
+        dxs = [dx[i * per:(i + 1) * per].clone() for i in range(n)]
         d = [sgs.AuxDesc(kind=SGS_AUX_LINEAR, dtype=sgs.SGS_BF16, N=per, H=1, W=1, C=C, K=K, ld=ld, act=0)] * n
-        a = [sgs.AuxArgs(x=dx[i * per:].data_ptr(), y=dy[i * per:].data_ptr(), w=dw.data_ptr(), bias=db.data_ptr()) for i in range(n)]
+        a = [sgs.AuxArgs(x=dxs[i].data_ptr(), y=dy[i].data_ptr(), w=dw.data_ptr(), bias=db.data_ptr()) for i in range(n)]
         sgs.aux_op(d, a, grouped, torch.cuda.current_stream().cuda_stream)
         torch.cuda.synchronize()
-        assert np.abs(dy.cpu().numpy() - ref).max() <= 2e-5 * np.abs(ref).max()
+        assert np.abs(torch.cat(dy).cpu().numpy() - ref).max() <= 2e-5 * np.abs(ref).max()
 
 
 @pytest.mark.parametrize("k", [1, 3, 5])
