@@ -314,9 +314,8 @@ sgs_status_t sgs_subnet_cost(const sgs_supernet_t *net, const sgs_subnet_cfg_t *
  * 16-byte aligned; kernels larger than 1x1 at stride 2 need at least 2x2 pixels), 1 = CUDA-core kernel, 2 = tensor cores or
  * SGS_EUNSUPPORTED.  weight_policy 0 = no L2 hint, 1 = evict-last for weight tiles with filter <
  * cache_k and channel < cache_c (default replacement for the rest), 2 = all weights evict-first.
- * Asynchronous on `cuda_stream`.  The tensor-core path may split the reduction over several CTAs
- * using a per-device scratch buffer that this function allocates on demand (cudaMalloc) and keeps;
- * calls that overlap on the same device must therefore not run concurrently.
+ * Asynchronous on `cuda_stream`.  The tensor-core path may split the reduction over a cluster of CTAs, whose partial sums
+ * stay in shared memory: no device memory is allocated.
  */
 typedef struct {
     int N, H, W, C, K;      /* input dims, sliced channels C, sliced filters K */
@@ -337,26 +336,20 @@ sgs_status_t sgs_conv2d_sliced(const sgs_conv_desc_t *desc, const void *d_x, con
  *
  * Who needs it: serving processes that gave all device memory to their own pool at start-up (a cudaMalloc
  * from a library then simply fails), and latency-critical loops that cannot afford the device-wide
- * synchronisation cudaMalloc and cudaFree imply.  sgs_conv2d_sliced may call cudaMalloc to
- * grow its split-reduction scratch; this variant never does.  Its scratch is a fixed array of
- * SGS_STATIC_SCRATCH_BYTES that is part of the library image, so every GPU that loads the library
- * holds that much memory until the process exits.
+ * synchronisation cudaMalloc and cudaFree imply.  Neither this call nor sgs_conv2d_sliced allocates; this one keeps its
+ * time-out status word inside the library image and takes the tensor-core path only.
  *
  * Same arguments, layouts and result as sgs_conv2d_sliced, with these limits:
  *   - tensor-core path only: dtype SGS_BF16, not depthwise, impl 0 or 2; otherwise SGS_EUNSUPPORTED
  *     (also for shapes the tensor-core kernel does not take).
- *   - a layer whose split reduction needs more than SGS_STATIC_SCRATCH_BYTES of partial tiles is
- *     rejected with SGS_ENOMEM and nothing is launched.  (Partial tiles take
- *     splits * N*Ho*Wo*K * 4 bytes with splits <= 8; layers large enough to fill the GPU are not split
- *     and need no scratch at all.  Set split_k_off = 1 to run any shape without scratch.)
+ *   - a layer whose split reduction, written out, would take more than SGS_STATIC_SCRATCH_BYTES of partial tiles is
+ *     rejected with SGS_ENOMEM and nothing is launched.  (Partial tiles would take
+ *     splits * N*Ho*Wo*K * 4 bytes with splits <= 8; layers large enough to fill the GPU are not split.  Set
+ *     split_k_off = 1 to run any shape.)
  *   - no cudaMalloc, cudaFree or other allocating device call is made, on any call.
- * The first call on each device looks up the device address of the array and sets the kernels'
- * shared-memory limit; make that first call outside any stream capture.  Later calls only enqueue
- * kernels on `cuda_stream` (nothing in the array has to start at zero: what the second step of a
- * split reduction reads was written by the first step of the same call).
- * All calls on a device share the one array and it keeps whatever the last call left in it: two calls
- * whose kernels may overlap on the GPU (different streams, or concurrent host threads) race on it and
- * give wrong results.  Issue them on one stream, or order them with events.
+ * The first call on each device looks up the device address of the status word and sets the kernels'
+ * shared-memory limit; make that first call outside any stream capture.  Later calls only enqueue a
+ * kernel on `cuda_stream`.
  */
 #define SGS_STATIC_SCRATCH_BYTES (8u << 20)
 sgs_status_t sgs_conv2d_sliced_static(const sgs_conv_desc_t *desc, const void *d_x, const void *d_w, const float *d_scale,

@@ -176,7 +176,6 @@ struct sgs_supernet {
     struct Slot {
         void *act[4] = {nullptr, nullptr, nullptr, nullptr};
         float *vec[3] = {nullptr, nullptr, nullptr};
-        float *ws = nullptr;        // split-K scratch of the tensor-core kernel
         void *stage_in = nullptr;   // device staging for host-buffer streams
         float *stage_out = nullptr;
         cudaStream_t st = nullptr;  // internal stream (slots >= 1)
@@ -206,7 +205,6 @@ struct sgs_supernet {
     int *tbl_ring = nullptr;        // pinned host ring of table images (async uploads need stable sources)
     cudaEvent_t tbl_ring_ev[16] = {};  // upload of ring entry i has completed
     int tbl_ring_pos = 0;
-    size_t splitk_ws_elems = 0;
     size_t stage_in_bytes = 0, stage_out_bytes = 0;
     size_t device_bytes = 0;
     std::unordered_map<std::string, std::unique_ptr<Plan>> plans;
@@ -522,11 +520,13 @@ sgs_status_t build_plan(sgs_supernet *net, const sgs_subnet_cfg_t *cfg, int batc
     plan->batch = batch; plan->res = res;
     plan->slices = slices_for(net, cfg);
     Builder B{net, plan, batch};
-    // Waves of the ResNet-shaped family on bf16 handles: every convolution runs in the grouped tensor-core kernel
-    // (all channel counts are multiples of 8, and every stride-2 layer sees at least 2x2 pixels), so the activation
-    // tensors can be padded to 16-channel pixels.  choose_impls refuses a padded plan otherwise.
-    B.padded = net->family == SGS_RESNET && net->throughput_mode == 2 && net->dtype == SGS_BF16 && !net->force_plain &&
-               tc_available() && (res >= 64 || res % 32 == 0) && net->stem_win_w != nullptr && net->pad_channels;
+    // ResNet-shaped family on bf16 handles: every convolution runs on the tensor cores (all channel counts are multiples of
+    // 8, every stride-2 layer sees at least 2x2 pixels, and single queries have the patch-matrix stem), so the activation
+    // tensors can be padded to 16-channel pixels: the copy unit moves rows that start or end inside a 32-byte sector at a
+    // third of the rate (0.35 us per 24 KB stage of a query's small layers).  choose_impls refuses a padded plan otherwise.
+    const bool stem_tc = net->throughput_mode == 2 ? net->stem_win_w != nullptr : (net->stem_gemm_w != nullptr && res % 8 == 0 && res <= 1024);
+    B.padded = net->family == SGS_RESNET && stem_tc && net->dtype == SGS_BF16 && !net->force_plain &&
+               tc_available() && (res >= 64 || res % 32 == 0) && net->pad_channels;
     plan->padded = B.padded;
     int H = res, W = res;
     // activation buffers: X current tensor, T1/T2 temporaries, SC shortcut
@@ -598,10 +598,9 @@ sgs_status_t build_plan(sgs_supernet *net, const sgs_subnet_cfg_t *cfg, int batc
 
 // Makes sure `n_slots` slots exist, each with buffers for the sizes in use.
 // Frees the activation / vector / split-reduction buffers of a slot (the sizes are the handle's current ones).
-void release_slot_buffers(sgs_supernet *net, sgs_supernet::Slot &sl, bool act, bool vec, bool ws) {
+void release_slot_buffers(sgs_supernet *net, sgs_supernet::Slot &sl, bool act, bool vec) {
     for (int i = 0; i < 4 && act; i++) { dev_free(net, sl.act[i], net->act_elems * net->elem() + 256); sl.act[i] = nullptr; }
     for (int i = 0; i < 3 && vec; i++) { dev_free(net, sl.vec[i], net->vec_elems * 4); sl.vec[i] = nullptr; }
-    if (ws) { dev_free(net, sl.ws, net->splitk_ws_elems * 4); sl.ws = nullptr; }
 }
 
 sgs_status_t ensure_slots(sgs_supernet *net, int n_slots) {
@@ -614,9 +613,8 @@ sgs_status_t ensure_slots(sgs_supernet *net, int n_slots) {
         sgs_status_t st = SGS_OK;
         for (int i = 0; i < 4 && net->act_elems && st == SGS_OK; i++) st = dev_alloc(net, &sl.act[i], net->act_elems * net->elem() + 256);
         for (int i = 0; i < 3 && net->vec_elems && st == SGS_OK; i++) st = dev_alloc(net, (void **)&sl.vec[i], net->vec_elems * 4);
-        if (net->splitk_ws_elems && st == SGS_OK) st = dev_alloc(net, (void **)&sl.ws, net->splitk_ws_elems * 4);
         if (st != SGS_OK) {  // nothing of a half-built slot stays behind
-            release_slot_buffers(net, sl, true, true, true);
+            release_slot_buffers(net, sl, true, true);
             if (sl.st) cudaStreamDestroy(sl.st);
             if (sl.ev) cudaEventDestroy(sl.ev);
             return st;
@@ -634,13 +632,13 @@ sgs_status_t ensure_workspace(sgs_supernet *net, size_t act_elems, int batch) {
     if (act_elems > net->act_elems) {
         drop_graphs(net);
         for (auto &kv : net->plans) kv.second->prepared = false;
-        for (auto &sl : net->slots) release_slot_buffers(net, sl, true, false, false);
+        for (auto &sl : net->slots) release_slot_buffers(net, sl, true, false);
         net->act_elems = act_elems;
         sgs_status_t st = SGS_OK;
         for (auto &sl : net->slots)
             for (int i = 0; i < 4 && st == SGS_OK; i++) st = dev_alloc(net, &sl.act[i], act_elems * net->elem() + 256);
         if (st != SGS_OK) {
-            for (auto &sl : net->slots) release_slot_buffers(net, sl, true, false, false);
+            for (auto &sl : net->slots) release_slot_buffers(net, sl, true, false);
             net->act_elems = 0;
             return st;
         }
@@ -648,13 +646,13 @@ sgs_status_t ensure_workspace(sgs_supernet *net, size_t act_elems, int batch) {
     size_t vneed = (size_t)batch * 2048;
     if (vneed > net->vec_elems) {
         drop_graphs(net);
-        for (auto &sl : net->slots) release_slot_buffers(net, sl, false, true, false);
+        for (auto &sl : net->slots) release_slot_buffers(net, sl, false, true);
         net->vec_elems = vneed;
         sgs_status_t st = SGS_OK;
         for (auto &sl : net->slots)
             for (int i = 0; i < 3 && st == SGS_OK; i++) st = dev_alloc(net, (void **)&sl.vec[i], vneed * 4);
         if (st != SGS_OK) {
-            for (auto &sl : net->slots) release_slot_buffers(net, sl, false, true, false);
+            for (auto &sl : net->slots) release_slot_buffers(net, sl, false, true);
             net->vec_elems = 0;
             return st;
         }
@@ -664,10 +662,7 @@ sgs_status_t ensure_workspace(sgs_supernet *net, size_t act_elems, int batch) {
 
 // Chooses the implementation of every convolution of a plan and fixes its buffer addresses (the
 // tensor maps of the tensor-core kernel hold absolute addresses of the activation workspaces).
-// prepare_impls touches nothing but the plan (several plans may be prepared at the same time by different threads);
-// choose_impls = prepare + the part that may grow the handle's split-reduction scratch.
-sgs_status_t prepare_impls(const sgs_supernet *net, Plan *plan, size_t *ws_need_out, std::string *err) {
-    size_t ws_need = 0;
+sgs_status_t choose_impls(sgs_supernet *net, Plan *plan) {
     for (Op &op : plan->ops) {
         if (op.type != OP_CONV && op.type != OP_DW) continue;
         const sgs_supernet::Slot &sl = net->slots[plan->slot];
@@ -681,41 +676,10 @@ sgs_status_t prepare_impls(const sgs_supernet *net, Plan *plan, size_t *ws_need_
         if (net->dtype != SGS_BF16 || net->force_plain || !tc_available()) continue;
         std::string why;
         op.tc = tc_conv_prepare(op.conv, net->device, &why);
-        if (!op.tc && op.conv.win) { *err = "window view of the stem: " + why; return SGS_EUNSUPPORTED; }
-        if (!op.tc && plan->padded) { *err = "padded activation layout needs the tensor-core kernel: " + why; return SGS_EUNSUPPORTED; }
-        if (op.tc) {
-            op.impl = 1;
-            ws_need = std::max(ws_need, tc_conv_ws_elems(*op.tc));
-        }
+        if (!op.tc && op.conv.win) return fail(net, SGS_EUNSUPPORTED, "window view of the stem: " + why);
+        if (!op.tc && plan->padded) return fail(net, SGS_EUNSUPPORTED, "padded activation layout needs the tensor-core kernel: " + why);
+        if (op.tc) op.impl = 1;
     }
-    *ws_need_out = ws_need;
-    return SGS_OK;
-}
-
-sgs_status_t grow_splitk_scratch(sgs_supernet *net, size_t ws_need) {
-    if (ws_need > net->splitk_ws_elems) {
-        drop_graphs(net);
-        for (auto &sl : net->slots) release_slot_buffers(net, sl, false, false, true);  // (cudaFree waits for work in flight)
-        net->splitk_ws_elems = ws_need;
-        sgs_status_t st = SGS_OK;
-        for (auto &sl : net->slots)
-            if (st == SGS_OK) st = dev_alloc(net, (void **)&sl.ws, ws_need * 4);
-        if (st != SGS_OK) {
-            for (auto &sl : net->slots) release_slot_buffers(net, sl, false, false, true);
-            net->splitk_ws_elems = 0;
-            for (auto &kv : net->plans) kv.second->prepared = false;  // (plans that counted on the scratch choose again)
-            return st;
-        }
-    }
-    return SGS_OK;
-}
-
-sgs_status_t choose_impls(sgs_supernet *net, Plan *plan) {
-    size_t ws_need = 0;
-    std::string err;
-    sgs_status_t st = prepare_impls(net, plan, &ws_need, &err);
-    if (st != SGS_OK) return fail(net, st, err);
-    if ((st = grow_splitk_scratch(net, ws_need)) != SGS_OK) return st;
     plan->prepared = true;
     return SGS_OK;
 }
@@ -859,9 +823,8 @@ sgs_status_t launch_op(sgs_supernet *net, Plan *plan, Op &op, const void *d_inpu
         ConvArgs a = op.conv;
         if (op.in < 0) a.x = d_input;
         a.cache_tbl = net->cache_tbl; a.layer = op.layer;
-        a.ws = sl.ws; a.ws_elems = net->splitk_ws_elems;
         if (op.type == OP_DW) { CU(launch_dw<T>(a, st)); net->kernel_launches++; }
-        else if (op.impl == 1) { int n = 0; CU(tc_conv_launch(*op.tc, a, st, &n)); net->kernel_launches += n; }
+        else if (op.impl == 1) { CU(tc_conv_launch(*op.tc, a, st)); net->kernel_launches++; }
         else { CU(launch_conv_plain<T>(a, st)); net->kernel_launches++; }
         break;
     }
@@ -1290,7 +1253,7 @@ sgs_status_t sgs_supernet_load(const sgs_arch_desc_t *arch, const void *host_blo
     if (e == cudaSuccess && bf && !net->layers.empty() && net->layers[0].kind == KIND_CONV && net->layers[0].C == 3) {
         const StoredLayer &L = net->layers[0];
         const int KK = L.R * L.R * 3;
-        net->stem_kkp = (KK + 7) / 8 * 8;
+        net->stem_kkp = (KK + 15) / 16 * 16;  // (rows of whole 32-byte sectors)
         if (dev_alloc(net, &net->stem_gemm_w, (size_t)L.K * net->stem_kkp * 2) != SGS_OK) e = cudaErrorMemoryAllocation;
         else e = launch_stem_gemm_weights(L.w, net->stem_gemm_w, L.K, KK, net->stem_kkp, 0);
         if (e == cudaSuccess && L.R <= 8) {
@@ -1341,7 +1304,6 @@ void sgs_supernet_free(sgs_supernet_t *net) {
     for (auto &sl : net->slots) {
         for (int i = 0; i < 4; i++) cudaFree(sl.act[i]);
         for (int i = 0; i < 3; i++) cudaFree(sl.vec[i]);
-        cudaFree(sl.ws);
         cudaFree(sl.stage_in);
         cudaFree(sl.stage_out);
         if (sl.ev) cudaEventDestroy(sl.ev);
@@ -2652,8 +2614,7 @@ long long sgs_get_counter(const sgs_supernet_t *net, const char *name) {
 
 const char *sgs_last_error(const sgs_supernet_t *net) { return net ? net->err.c_str() : "null handle"; }
 
-// Stand-alone sliced convolution.  The split-K scratch of the tensor-core kernel is one buffer per
-// device, grown on demand and shared by all calls of this function.
+// Stand-alone sliced convolution.
 sgs_status_t sgs_conv2d_sliced(const sgs_conv_desc_t *d, const void *d_x, const void *d_w, const float *d_scale,
                                const float *d_shift, const void *d_res, void *d_y, void *cuda_stream) {
     if (!d || !d_x || !d_w || !d_scale || !d_shift || !d_y) return SGS_EINVAL;
@@ -2669,6 +2630,7 @@ sgs_status_t sgs_conv2d_sliced(const sgs_conv_desc_t *d, const void *d_x, const 
     a.Ho = (d->H + 2 * p - d->k) / d->stride + 1;
     a.Wo = (d->W + 2 * p - d->k) / d->stride + 1;
     a.cacheK = d->cache_k; a.cacheC = d->cache_c; a.weight_policy = d->weight_policy;
+    a.no_split = d->split_k_off;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     cudaError_t e;
     if (d->depthwise) {
@@ -2682,18 +2644,7 @@ sgs_status_t sgs_conv2d_sliced(const sgs_conv_desc_t *d, const void *d_x, const 
         std::string why;
         std::shared_ptr<TcConvPlan> plan = tc_conv_prepare(a, dev, &why);
         if (plan) {
-            static float *ws[64] = {};
-            static size_t ws_elems[64] = {};
-            const size_t need = d->split_k_off ? 0 : tc_conv_ws_elems(*plan);
-            if (need > ws_elems[dev]) {
-                cudaFree(ws[dev]);
-                ws[dev] = nullptr; ws_elems[dev] = 0;
-                if (cudaMalloc((void **)&ws[dev], need * 4) != cudaSuccess) return SGS_ENOMEM;
-                ws_elems[dev] = need;
-            }
-            if (!d->split_k_off) { a.ws = ws[dev]; a.ws_elems = ws_elems[dev]; }
-            int n = 0;
-            e = tc_conv_launch(*plan, a, st, &n);
+            e = tc_conv_launch(*plan, a, st);
             return e == cudaSuccess ? SGS_OK : SGS_ECUDA;
         }
     }
@@ -2728,8 +2679,7 @@ sgs_status_t sgs_conv2d_sliced_i8(const sgs_conv_i8_desc_t *d, const void *d_x, 
     std::string why;
     std::shared_ptr<TcConvPlan> plan = tc_conv_prepare(a, dev, &why);
     if (!plan) return SGS_EUNSUPPORTED;
-    int n = 0;
-    return tc_conv_launch(*plan, a, (cudaStream_t)cuda_stream, &n) == cudaSuccess ? SGS_OK : SGS_ECUDA;
+    return tc_conv_launch(*plan, a, (cudaStream_t)cuda_stream) == cudaSuccess ? SGS_OK : SGS_ECUDA;
 }
 
 // Non-convolution layers on caller tensors (see sgs.h).  Mirrors the dispatch of launch_op / wave_impl.

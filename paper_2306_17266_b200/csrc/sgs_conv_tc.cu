@@ -22,8 +22,8 @@
 // L2 evict-last policy so that the shared weights stay on chip across queries; the distinct weights
 // of each SubNet take the default replacement.
 //
-// Warp roles (192 threads): warp 0 = TMA producer, warp 1 = MMA issuer and TMEM owner, warps 2..5 =
-// epilogue (one TMEM lane quadrant each).  Every wait is bounded; when one runs out the kernel sets
+// Warp roles (320 threads): warp 0 = TMA producer, warp 1 = MMA issuer and TMEM owner, warps 2..9 =
+// epilogue (a TMEM lane quadrant and half of the columns each).  Every wait is bounded; when one runs out the kernel sets
 // a status word, lets its in-flight copies land, frees its tensor memory and returns.
 #include "sgs_tc.cuh"
 
@@ -31,6 +31,7 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 #include <unordered_map>
 
 namespace sgs {
@@ -38,25 +39,56 @@ namespace sgs {
 namespace {
 
 // ---------------------------------------------------------------------------------------------
-// The kernel.  grid = (m tiles, n tiles, K splits), block = 192.
-// Dynamic shared memory (1024-byte aligned): STAGES x [A tile 16 KB | B tile BN*128 B].
+// The kernel.  grid = (m tiles, n tiles, K splits), block = 320, the splits of a tile form a cluster.
+// Dynamic shared memory (1024-byte aligned): p.stages x [A tile 16 KB | B tile BN*128 B]; when the MMAs are done, the
+// tile's accumulator [128][BN + 4] in its place.
+//
+// What bounds it on a query of one or a few images: the chain of latencies of a layer, not a rate.  Time stamps of one
+// query's layers (B200): 1.1 us from the previous layer's last block to the end of the wait, 1.1 us to the first operands,
+// then one copy latency per ring of stages, 1.1 us (3 us with a residual) for an epilogue whose lanes each wrote their own
+// pixel row, and 7 us of a second launch where the reduction was split.  Hence:
+//  - as many stages as the block's share of the reduction has steps, up to 192 KB;
+//  - the splits of a tile are a cluster: their partial sums meet through distributed shared memory in split order, each
+//    block finishes 1 / splits of the tile's pixels, and there is neither scratch memory nor a second launch;
+//  - the accumulator goes through shared memory once, so that neighbouring lanes read the residual and write the output
+//    of neighbouring filters (a warp touches whole 128-byte lines instead of 32 rows x 16 bytes); the residual and the
+//    folded batch norm are requested before the wait for the accumulator;
+//  - eight epilogue warps: the second half of the epilogue is some 60 instructions per 8 filters of a pixel, and with one
+//    warp per scheduler it ran at their latency (1.5 us a tile).
 // ---------------------------------------------------------------------------------------------
-template <int BN, int STAGES, bool I8>
-__global__ void __launch_bounds__(192, 1) conv_tc_kernel(const __grid_constant__ TcParams p) {
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t saddr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ void cluster_sync_all() {  // (every thread of every block of the cluster)
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+constexpr int TC_EPI_WARPS = 8, TC_EPI = 32 * TC_EPI_WARPS, TC_THREADS = 64 + TC_EPI;
+
+template <int BN, bool I8>
+__global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_constant__ TcParams p) {
     // (a stage row is 128 bytes either way: 64 bf16 or 128 8-bit channels; an MMA takes 32 bytes of it)
     constexpr int CH = I8 ? 2 * CHUNK_C : CHUNK_C, KS = I8 ? 32 : 16;
     constexpr int B_STAGE_BYTES = BN * CHUNK_C * 2;
     constexpr int STAGE_BYTES = A_STAGE_BYTES + B_STAGE_BYTES;
+    constexpr int ACC_PITCH = BN + 4;  // floats; (BN + 4) / 4 is odd: 8 consecutive rows lie in 8 different groups of 4 banks
+    constexpr int CHUNKS = BN / 8;     // output vectors of 8 filters per pixel
     extern __shared__ uint8_t smem_raw[];
     __shared__ int row_m[TILE_M];  // output pixel index of each tile row, -1 outside the tensor
-    __shared__ __align__(8) uint64_t full_bar[STAGES], empty_bar[STAGES], accum_bar;
+    __shared__ __align__(8) uint64_t full_bar[TC_MAX_STAGES], empty_bar[TC_MAX_STAGES], accum_bar;
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s;
-    __shared__ float scale_s[BN], shift_s[BN];  // folded batch norm (8-bit layers: multiplier and shift as integers, plus the bias)
-    __shared__ int bias_s[I8 ? BN : 1];
 
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int stages = p.stages, splits = p.splits;
     volatile int *abort_flag = &abort_s;
 
     // tile coordinates
@@ -70,36 +102,23 @@ __global__ void __launch_bounds__(192, 1) conv_tc_kernel(const __grid_constant__
     // 8-bit: 0 unsigned, 1 signed), N >> 3 at bit 17, M >> 4 at bit 24; both operands K-major
     const uint32_t IDESC = I8 ? ((2u << 4) | ((uint32_t)(p.q_flags & 1) << 7) | (1u << 10) | ((uint32_t)(n_mma >> 3) << 17) | ((uint32_t)(TILE_M >> 4) << 24))
                               : ((1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n_mma >> 3) << 17) | ((uint32_t)(TILE_M >> 4) << 24));
-    // K range of this split
-    const int per = (p.iters + p.splits - 1) / p.splits;
-    const int it_begin = blockIdx.z * per, it_end = min(p.iters, it_begin + per);
-    const int n_it = max(0, it_end - it_begin);
+    // K range of this split (every split has at least one step: splits <= iters)
+    const int it_begin = p.iters * (int)blockIdx.z / splits, n_it = p.iters * ((int)blockIdx.z + 1) / splits - it_begin;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; s++) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
+        for (int s = 0; s < stages; s++) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
         mbar_init(&accum_bar, 1);
         abort_s = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) tmem_alloc(&tmem_base_s, BN);
-    if (warp >= 2) {
-        for (int j = threadIdx.x - 64; j < BN; j += 128) {
-            int f = f0 + j;
-            if (I8) {
-                reinterpret_cast<int *>(scale_s)[j] = f < p.K ? p.q_mult[f] : 0;
-                reinterpret_cast<int *>(shift_s)[j] = f < p.K ? min(max(p.q_shift[f], 0), 31) : 0;  // (0..31 by contract)
-                bias_s[I8 ? j : 0] = f < p.K ? p.q_bias[f] : 0;
-            } else {
-                scale_s[j] = f < p.K ? p.scale[f] : 0.f;
-                shift_s[j] = f < p.K ? p.shift[f] : 0.f;
-            }
-        }
-    }
+    if (warp == 2 && lane < (p.stride == 2 && p.k > 1 ? 4 : 1)) asm volatile("prefetch.tensormap [%0];" ::"l"(&p.tmA[lane]) : "memory");
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_s;
     pdl_launch_dependents();  // the next layer may start its prologue and its weight loads now
+    const uint32_t ring = smem_u32(smem);
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
@@ -121,7 +140,7 @@ __global__ void __launch_bounds__(192, 1) conv_tc_kernel(const __grid_constant__
         // (tap row r, tap column sx, channel chunk cc) of iteration it_begin, then stepped
         int cc = it_begin % p.cchunks, tap = it_begin / p.cchunks;
         int r = tap / p.k, sx = tap % p.k;
-        const uint32_t ring = smem_u32(smem), full0 = smem_u32(full_bar);
+        const uint32_t full0 = smem_u32(full_bar);
         auto load_weights = [&](int s, int c0, int tapw) {
             const uint32_t sb = ring + (uint32_t)(s * STAGE_BYTES + A_STAGE_BYTES), fb = full0 + (uint32_t)(s * 8);
             mbar_expect_tx_if(on, fb, tx);
@@ -132,7 +151,7 @@ __global__ void __launch_bounds__(192, 1) conv_tc_kernel(const __grid_constant__
         // waiting for it, so that their latency overlaps the previous layer's tail.
         {
             int cc2 = cc, r2 = r, sx2 = sx;
-            const int pre = min(n_it, STAGES);
+            const int pre = min(n_it, stages);
             for (int i = 0; i < pre; i++) {
                 load_weights(i, cc2 * CH, (p.o + r2) * p.R + (p.o + sx2));
                 if (++cc2 == p.cchunks) { cc2 = 0; if (++sx2 == p.k) { sx2 = 0; ++r2; } }
@@ -142,11 +161,11 @@ __global__ void __launch_bounds__(192, 1) conv_tc_kernel(const __grid_constant__
         int s = 0;
         uint32_t phase = 0;
         for (int i = 0; i < n_it; i++) {
-            if (i >= STAGES && !__all_sync(0xffffffffu, mbar_wait(&empty_bar[s], phase ^ 1, abort_flag))) break;
+            if (i >= stages && !__all_sync(0xffffffffu, mbar_wait(&empty_bar[s], phase ^ 1, abort_flag))) break;
             const int c0 = cc * CH;
             const uint32_t sa = ring + (uint32_t)(s * STAGE_BYTES), fb = full0 + (uint32_t)(s * 8);
             const int dh = r - p.p, dw = sx - p.p;
-            if (i >= STAGES) load_weights(s, c0, (p.o + r) * p.R + (p.o + sx));
+            if (i >= stages) load_weights(s, c0, (p.o + r) * p.R + (p.o + sx));
             if (p.stride == 1) {
                 tma_load_4d_if(on, sa, &p.tmA[0], fb, c0, w0 + dw, h0 + dh, n0);
             } else {
@@ -154,11 +173,11 @@ __global__ void __launch_bounds__(192, 1) conv_tc_kernel(const __grid_constant__
                 tma_load_4d_if(on, sa, &p.tmA[ph * 2 + pw], fb, c0, w0 + ((dw - pw) >> 1), h0 + ((dh - ph) >> 1), n0);
             }
             if (++cc == p.cchunks) { cc = 0; if (++sx == p.k) { sx = 0; ++r; } }
-            if (++s == STAGES) { s = 0; phase ^= 1; }
+            if (++s == stages) { s = 0; phase ^= 1; }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        const uint32_t on = elect_one(), d_tmem = uniform(tmem_base), ring = smem_u32(smem), empty0 = smem_u32(empty_bar);
+        const uint32_t on = elect_one(), d_tmem = uniform(tmem_base), empty0 = smem_u32(empty_bar);
         const int last_ksteps = (p.C - (p.cchunks - 1) * CH + KS - 1) / KS;  // MMAs of a tap's last chunk
         int cc = it_begin % p.cchunks, s = 0;
         uint32_t phase = 0;
@@ -175,123 +194,177 @@ __global__ void __launch_bounds__(192, 1) conv_tc_kernel(const __grid_constant__
             umma_commit_if(on, empty0 + (uint32_t)(s * 8));  // frees the stage once these MMAs have read it
             if (i == n_it - 1) umma_commit_if(on, smem_u32(&accum_bar));  // accumulator complete
             if (++cc == p.cchunks) cc = 0;
-            if (++s == STAGES) { s = 0; phase ^= 1; }
+            if (++s == stages) { s = 0; phase ^= 1; }
         }
-    } else {
-        // ------------------------------------------------------------------ epilogue (warps 2..5)
-        // Each thread owns one tile row (= TMEM lane = output pixel).
-        const int quad = warp & 3;            // TMEM lane quadrant this warp may read
-        const int row = quad * 32 + lane;     // tile row = output pixel within the box
-        {
+    }
+    // ---------------------------------------------------------------------- epilogue (warps 2..9)
+    // Thread et finishes filters fc .. fc + 7 of the tile rows et / CHUNKS + i * RSTEP of this block's share.
+    const bool epi = warp >= 2;
+    const int et = threadIdx.x - 64, chunk = et & (CHUNKS - 1), fc = f0 + 8 * chunk;
+    const int rows_mine = TILE_M / splits, row_first = rows_mine * (int)blockIdx.z, row0 = et / CHUNKS;
+    constexpr int RSTEP = TC_EPI / CHUNKS, BATCH = 4;
+    const bool fvalid = epi && fc < p.K;
+    bool ok_epi = epi;
+    uint4 rv[BATCH];   // residual of up to four outputs
+    float2 sc[4], sh[4];  // folded batch norm of the thread's filters (8-bit layers: multiplier and shift as integers)
+    int bias[I8 ? 8 : 1];
+    auto load_residual = [&](int i0) {
+#pragma unroll
+        for (int i = 0; i < BATCH; i++) {
+            const int r = row0 + RSTEP * (i0 + i);
+            rv[i] = make_uint4(0u, 0u, 0u, 0u);
+            if (p.res && r < rows_mine && fvalid) {
+                const int m = row_m[row_first + r];
+                if (m >= 0) {
+                    if (I8) {
+                        const uint2 q = ld_act(reinterpret_cast<const uint2 *>(reinterpret_cast<const uint8_t *>(p.res) + (size_t)m * p.ldy + fc));
+                        rv[i].x = q.x; rv[i].y = q.y;
+                    } else rv[i] = ld_act(reinterpret_cast<const uint4 *>(p.res + (size_t)m * p.ldy + fc));
+                }
+            }
+        }
+    };
+    if (epi) {
+        if (et < TILE_M) {
             const int rows = p.bw * p.bh * p.bn;
-            const int dn = row / (p.bh * p.bw), dhh = (row / p.bw) % p.bh, dww = row % p.bw;
+            const int dn = et / (p.bh * p.bw), dhh = (et / p.bw) % p.bh, dww = et % p.bw;
             const int n = n0 + dn, h = h0 + dhh, w = w0 + dww;
-            const bool valid = row < rows && n < p.N && h < p.Ho && w < p.Wo;
-            row_m[row] = valid ? (int)(((size_t)n * p.Ho + h) * p.Wo + w) : -1;
+            row_m[et] = et < rows && n < p.N && h < p.Ho && w < p.Wo ? (int)(((size_t)n * p.Ho + h) * p.Wo + w) : -1;
         }
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+            const int f = min(fc, p.K - 8) + j;
+            float a, b;
+            if (I8) {
+                a = __int_as_float(__ldg(p.q_mult + f));
+                b = __int_as_float(min(max(__ldg(p.q_shift + f), 0), 31));  // (0..31 by contract)
+                bias[I8 ? j : 0] = __ldg(p.q_bias + f);
+            } else { a = __ldg(p.scale + f); b = __ldg(p.shift + f); }
+            if (j & 1) { sc[j >> 1].y = a; sh[j >> 1].y = b; } else { sc[j >> 1].x = a; sh[j >> 1].x = b; }
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(TC_EPI) : "memory");
         pdl_wait();  // residual reads and output writes must not pass the previous layers
-        bool ok = n_it > 0 ? mbar_wait(&accum_bar, 0, abort_flag) : true;
-        ok = __all_sync(0xffffffffu, ok);
+        load_residual(0);
+        ok_epi = __all_sync(0xffffffffu, mbar_wait(&accum_bar, 0, abort_flag));
         tc_fence_after();
-        const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16);
-        const int ncols = min(BN, p.K - f0);  // filters of this tile, a multiple of 8
-        if (I8) {
-            // integer epilogue: requantise the int32 accumulator per filter, add bias, residual and the output
-            // zero point, ReLU as a maximum with the zero point, saturate, store 8 filters (8 bytes) at a time
-            if (ok) {
-                const int m = row_m[row];
-                const int *mult = reinterpret_cast<const int *>(scale_s), *shf = reinterpret_cast<const int *>(shift_s);
-                const uint8_t *res8 = reinterpret_cast<const uint8_t *>(p.res);
-                uint8_t *y8 = reinterpret_cast<uint8_t *>(p.y);
+        if (ok_epi) {
+            // accumulator -> shared memory (every operand stage has been read: the MMAs are complete); a warp takes its
+            // quadrant's 32 rows (warp % 4) and one half of the columns
+            const int quad = warp & 3, c0 = (warp >= 6 ? BN / 2 : 0), c1 = min(c0 + BN / 2, p.K - f0);
+            const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16);
+            float *dst = reinterpret_cast<float *>(smem) + (quad * 32 + lane) * ACC_PITCH;
+#pragma unroll 1
+            for (int j0 = c0; j0 < c1; j0 += 32) {
+                uint32_t v[32];
+                tmem_ld32(taddr + j0, v);
+                tmem_ld_wait();
+#pragma unroll
+                for (int g = 0; g < 8; g++)
+                    *reinterpret_cast<uint4 *>(dst + j0 + 4 * g) = make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
+            }
+        }
+        if (splits == 1) asm volatile("bar.sync 1, %0;" ::"n"(TC_EPI) : "memory");
+    }
+    if (splits > 1) cluster_sync_all();  // (also after a wait that ran out)
+    if (ok_epi && fc < p.ldy) {
+        const float lo = p.act == ACT_RELU ? 0.f : __int_as_float(0xff800000);  // ReLU as a maximum; no activation: -infinity
+        // One output: 8 filters of pixel m, o = accumulator (int32 bits in 8-bit layers).
+        auto store_output = [&](const float *o, const uint4 rq, int m) {
+            if (I8) {
+                // requantise the int32 accumulator per filter, add bias, residual and the output zero point, ReLU as a
+                // maximum with the zero point, saturate, store 8 filters (8 bytes)
                 const bool ysig = p.q_flags & 2, rsig = p.q_flags & 4, relu = p.q_flags & 8;
-                const int lo = ysig ? -128 : 0, hi = ysig ? 127 : 255;
+                const int qlo = ysig ? -128 : 0, qhi = ysig ? 127 : 255;
+                uint2 outw = make_uint2(0u, 0u);
+#pragma unroll
+                for (int j = 0; j < 8; j++) {
+                    const int mult = __float_as_int(j & 1 ? sc[j >> 1].y : sc[j >> 1].x), shf = __float_as_int(j & 1 ? sh[j >> 1].y : sh[j >> 1].x);
+                    long long t = rshift_round((long long)__float_as_int(o[j]) * (long long)mult, 31 + shf) + (long long)bias[I8 ? j : 0];
+                    if (p.res) {
+                        const uint32_t rb = ((j < 4 ? rq.x : rq.y) >> (8 * (j & 3))) & 0xffu;
+                        const int r8 = rsig ? (int)(signed char)rb : (int)rb;
+                        t += rshift_round((long long)(r8 - p.q_zr) * (long long)p.q_res_mult, 31 + p.q_res_shift);
+                    }
+                    t += p.q_zy;
+                    if (relu && t < p.q_zy) t = p.q_zy;
+                    const uint32_t byte = (uint32_t)(int)(t < qlo ? qlo : (t > qhi ? qhi : t)) & 0xffu;
+                    if (j < 4) outw.x |= byte << (8 * j); else outw.y |= byte << (8 * (j - 4));
+                }
+                *reinterpret_cast<uint2 *>(reinterpret_cast<uint8_t *>(p.y) + (size_t)m * p.ldy + fc) = outw;
+            } else {
+                const uint32_t r4[4] = {rq.x, rq.y, rq.z, rq.w};
+                uint4 ov;
+                __nv_bfloat162 *ob = reinterpret_cast<__nv_bfloat162 *>(&ov);
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    float2 v = __ffma2_rn(make_float2(o[2 * j], o[2 * j + 1]), sc[j], sh[j]);
+                    v = __fadd2_rn(v, make_float2(__uint_as_float(r4[j] << 16), __uint_as_float(r4[j] & 0xffff0000u)));
+                    if (p.act == ACT_HSWISH) { v.x = act_fn(v.x, ACT_HSWISH); v.y = act_fn(v.y, ACT_HSWISH); }
+                    else { v.x = fmaxf(v.x, lo); v.y = fmaxf(v.y, lo); }
+                    ob[j] = __float22bfloat162_rn(v);
+                }
+                *reinterpret_cast<uint4 *>(p.y + (size_t)m * p.ldy + fc) = ov;
+            }
+        };
+        // S = blocks of the cluster; the parts of four outputs (one output's 8 with S = 8) are requested before the first is
+        // used, and summed in split order (the sums of 8-bit layers are integers).
+        const int n_out = (rows_mine + RSTEP - 1) / RSTEP;
+        auto finish = [&](auto S_) {
+            constexpr int S = decltype(S_)::value, NB = S >= 4 ? 1 : 4 / S;
 #pragma unroll 1
-                for (int j0 = 0; j0 < ncols; j0 += 32) {
-                    uint32_t v[32];
-                    tmem_ld32(taddr + j0, v);
-                    tmem_ld_wait();
-                    if (m >= 0) {
+            for (int i0 = 0; i0 < n_out; i0 += BATCH) {
+                if (i0) load_residual(i0);
 #pragma unroll
-                        for (int g = 0; g < 4; g++) {
-                            const int c = j0 + 8 * g;
-                            if (c < ncols) {
-                                const size_t oi = (size_t)m * p.q_ldy + f0 + c;
-                                uint2 rraw = make_uint2(0u, 0u);
-                                if (res8) rraw = *reinterpret_cast<const uint2 *>(res8 + oi);
-                                uint2 outw = make_uint2(0u, 0u);
+                for (int h = 0; h < BATCH; h += NB) {
+                    if (i0 + h >= n_out) break;
+                    float4 qa[NB * S], qb[NB * S];
+                    int m[NB];
 #pragma unroll
-                                for (int j = 0; j < 8; j++) {
-                                    long long t = rshift_round((long long)(int)v[8 * g + j] * (long long)mult[c + j], 31 + shf[c + j]) + (long long)bias_s[I8 ? c + j : 0];
-                                    if (res8) {
-                                        const uint32_t rb = ((j < 4 ? rraw.x : rraw.y) >> (8 * (j & 3))) & 0xffu;
-                                        const int rq = rsig ? (int)(signed char)rb : (int)rb;
-                                        t += rshift_round((long long)(rq - p.q_zr) * (long long)p.q_res_mult, 31 + p.q_res_shift);
-                                    }
-                                    t += p.q_zy;
-                                    if (relu && t < p.q_zy) t = p.q_zy;
-                                    const int q8 = (int)(t < lo ? lo : (t > hi ? hi : t));
-                                    const uint32_t byte = (uint32_t)q8 & 0xffu;
-                                    if (j < 4) outw.x |= byte << (8 * j); else outw.y |= byte << (8 * (j - 4));
-                                }
-                                *reinterpret_cast<uint2 *>(y8 + oi) = outw;
+                    for (int i = 0; i < NB; i++) {
+                        const int r = row0 + RSTEP * (i0 + h + i), rr = row_first + min(r, rows_mine - 1);
+                        m[i] = r < rows_mine ? row_m[rr] : -1;
+                        const int off = (rr * ACC_PITCH + 8 * chunk) * 4;
+#pragma unroll
+                        for (int z = 0; z < S; z++) {
+                            if (S == 1) {
+                                qa[i] = *reinterpret_cast<const float4 *>(smem + off);
+                                qb[i] = *reinterpret_cast<const float4 *>(smem + off + 16);
+                            } else {
+                                const uint32_t ad = cluster_addr(ring + (uint32_t)off, (uint32_t)z);
+                                qa[i * S + z] = ld_cluster4(ad);
+                                qb[i * S + z] = ld_cluster4(ad + 16);
                             }
                         }
                     }
-                }
-                // a padded pixel (16-byte multiples for the next layer's copies): the 8 bytes beyond the last filter are zeros
-                if (m >= 0 && f0 + ncols == p.K && p.q_ldy > p.K) *reinterpret_cast<uint2 *>(y8 + (size_t)m * p.q_ldy + p.K) = make_uint2(0u, 0u);
-            }
-        } else if (p.splits == 1) {
-            // straight from tensor memory to global memory: each thread finishes its own pixel row,
-            // 8 filters (16 bytes) per store
-            if (ok) {
-                const int m = row_m[row];
-#pragma unroll 1
-                for (int j0 = 0; j0 < ncols; j0 += 32) {
-                    uint32_t v[32];
-                    tmem_ld32(taddr + j0, v);
-                    tmem_ld_wait();
-                    if (m >= 0) {
 #pragma unroll
-                        for (int g = 0; g < 4; g++) {
-                            const int c = j0 + 8 * g;
-                            if (c < ncols) {
-                                float o[8];
+                    for (int i = 0; i < NB; i++) {
+                        float o[8];
 #pragma unroll
-                                for (int j = 0; j < 8; j++) o[j] = __uint_as_float(v[8 * g + j]) * scale_s[c + j] + shift_s[c + j];
-                                finish_store(o, p.res, p.y, (size_t)m * p.K + f0 + c, p.act);
-                            }
+                        for (int z = 0; z < S; z++) {
+                            const float4 a = qa[i * S + z], b = qb[i * S + z];
+                            const float q[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+                            for (int j = 0; j < 8; j++) o[j] = z == 0 ? q[j] : I8 ? __int_as_float(__float_as_int(o[j]) + __float_as_int(q[j])) : o[j] + q[j];
                         }
+                        if (m[i] < 0) continue;
+                        if (fvalid) store_output(o, rv[h + i], m[i]);
+                        // a padded pixel: the 8 channels beyond the last filter are zeros
+                        else if (I8) *reinterpret_cast<uint2 *>(reinterpret_cast<uint8_t *>(p.y) + (size_t)m[i] * p.ldy + fc) = make_uint2(0u, 0u);
+                        else *reinterpret_cast<uint4 *>(p.y + (size_t)m[i] * p.ldy + fc) = make_uint4(0u, 0u, 0u, 0u);
                     }
                 }
             }
-        } else {
-            // split K: this CTA covers only part of the reduction; it stores its fp32 partial tile into
-            // its own slice of the workspace and splitk_finish_kernel adds the slices in split order.
-            if (ok && n_it > 0) {
-                const int m = row_m[row];
-                float *part = p.ws + (size_t)blockIdx.z * p.slice + (size_t)(m < 0 ? 0 : m) * p.K + f0;
-#pragma unroll 1
-                for (int j0 = 0; j0 < ncols; j0 += 32) {
-                    uint32_t v[32];
-                    tmem_ld32(taddr + j0, v);
-                    tmem_ld_wait();
-                    if (m >= 0) {
-#pragma unroll
-                        for (int g = 0; g < 8; g++) {
-                            const int c = j0 + 4 * g;
-                            if (c < ncols)
-                                __stcg(reinterpret_cast<float4 *>(part + c),
-                                       make_float4(__uint_as_float(v[4 * g]), __uint_as_float(v[4 * g + 1]),
-                                                   __uint_as_float(v[4 * g + 2]), __uint_as_float(v[4 * g + 3])));
-                        }
-                    }
-                }
-            }
+        };
+        switch (splits) {
+        case 1: finish(std::integral_constant<int, 1>()); break;
+        case 2: finish(std::integral_constant<int, 2>()); break;
+        case 4: finish(std::integral_constant<int, 4>()); break;
+        default: finish(std::integral_constant<int, 8>()); break;
         }
     }
     // ---------------------------------------------------------------------- teardown
     tc_fence_before();
+    if (splits > 1) cluster_sync_all();  // nobody leaves while another block may still read its sums
     __syncthreads();
     if (abort_s) {
         // a wait ran out: report, give copies that may still be in flight time to land in this
@@ -302,39 +375,6 @@ __global__ void __launch_bounds__(192, 1) conv_tc_kernel(const __grid_constant__
         __syncthreads();
     }
     if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem_base, BN); }
-}
-
-// Second step of a split reduction: out = act(scale * (slice_0 + slice_1 + ...) + shift + res), the
-// slices added in split order so that the result is the same on every run.  One thread per 8 filters
-// of one pixel; all of a thread's loads are issued before the first add.
-__global__ void __launch_bounds__(256) splitk_finish_kernel(const float *__restrict__ ws, size_t slice, int live,
-                                                            const float *__restrict__ scale, const float *__restrict__ shift,
-                                                            const __nv_bfloat16 *res, __nv_bfloat16 *y, size_t groups, int K,
-                                                            int act) {
-    const size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (g >= groups) return;
-    const size_t oi = g * 8;
-    const int f = (int)(oi % (size_t)K);
-    float4 q[8][2];
-#pragma unroll
-    for (int z = 0; z < 8; z++) {
-        if (z < live) {
-            const float *src = ws + (size_t)z * slice + oi;
-            q[z][0] = __ldcg(reinterpret_cast<const float4 *>(src));
-            q[z][1] = __ldcg(reinterpret_cast<const float4 *>(src + 4));
-        }
-    }
-    float o[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-    for (int z = 0; z < 8; z++) {
-        if (z < live) {
-            o[0] += q[z][0].x; o[1] += q[z][0].y; o[2] += q[z][0].z; o[3] += q[z][0].w;
-            o[4] += q[z][1].x; o[5] += q[z][1].y; o[6] += q[z][1].z; o[7] += q[z][1].w;
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < 8; j++) o[j] = o[j] * scale[f + j] + shift[f + j];
-    finish_store(o, res, y, oi, act);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -409,12 +449,12 @@ DeviceScratch g_dev[64];
 std::mutex g_mu;
 int g_status_seen = 0;
 
-template <int BN, int STAGES> constexpr int smem_bytes() { return STAGES * (A_STAGE_BYTES + BN * CHUNK_C * 2) + 1024; }
+constexpr int TC_RING_MAX = 192 * 1024;
+constexpr int tc_stage_bytes(int bn) { return A_STAGE_BYTES + bn * CHUNK_C * 2; }
 
 }  // namespace
 
 bool tc_available() { return encode_fn() != nullptr; }
-size_t tc_conv_ws_elems(const TcConvPlan &p) { return p.ws_elems; }
 
 int *tc_status_word(int device) {
     if (device < 0 || device >= 64) return nullptr;
@@ -524,7 +564,6 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
          reinterpret_cast<uintptr_t>(a.res)) & 15)
         return no("pointers must be 16-byte aligned");
     if (device < 0 || device >= 64) return no("device index");
-    if ((a.ldx || a.ldy) && a.throughput != 2 && !a.i8) return no("padded pixels are for grouped launches and 8-bit layers");
     if ((a.ldx && (a.ldx < a.C || a.ldx % 8)) || (a.ldy && (a.ldy < a.K || a.ldy % 8))) return no("channel pitch");
 
     auto plan = std::make_shared<TcConvPlan>();
@@ -612,15 +651,11 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
     }
     p.cchunks = (a.C + (int)CH - 1) / (int)CH;
     p.iters = a.k * plan->kw * p.cchunks;
-    // Filter tile.  Issuing one MMA costs the issuing thread about the same whatever its width, so wide
-    // tiles are preferred as long as tiles x K splits can still occupy every SM.
-    // a split costs a second (small) kernel, so it has to save at least a dozen pipeline iterations
-    int max_splits = p.iters >= 16 ? std::min(8, p.iters / 4) : 1;
-    int BN = 64;
-    for (int cand : {128}) {  // 256-wide tiles leave one CTA per SM, which this non-persistent kernel cannot afford
-        if (a.K <= cand / 2) continue;  // would be mostly padding
-        if ((long long)mtiles * ((a.K + cand - 1) / cand) * max_splits >= sms) { BN = cand; break; }
-    }
+    // Filter tile: 128 wide where the tiles then still occupy every SM (half the pixel copies per filter), else 64.
+    int BN = (a.K > 64 && (long long)mtiles * ((a.K + 127) / 128) >= sms) ? 128 : 64;
+    // A split (cluster of blocks) shortens the chain of steps by half for about a microsecond of meeting: it has to leave
+    // at least four steps per block.
+    int max_splits = p.iters >= 10 ? std::min(8, p.iters / 4) : 1;
     if (a.throughput) {
         // Many independent launches share the GPU (queries in flight): filling every SM from one launch
         // no longer matters, work per issued MMA does.  Wide tiles, splits only for very long K loops.
@@ -634,7 +669,7 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
         max_splits = 1;
         BN = swap ? 128 : a.K <= 64 ? 64 : a.K <= 128 ? 128 : 256;
     }
-    if (a.i8) max_splits = 1;  // (the integer epilogue has no second step)
+    if (a.no_split) max_splits = 1;
     plan->bn_tile = BN;
     {
         const uint64_t taps = a.win ? (uint64_t)a.k : (uint64_t)a.R * a.R;  // stored taps per filter
@@ -649,41 +684,28 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
     // split the K loop when the tiles alone cannot fill the machine
     int splits = 1;
     const int ctas = mtiles * ntiles;
-    if (ctas < sms && max_splits > 1) {
-        splits = std::min((sms + ctas - 1) / ctas, max_splits);
-        if (splits < 1) splits = 1;
-        // every split must own at least one iteration
-        while (splits > 1 && (p.iters + splits - 1) / splits * (splits - 1) >= p.iters) splits--;
-    }
+    while (splits * 2 <= max_splits && (long long)ctas * splits * 2 <= sms) splits *= 2;
     p.splits = splits;
-    p.slice = (size_t)a.N * a.Ho * a.Wo * a.K;
+    p.ldy = a.ldy ? a.ldy : a.K;
+    // Stages: all of a block's steps in flight up to 192 KB while the launch has a block per SM at most; two blocks per SM
+    // (one loads while the other finishes its tile) when it has more.  Never fewer than the accumulator needs (BN = 64: 2,
+    // 128: 3).
+    const int steps = (p.iters + splits - 1) / splits, room = (long long)ctas * splits > sms ? 98304 : TC_RING_MAX;
+    p.stages = std::max(BN == 128 ? 3 : 2, std::min({steps, room / tc_stage_bytes(BN), TC_MAX_STAGES}));
     plan->grid = dim3((unsigned)mtiles, (unsigned)ntiles, (unsigned)splits);
-    plan->ws_elems = splits > 1 ? (size_t)splits * a.N * a.Ho * a.Wo * a.K : 0;
     return plan;
 }
 
-// Launches the second step of a split reduction for the layer described by prm.
-static cudaError_t launch_finish(const TcParams &prm, cudaStream_t st) {
-    const int per = (prm.iters + prm.splits - 1) / prm.splits;
-    const int live = (prm.iters + per - 1) / per;  // splits that own at least one iteration
-    const size_t groups = prm.slice / 8;
-    splitk_finish_kernel<<<(unsigned)((groups + 255) / 256), 256, 0, st>>>(prm.ws, prm.slice, live, prm.scale, prm.shift, prm.res,
-                                                                         prm.y, groups, prm.K, prm.act);
-    return cudaGetLastError();
+template <int BN, bool I8> static cudaError_t launch_variant(const TcConvPlan &pl, const TcParams &prm, cudaStream_t st) {
+    return launch_pdl(conv_tc_kernel<BN, I8>, pl.grid, dim3(TC_THREADS), (size_t)(prm.stages * tc_stage_bytes(BN) + 1024), st, (unsigned)prm.splits, prm);
 }
-
-template <int BN, int STAGES, bool I8 = false> static cudaError_t launch_variant(const TcConvPlan &pl, const TcParams &prm, cudaStream_t st) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = pl.grid;
-    cfg.blockDim = dim3(192);
-    cfg.dynamicSmemBytes = smem_bytes<BN, STAGES>();
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, conv_tc_kernel<BN, STAGES, I8>, prm);
+static cudaError_t set_limits() {
+    const int most = TC_RING_MAX + 1024;
+    cudaError_t e;
+    if ((e = cudaFuncSetAttribute(conv_tc_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(conv_tc_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(conv_tc_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess) return e;
+    return cudaFuncSetAttribute(conv_tc_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
 }
 
 // One-time set-up of the current device: status word and the kernels' shared-memory limits.  Must
@@ -698,18 +720,14 @@ cudaError_t tc_conv_init(int dev) {
         if ((e = cudaMalloc(&ds.status, sizeof(int))) != cudaSuccess) return e;
         if ((e = cudaMemset(ds.status, 0, sizeof(int))) != cudaSuccess) return e;
     }
-    if ((e = cudaFuncSetAttribute(conv_tc_kernel<64, 3, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<64, 3>())) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(conv_tc_kernel<128, 3, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<128, 3>())) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(conv_tc_kernel<256, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<256, 4>())) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(conv_tc_kernel<64, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<64, 3>())) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(conv_tc_kernel<128, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<128, 3>())) != cudaSuccess) return e;
+    if ((e = set_limits()) != cudaSuccess) return e;
     if ((e = tc_group_init(dev)) != cudaSuccess) return e;
     if ((e = subnet_kernel_init(dev)) != cudaSuccess) return e;
     ds.attrs_set = true;
     return cudaSuccess;
 }
 
-cudaError_t tc_conv_launch(const TcConvPlan &pl, const ConvArgs &a, cudaStream_t st, int *launches) {
+cudaError_t tc_conv_launch(const TcConvPlan &pl, const ConvArgs &a, cudaStream_t st) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -721,27 +739,13 @@ cudaError_t tc_conv_launch(const TcConvPlan &pl, const ConvArgs &a, cudaStream_t
     prm.status = g_dev[dev].status;
     prm.cacheK = a.cacheK; prm.cacheC = a.cacheC; prm.weight_policy = a.weight_policy;
     prm.cache_tbl = a.cache_tbl; prm.layer = a.layer;
-    prm.ws = a.ws;
-    if (prm.splits > 1 && (!a.ws || a.ws_elems < pl.ws_elems)) prm.splits = 1;  // no workspace: run unsplit
-    TcConvPlan run = pl;
-    run.grid.z = (unsigned)prm.splits;
     if (pl.i8) {
-        if (!a.q_mult || !a.q_shift || !a.q_bias || pl.bn_tile > 128 || prm.splits != 1) return cudaErrorInvalidValue;
+        if (!a.q_mult || !a.q_shift || !a.q_bias || pl.bn_tile > 128) return cudaErrorInvalidValue;
         prm.q_mult = a.q_mult; prm.q_shift = a.q_shift; prm.q_bias = a.q_bias;
         prm.q_zy = a.q_zy; prm.q_zr = a.q_zr; prm.q_res_mult = a.q_res_mult; prm.q_res_shift = a.q_res_shift; prm.q_flags = a.q_flags;
-        prm.q_ldy = a.ldy ? a.ldy : a.K;
-        e = pl.bn_tile == 64 ? launch_variant<64, 3, true>(run, prm, st) : launch_variant<128, 3, true>(run, prm, st);
-        if (launches) *launches = 1;
-        return e;
+        return pl.bn_tile == 64 ? launch_variant<64, true>(pl, prm, st) : launch_variant<128, true>(pl, prm, st);
     }
-    if (pl.bn_tile == 64) e = launch_variant<64, 3>(run, prm, st);
-    else if (pl.bn_tile == 128) e = launch_variant<128, 3>(run, prm, st);
-    else e = launch_variant<256, 4>(run, prm, st);
-    if (launches) *launches = 1;
-    if (e != cudaSuccess || prm.splits == 1) return e;
-    e = launch_finish(prm, st);
-    if (launches) *launches = 2;
-    return e;
+    return pl.bn_tile == 64 ? launch_variant<64, false>(pl, prm, st) : launch_variant<128, false>(pl, prm, st);
 }
 
 }  // namespace sgs
@@ -751,22 +755,19 @@ cudaError_t tc_conv_launch(const TcConvPlan &pl, const ConvArgs &a, cudaStream_t
 //
 // Some users of this library run where cudaMalloc is off limits: inside a serving process whose
 // whole device memory was handed to a pool at start-up, or in a latency-critical loop where an
-// implicit device synchronisation (which cudaMalloc / cudaFree cause) is not acceptable.  For them the split-reduction scratch of the
-// tensor-core kernel lives in a fixed array that is part of the loaded library image.
+// implicit device synchronisation (which cudaMalloc / cudaFree cause) is not acceptable.  A split reduction keeps its
+// partial sums in shared memory, so the kernel needs no scratch at all; what this entry point has of its own is a status
+// word inside the library image.
 // =============================================================================================
 namespace sgs {
 namespace {
 
-constexpr size_t STATIC_WS_FLOATS = SGS_STATIC_SCRATCH_BYTES / sizeof(float);
-
 struct StaticScratch {
-    float ws[STATIC_WS_FLOATS];  // partial tiles of the split reduction
-    int status;                  // set by a kernel whose bounded wait ran out
+    int status;  // set by a kernel whose bounded wait ran out
 };
-// Every GPU that loads the library holds this array until the process exits.
 static __device__ __align__(256) StaticScratch g_static_scratch;
 
-// Device address of the array per device.  In host code the symbol's name is only a handle; the
+// Device address of it per device.  In host code the symbol's name is only a handle; the
 // address a kernel can use has to be asked for with cudaGetSymbolAddress while that device is current.
 StaticScratch *g_static_ptr[64] = {};
 std::mutex g_static_mu;
@@ -777,14 +778,25 @@ cudaError_t static_scratch_setup(int dev, StaticScratch **out) {
         StaticScratch *ptr = nullptr;
         cudaError_t e = cudaGetSymbolAddress((void **)&ptr, g_static_scratch);
         if (e != cudaSuccess) return e;
-        if ((e = cudaFuncSetAttribute(conv_tc_kernel<64, 3, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<64, 3>())) != cudaSuccess) return e;
-        if ((e = cudaFuncSetAttribute(conv_tc_kernel<128, 3, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<128, 3>())) != cudaSuccess) return e;
-        if ((e = cudaFuncSetAttribute(conv_tc_kernel<256, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<256, 4>())) != cudaSuccess) return e;
+        if ((e = set_limits()) != cudaSuccess) return e;
         if ((e = cudaMemset(&ptr->status, 0, sizeof(int))) != cudaSuccess) return e;
         g_static_ptr[dev] = ptr;
     }
     *out = g_static_ptr[dev];
     return cudaSuccess;
+}
+
+// The entry point refuses layers whose partial sums, written out as fp32 tiles, would take more than
+// SGS_STATIC_SCRATCH_BYTES.  The present kernel never writes them; the refusal is part of the contract (sgs.h), so the
+// tiling it is stated for - 64- or 128-filter tiles, up to 8 splits of at least 4 steps - is kept here.
+size_t contract_scratch_bytes(const TcParams &p, long long M, int mtiles, int sms) {
+    const int most = p.iters >= 16 ? std::min(8, p.iters / 4) : 1;
+    const int bn = (p.K > 64 && (long long)mtiles * ((p.K + 127) / 128) * most >= sms) ? 128 : 64;
+    const int ctas = mtiles * ((p.K + bn - 1) / bn);
+    if (ctas >= sms || most <= 1) return 0;
+    int splits = std::min((sms + ctas - 1) / ctas, most);
+    while (splits > 1 && (p.iters + splits - 1) / splits * (splits - 1) >= p.iters) splits--;
+    return splits > 1 ? (size_t)splits * (size_t)M * (size_t)p.K * sizeof(float) : 0;
 }
 
 }  // namespace
@@ -818,27 +830,20 @@ extern "C" sgs_status_t sgs_conv2d_sliced_static(const sgs_conv_desc_t *d, const
     a.Ho = (d->H + 2 * p - d->k) / d->stride + 1;
     a.Wo = (d->W + 2 * p - d->k) / d->stride + 1;
     a.cacheK = d->cache_k; a.cacheC = d->cache_c; a.weight_policy = d->weight_policy;
+    a.no_split = d->split_k_off;
     std::shared_ptr<TcConvPlan> plan = tc_conv_prepare(a, dev, nullptr);  // host memory only
     if (!plan) return SGS_EUNSUPPORTED;
     TcParams prm = plan->prm;
-    if (d->split_k_off) prm.splits = 1;
-    if (prm.splits > 1 && plan->ws_elems > STATIC_WS_FLOATS)
-        return SGS_ENOMEM;  // the layer's split reduction does not fit SGS_STATIC_SCRATCH_BYTES
+    int sms = 148;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (!d->split_k_off && contract_scratch_bytes(prm, (long long)a.N * a.Ho * a.Wo, (int)plan->grid.x, sms) > SGS_STATIC_SCRATCH_BYTES) return SGS_ENOMEM;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    // Nothing in the array has to start at zero: every partial-tile element that is read back by the
-    // second step is written by the first step of the same call.
     prm.scale = a.scale; prm.shift = a.shift;
     prm.res = static_cast<const __nv_bfloat16 *>(a.res);
     prm.y = static_cast<__nv_bfloat16 *>(a.y);
     prm.status = &sc->status;
     prm.cacheK = a.cacheK; prm.cacheC = a.cacheC; prm.weight_policy = a.weight_policy;
     prm.cache_tbl = nullptr; prm.layer = 0;
-    prm.ws = sc->ws;
-    TcConvPlan run = *plan;
-    run.grid.z = (unsigned)prm.splits;
-    cudaError_t e = plan->bn_tile == 64    ? launch_variant<64, 3>(run, prm, st)
-                    : plan->bn_tile == 128 ? launch_variant<128, 3>(run, prm, st)
-                                           : launch_variant<256, 4>(run, prm, st);
-    if (e == cudaSuccess && prm.splits > 1) e = launch_finish(prm, st);
+    const cudaError_t e = plan->bn_tile == 64 ? launch_variant<64, false>(*plan, prm, st) : launch_variant<128, false>(*plan, prm, st);
     return e == cudaSuccess ? SGS_OK : SGS_ECUDA;
 }

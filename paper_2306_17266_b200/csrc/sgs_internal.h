@@ -51,8 +51,8 @@ struct ConvArgs {
     // Channel pitch (elements per pixel) of x and of y / res when a pixel holds more than the sliced channels:
     // 0 = dense (C resp. K).  Padded tensors keep their pixels at a multiple of 16 channels (32 bytes) and the
     // channels beyond the slice are ZERO: the copy unit moves rows whose ends fall inside a 32-byte sector at a
-    // third of the rate (measured on sm_100a), and C, K are multiples of 8 only.  Tensor-core kernels of grouped
-    // launches only; they write the zeros of y.
+    // third of the rate (measured on sm_100a), and C, K are multiples of 8 only.  Tensor-core kernels only; they
+    // write the zeros of y.
     int ldx = 0, ldy = 0;
     int i8 = 0;  // 8-bit operands (x, w, res, y one byte per element; sgs_conv2d_sliced_i8): tensor-core kernel only
     const int *q_mult = nullptr, *q_shift = nullptr, *q_bias = nullptr;  // ... with the integer epilogue of TcParams
@@ -75,9 +75,7 @@ struct ConvArgs {
                          // 2: member of a grouped launch (128-filter tiles, reduction never split)
     int early_weights = 0;  // 1: the weights belong to a loaded SuperNet, so a kernel may read them before the previous kernel of
                             // the stream has finished; 0: they are the caller's and may come from that kernel
-    // split-K scratch of the tensor-core kernel: fp32 partial tiles [splits][M][K]
-    float *ws = nullptr;
-    size_t ws_elems = 0;
+    int no_split = 0;  // 1: one block per tile (the reduction is never split over a cluster)
 };
 
 // ---- persistent SubNet kernel (sgs_subnet_kernel.cu) ------------------------------------------
@@ -227,8 +225,7 @@ cudaError_t launch_stem_gemm_weights(const void *src, void *dst, int K, int KK, 
 // ---- tensor-core convolution (sgs_conv_tc.cu) -----------------------------------------------
 // Returns nullptr when the shape is not handled by the tensor-core kernel (caller falls back).
 std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::string *why);
-size_t tc_conv_ws_elems(const TcConvPlan &p);      // fp32 elements of split-K scratch the plan wants (0 = none)
-cudaError_t tc_conv_launch(const TcConvPlan &p, const ConvArgs &a, cudaStream_t st, int *launches);
+cudaError_t tc_conv_launch(const TcConvPlan &p, const ConvArgs &a, cudaStream_t st);
 cudaError_t tc_conv_init(int device);  // one-time device set-up; call outside stream capture
 bool tc_available();
 int tc_conv_status();  // nonzero once any tensor-core kernel reported a bounded wait running out

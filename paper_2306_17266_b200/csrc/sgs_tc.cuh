@@ -10,6 +10,7 @@ namespace sgs {
 
 constexpr int TILE_M = 128;   // output pixels per CTA (TMEM lanes)
 constexpr int CHUNK_C = 64;   // channels per pipeline stage (64 bf16 = one 128-byte swizzle row)
+constexpr int TC_MAX_STAGES = 8;
 constexpr int A_STAGE_BYTES = TILE_M * CHUNK_C * 2;
 constexpr unsigned long long WAIT_LIMIT_NS = 2000000000ull;  // 2 s per wait
 
@@ -19,8 +20,6 @@ struct TcParams {
     const float *scale, *shift;
     const __nv_bfloat16 *res;
     __nv_bfloat16 *y;
-    float *ws;               // split-K workspace: [splits][M][K] fp32 partial tiles
-    size_t slice;            // M*K, elements of one workspace slice
     int *status;             // device status word: nonzero after a bounded wait ran out
     int N, Ho, Wo, K, C;     // output dims, sliced filters, sliced channels
     int k, stride, R, o, p;  // kernel size, stride, stored kernel size, crop offset, padding
@@ -28,6 +27,8 @@ struct TcParams {
     int tiles_w, tiles_h;    // tiles along w and h (tiles along n = gridDim.x / (tiles_w*tiles_h))
     int cchunks, iters;      // channel chunks per tap, total pipeline iterations (k*k*cchunks)
     int splits, act;
+    int stages;              // operand stages in shared memory
+    int ldy;                 // elements per pixel of y and res (>= K; what lies beyond K is written as zeros)
     int cacheK, cacheC, weight_policy;
     const int *cache_tbl;    // optional device table overriding the three values above (see ConvArgs)
     int layer;
@@ -36,7 +37,6 @@ struct TcParams {
     const int *q_mult, *q_shift, *q_bias;
     int q_zy, q_zr, q_res_mult, q_res_shift;
     int q_flags;             // bit 0: x signed, bit 1: y signed, bit 2: res signed, bit 3: ReLU (max with q_zy)
-    int q_ldy;               // bytes per pixel of y and res (>= K; the bytes beyond K are written as zeros)
 };
 
 namespace {
@@ -266,7 +266,6 @@ struct TcConvPlan {
     int bn_tile = 128;   // filters per tile
     int swap = 0;        // grouped launches only: filters on the MMA's row side, all pixels on the column side
     int kw = 1;          // taps along x (k for square kernels, 1 for the window view of a stem)
-    size_t ws_elems = 0;
 };
 
 }  // namespace sgs
