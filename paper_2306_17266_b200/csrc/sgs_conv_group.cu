@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
                 const uint64_t da = smem_desc_sw128(sx_), db = smem_desc_sw128(sx_ + G_X_BYTES);
 #pragma unroll
                 for (int q = 0; q < CHUNK_C / 16; q++)
-                    umma_if<false>(q < ksteps ? on : 0u, d_tmem, da + (uint64_t)(2 * q), db + (uint64_t)(2 * q), idesc, (i > 0 || q > 0) ? 1u : 0u);
+                    if (q < ksteps) umma_if<false>(on, d_tmem, da + (uint64_t)(2 * q), db + (uint64_t)(2 * q), idesc, (i > 0 || q > 0) ? 1u : 0u);
                 umma_commit_if(on, empty0 + (uint32_t)(s * 8));  // frees the stage once these MMAs have read it
                 if (i == iters - 1) umma_commit_if(on, smem_u32(&acc_full[buf]));  // accumulator complete
                 if (++cc == cchunks) cc = 0;

@@ -190,12 +190,17 @@ __global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_con
             const uint64_t da = smem_desc_sw128(sa), db = smem_desc_sw128(sa + A_STAGE_BYTES);
 #pragma unroll
             for (int q = 0; q < CH / KS; q++)
-                umma_if<I8>(q < ksteps ? on : 0u, d_tmem, da + (uint64_t)(2 * q), db + (uint64_t)(2 * q), IDESC, (i > 0 || q > 0) ? 1u : 0u);
+                if (q < ksteps) umma_if<I8>(on, d_tmem, da + (uint64_t)(2 * q), db + (uint64_t)(2 * q), IDESC, (i > 0 || q > 0) ? 1u : 0u);
             umma_commit_if(on, empty0 + (uint32_t)(s * 8));  // frees the stage once these MMAs have read it
             if (i == n_it - 1) umma_commit_if(on, smem_u32(&accum_bar));  // accumulator complete
             if (++cc == p.cchunks) cc = 0;
             if (++s == stages) { s = 0; phase ^= 1; }
         }
+        // Only this warp polls for the accumulator; the epilogue warps sleep in a hardware barrier meanwhile (eight polling
+        // warps take the schedulers and the shared-memory pipe from the issuing ones).
+        if (!*abort_flag) mbar_wait(&accum_bar, 0, abort_flag);
+        tc_fence_before();
+        asm volatile("bar.arrive 2, %0;" ::"n"(TC_EPI + 32) : "memory");
     }
     // ---------------------------------------------------------------------- epilogue (warps 2..9)
     // Thread et finishes filters fc .. fc + 7 of the tile rows et / CHUNKS + i * RSTEP of this block's share.
@@ -245,7 +250,8 @@ __global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_con
         asm volatile("bar.sync 1, %0;" ::"n"(TC_EPI) : "memory");
         pdl_wait();  // residual reads and output writes must not pass the previous layers
         load_residual(0);
-        ok_epi = __all_sync(0xffffffffu, mbar_wait(&accum_bar, 0, abort_flag));
+        asm volatile("bar.sync 2, %0;" ::"n"(TC_EPI + 32) : "memory");
+        ok_epi = *abort_flag == 0;
         tc_fence_after();
         if (ok_epi) {
             // accumulator -> shared memory (every operand stage has been read: the MMAs are complete); a warp takes its

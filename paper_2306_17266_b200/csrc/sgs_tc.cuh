@@ -71,10 +71,12 @@ __device__ __forceinline__ unsigned long long global_ns() {
     asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
     return t;
 }
-// Bounded wait: false if the phase did not complete within limit_ns or another role gave up.
+// Bounded wait: false if the phase did not complete within limit_ns or another role gave up.  The time is read only after
+// some hundred tries: %globaltimer takes longer to read than most waits of a pipeline last.
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag,
                                           unsigned long long limit_ns = WAIT_LIMIT_NS) {
-    if (mbar_try_wait(bar, parity)) return true;
+    for (int i = 0; i < 256; i++)
+        if (mbar_try_wait(bar, parity)) return true;
     const unsigned long long t0 = global_ns();
     for (;;) {
         for (int i = 0; i < 64; i++)
@@ -117,7 +119,8 @@ __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, u
 // as divergent, and then every descriptor, barrier address and coordinate (operands the tensor and copy units take from
 // the uniform registers) is moved there one by one in front of every instruction.  Measured (B200, all SMs, 64 channels a
 // stage, wait + four MMAs + commit): 624 -> 353 clocks a stage with 64 or 128 columns, 675 -> 518 with 256 columns, where
-// the tensor unit itself needs 512.
+// the tensor unit itself needs 512.  The predicate has to be the elected lane's alone: combined with a condition on the
+// step (`q < ksteps ? on : 0`) the same loop takes 536 clocks, with a branch on that uniform condition 360.
 __device__ __forceinline__ void mbar_expect_tx_if(uint32_t on, uint32_t bar, uint32_t bytes) {
     asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}" ::"r"(bar), "r"(bytes), "r"(on) : "memory");
 }
