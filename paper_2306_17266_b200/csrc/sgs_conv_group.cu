@@ -5,10 +5,9 @@
 // form one list of tiles; persistent CTAs (one per SM) walk that list with a fixed stride.
 //
 // Per CTA: warp 0 = weight producer, warp 10 = activation producer, warp 1 = MMA issuer, warps 2..9 =
-// two epilogue groups.  The shared-memory ring of operand stages runs on across tiles, and the fp32
-// accumulator in tensor memory is double buffered (2 x 256 columns, one buffer per epilogue group), so the
-// epilogues of tiles j and j + 1 (tensor memory -> folded batch norm -> residual -> activation -> bf16
-// NHWC) overlap each other and the loads and MMAs of the tiles that follow.
+// epilogue.  The shared-memory ring of operand stages runs on across tiles, and the fp32 accumulator in tensor memory
+// is double buffered (2 x 256 columns), so the epilogue of a tile (tensor memory -> folded batch norm -> residual ->
+// activation -> bf16 NHWC) overlaps the loads and MMAs of the tiles that follow.
 //
 // The arithmetic of one tile is that of conv_tc_kernel (sgs_conv_tc.cu): implicit GEMM with
 // 128 output pixels x up to 256 filters, 64 channels per stage, slicing through the tensor maps'
@@ -25,9 +24,11 @@ namespace {
 constexpr int G_MAX_STAGES = 8;
 constexpr int G_X_BYTES = 128 * CHUNK_C * 2;  // operand on the MMA's row side: 128 rows
 constexpr int G_RING_BYTES = 192 * 1024;      // operand ring: 8 stages of 16 + 8 KB (tiles of at most 64 columns), 6 of 16 + 16 KB, or 4 of 16 + 32 KB (256-column tiles)
-constexpr int G_SMEM_BYTES = G_RING_BYTES + 1024;
 constexpr int G_ACC_COLS = 256;                   // tensor-memory columns of one accumulator buffer
-constexpr int G_EPI_WARPS = 8;                    // two groups of four (one warp per tensor-memory lane quadrant)
+constexpr int G_EPI_WARPS = 8;                    // two per tensor-memory lane quadrant
+constexpr int G_EPI_PITCH = 36;                   // floats per staged row of 32 columns: 8 consecutive rows lie in 8 different groups of 4 banks
+constexpr int G_EPI_FLOATS = 16 * G_EPI_PITCH;    // a warp's staging area: 16 rows
+constexpr int G_SMEM_BYTES = 1024 + G_RING_BYTES + G_EPI_WARPS * G_EPI_FLOATS * 4;
 constexpr int G_THREADS = 64 + 32 * G_EPI_WARPS + 32;  // weight producer, MMA warp, epilogue warps, pixel producer
 constexpr int G_PIX_WARP = 2 + G_EPI_WARPS;
 
@@ -83,8 +84,6 @@ __device__ __forceinline__ int tile_entry(const GroupEntry *es, int n, int t, in
     return es[i].second ? i - 1 : i;
 }
 
-// Named barrier of one epilogue group (4 warps): id 1 or 2.
-__device__ __forceinline__ void group_bar(int grp) { asm volatile("bar.sync %0, 128;" ::"r"(grp + 1) : "memory"); }
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap *m) { asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory"); }
 
 
@@ -108,7 +107,6 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
     int *status = P.status;
     extern __shared__ uint8_t smem_raw[];
     __shared__ GroupEntry es[TC_GROUP_MAX_ENTRIES];
-    __shared__ float scale_s[2][2][G_ACC_COLS], shift_s[2][2][G_ACC_COLS];  // per epilogue group: folded batch norm of its current / next tile's filters
     __shared__ __align__(8) uint64_t full_bar[G_MAX_STAGES], empty_bar[G_MAX_STAGES], acc_full[2], acc_empty[2];
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s;
@@ -123,7 +121,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
         reinterpret_cast<uint4 *>(es)[i] = __ldg(reinterpret_cast<const uint4 *>(entries) + i);
     if (threadIdx.x == 0) {
         for (int s = 0; s < G_MAX_STAGES; s++) { mbar_init(&full_bar[s], 2); mbar_init(&empty_bar[s], 1); }  // (full: both producers arrive)
-        for (int b = 0; b < 2; b++) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], G_EPI_WARPS / 2); }
+        for (int b = 0; b < 2; b++) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], G_EPI_WARPS); }
         abort_s = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -252,112 +250,117 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
         }
     } else {
         // ------------------------------------------------------------------ epilogue (warps 2..9)
-        // Two groups of four warps (one per tensor-memory lane quadrant).  Group g owns accumulator buffer g
-        // and takes the CTA's tiles j with j % 2 == g, so the epilogues of two consecutive tiles run side by
-        // side; a thread handles one accumulator row and all of the tile's columns, 32 at a time.
+        // All eight warps work on every tile: a warp takes its tensor-memory lane quadrant (warp % 4) and every other block
+        // of 32 columns; the accumulator is double buffered, so the main loop of the next tile runs meanwhile.
+        //
+        // What bounds it: the memory pipe, then issue slots.  When a lane stored its own pixel row, 16 bytes at a time, a
+        // warp's store touched 32 lines and a 128 x 256 tile took 10.8k clocks (20k with a residual) against 512 clocks of
+        // tensor time per 64 channels - most launches were bound by that.  So each block goes through a few KB of shared
+        // memory private to the warp (fp32, 16 rows at a time): afterwards four neighbouring lanes own 32 neighbouring
+        // filters of a pixel, residual reads and output writes are runs of 64 bytes, and a lane keeps the folded batch norm
+        // of its 8 filters in registers for all of the block's rows.
         const int quad = warp & 3;                // tensor-memory lane quadrant this warp may read
-        const int grp = (warp - 2) >> 2;          // epilogue group = accumulator buffer
+        const int half = (warp - 2) >> 2;         // which of every two column blocks
         const int row_all = quad * 32 + lane;     // accumulator row: output pixel (normal) or filter (swapped)
-        const int et = (threadIdx.x - 64) & 127;  // thread within the group
-        float(*scale_g)[G_ACC_COLS] = scale_s[grp];
-        float(*shift_g)[G_ACC_COLS] = shift_s[grp];
-        const int stride2 = 2 * (int)gridDim.x;
+        const int lr = lane >> 2, lc = lane & 3;  // in the staged form: row within 8, 8-filter chunk within 32
+        float *stage = reinterpret_cast<float *>(smem + G_RING_BYTES) + (warp - 2) * G_EPI_FLOATS;
         pdl_wait();  // residual reads and output writes must not pass the previous layers
-        bool alive = true;  // after a failed wait the warp only keeps the named barrier in step
-        // folded batch norm of a normal tile: thread et fetches the scale and shift of filters et and et + 128
-        auto fetch_bn = [&](int tile, float *v) {
-            v[0] = v[1] = v[2] = v[3] = 0.f;
-            if (tile >= total_tiles) return;
-            const GroupEntry &e = es[tile_entry(es, n_entries, tile, lane)];
-            if (e.swap) return;
-            const int f = ((tile - e.tile_begin) / e.mtiles) * e.bn_tile + et;
-            if (et < e.bn_tile && f < e.K) { v[0] = __ldg(e.scale + f); v[1] = __ldg(e.shift + f); }
-            if (et + 128 < e.bn_tile && f + 128 < e.K) { v[2] = __ldg(e.scale + f + 128); v[3] = __ldg(e.shift + f + 128); }
-        };
-        auto store_bn = [&](int b, const float *v) {
-            scale_g[b][et] = v[0]; shift_g[b][et] = v[1]; scale_g[b][et + 128] = v[2]; shift_g[b][et + 128] = v[3];
-        };
-        {
-            float v[4];
-            fetch_bn((int)blockIdx.x + grp * (int)gridDim.x, v);
-            store_bn(0, v);
-        }
-        int jj = 0;  // tiles this group has taken
-        for (int t = (int)blockIdx.x + grp * (int)gridDim.x; t < total_tiles; t += stride2, jj++) {
+        int j = 0;   // tiles of this CTA so far
+        for (int t = (int)blockIdx.x; t < total_tiles; t += (int)gridDim.x, j++) {
             const GroupEntry &e0 = es[tile_entry(es, n_entries, t, lane)];
             const int local = t - e0.tile_begin, nt = local / e0.mtiles, mt = local % e0.mtiles;
             // rows 64..127 of a pair's tile belong to the second member (a warp lies on one side)
             const bool second_half = e0.pair && quad >= 2;
             const GroupEntry &e = second_half ? (&e0)[1] : e0;
             const int row = second_half ? row_all - 64 : row_all;
-            const int K = e.K, ldk = e.ldk, act = e.act;
+            const int K = e.K, ldk = e.ldk, act = e.act, buf = j & 1;
             const __nv_bfloat16 *res = e.res;
             __nv_bfloat16 *y = e.y;
-            const int sb = jj & 1;  // which of the group's two scale / shift tables
-            const uint32_t tacc = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(grp * G_ACC_COLS);
-            float nbn[4];
-            fetch_bn(t + stride2, nbn);  // requested now, stored after this tile's work
+            const uint32_t tacc = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * G_ACC_COLS);
             if (!e.swap) {
-                // ---- normal tile: this thread owns output pixel `m`, columns are filters
+                // ---- normal tile: rows are output pixels, columns are filters
                 const int n0 = (mt / e.tiles_hw) * e.bn, h0 = ((mt % e.tiles_hw) / e.tiles_w) * e.bh, w0 = (mt % e.tiles_w) * e.bw;
                 const int f0 = nt * e0.bn_tile;
-                int m;
+                // offset of the four rows this lane finishes (lr + 8 i), in vectors of 8 channels; ~0: outside the tensor
+                uint32_t off[4];
                 {
                     const int dn = row / (e.bh * e.bw), dhh = (row / e.bw) % e.bh, dww = row % e.bw;
                     const int n = n0 + dn, h = h0 + dhh, w = w0 + dww;
                     const bool valid = row < e.pix_rows && n < e.N && h < e.Ho && w < e.Wo;
-                    m = valid ? (int)(((size_t)n * e.Ho + h) * e.Wo + w) : -1;
-                }
-                const int cend = min((int)e0.bn_tile, K - f0);  // filters of this tile, a multiple of 8 (<= 0: none of this member's)
-                const int cpad = min((int)e0.bn_tile, ldk - f0);  // ... and the end of the pixel's padding, written as zeros
-                const size_t obase = (size_t)(m < 0 ? 0 : m) * ldk + f0;
-                // the residual does not depend on the accumulator: the first 64 columns' part is requested
-                // before waiting, every further part two steps ahead of its use (a thread then has 8 loads of
-                // 16 bytes in flight: the epilogue of a tile with a residual is bound by their latency).
-                // (Measured alternative: transposing the accesses through a warp-private staging block so that a
-                // warp touches 8 rows x 64 contiguous bytes instead of 32 rows x 16 bytes changed no layer's time
-                // at 16 images per member and cost 1.7 % on the batch-1 stream.)
-                auto load_res = [&](int c0, uint4 *rv) {
+                    const uint32_t mine = valid ? (uint32_t)(((size_t)((size_t)n * e.Ho + h) * e.Wo + w) * (size_t)(ldk >> 3)) + (uint32_t)(f0 >> 3) : 0xffffffffu;
 #pragma unroll
-                    for (int g = 0; g < 4; g++) {
-                        const int c = c0 + 8 * g;
-                        rv[g] = (res && m >= 0 && c < cend) ? ld_act(reinterpret_cast<const uint4 *>(res + obase + c)) : make_uint4(0u, 0u, 0u, 0u);
+                    for (int i = 0; i < 4; i++) off[i] = __shfl_sync(0xffffffffu, mine, lr + 8 * i);
+                }
+                const int cend = min((int)e0.bn_tile, K - f0);    // filters of this tile, a multiple of 8 (<= 0: none of this member's)
+                const int cpad = min((int)e0.bn_tile, ldk - f0);  // ... and the end of the pixel's padding, written as zeros
+                const float lo = act == ACT_RELU ? 0.f : __int_as_float(0xff800000);  // ReLU as a maximum; no activation: -infinity
+                auto load_bn = [&](int c0, float2 *sc, float2 *sh) {
+                    const int f = f0 + min(c0 + 8 * lc, max(cend, 8) - 8);
+#pragma unroll
+                    for (int q = 0; q < 4; q++) {
+                        sc[q] = __ldg(reinterpret_cast<const float2 *>(e.scale + f) + q);
+                        sh[q] = __ldg(reinterpret_cast<const float2 *>(e.shift + f) + q);
                     }
                 };
-                uint4 rv[4], rn[4];
-                load_res(0, rv);
-                load_res(32, rn);
-                group_bar(grp);  // this tile's scale / shift (written during the group's previous tile) are visible
-                const float *sc = scale_g[sb], *sh = shift_g[sb];
-                if (alive) alive = __all_sync(0xffffffffu, mbar_wait(&acc_full[grp], jj & 1, abort_flag));
-                if (alive) {
-                    tc_fence_after();
-#pragma unroll 1
-                    for (int c0 = 0; c0 < cpad; c0 += 32) {
-                        uint32_t v[32];
-                        tmem_ld32(tacc + c0, v);
-                        uint4 rf[4];
-                        load_res(c0 + 64, rf);
-                        tmem_ld_wait();
-                        if (m >= 0) {
+                auto load_res = [&](int c0, int i) -> uint4 {
+                    return (c0 + 8 * lc < cend && off[i] != 0xffffffffu) ? ld_act(reinterpret_cast<const uint4 *>(res) + off[i] + (uint32_t)((c0 >> 3) + lc)) : make_uint4(0u, 0u, 0u, 0u);
+                };
+                float2 sc[4], sh[4];
+                uint4 rv[4];
+                if (half * 32 < cend) {
+                    load_bn(half * 32, sc, sh);
+                    if (res) {
 #pragma unroll
-                            for (int g = 0; g < 4; g++) {
-                                const int c = c0 + 8 * g;
-                                if (c >= cend && c < cpad) *reinterpret_cast<uint4 *>(y + obase + c) = make_uint4(0u, 0u, 0u, 0u);
-                                if (c < cend) {
-                                    float ov[8];
-#pragma unroll
-                                    for (int q = 0; q < 8; q++) ov[q] = __uint_as_float(v[8 * g + q]) * sc[c + q] + sh[c + q];
-                                    const __nv_bfloat162 *rb = reinterpret_cast<const __nv_bfloat162 *>(&rv[g]);
-#pragma unroll
-                                    for (int q = 0; q < 4; q++) { const float2 f2 = __bfloat1622float2(rb[q]); ov[2 * q] += f2.x; ov[2 * q + 1] += f2.y; }
-                                    finish_store(ov, nullptr, y, obase + c, act);
-                                }
-                            }
-                        }
-#pragma unroll
-                        for (int g = 0; g < 4; g++) { rv[g] = rn[g]; rn[g] = rf[g]; }
+                        for (int i = 0; i < 4; i++) rv[i] = load_res(half * 32, i);
                     }
+                }
+                if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[buf], (j >> 1) & 1, abort_flag))) break;
+                tc_fence_after();
+#pragma unroll 1
+                for (int c0 = half * 32; c0 < cpad; c0 += 64) {
+                    uint32_t v[32];
+                    tmem_ld32(tacc + c0, v);
+                    const int c = c0 + 8 * lc;  // this lane's 8 filters
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int hr = 0; hr < 2; hr++) {
+                        __syncwarp();
+                        if ((lane >> 4) == hr) {
+#pragma unroll
+                            for (int g = 0; g < 8; g++)
+                                *reinterpret_cast<uint4 *>(stage + (lane & 15) * G_EPI_PITCH + 4 * g) = make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
+                        }
+                        __syncwarp();
+#pragma unroll
+                        for (int i2 = 0; i2 < 2; i2++) {
+                            const int i = hr * 2 + i2;
+                            const float4 qa = *reinterpret_cast<const float4 *>(stage + (lr + 8 * i2) * G_EPI_PITCH + 8 * lc);
+                            const float4 qb = *reinterpret_cast<const float4 *>(stage + (lr + 8 * i2) * G_EPI_PITCH + 8 * lc + 4);
+                            float2 o[4] = {make_float2(qa.x, qa.y), make_float2(qa.z, qa.w), make_float2(qb.x, qb.y), make_float2(qb.z, qb.w)};
+#pragma unroll
+                            for (int q = 0; q < 4; q++) o[q] = __ffma2_rn(o[q], sc[q], sh[q]);
+                            if (res) {
+                                const uint32_t r4[4] = {rv[i].x, rv[i].y, rv[i].z, rv[i].w};
+#pragma unroll
+                                for (int q = 0; q < 4; q++) o[q] = __fadd2_rn(o[q], make_float2(__uint_as_float(r4[q] << 16), __uint_as_float(r4[q] & 0xffff0000u)));
+                                rv[i] = load_res(c0 + 64, i);  // the next block's, used after its tensor-memory load
+                            }
+                            if (act == ACT_HSWISH) {
+#pragma unroll
+                                for (int q = 0; q < 4; q++) { o[q].x = act_fn(o[q].x, ACT_HSWISH); o[q].y = act_fn(o[q].y, ACT_HSWISH); }
+                            } else {
+#pragma unroll
+                                for (int q = 0; q < 4; q++) { o[q].x = fmaxf(o[q].x, lo); o[q].y = fmaxf(o[q].y, lo); }
+                            }
+                            uint4 out;
+                            __nv_bfloat162 *ob = reinterpret_cast<__nv_bfloat162 *>(&out);
+#pragma unroll
+                            for (int q = 0; q < 4; q++) ob[q] = __float22bfloat162_rn(o[q]);
+                            if (c >= cend) out = make_uint4(0u, 0u, 0u, 0u);  // (the pixel's padding)
+                            if (c < cpad && off[i] != 0xffffffffu) reinterpret_cast<uint4 *>(y)[off[i] + (uint32_t)(c >> 3)] = out;
+                        }
+                    }
+                    if (c0 + 64 < cend) load_bn(c0 + 64, sc, sh);
                 }
             } else {
                 // ---- swapped tile: this thread owns filter `f`, columns are the member's output pixels
@@ -367,58 +370,28 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
                 float sc = 0.f, sh = 0.f;
                 if (fvalid) { sc = __ldg(e.scale + f); sh = __ldg(e.shift + f); }
                 const unsigned short *resu = reinterpret_cast<const unsigned short *>(res);
-                auto load_res = [&](int c0, uint32_t *rv) {  // 32 pixels, two per register
-#pragma unroll
-                    for (int q = 0; q < 16; q++) {
-                        const int p0 = c0 + 2 * q;
-                        uint32_t lo = 0, hi = 0;
-                        if (res && fvalid && p0 < cend) lo = ld_act(resu + (size_t)p0 * ldk + f);
-                        if (res && fvalid && p0 + 1 < cend) hi = ld_act(resu + (size_t)(p0 + 1) * ldk + f);
-                        rv[q] = lo | (hi << 16);
-                    }
-                };
-                uint32_t rv[16];
-                load_res(0, rv);
-                group_bar(grp);
-                if (alive) alive = __all_sync(0xffffffffu, mbar_wait(&acc_full[grp], jj & 1, abort_flag));
-                if (alive) {
-                    tc_fence_after();
+                if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[buf], (j >> 1) & 1, abort_flag))) break;
+                tc_fence_after();
 #pragma unroll 1
-                    for (int c0 = 0; c0 < cend; c0 += 32) {
-                        uint32_t v[32];
-                        tmem_ld32(tacc + c0, v);
-                        uint32_t rn[16];
-                        load_res(c0 + 32, rn);
-                        tmem_ld_wait();
-                        if (fvalid) {
+                for (int c0 = half * 16; c0 < cend; c0 += 32) {  // (at most 32 pixels: one block of 16 per warp)
+                    uint32_t v[16];
+                    tmem_ld16(tacc + c0, v);
+                    unsigned short rv[16];
 #pragma unroll
-                            for (int q = 0; q < 32; q++) {
-                                const int px = c0 + q;
-                                if (px < cend) {
-                                    const uint32_t rbits = (q & 1) ? (rv[q >> 1] & 0xffff0000u) : (rv[q >> 1] << 16);
-                                    const float o = act_fn(__uint_as_float(v[q]) * sc + sh + __uint_as_float(rbits), act);
-                                    y[(size_t)px * ldk + f] = __float2bfloat16_rn(o);
-                                }
-                            }
-                        } else if (fpad) {
+                    for (int q = 0; q < 16; q++) rv[q] = (res && fvalid && c0 + q < cend) ? ld_act(resu + (size_t)(c0 + q) * ldk + f) : (unsigned short)0;
+                    tmem_ld_wait();
+                    if (fvalid || fpad) {
 #pragma unroll
-                            for (int q = 0; q < 32; q++)
-                                if (c0 + q < cend) y[(size_t)(c0 + q) * ldk + f] = __float2bfloat16_rn(0.f);
-                        }
-#pragma unroll
-                        for (int q = 0; q < 16; q++) rv[q] = rn[q];
+                        for (int q = 0; q < 16; q++)
+                            if (c0 + q < cend)
+                                y[(size_t)(c0 + q) * ldk + f] = __float2bfloat16_rn(fvalid ? act_fn(__uint_as_float(v[q]) * sc + sh + __uint_as_float((uint32_t)rv[q] << 16), act) : 0.f);
                     }
                 }
             }
-            if (alive) {
-                // hand the accumulator buffer back to the MMA warp
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&acc_empty[grp]);
-            }
-            // the group read table sb ^ 1 for the last time during its previous tile, which all of its
-            // threads have left (barrier above)
-            store_bn(sb ^ 1, nbn);
+            // hand the accumulator buffer back to the MMA warp
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&acc_empty[buf]);
         }
     }
     // ---------------------------------------------------------------------- teardown
