@@ -456,8 +456,8 @@ sgs_status_t sgs_debug_expire_wait(unsigned limit_us, void *cuda_stream);
  * at 16-channel pixels (zeros beyond the slice), 0 = dense pixels; "cache_mechanism" how grouped launches keep the cached SubGraph in L2: 0 (default) = an evict-last
  * hint on every weight tile inside the SubGraph's box, 1 = an access-policy window on the launch (the cached filter
  * prefix of the launch's stored layer, persisting; the persisting-L2 carve-out of the process is sized to the cache
- * budget), 2 = both; "dw_walk" N = stride-1 depthwise launches of at least N million output
- * elements take the walking kernel (default 48; 0 never, negative always; process-wide); "persistent_held_kb" n = shared memory per SM that persistent
+ * budget), 2 = both; "dw_walk" is accepted and has no effect (there is one depthwise
+ * kernel); "persistent_held_kb" n = shared memory per SM that persistent
  * execution spends on the cached SubGraph's first pointwise layers (default 16, 0 = none); "nvtx" 1 = an NVTX range named after the stored layer around
  * every launch (for timeline tools); "fail_alloc_after" n = the handle's device allocations fail from
  * the (n+1)-th on with SGS_ENOMEM (fault injection on the host, -1 = off); "drop_plans" forgets every cached plan (measuring what a never-seen config costs); "profile" see

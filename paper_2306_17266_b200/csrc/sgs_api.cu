@@ -2580,10 +2580,7 @@ sgs_status_t sgs_set_option(sgs_supernet_t *net, const char *name, long long val
         net->plans.clear();
         return SGS_OK;
     }
-    if (n == "dw_walk") {  // tuning aid (process-wide)
-        dw_set_walk((int)value);
-        return SGS_OK;
-    }
+    if (n == "dw_walk") return SGS_OK;  // (accepted for compatibility: there is one depthwise kernel)
     if (n == "stage_group") {  // (accepted for compatibility: every stage of the grouped convolution kernel has its own barriers)
         if (value < 0 || value > 4) return fail(net, SGS_EINVAL, "stage_group");
         return SGS_OK;

@@ -1,5 +1,5 @@
-// CUDA-core kernels other than the convolution (sgs_conv_simt.cu): depthwise convolution with centre-cropped
-// kernels, pooling, squeeze-excite, linear layers, and the load-time re-layout / batch-norm folding kernels.
+// CUDA-core kernels other than the convolutions (sgs_conv_simt.cu, sgs_dw.cu): plain depthwise convolution, pooling,
+// squeeze-excite, linear layers, and the load-time re-layout / batch-norm folding kernels.
 #include "sgs_internal.h"
 #include "sgs_pdl.cuh"
 
@@ -62,562 +62,10 @@ __global__ void __launch_bounds__(256) dw_plain_kernel(ConvArgs a) {
     }
 }
 
-// Vectorised bf16 depthwise convolution.  A thread owns 8 channels (one 16-byte vector) of TW = 4
-// neighbouring output pixels of one output row: per filter row it loads the (TW-1)*ST + K input
-// columns once and uses each for every tap it belongs to, so global loads per output drop from K*K
-// to about K*(1 + (K-1)/(TW*ST)); neighbouring threads cover neighbouring channel vectors, so every
-// load and store of a warp is one contiguous run.  fp32 accumulation with packed 2-wide FMAs.
-// HBM traffic per output element: 2 B read + 2 B written (rows are re-read from L1/L2, not DRAM).
-__device__ __forceinline__ float2 bf2_lo(uint32_t u) { return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u)); }
-
-// Argument record of a depthwise kernel: by value, or (GROUP: one launch for many queries in flight) from a
-// device table with DW_ENTRY_BYTES per member, blockIdx.z = member * images + image.
-#define SGS_DW_ARGS()                                                                                          \
-    __shared__ __align__(16) unsigned char a_raw_[sizeof(ConvArgs)];                                           \
-    if (GROUP) {                                                                                               \
-        const uint32_t *src_ = reinterpret_cast<const uint32_t *>(tbl + (size_t)(blockIdx.z / n_img) * DW_ENTRY_BYTES); \
-        for (int i_ = threadIdx.x; i_ < (int)(sizeof(ConvArgs) / 4); i_ += blockDim.x) reinterpret_cast<uint32_t *>(a_raw_)[i_] = __ldg(src_ + i_); \
-        __syncthreads();                                                                                       \
-    }                                                                                                          \
-    const ConvArgs &a = GROUP ? *reinterpret_cast<const ConvArgs *>(a_raw_) : a1;                              \
-    if (!a.early_weights) pdl_wait();                                                                          \
-    const int n = GROUP ? (int)(blockIdx.z % n_img) : (int)blockIdx.z;
-static_assert(sizeof(ConvArgs) % 4 == 0 && sizeof(ConvArgs) <= DW_ENTRY_BYTES, "depthwise table record");
-
-template <int K, int ST>
-__device__ __forceinline__ void dw_vec_body(const ConvArgs &a, const int n) {
-    constexpr int TW = 4, NCOL = (TW - 1) * ST + K, P = (K - 1) / 2;
-    // grid: x covers (channel vector, pixel block) of one output row, y = output row, z = image;
-    // all index arithmetic stays in 32 bits
-    const int groups = a.K / 8, wblocks = (a.Wo + TW - 1) / TW;
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= groups * wblocks) return;
-    const int cg = idx % groups, wb = idx / groups;
-    const int ho = blockIdx.y;
-    const int c0 = cg * 8, wo0 = wb * TW, o = (a.R - K) / 2;
-    const __nv_bfloat16 *x = static_cast<const __nv_bfloat16 *>(a.x);
-    const __nv_bfloat16 *__restrict__ w = static_cast<const __nv_bfloat16 *>(a.w);
-
-    float2 acc[TW][4];
-#pragma unroll
-    for (int t = 0; t < TW; t++)
-#pragma unroll
-        for (int j = 0; j < 4; j++) acc[t][j] = make_float2(0.f, 0.f);
-
-    const __nv_bfloat16 *ximg = x + ((size_t)n * a.H) * a.W * a.K + c0;
-    pdl_wait();
-#pragma unroll
-    for (int r = 0; r < K; r++) {
-        const int hi = ho * ST + r - P;
-        if (hi < 0 || hi >= a.H) continue;
-        const __nv_bfloat16 *xrow = ximg + (size_t)hi * a.W * a.K;
-        uint4 col[NCOL];
-#pragma unroll
-        for (int j = 0; j < NCOL; j++) {
-            const int wi = wo0 * ST + j - P;
-            col[j] = (wi >= 0 && wi < a.W) ? ld_act(reinterpret_cast<const uint4 *>(xrow + wi * a.K)) : make_uint4(0u, 0u, 0u, 0u);
-        }
-        const __nv_bfloat16 *wrow = w + ((o + r) * a.R + o) * a.Kmax + c0;
-#pragma unroll
-        for (int s = 0; s < K; s++) {
-            const uint4 wv = __ldg(reinterpret_cast<const uint4 *>(wrow + s * a.Kmax));
-            const float2 w0 = bf2_lo(wv.x), w1 = bf2_lo(wv.y), w2 = bf2_lo(wv.z), w3 = bf2_lo(wv.w);
-#pragma unroll
-            for (int t = 0; t < TW; t++) {
-                const uint4 xv = col[t * ST + s];
-                acc[t][0] = __ffma2_rn(bf2_lo(xv.x), w0, acc[t][0]);
-                acc[t][1] = __ffma2_rn(bf2_lo(xv.y), w1, acc[t][1]);
-                acc[t][2] = __ffma2_rn(bf2_lo(xv.z), w2, acc[t][2]);
-                acc[t][3] = __ffma2_rn(bf2_lo(xv.w), w3, acc[t][3]);
-            }
-        }
-    }
-    const float4 s0 = __ldg(reinterpret_cast<const float4 *>(a.scale + c0)), s1 = __ldg(reinterpret_cast<const float4 *>(a.scale + c0 + 4));
-    const float4 h0 = __ldg(reinterpret_cast<const float4 *>(a.shift + c0)), h1 = __ldg(reinterpret_cast<const float4 *>(a.shift + c0 + 4));
-    __nv_bfloat16 *yrow = static_cast<__nv_bfloat16 *>(a.y) + (((size_t)n * a.Ho + ho) * a.Wo) * a.K + c0;
-#pragma unroll
-    for (int t = 0; t < TW; t++) {
-        const int wo = wo0 + t;
-        if (wo >= a.Wo) break;
-        float v[8] = {acc[t][0].x * s0.x + h0.x, acc[t][0].y * s0.y + h0.y, acc[t][1].x * s0.z + h0.z, acc[t][1].y * s0.w + h0.w,
-                      acc[t][2].x * s1.x + h1.x, acc[t][2].y * s1.y + h1.y, acc[t][3].x * s1.z + h1.z, acc[t][3].y * s1.w + h1.w};
-        uint4 ov;
-        __nv_bfloat162 *ob = reinterpret_cast<__nv_bfloat162 *>(&ov);
-#pragma unroll
-        for (int j = 0; j < 4; j++) ob[j] = __floats2bfloat162_rn(apply_act(v[2 * j], a.act), apply_act(v[2 * j + 1], a.act));
-        *reinterpret_cast<uint4 *>(yrow + wo * a.K) = ov;
-    }
-}
-template <int K, int ST, bool GROUP>
-__global__ void __launch_bounds__(256) dw_vec_kernel(const ConvArgs a1, const char *__restrict__ tbl, int n_img) {
-    pdl_launch_dependents();
-    SGS_DW_ARGS()
-    dw_vec_body<K, ST>(a, n);
-}
-
-// Tiled variant: a thread owns 8 channels of a TH x TW patch of output pixels.  Every vector of the
-// patch's halo is loaded and unpacked ONCE and used for all the output rows and taps it belongs to, so
-// the instruction count per output element (the limit of the row-at-a-time kernel above) drops to about
-// ((TH-1)*ST+K)*((TW-1)*ST+K)/(TH*TW) unpacks + K*K packed FMAs per 8 channels.  With PRELOAD every load
-// of the halo is issued before the first use (memory latency is then hidden by the loads a thread has
-// in flight, not by occupancy).  Patches whose halo lies inside the image take a path without bounds
-// tests.  The epilogue is packed: one FMA for the folded batch norm per channel pair, and h-swish as
-// x * clamp(x / 6 + 0.5, 0, 1) (= x * relu6(x + 3) / 6): one saturating FMA and one packed multiply.
-template <int K, int ST, int TH, int TW, bool PRELOAD, int ACT>
-__device__ __forceinline__ void dw_tile_body(const ConvArgs &a, const int n) {
-    constexpr int P = (K - 1) / 2, NCOL = (TW - 1) * ST + K, NROW = (TH - 1) * ST + K;
-    const int groups = a.K / 8, wblocks = (a.Wo + TW - 1) / TW;
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= groups * wblocks || (int)blockIdx.y * TH >= a.Ho) return;
-    const int cg = idx % groups, wb = idx / groups;
-    const int ho0 = blockIdx.y * TH;
-    const int c0 = cg * 8, wo0 = wb * TW, o = (a.R - K) / 2;
-    const __nv_bfloat16 *x = static_cast<const __nv_bfloat16 *>(a.x);
-    const __nv_bfloat16 *__restrict__ w = static_cast<const __nv_bfloat16 *>(a.w);
-
-    // weights stay packed in registers and are unpacked at use
-    constexpr bool WUNPACK = false;  // (unpacking the weights once costs 72 registers for K = 3 and measured slower)
-    uint4 wv[WUNPACK ? 1 : K * K];
-    float2 wf[WUNPACK ? K * K : 1][4];
-#pragma unroll
-    for (int r = 0; r < K; r++)
-#pragma unroll
-        for (int s = 0; s < K; s++) {
-            const uint4 q = __ldg(reinterpret_cast<const uint4 *>(w + ((o + r) * a.R + o + s) * a.Kmax + c0));
-            if (WUNPACK) {
-                float2 *d = wf[WUNPACK ? r * K + s : 0];
-                d[0] = bf2_lo(q.x); d[1] = bf2_lo(q.y); d[2] = bf2_lo(q.z); d[3] = bf2_lo(q.w);
-            } else {
-                wv[WUNPACK ? 0 : r * K + s] = q;
-            }
-        }
-
-    float2 acc[TH][TW][4];
-#pragma unroll
-    for (int i = 0; i < TH; i++)
-#pragma unroll
-        for (int t = 0; t < TW; t++)
-#pragma unroll
-            for (int j = 0; j < 4; j++) acc[i][t][j] = make_float2(0.f, 0.f);
-
-    const __nv_bfloat16 *ximg = x + ((size_t)n * a.H) * a.W * a.K + c0;
-    const int wi0 = wo0 * ST - P, hi0 = ho0 * ST - P;
-    const bool interior = hi0 >= 0 && hi0 + NROW <= a.H && wi0 >= 0 && wi0 + NCOL <= a.W;
-    uint4 raw[PRELOAD ? NROW : 1][NCOL];
-    pdl_wait();  // (the filters above do not depend on the previous layer)
-    if (PRELOAD) {
-#pragma unroll
-        for (int ir = 0; ir < NROW; ir++) {
-            const int hi = hi0 + ir;
-            const bool rok = hi >= 0 && hi < a.H;
-            const __nv_bfloat16 *xrow = ximg + (size_t)(rok ? hi : 0) * a.W * a.K;
-#pragma unroll
-            for (int j = 0; j < NCOL; j++) {
-                const int wi = wi0 + j;
-                raw[PRELOAD ? ir : 0][j] = (rok && wi >= 0 && wi < a.W) ? ld_act(reinterpret_cast<const uint4 *>(xrow + wi * a.K)) : make_uint4(0u, 0u, 0u, 0u);
-            }
-        }
-    }
-#pragma unroll
-    for (int ir = 0; ir < NROW; ir++) {
-        const int hi = hi0 + ir;
-        if (!PRELOAD && (hi < 0 || hi >= a.H)) continue;
-        const __nv_bfloat16 *xrow = ximg + (size_t)hi * a.W * a.K;
-        float2 xc[NCOL][4];
-#pragma unroll
-        for (int j = 0; j < NCOL; j++) {
-            const int wi = wi0 + j;
-            uint4 v;
-            if (PRELOAD) v = raw[PRELOAD ? ir : 0][j];
-            else if (interior) v = ld_act(reinterpret_cast<const uint4 *>(xrow + wi * a.K));
-            else v = (wi >= 0 && wi < a.W) ? ld_act(reinterpret_cast<const uint4 *>(xrow + wi * a.K)) : make_uint4(0u, 0u, 0u, 0u);
-            xc[j][0] = bf2_lo(v.x); xc[j][1] = bf2_lo(v.y); xc[j][2] = bf2_lo(v.z); xc[j][3] = bf2_lo(v.w);
-        }
-#pragma unroll
-        for (int oh = 0; oh < TH; oh++) {
-            const int r = ir - oh * ST;  // filter row this input row meets in output row oh
-            if (r < 0 || r >= K) continue;
-#pragma unroll
-            for (int s = 0; s < K; s++) {
-                float2 w0, w1, w2, w3;
-                if (WUNPACK) {
-                    const float2 *d = wf[WUNPACK ? r * K + s : 0];
-                    w0 = d[0]; w1 = d[1]; w2 = d[2]; w3 = d[3];
-                } else {
-                    const uint4 q = wv[WUNPACK ? 0 : r * K + s];
-                    w0 = bf2_lo(q.x); w1 = bf2_lo(q.y); w2 = bf2_lo(q.z); w3 = bf2_lo(q.w);
-                }
-#pragma unroll
-                for (int t = 0; t < TW; t++) {
-                    acc[oh][t][0] = __ffma2_rn(xc[t * ST + s][0], w0, acc[oh][t][0]);
-                    acc[oh][t][1] = __ffma2_rn(xc[t * ST + s][1], w1, acc[oh][t][1]);
-                    acc[oh][t][2] = __ffma2_rn(xc[t * ST + s][2], w2, acc[oh][t][2]);
-                    acc[oh][t][3] = __ffma2_rn(xc[t * ST + s][3], w3, acc[oh][t][3]);
-                }
-            }
-        }
-    }
-    const float4 s0 = __ldg(reinterpret_cast<const float4 *>(a.scale + c0)), s1 = __ldg(reinterpret_cast<const float4 *>(a.scale + c0 + 4));
-    const float4 h0 = __ldg(reinterpret_cast<const float4 *>(a.shift + c0)), h1 = __ldg(reinterpret_cast<const float4 *>(a.shift + c0 + 4));
-    const float2 sc[4] = {make_float2(s0.x, s0.y), make_float2(s0.z, s0.w), make_float2(s1.x, s1.y), make_float2(s1.z, s1.w)};
-    const float2 sh[4] = {make_float2(h0.x, h0.y), make_float2(h0.z, h0.w), make_float2(h1.x, h1.y), make_float2(h1.z, h1.w)};
-#pragma unroll
-    for (int oh = 0; oh < TH; oh++) {
-        const int ho = ho0 + oh;
-        if (ho >= a.Ho) break;
-        __nv_bfloat16 *yrow = static_cast<__nv_bfloat16 *>(a.y) + (((size_t)n * a.Ho + ho) * a.Wo) * a.K + c0;
-#pragma unroll
-        for (int t = 0; t < TW; t++) {
-            const int wo = wo0 + t;
-            if (wo >= a.Wo) break;
-            uint4 ov;
-            __nv_bfloat162 *ob = reinterpret_cast<__nv_bfloat162 *>(&ov);
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                float2 v = __ffma2_rn(acc[oh][t][j], sc[j], sh[j]);
-                if (ACT == ACT_RELU) { v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); }
-                if (ACT == ACT_HSWISH) {
-                    const float2 g = make_float2(__saturatef(fmaf(v.x, 1.f / 6.f, 0.5f)), __saturatef(fmaf(v.y, 1.f / 6.f, 0.5f)));
-                    v = __fmul2_rn(v, g);
-                }
-                ob[j] = __float22bfloat162_rn(v);
-            }
-            *reinterpret_cast<uint4 *>(yrow + wo * a.K) = ov;
-        }
-    }
-}
-template <int K, int ST, int TH, int TW, bool PRELOAD, int ACT, bool GROUP>
-__global__ void __launch_bounds__(128) dw_tile_kernel(const ConvArgs a1, const char *__restrict__ tbl, int n_img) {
-    pdl_launch_dependents();
-    SGS_DW_ARGS()
-    if (GROUP) { const ConvArgs al = a; dw_tile_body<K, ST, TH, TW, PRELOAD, ACT>(al, n); }  // (register copy, see dw_mixed_kernel)
-    else dw_tile_body<K, ST, TH, TW, PRELOAD, ACT>(a, n);
-}
-// Stride-1 depthwise convolution that WALKS down the image behind a ring of input rows in shared memory (the
-// B200 form of a line buffer: paper Section 4.2 keeps the rows a sliding window needs on chip).  A block owns 128
-// channels x a tile of 4 * TW output columns x a segment of SEG output rows.  Its 128 threads copy one input row of
-// the tile at a time into a ring of RING rows with 16-byte asynchronous copies (zero fill for rows, columns and
-// channels outside the tensor, so the arithmetic has no bounds tests), RING - 1 rows ahead of the row being used:
-// memory latency is covered by the ring, not by registers or occupancy.  A thread owns 4 channels (an 8-byte vector)
-// of a strip of TW columns: per input row it reads TW + K - 1 vectors from the ring, unpacks each ONCE, and
-// scatters it into the K output rows it belongs to.  The K live output rows rotate through K accumulator slots; the
-// row loop is unrolled by K so that every slot index is static: input row hi = base + u meets filter row r in output
-// row hi + P - r, slot (u - r) mod K.  Filter row 0 STARTS an output row (a product instead of an accumulate: slots
-// never need clearing, rows outside the segment never need a test), filter row K - 1 completes it.  The weights of
-// the block's 128 channels sit unpacked (fp32) in shared memory; a lane reads its four per tap with one 16-byte load.
-// Grid: x = channel blocks x column tiles, y = row segments, z = image (x member).
-#ifndef DW_WALK_SEG_ROWS
-#define DW_WALK_SEG_ROWS 56
-#endif
-constexpr int DW_WALK_SEG = DW_WALK_SEG_ROWS;  // output rows per segment (halo: K - 1 extra input rows per segment)
-template <int K> struct DwWalkShape {
-    static constexpr int TW = K == 3 ? 4 : 2;          // output columns per thread
-    static constexpr int ICOL = 4 * TW + K - 1;        // input columns of a block's tile
-    static constexpr int RING = K == 7 ? 6 : 8;        // input rows in the ring
-    static constexpr int ROW_BYTES = ICOL * 256;       // 128 channels x 2 bytes per column
-    static constexpr int SMEM = K * K * 128 * 4 + RING * ROW_BYTES;
-};
-
-__device__ __forceinline__ void cp_async16(void *dst, const void *src, bool valid) {
-    const unsigned n = valid ? 16u : 0u;  // 0 source bytes: the 16 destination bytes are zero-filled
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"(n) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
-template <int K, int ACT>
-__device__ __forceinline__ void dw_walk_body(const ConvArgs &a, const int n, unsigned char *smem, const int chblocks) {
-    using S = DwWalkShape<K>;
-    constexpr int TW = S::TW, P = (K - 1) / 2, NCOL = TW + K - 1, ICOL = S::ICOL, RING = S::RING;
-    float *wsm = reinterpret_cast<float *>(smem);
-    unsigned char *ring = smem + K * K * 128 * 4;
-    const int lane = threadIdx.x & 31, wrp = threadIdx.x >> 5;
-    const int groups = a.K / 4, tiles_w = (a.Wo + 4 * TW - 1) / (4 * TW);
-    // (chblocks = channel blocks of the GRID: a launch over several members is sized for the widest of them)
-    const int cb = blockIdx.x % chblocks, tb = blockIdx.x / chblocks;
-    const int ho_begin = blockIdx.y * DW_WALK_SEG, ho_end = min(a.Ho, ho_begin + DW_WALK_SEG);
-    if (cb * 32 >= groups || tb >= tiles_w || ho_begin >= a.Ho) return;  // (whole blocks only: no barrier is skipped)
-    const int o = (a.R - K) / 2;
-    const __nv_bfloat16 *__restrict__ w = static_cast<const __nv_bfloat16 *>(a.w);
-    // the block's weights: wsm[tap][lane * 4 + j] = w[o + r][o + s][cb * 128 + lane * 4 + j] (zero beyond the slice)
-    for (int i = threadIdx.x; i < K * K * 32; i += blockDim.x) {
-        const int tap = i >> 5, l = i & 31, c = cb * 128 + l * 4;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (c < a.K) {
-            const uint2 q = __ldg(reinterpret_cast<const uint2 *>(w + ((size_t)((o + tap / K) * a.R + o + tap % K)) * a.Kmax + c));
-            const float2 lo = bf2_lo(q.x), hi = bf2_lo(q.y);
-            v = make_float4(lo.x, lo.y, hi.x, hi.y);
-        }
-        reinterpret_cast<float4 *>(wsm)[tap * 32 + l] = v;
-    }
-    const int cg = cb * 32 + lane;
-    const int c0 = cg * 4, wt0 = tb * 4 * TW, wo0 = wt0 + wrp * TW;
-    const bool active = cg < groups;  // (lanes beyond the slice compute zeros and store nothing)
-    const __nv_bfloat16 *ximg = static_cast<const __nv_bfloat16 *>(a.x) + ((size_t)n * a.H) * a.W * a.K;
-    __nv_bfloat16 *yimg = static_cast<__nv_bfloat16 *>(a.y) + ((size_t)n * a.Ho) * a.Wo * a.K + c0;
-    float4 sc4 = make_float4(0.f, 0.f, 0.f, 0.f), sh4 = sc4;
-    if (active) { sc4 = __ldg(reinterpret_cast<const float4 *>(a.scale + c0)); sh4 = __ldg(reinterpret_cast<const float4 *>(a.shift + c0)); }
-    const float2 sc[2] = {make_float2(sc4.x, sc4.y), make_float2(sc4.z, sc4.w)}, sh[2] = {make_float2(sh4.x, sh4.y), make_float2(sh4.z, sh4.w)};
-    const float4 *wl = reinterpret_cast<const float4 *>(wsm) + lane;
-
-    const int hi_first = ho_begin - P, hi_last = ho_end - 1 + P;  // input rows that meet the segment (may lie outside the image)
-    // One input row of the tile -> ring slot (hi - hi_first) % RING, 16 chunks of 16 bytes per column.  A thread
-    // copies the same (column, channel) chunks of every row: their offsets and whether they lie inside the tensor
-    // are fixed before the row loop.
-    constexpr int NCH = (ICOL * 16 + 127) / 128;  // chunks per thread and row
-    int src_off[NCH], dst_off[NCH];               // element offset inside an input row (-1: outside), byte offset in the slot
-#pragma unroll
-    for (int i = 0; i < NCH; i++) {
-        const int q = threadIdx.x + i * 128;
-        const int j = q >> 4, part = q & 15;
-        const int wi = wt0 - P + j, c = cb * 128 + part * 8;
-        dst_off[i] = q < ICOL * 16 ? q * 16 : -1;
-        src_off[i] = (q < ICOL * 16 && wi >= 0 && wi < a.W && c < a.K) ? wi * a.K + c : -1;
-    }
-    auto copy_row = [&](int hi) {
-        if (hi <= hi_last) {
-            unsigned char *dst = ring + ((hi - hi_first) % RING) * S::ROW_BYTES;
-            const bool rok = hi >= 0 && hi < a.H;
-            const __nv_bfloat16 *xrow = ximg + (size_t)(rok ? hi : 0) * a.W * a.K;
-#pragma unroll
-            for (int i = 0; i < NCH; i++) {
-                if (dst_off[i] >= 0) {
-                    const bool ok = rok && src_off[i] >= 0;
-                    cp_async16(dst + dst_off[i], ok ? (const void *)(xrow + src_off[i]) : (const void *)ximg, ok);
-                }
-            }
-        }
-        cp_async_commit();  // (a group per row, also when it is empty: the wait below counts groups)
-    };
-    pdl_wait();  // (the filters above do not depend on the previous layer)
-#pragma unroll 1
-    for (int d = 0; d < RING - 1; d++) copy_row(hi_first + d);
-
-    float2 acc[K][TW][2];
-    for (int base = hi_first; base <= hi_last; base += K) {
-#pragma unroll
-        for (int u = 0; u < K; u++) {
-            const int hi = base + u;
-            if (hi <= hi_last) {  // (block-uniform)
-                cp_async_wait<RING - 2>();  // this thread's copies of row hi have landed ...
-                __syncthreads();            // ... and everybody's; everybody has also finished with row hi - 1
-                copy_row(hi + RING - 1);    // into the slot row hi - 1 used
-                const unsigned char *row = ring + ((hi - hi_first) % RING) * S::ROW_BYTES + (wrp * TW) * 256 + lane * 8;
-                float2 xc[NCOL][2];
-#pragma unroll
-                for (int j = 0; j < NCOL; j++) {
-                    const uint2 v = *reinterpret_cast<const uint2 *>(row + j * 256);
-                    xc[j][0] = bf2_lo(v.x); xc[j][1] = bf2_lo(v.y);
-                }
-#pragma unroll
-                for (int r = 0; r < K; r++) {
-                    constexpr int KK = K;
-                    const int slot = ((u - r) % KK + KK) % KK;
-#pragma unroll
-                    for (int s2 = 0; s2 < K; s2++) {
-                        const float4 wq = wl[(r * K + s2) * 32];
-                        const float2 w0 = make_float2(wq.x, wq.y), w1 = make_float2(wq.z, wq.w);
-#pragma unroll
-                        for (int t = 0; t < TW; t++) {
-                            if (r == 0 && s2 == 0) {
-                                acc[slot][t][0] = __fmul2_rn(xc[t + s2][0], w0);
-                                acc[slot][t][1] = __fmul2_rn(xc[t + s2][1], w1);
-                            } else {
-                                acc[slot][t][0] = __ffma2_rn(xc[t + s2][0], w0, acc[slot][t][0]);
-                                acc[slot][t][1] = __ffma2_rn(xc[t + s2][1], w1, acc[slot][t][1]);
-                            }
-                        }
-                    }
-                }
-                // the output row this input row completes (filter row K - 1): hi - P
-                const int oh = hi - P;
-                if (active && oh >= ho_begin && oh < ho_end) {
-                    constexpr int KK = K;
-                    const int slot = ((u - (K - 1)) % KK + KK) % KK;
-                    __nv_bfloat16 *yrow = yimg + (size_t)oh * a.Wo * a.K;
-#pragma unroll
-                    for (int t = 0; t < TW; t++) {
-                        if (wo0 + t < a.Wo) {
-                            uint2 ov;
-                            __nv_bfloat162 *ob = reinterpret_cast<__nv_bfloat162 *>(&ov);
-#pragma unroll
-                            for (int j = 0; j < 2; j++) {
-                                float2 v = __ffma2_rn(acc[slot][t][j], sc[j], sh[j]);
-                                if (ACT == ACT_RELU) { v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); }
-                                if (ACT == ACT_HSWISH) {
-                                    const float2 g = make_float2(__saturatef(fmaf(v.x, 1.f / 6.f, 0.5f)), __saturatef(fmaf(v.y, 1.f / 6.f, 0.5f)));
-                                    v = __fmul2_rn(v, g);
-                                }
-                                ob[j] = __float22bfloat162_rn(v);
-                            }
-                            *reinterpret_cast<uint2 *>(yrow + (size_t)(wo0 + t) * a.K) = ov;
-                        }
-                    }
-                }
-            }
-        }
-    }
-    cp_async_wait<0>();
-}
-template <int K, int ACT, bool GROUP>
-__global__ void __launch_bounds__(128, K == 7 ? 3 : 4) dw_walk_kernel(const ConvArgs a1, const char *__restrict__ tbl, int n_img, int chblocks) {
-    pdl_launch_dependents();
-    __shared__ __align__(16) unsigned char smem[DwWalkShape<K>::SMEM];
-    SGS_DW_ARGS()
-    if (GROUP) { const ConvArgs al = a; dw_walk_body<K, ACT>(al, n, smem, chblocks); }
-    else dw_walk_body<K, ACT>(a, n, smem, chblocks);
-}
-// grid of the walking kernel for a member with `kmax` channels at most
-static dim3 dw_walk_grid(const ConvArgs &a, int kmax, int TW, int images) {
-    const int chblocks = (kmax / 4 + 31) / 32, tiles_w = (a.Wo + 4 * TW - 1) / (4 * TW);
-    return dim3((unsigned)(chblocks * tiles_w), (unsigned)((a.Ho + DW_WALK_SEG - 1) / DW_WALK_SEG), (unsigned)images);
-}
-
-// Members of one launch with different kernel sizes (a wave's depthwise layer: every member crops its own
-// k x k window out of the stored 7x7): each block runs the body of its member's kernel size.  The grid
-// covers the largest member; blocks beyond a member's own extent leave at once.
-// Stride 1: the walking bodies on the walking kernel's grid (sized for strips of 2 columns and the widest member);
-// stride 2: the patch / row bodies on their grid.
-template <int ST, int ACT, bool WALK> __device__ __forceinline__ void dw_mixed_dispatch(const ConvArgs &a, const int n, unsigned char *wsm, int chblocks);
-template <int ST, int ACT, bool WALK>
-__global__ void __launch_bounds__(128, 3) dw_mixed_kernel(const char *__restrict__ tbl, int n_img, int chblocks) {
-    pdl_launch_dependents();
-    constexpr bool GROUP = true;
-    __shared__ __align__(16) unsigned char wsm[WALK ? DwWalkShape<7>::SMEM : 16];  // (7x7 needs the most; 5x5: 37376, 3x3: 41472 bytes)
-    static_assert(DwWalkShape<7>::SMEM >= DwWalkShape<5>::SMEM && DwWalkShape<7>::SMEM >= DwWalkShape<3>::SMEM && DwWalkShape<7>::SMEM <= 48 * 1024, "ring sizes");
-    const ConvArgs a1 = ConvArgs();
-    SGS_DW_ARGS()
-    const ConvArgs al = a;  // (a copy in registers: reading the fields from shared memory at every use costs the tiled bodies 100 registers more)
-    dw_mixed_dispatch<ST, ACT, WALK>(al, n, wsm, chblocks);
-}
-template <int ST, int ACT, bool WALK>
-__device__ __forceinline__ void dw_mixed_dispatch(const ConvArgs &a, const int n, unsigned char *wsm, int chblocks) {
-    if (WALK) {
-        if (a.k == 3) dw_walk_body<3, ACT>(a, n, wsm, chblocks);
-        else if (a.k == 5) dw_walk_body<5, ACT>(a, n, wsm, chblocks);
-        else dw_walk_body<7, ACT>(a, n, wsm, chblocks);
-    } else if (ST == 1) {
-        if (a.k == 3) dw_tile_body<3, 1, 2, 4, true, ACT>(a, n);
-        else if (a.k == 5) dw_tile_body<5, 1, 1, 4, true, ACT>(a, n);
-        else dw_vec_body<7, 1>(a, n);
-    } else {
-        if (a.k == 3) dw_tile_body<3, 2, 1, 4, false, ACT>(a, n);
-        else if (a.k == 5) dw_vec_body<5, 2>(a, n);
-        else dw_vec_body<7, 2>(a, n);
-    }
-}
-
-// `a` = the (first) member; grouped: kmax = the widest member's channel count, tbl = device table, members > 0
-template <int K, int ST, int TH, int TW, bool PRELOAD, bool GROUP>
-static cudaError_t launch_dw_tile(const ConvArgs &a, int kmax, const char *tbl, int members, cudaStream_t st) {
-    const int per_row = ((a.Wo + TW - 1) / TW) * (kmax / 8);
-    dim3 grid((per_row + 127) / 128, (a.Ho + TH - 1) / TH, a.N * (GROUP ? members : 1));
-    if (a.act == ACT_RELU) SGS_LAUNCH((dw_tile_kernel<K, ST, TH, TW, PRELOAD, ACT_RELU, GROUP>), grid, dim3(128), 0, st, a, tbl, a.N);
-    else if (a.act == ACT_HSWISH) SGS_LAUNCH((dw_tile_kernel<K, ST, TH, TW, PRELOAD, ACT_HSWISH, GROUP>), grid, dim3(128), 0, st, a, tbl, a.N);
-    else SGS_LAUNCH((dw_tile_kernel<K, ST, TH, TW, PRELOAD, ACT_NONE, GROUP>), grid, dim3(128), 0, st, a, tbl, a.N);
-    return cudaGetLastError();
-}
-
-template <int K, bool GROUP>
-static cudaError_t launch_dw_walk(const ConvArgs &a, int kmax, const char *tbl, int members, cudaStream_t st) {
-    const dim3 grid = dw_walk_grid(a, kmax, DwWalkShape<K>::TW, a.N * (GROUP ? members : 1));
-    const int chblocks = (kmax / 4 + 31) / 32;
-    if (a.act == ACT_RELU) SGS_LAUNCH((dw_walk_kernel<K, ACT_RELU, GROUP>), grid, dim3(128), 0, st, a, tbl, a.N, chblocks);
-    else if (a.act == ACT_HSWISH) SGS_LAUNCH((dw_walk_kernel<K, ACT_HSWISH, GROUP>), grid, dim3(128), 0, st, a, tbl, a.N, chblocks);
-    else SGS_LAUNCH((dw_walk_kernel<K, ACT_NONE, GROUP>), grid, dim3(128), 0, st, a, tbl, a.N, chblocks);
-    return cudaGetLastError();
-}
-
-template <int K, int ST, bool GROUP>
-static cudaError_t launch_dw_vec(const ConvArgs &a, int kmax, const char *tbl, int members, cudaStream_t st) {
-    const int per_row = ((a.Wo + 3) / 4) * (kmax / 8);
-    const int block = per_row >= 256 ? 256 : per_row >= 128 ? 128 : 64;
-    dim3 grid((per_row + block - 1) / block, a.Ho, a.N * (GROUP ? members : 1));
-    SGS_LAUNCH((dw_vec_kernel<K, ST, GROUP>), grid, block, 0, st, a, tbl, a.N);
-    return cudaGetLastError();
-}
-
-static bool dw_vec_eligible(const ConvArgs &a) {
-    return a.K % 8 == 0 && a.Kmax % 8 == 0 && (a.stride == 1 || a.stride == 2) && a.Ho <= 65535 && a.N <= 65535 &&
-           (size_t)a.W * a.K < (1u << 30) &&
-           ((reinterpret_cast<uintptr_t>(a.x) | reinterpret_cast<uintptr_t>(a.w) | reinterpret_cast<uintptr_t>(a.y)) & 15) == 0 &&
-           ((reinterpret_cast<uintptr_t>(a.scale) | reinterpret_cast<uintptr_t>(a.shift)) & 15) == 0;
-}
-
-// Stride-1 layers take the walking kernel when the launch is large: at least this many million output elements over
-// all images and members, on maps at least 28 wide.  A block walks up to 56 rows one after the other, which pays on
-// working sets that stream from HBM (64 x 56 x 56 x 480: +6 % for 3x3, +13 % for 7x7 over the patch / row kernels) and
-// loses on the small launches of batch-1 waves (MobileNetV3-shaped stream: 34.7k queries/s without it, 32.3k with it
-// everywhere), where the patch kernels' many short threads win.  0 = never, negative = always; tuning aid.
-static int g_dw_walk_min_melems = 48;
-void dw_set_walk(int min_million_elements) { g_dw_walk_min_melems = min_million_elements; }
-static bool dw_walks(const ConvArgs &a, int kmax, int members) {
-    if (g_dw_walk_min_melems < 0) return true;  // (tests: every stride-1 shape through the walking kernel)
-    return g_dw_walk_min_melems > 0 && a.Wo >= 28 &&
-           (long long)a.N * members * a.Ho * a.Wo * kmax >= (long long)g_dw_walk_min_melems * 1000000ll;
-}
-
-// The vectorised bf16 kernel of a (kernel size, stride) pair; measured on working sets beyond L2
-// (N64 56x56 C480) the tiled kernel wins for k3 and for k5 stride 1.
-template <bool GROUP>
-static cudaError_t launch_dw_bf16(const ConvArgs &a, int kmax, const char *tbl, int members, cudaStream_t st) {
-    switch (a.k * 10 + a.stride) {
-    case 31: return dw_walks(a, kmax, GROUP ? members : 1) ? launch_dw_walk<3, GROUP>(a, kmax, tbl, members, st) : launch_dw_tile<3, 1, 2, 4, true, GROUP>(a, kmax, tbl, members, st);
-    case 32: return launch_dw_tile<3, 2, 1, 4, false, GROUP>(a, kmax, tbl, members, st);
-    case 51: return dw_walks(a, kmax, GROUP ? members : 1) ? launch_dw_walk<5, GROUP>(a, kmax, tbl, members, st) : launch_dw_tile<5, 1, 1, 4, true, GROUP>(a, kmax, tbl, members, st);
-    case 52: return launch_dw_vec<5, 2, GROUP>(a, kmax, tbl, members, st);
-    case 71: return dw_walks(a, kmax, GROUP ? members : 1) ? launch_dw_walk<7, GROUP>(a, kmax, tbl, members, st) : launch_dw_vec<7, 1, GROUP>(a, kmax, tbl, members, st);
-    case 72: return launch_dw_vec<7, 2, GROUP>(a, kmax, tbl, members, st);
-    default: return cudaErrorNotSupported;
-    }
-}
-
-cudaError_t launch_dw_group(const char *h_tbl, const char *d_tbl, int members, cudaStream_t st) {
-    if (members <= 0) return cudaSuccess;
-    const ConvArgs &a0 = *reinterpret_cast<const ConvArgs *>(h_tbl);
-    int kmax = 0;
-    bool mixed = false;
-    for (int i = 0; i < members; i++) {
-        const ConvArgs &a = *reinterpret_cast<const ConvArgs *>(h_tbl + (size_t)i * DW_ENTRY_BYTES);
-        if (!dw_vec_eligible(a) || (a.k != 3 && a.k != 5 && a.k != 7) || a.stride != a0.stride || a.act != a0.act || a.N != a0.N ||
-            a.H != a0.H || a.W != a0.W)
-            return cudaErrorNotSupported;
-        kmax = std::max(kmax, a.K);
-        mixed = mixed || a.k != a0.k;
-    }
-    if ((long long)a0.N * members > 65535) return cudaErrorNotSupported;
-    if (!mixed) return launch_dw_bf16<true>(a0, kmax, d_tbl, members, st);
-    // (same input size and stride, odd kernels with padding (k - 1) / 2: every member has the same output size)
-    const int per_row = ((a0.Wo + 3) / 4) * (kmax / 8);
-    const int chblocks = (kmax / 4 + 31) / 32;
-    if (a0.stride == 1 && dw_walks(a0, kmax, members)) {
-        const dim3 grid = dw_walk_grid(a0, kmax, 2, a0.N * members);
-        if (a0.act == ACT_RELU) SGS_LAUNCH((dw_mixed_kernel<1, ACT_RELU, true>), grid, dim3(128), 0, st, d_tbl, a0.N, chblocks);
-        else if (a0.act == ACT_HSWISH) SGS_LAUNCH((dw_mixed_kernel<1, ACT_HSWISH, true>), grid, dim3(128), 0, st, d_tbl, a0.N, chblocks);
-        else SGS_LAUNCH((dw_mixed_kernel<1, ACT_NONE, true>), grid, dim3(128), 0, st, d_tbl, a0.N, chblocks);
-    } else if (a0.stride == 1) {
-        // (the patch bodies of 3x3 and 5x5 own 2 resp. 1 output rows per block row: the grid covers single rows,
-        // blocks beyond a member's own extent leave at once)
-        dim3 grid((per_row + 127) / 128, a0.Ho, a0.N * members);
-        if (a0.act == ACT_RELU) SGS_LAUNCH((dw_mixed_kernel<1, ACT_RELU, false>), grid, dim3(128), 0, st, d_tbl, a0.N, chblocks);
-        else if (a0.act == ACT_HSWISH) SGS_LAUNCH((dw_mixed_kernel<1, ACT_HSWISH, false>), grid, dim3(128), 0, st, d_tbl, a0.N, chblocks);
-        else SGS_LAUNCH((dw_mixed_kernel<1, ACT_NONE, false>), grid, dim3(128), 0, st, d_tbl, a0.N, chblocks);
-    } else {
-        dim3 grid((per_row + 127) / 128, a0.Ho, a0.N * members);
-        if (a0.act == ACT_RELU) SGS_LAUNCH((dw_mixed_kernel<2, ACT_RELU, false>), grid, dim3(128), 0, st, d_tbl, a0.N, chblocks);
-        else if (a0.act == ACT_HSWISH) SGS_LAUNCH((dw_mixed_kernel<2, ACT_HSWISH, false>), grid, dim3(128), 0, st, d_tbl, a0.N, chblocks);
-        else SGS_LAUNCH((dw_mixed_kernel<2, ACT_NONE, false>), grid, dim3(128), 0, st, d_tbl, a0.N, chblocks);
-    }
-    return cudaGetLastError();
-}
-
 template <typename T> cudaError_t launch_dw(const ConvArgs &a, cudaStream_t st) {
     size_t total = (size_t)a.N * a.Ho * a.Wo * a.K;
     if (!total) return cudaSuccess;
-    if (sizeof(T) == 2 && dw_vec_eligible(a)) {
-        cudaError_t e = launch_dw_bf16<false>(a, a.K, nullptr, 1, st);
-        if (e != cudaErrorNotSupported) return e;
-    }
+    if (sizeof(T) == 2 && dw_eligible(a)) return launch_dw_single(a, st);
     int blocks = (int)std::min<size_t>((total + 255) / 256, 148 * 16);
     SGS_LAUNCH((dw_plain_kernel<T>), dim3(blocks), dim3(256), 0, st, a);
     return cudaGetLastError();
