@@ -305,19 +305,6 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
                 auto load_res = [&](int c0, int i) -> uint4 {
                     return (c0 + 8 * lc < cend && off[i] != 0xffffffffu) ? ld_act(reinterpret_cast<const uint4 *>(res) + off[i] + (uint32_t)((c0 >> 3) + lc)) : make_uint4(0u, 0u, 0u, 0u);
                 };
-                // The residual of this member's next tile on this CTA is brought to L2 one tile ahead: with streaming working
-                // sets its latency is several blocks long (1300 of the 2300 clocks of a block were spent waiting for it).
-                const int tn = t + (int)gridDim.x;
-                if (res && !second_half && !e.pair && tn < total_tiles && tn - e.tile_begin < e.mtiles * ((K + e.bn_tile - 1) / e.bn_tile)) {
-                    const int nl = tn - e.tile_begin, nnt = nl / e.mtiles, nmt = nl % e.mtiles;
-                    const int dn = row / (e.bh * e.bw), dhh = (row / e.bw) % e.bh, dww = row % e.bw;
-                    const int n = (nmt / e.tiles_hw) * e.bn + dn, h = ((nmt % e.tiles_hw) / e.tiles_w) * e.bh + dhh, w = (nmt % e.tiles_w) * e.bw + dww;
-                    if (row < e.pix_rows && n < e.N && h < e.Ho && w < e.Wo) {
-                        const __nv_bfloat16 *r0 = res + (((size_t)n * e.Ho + h) * e.Wo + w) * (size_t)ldk + nnt * e.bn_tile;
-                        const int cols = min((int)e.bn_tile, K - nnt * e.bn_tile);
-                        for (int c = half * 64; c < cols; c += 128) prefetch_l2(r0 + c);
-                    }
-                }
                 float2 sc[4], sh[4];
                 uint4 rv[4];
                 if (half * 32 < cend) {
@@ -334,16 +321,6 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
                     uint32_t v[32];
                     tmem_ld32(tacc + c0, v);
                     const int c = c0 + 8 * lc;  // this lane's 8 filters
-                    // the next block's parameters and residual (an L2 latency is as long as a block's work)
-                    float2 nsc[4], nsh[4];
-                    uint4 rn[4];
-                    if (c0 + 64 < cend) {
-                        load_bn(c0 + 64, nsc, nsh);
-                        if (res) {
-#pragma unroll
-                            for (int i = 0; i < 4; i++) rn[i] = load_res(c0 + 64, i);
-                        }
-                    }
                     tmem_ld_wait();
 #pragma unroll
                     for (int hr = 0; hr < 2; hr++) {
@@ -354,22 +331,19 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
                                 *reinterpret_cast<uint4 *>(stage + (lane & 15) * G_EPI_PITCH + 4 * g) = make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
                         }
                         __syncwarp();
-                        float4 qa[2], qb[2];
-#pragma unroll
-                        for (int i2 = 0; i2 < 2; i2++) {
-                            qa[i2] = *reinterpret_cast<const float4 *>(stage + (lr + 8 * i2) * G_EPI_PITCH + 8 * lc);
-                            qb[i2] = *reinterpret_cast<const float4 *>(stage + (lr + 8 * i2) * G_EPI_PITCH + 8 * lc + 4);
-                        }
 #pragma unroll
                         for (int i2 = 0; i2 < 2; i2++) {
                             const int i = hr * 2 + i2;
-                            float2 o[4] = {make_float2(qa[i2].x, qa[i2].y), make_float2(qa[i2].z, qa[i2].w), make_float2(qb[i2].x, qb[i2].y), make_float2(qb[i2].z, qb[i2].w)};
+                            const float4 qa = *reinterpret_cast<const float4 *>(stage + (lr + 8 * i2) * G_EPI_PITCH + 8 * lc);
+                            const float4 qb = *reinterpret_cast<const float4 *>(stage + (lr + 8 * i2) * G_EPI_PITCH + 8 * lc + 4);
+                            float2 o[4] = {make_float2(qa.x, qa.y), make_float2(qa.z, qa.w), make_float2(qb.x, qb.y), make_float2(qb.z, qb.w)};
 #pragma unroll
                             for (int q = 0; q < 4; q++) o[q] = __ffma2_rn(o[q], sc[q], sh[q]);
                             if (res) {
                                 const uint32_t r4[4] = {rv[i].x, rv[i].y, rv[i].z, rv[i].w};
 #pragma unroll
                                 for (int q = 0; q < 4; q++) o[q] = __fadd2_rn(o[q], make_float2(__uint_as_float(r4[q] << 16), __uint_as_float(r4[q] & 0xffff0000u)));
+                                rv[i] = load_res(c0 + 64, i);  // the next block's, used after its tensor-memory load
                             }
                             if (act == ACT_HSWISH) {
 #pragma unroll
@@ -383,11 +357,10 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
 #pragma unroll
                             for (int q = 0; q < 4; q++) ob[q] = __float22bfloat162_rn(o[q]);
                             if (c >= cend) out = make_uint4(0u, 0u, 0u, 0u);  // (the pixel's padding)
-                            if (c < cpad && off[i] != 0xffffffffu) st_act(reinterpret_cast<uint4 *>(y) + off[i] + (uint32_t)(c >> 3), out);
+                            if (c < cpad && off[i] != 0xffffffffu) reinterpret_cast<uint4 *>(y)[off[i] + (uint32_t)(c >> 3)] = out;
                         }
                     }
-#pragma unroll
-                    for (int q = 0; q < 4; q++) { sc[q] = nsc[q]; sh[q] = nsh[q]; rv[q] = rn[q]; }
+                    if (c0 + 64 < cend) load_bn(c0 + 64, sc, sh);
                 }
             } else {
                 // ---- swapped tile: this thread owns filter `f`, columns are the member's output pixels

@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_con
                     else { v.x = fmaxf(v.x, lo); v.y = fmaxf(v.y, lo); }
                     ob[j] = __float22bfloat162_rn(v);
                 }
-                st_act(reinterpret_cast<uint4 *>(p.y + (size_t)m * p.ldy + fc), ov);
+                *reinterpret_cast<uint4 *>(p.y + (size_t)m * p.ldy + fc) = ov;
             }
         };
         // S = blocks of the cluster; the parts of four outputs (one output's 8 with S = 8) are requested before the first is

@@ -45,13 +45,6 @@ __device__ __forceinline__ unsigned short ld_act(const unsigned short *p) {
 }
 __device__ __forceinline__ __nv_bfloat16 ld_act(const __nv_bfloat16 *p) { return __ushort_as_bfloat16(ld_act(reinterpret_cast<const unsigned short *>(p))); }
 
-// Store of an output vector that this kernel does not read back: unlike a store through a pointer it does not keep the
-// compiler from moving later shared-memory reads in front of it.
-__device__ __forceinline__ void st_act(uint4 *p, uint4 v) {
-    asm volatile("st.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w));
-}
-__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-
 // Launches `kernel` so that it may start while the previous kernel of the stream drains; cluster_z > 1: clusters along z.
 template <typename... P, typename... A>
 cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, unsigned cluster_z, A &&...args) {
