@@ -72,6 +72,24 @@ __device__ __forceinline__ void cluster_sync_all() {  // (every thread of every 
 
 constexpr int TC_EPI_WARPS = 8, TC_EPI = 32 * TC_EPI_WARPS, TC_THREADS = 64 + TC_EPI;
 
+// Requantisation of 8 filters in 64-bit arithmetic, for scales, biases and zero points that 32 bits do not hold.  Out of
+// line: inlined at every output it was most of the kernel's code, which then missed the instruction cache (3.5 of 14 stall
+// cycles per instruction; 32x56x56, 64 -> 128 filters, 1x1: 34.8 us, now 22.7).
+struct QuantWide { int acc[8], mult[8], shf[8], bias[8]; };  // acc: sums in, results (saturated to 32 bits) out
+__device__ __noinline__ void requantise_wide(const TcParams &p, QuantWide &t, uint4 rq) {
+#pragma unroll 1
+    for (int j = 0; j < 8; j++) {
+        long long v = rshift_round((long long)t.acc[j] * (long long)t.mult[j], 31 + t.shf[j]) + (long long)t.bias[j];
+        if (p.res) {
+            const uint32_t rb = ((j < 4 ? rq.x : rq.y) >> (8 * (j & 3))) & 0xffu;
+            const int r8 = p.q_flags & 4 ? (int)(signed char)rb : (int)rb;
+            v += rshift_round((long long)(r8 - p.q_zr) * (long long)p.q_res_mult, 31 + p.q_res_shift);
+        }
+        v += p.q_zy;
+        t.acc[j] = (int)(v < -2147483647ll ? -2147483647ll : (v > 2147483647ll ? 2147483647ll : v));
+    }
+}
+
 template <int BN, bool I8>
 __global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_constant__ TcParams p) {
     // (a stage row is 128 bytes either way: 64 bf16 or 128 8-bit channels; an MMA takes 32 bytes of it)
@@ -79,7 +97,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_con
     constexpr int B_STAGE_BYTES = BN * CHUNK_C * 2;
     constexpr int STAGE_BYTES = A_STAGE_BYTES + B_STAGE_BYTES;
     constexpr int ACC_PITCH = BN + 4;  // floats; (BN + 4) / 4 is odd: 8 consecutive rows lie in 8 different groups of 4 banks
-    constexpr int CHUNKS = BN / 8;     // output vectors of 8 filters per pixel
+    constexpr int CHUNKS_LOG = BN == 128 ? 4 : 3;  // output vectors of 8 filters per pixel
     extern __shared__ uint8_t smem_raw[];
     __shared__ int row_m[TILE_M];  // output pixel index of each tile row, -1 outside the tensor
     __shared__ __align__(8) uint64_t full_bar[TC_MAX_STAGES], empty_bar[TC_MAX_STAGES], accum_bar;
@@ -203,20 +221,24 @@ __global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_con
         asm volatile("bar.arrive 2, %0;" ::"n"(TC_EPI + 32) : "memory");
     }
     // ---------------------------------------------------------------------- epilogue (warps 2..9)
-    // Thread et finishes filters fc .. fc + 7 of the tile rows et / CHUNKS + i * RSTEP of this block's share.
+    // Thread et finishes filters fc .. fc + 7 of the tile rows row0 + i * rstep of this block's share; a narrow last tile gives
+    // its rows to fewer lanes each (the 48 filters beyond 128 of 176: half the steps).
     const bool epi = warp >= 2;
-    const int et = threadIdx.x - 64, chunk = et & (CHUNKS - 1), fc = f0 + 8 * chunk;
-    const int rows_mine = TILE_M / splits, row_first = rows_mine * (int)blockIdx.z, row0 = et / CHUNKS;
-    constexpr int RSTEP = TC_EPI / CHUNKS, BATCH = 4;
+    const int et = threadIdx.x - 64, csh = CHUNKS_LOG - (p.ldy - f0 <= BN / 2) - (p.ldy - f0 <= BN / 4), chunk = et & ((1 << csh) - 1), fc = f0 + 8 * chunk;
+    const int rows_mine = TILE_M / splits, row_first = rows_mine * (int)blockIdx.z, row0 = et >> csh, rstep = TC_EPI >> csh;
+    constexpr int BATCH = 4;
     const bool fvalid = epi && fc < p.K;
     bool ok_epi = epi;
     uint4 rv[BATCH];   // residual of up to four outputs
     float2 sc[4], sh[4];  // folded batch norm of the thread's filters (8-bit layers: multiplier and shift as integers)
     int bias[I8 ? 8 : 1];
+    // 8-bit layers: the requantised sums of this thread's filters fit 32 bits (shifts of 33 and more, which every scale below
+    // a quarter has, and terms within 2^28); 64-bit arithmetic otherwise.
+    bool q_narrow = I8 && abs(p.q_zy) < (1 << 28) && abs(p.q_zr) < (1 << 28) && p.q_res_shift >= 0;
     auto load_residual = [&](int i0) {
 #pragma unroll
         for (int i = 0; i < BATCH; i++) {
-            const int r = row0 + RSTEP * (i0 + i);
+            const int r = row0 + rstep * (i0 + i);
             rv[i] = make_uint4(0u, 0u, 0u, 0u);
             if (p.res && r < rows_mine && fvalid) {
                 const int m = row_m[row_first + r];
@@ -244,6 +266,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_con
                 a = __int_as_float(__ldg(p.q_mult + f));
                 b = __int_as_float(min(max(__ldg(p.q_shift + f), 0), 31));  // (0..31 by contract)
                 bias[I8 ? j : 0] = __ldg(p.q_bias + f);
+                q_narrow = q_narrow && __float_as_int(b) >= 2 && bias[I8 ? j : 0] > -(1 << 28) && bias[I8 ? j : 0] < (1 << 28);
             } else { a = __ldg(p.scale + f); b = __ldg(p.shift + f); }
             if (j & 1) { sc[j >> 1].y = a; sh[j >> 1].y = b; } else { sc[j >> 1].x = a; sh[j >> 1].x = b; }
         }
@@ -279,23 +302,40 @@ __global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_con
             if (I8) {
                 // requantise the int32 accumulator per filter, add bias, residual and the output zero point, ReLU as a
                 // maximum with the zero point, saturate, store 8 filters (8 bytes)
-                const bool ysig = p.q_flags & 2, rsig = p.q_flags & 4, relu = p.q_flags & 8;
-                const int qlo = ysig ? -128 : 0, qhi = ysig ? 127 : 255;
-                uint2 outw = make_uint2(0u, 0u);
+                const bool rsig = p.q_flags & 4;
+                const int qlo = p.q_flags & 2 ? -128 : 0, qhi = qlo + 255, least = p.q_flags & 8 ? max(qlo, min(p.q_zy, qhi)) : qlo;
+                int v[8];
+                if (!q_narrow) {
+                    QuantWide t;
 #pragma unroll
-                for (int j = 0; j < 8; j++) {
-                    const int mult = __float_as_int(j & 1 ? sc[j >> 1].y : sc[j >> 1].x), shf = __float_as_int(j & 1 ? sh[j >> 1].y : sh[j >> 1].x);
-                    long long t = rshift_round((long long)__float_as_int(o[j]) * (long long)mult, 31 + shf) + (long long)bias[I8 ? j : 0];
-                    if (p.res) {
-                        const uint32_t rb = ((j < 4 ? rq.x : rq.y) >> (8 * (j & 3))) & 0xffu;
-                        const int r8 = rsig ? (int)(signed char)rb : (int)rb;
-                        t += rshift_round((long long)(r8 - p.q_zr) * (long long)p.q_res_mult, 31 + p.q_res_shift);
+                    for (int j = 0; j < 8; j++) {
+                        t.acc[j] = __float_as_int(o[j]);
+                        t.mult[j] = __float_as_int(j & 1 ? sc[j >> 1].y : sc[j >> 1].x);
+                        t.shf[j] = __float_as_int(j & 1 ? sh[j >> 1].y : sh[j >> 1].x);
+                        t.bias[j] = bias[I8 ? j : 0];
                     }
-                    t += p.q_zy;
-                    if (relu && t < p.q_zy) t = p.q_zy;
-                    const uint32_t byte = (uint32_t)(int)(t < qlo ? qlo : (t > qhi ? qhi : t)) & 0xffu;
-                    if (j < 4) outw.x |= byte << (8 * j); else outw.y |= byte << (8 * (j - 4));
+                    requantise_wide(p, t, rq);
+#pragma unroll
+                    for (int j = 0; j < 8; j++) v[j] = t.acc[j];
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 8; j++) {
+                        const int mult = __float_as_int(j & 1 ? sc[j >> 1].y : sc[j >> 1].x), shf = __float_as_int(j & 1 ? sh[j >> 1].y : sh[j >> 1].x);
+                        // floor((p + 2^(s-1)) / 2^s) = floor((floor(p / 2^(s-1)) + 1) / 2), and s - 1 >= 32 here: the product's high word is enough
+                        v[j] = (((__mulhi(__float_as_int(o[j]), mult) >> (shf - 2)) + 1) >> 1) + bias[I8 ? j : 0] + p.q_zy;
+                    }
+                    if (p.res) {
+#pragma unroll
+                        for (int j = 0; j < 8; j++) {
+                            const uint32_t rb = ((j < 4 ? rq.x : rq.y) >> (8 * (j & 3))) & 0xffu;
+                            const int r8 = rsig ? (int)(signed char)rb : (int)rb;
+                            v[j] += (int)rshift_round((long long)(r8 - p.q_zr) * (long long)p.q_res_mult, 31 + p.q_res_shift);
+                        }
+                    }
                 }
+#pragma unroll
+                for (int j = 0; j < 8; j++) v[j] = min(max(v[j], least), qhi) & 0xff;
+                const uint2 outw = make_uint2((uint32_t)(v[0] | v[1] << 8 | v[2] << 16 | v[3] << 24), (uint32_t)(v[4] | v[5] << 8 | v[6] << 16 | v[7] << 24));
                 *reinterpret_cast<uint2 *>(reinterpret_cast<uint8_t *>(p.y) + (size_t)m * p.ldy + fc) = outw;
             } else {
                 const uint32_t r4[4] = {rq.x, rq.y, rq.z, rq.w};
@@ -314,9 +354,9 @@ __global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_con
         };
         // S = blocks of the cluster; the parts of four outputs (one output's 8 with S = 8) are requested before the first is
         // used, and summed in split order (the sums of 8-bit layers are integers).
-        const int n_out = (rows_mine + RSTEP - 1) / RSTEP;
+        const int n_out = (rows_mine + rstep - 1) / rstep;
         auto finish = [&](auto S_) {
-            constexpr int S = decltype(S_)::value, NB = S >= 4 ? 1 : 4 / S;
+            constexpr int S = decltype(S_)::value, NB = I8 ? (S == 1 ? 2 : 1) : S >= 4 ? 1 : 4 / S;  // (8-bit outputs take more registers each)
 #pragma unroll 1
             for (int i0 = 0; i0 < n_out; i0 += BATCH) {
                 if (i0) load_residual(i0);
@@ -327,7 +367,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_con
                     int m[NB];
 #pragma unroll
                     for (int i = 0; i < NB; i++) {
-                        const int r = row0 + RSTEP * (i0 + h + i), rr = row_first + min(r, rows_mine - 1);
+                        const int r = row0 + rstep * (i0 + h + i), rr = row_first + min(r, rows_mine - 1);
                         m[i] = r < rows_mine ? row_m[rr] : -1;
                         const int off = (rr * ACC_PITCH + 8 * chunk) * 4;
 #pragma unroll
@@ -659,6 +699,9 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
     p.iters = a.k * plan->kw * p.cchunks;
     // Filter tile: 128 wide where the tiles then still occupy every SM (half the pixel copies per filter), else 64.
     int BN = (a.K > 64 && (long long)mtiles * ((a.K + 127) / 128) >= sms) ? 128 : 64;
+    // 8-bit layers whose 64-wide tiles are all resident at two blocks per SM take those: no SM then gets two 128-wide tiles
+    // while others have one (16x28x28, 176 -> 176, 3x3: 25.0 -> 22.9 us).
+    if (a.i8 && (long long)mtiles * ((a.K + 63) / 64) <= 2 * sms) BN = 64;
     // A split (cluster of blocks) shortens the chain of steps by half for about a microsecond of meeting: it has to leave
     // at least four steps per block.
     int max_splits = p.iters >= 10 ? std::min(8, p.iters / 4) : 1;
