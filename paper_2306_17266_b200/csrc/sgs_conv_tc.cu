@@ -221,10 +221,11 @@ __global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_con
         asm volatile("bar.arrive 2, %0;" ::"n"(TC_EPI + 32) : "memory");
     }
     // ---------------------------------------------------------------------- epilogue (warps 2..9)
-    // Thread et finishes filters fc .. fc + 7 of the tile rows row0 + i * rstep of this block's share; a narrow last tile gives
-    // its rows to fewer lanes each (the 48 filters beyond 128 of 176: half the steps).
+    // Thread et finishes filters fc .. fc + 7 of the tile rows row0 + i * rstep of this block's share.  In 8-bit layers a narrow
+    // last tile gives its rows to fewer lanes each (the 48 filters beyond 128 of 176: half the steps of a requantisation); for
+    // bf16 the split is the compiler's to know (a single ResNet query: 268 us, 290 with one chosen at run time).
     const bool epi = warp >= 2;
-    const int et = threadIdx.x - 64, csh = CHUNKS_LOG - (p.ldy - f0 <= BN / 2) - (p.ldy - f0 <= BN / 4), chunk = et & ((1 << csh) - 1), fc = f0 + 8 * chunk;
+    const int et = threadIdx.x - 64, csh = CHUNKS_LOG - (I8 ? (p.ldy - f0 <= BN / 2) + (p.ldy - f0 <= BN / 4) : 0), chunk = et & ((1 << csh) - 1), fc = f0 + 8 * chunk;
     const int rows_mine = TILE_M / splits, row_first = rows_mine * (int)blockIdx.z, row0 = et >> csh, rstep = TC_EPI >> csh;
     constexpr int BATCH = 4;
     const bool fvalid = epi && fc < p.K;
