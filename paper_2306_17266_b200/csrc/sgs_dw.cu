@@ -2,16 +2,17 @@
 // norm and the activation, for one tensor or for all members of a wave (paper Section 2.1: elastic kernel = centre window;
 // Section 4.2: a line buffer keeps the rows a sliding window needs on chip).
 //
-// A block owns 64 channels x nw strips of TW output columns x a segment of output rows and walks down the input rows behind
-// a ring of rows in shared memory, filled RING - 1 rows ahead by 16-byte asynchronous copies (zero fill outside the tensor,
-// so the arithmetic has no bounds tests).  A warp is one strip, a lane two channels: an input vector is one conflict-free
-// 4-byte read, unpacked once and used for every output row and tap it belongs to; ceil(k / stride) output rows are live:
-// filter row 0 starts one with a product, filter row k - 1 completes the oldest.
+// A warp owns 64 channels x TW output columns x a segment of output rows and walks down it two output rows a step, behind a
+// ring of input rows of its own in shared memory; the next step's rows are in flight as 16-byte asynchronous copies (zero
+// fill outside the tensor, so the arithmetic has no bounds tests).  A lane owns two channels: an input vector is one
+// conflict-free 4-byte read, unpacked once and used for all its taps in both rows; a weight is one 8-byte read (fp32, of the
+// block) and used for 2 TW outputs.  Warps meet only once, when the block's weights are in place.
 //
-// What bounds it: the fp32 multiply-adds for k = 5 and 7 (packed, two per instruction), HBM for k = 3.  The kernel this one
-// replaces kept the weights in shared memory and read 16 bytes of them per tap for 4 packed multiply-adds, which took the
-// shared-memory pipe twice as long as the arithmetic; here a lane keeps its k * k packed weights in registers and a weight
-// serves TW outputs.
+// What bounds it: instruction issue (2.3 of 4 a cycle; half of them the packed multiply-adds and the unpacking of inputs,
+// both at the rate of their pipes half the time).  Measured on 64x56x56x480, 5x5, stride 1, h-swish: 177 us against 228 us
+// of the kernel that it replaces, which kept weights in shared memory too but read 16 bytes of them for 4 packed
+// multiply-adds.  Slower forms of this one: a ring shared by the block (a barrier a step) 194 us; weights in registers
+// (128 of them, spills) 198 us; all live output rows in registers, one input row a step (188 registers, 7 warps per SM) 365 us.
 #include "sgs_internal.h"
 #include "sgs_pdl.cuh"
 
@@ -212,9 +213,10 @@ cudaError_t launch_shape(const ConvArgs &a, int kmin, int kmax, int ch, const ch
     const int seg = ((a.Ho + nseg - 1) / nseg + 1) & ~1;
     int smem = 0;
     for (int k = kmin; k <= kmax; k += 2) smem = std::max(smem, block_bytes<ST, WIDE>(k));
+    const int most = std::max({block_bytes<ST, WIDE>(3), block_bytes<ST, WIDE>(5), block_bytes<ST, WIDE>(7)});
     const DwKernel kern = kmin != kmax ? dw_mixed_kernel<ST, WIDE> : kmin == 3 ? dw_kernel<3, ST, WIDE> : kmin == 5 ? dw_kernel<5, ST, WIDE> : dw_kernel<7, ST, WIDE>;
     if (smem + (int)sizeof(ConvArgs) > 47 * 1024) {  // (the static record counts too)
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most);  // (one value for all callers: threads may meet here)
         if (e != cudaSuccess) return e;
     }
     const long long units = (long long)((a.Wo + tw - 1) / tw) * ((a.Ho + seg - 1) / seg);
