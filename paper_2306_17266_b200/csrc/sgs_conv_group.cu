@@ -63,24 +63,12 @@ struct __align__(16) GroupEntry {
 };
 static_assert(sizeof(GroupEntry) == TC_GROUP_ENTRY_BYTES, "entry size");
 
-// Index of the entry that owns tile t (entries are sorted by tile_begin); the whole warp calls it.
-__device__ __forceinline__ int find_entry(const GroupEntry *es, int n, int t, int lane) {
-    const unsigned b0 = __ballot_sync(0xffffffffu, lane < n && es[lane].tile_begin <= t);
-    const unsigned b1 = __ballot_sync(0xffffffffu, lane + 32 < n && es[lane + 32].tile_begin <= t);
-    return __popc(b0) + __popc(b1) - 1;
-}
-// Same for one thread.
-__device__ __forceinline__ int find_entry_serial(const GroupEntry *es, int n, int t) {
-    int lo = 0, hi = n - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (es[mid].tile_begin <= t) lo = mid; else hi = mid - 1;
-    }
-    return es[lo].second ? lo - 1 : lo;
-}
-// The entry that owns tile t's geometry (the first member of a pair); the whole warp calls it.
-__device__ __forceinline__ int tile_entry(const GroupEntry *es, int n, int t, int lane) {
-    const int i = find_entry(es, n, t, lane);
+// Index of the entry that owns tile t's geometry (the first member of a pair); the whole warp calls it.  begin[]: the entries'
+// first tiles, sorted, INT_MAX beyond the last (an array of its own: read out of the 128-byte records, the 32 lanes' words
+// would lie in one bank).
+__device__ __forceinline__ int tile_entry(const GroupEntry *es, const int *begin, int t, int lane) {
+    const unsigned b0 = __ballot_sync(0xffffffffu, begin[lane] <= t), b1 = __ballot_sync(0xffffffffu, begin[lane + 32] <= t);
+    const int i = __popc(b0) + __popc(b1) - 1;
     return es[i].second ? i - 1 : i;
 }
 
@@ -107,6 +95,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
     int *status = P.status;
     extern __shared__ uint8_t smem_raw[];
     __shared__ GroupEntry es[TC_GROUP_MAX_ENTRIES];
+    __shared__ int begin[TC_GROUP_MAX_ENTRIES];
     __shared__ __align__(8) uint64_t full_bar[G_MAX_STAGES], empty_bar[G_MAX_STAGES], acc_full[2], acc_empty[2];
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s;
@@ -119,6 +108,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
     // the wait on the previous layer.
     for (int i = threadIdx.x; i < n_entries * (int)(sizeof(GroupEntry) / 16); i += blockDim.x)
         reinterpret_cast<uint4 *>(es)[i] = __ldg(reinterpret_cast<const uint4 *>(entries) + i);
+    for (int i = threadIdx.x; i < TC_GROUP_MAX_ENTRIES; i += blockDim.x) begin[i] = i < n_entries ? __ldg(&entries[i].tile_begin) : 0x7fffffff;
     if (threadIdx.x == 0) {
         for (int s = 0; s < G_MAX_STAGES; s++) { mbar_init(&full_bar[s], 2); mbar_init(&empty_bar[s], 1); }  // (full: both producers arrive)
         for (int b = 0; b < 2; b++) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], G_EPI_WARPS); }
@@ -145,7 +135,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
         uint32_t phase = 0;
         bool wrapped = false, ok = true;
         for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x) {
-            const GroupEntry &e = es[tile_entry(es, n_entries, t, lane)];
+            const GroupEntry &e = es[tile_entry(es, begin, t, lane)];
             const int nt = (t - e.tile_begin) / e.mtiles;
             const int wrows = e.swap ? 128 : e.bn_tile;  // rows of the weight box
             const int f0 = (int)uniform((uint32_t)(nt * wrows));
@@ -171,7 +161,10 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
                 }
             }
             const int tn = t + (int)gridDim.x;
-            if (ok && tn < total_tiles && on) prefetch_tensormap(&P.maps[es[find_entry_serial(es, n_entries, tn)].map_w]);
+            if (ok && tn < total_tiles) {
+                const int en = tile_entry(es, begin, tn, lane);
+                if (on) prefetch_tensormap(&P.maps[es[en].map_w]);
+            }
             __syncwarp();
         }
     } else if (warp == G_PIX_WARP) {
@@ -182,10 +175,10 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
         bool wrapped = false, ok = true;
         pdl_wait();  // activations (and the buffers this layer overwrites) belong to the previous layers until here
         for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x) {
-            const GroupEntry &e = es[tile_entry(es, n_entries, t, lane)];
-            const int mt = (t - e.tile_begin) % e.mtiles;
-            const int n0 = (int)uniform((uint32_t)((mt / e.tiles_hw) * e.bn)), h0 = (int)uniform((uint32_t)(((mt % e.tiles_hw) / e.tiles_w) * e.bh)),
-                      w0 = (int)uniform((uint32_t)((mt % e.tiles_w) * e.bw));
+            const GroupEntry &e = es[tile_entry(es, begin, t, lane)];
+            const int lt = t - e.tile_begin, mt = lt - lt / e.mtiles * e.mtiles;
+            const int tn_ = mt / e.tiles_hw, mhw = mt - tn_ * e.tiles_hw, th_ = mhw / e.tiles_w, tw_ = mhw - th_ * e.tiles_w;
+            const int n0 = (int)uniform((uint32_t)(tn_ * e.bn)), h0 = (int)uniform((uint32_t)(th_ * e.bh)), w0 = (int)uniform((uint32_t)(tw_ * e.bw));
             const bool pair = uniform(e.pair) != 0;
             const uint32_t pix_bytes = uniform((uint32_t)(e.pix_rows * CHUNK_C * 2) + (pair ? (uint32_t)((&e)[1].pix_rows * CHUNK_C * 2) : 0u));
             const uint32_t dst0 = uniform(ring + (e.swap ? (uint32_t)G_X_BYTES : 0u));
@@ -209,7 +202,10 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
                 }
             }
             const int tn = t + (int)gridDim.x;
-            if (ok && tn < total_tiles && on) prefetch_tensormap(&P.maps[es[find_entry_serial(es, n_entries, tn)].map_a]);
+            if (ok && tn < total_tiles) {
+                const int en = tile_entry(es, begin, tn, lane);
+                if (on) prefetch_tensormap(&P.maps[es[en].map_a]);
+            }
             __syncwarp();
         }
     } else if (warp == 1) {
@@ -219,7 +215,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
         uint32_t phase = 0;
         bool ok = true;
         for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x, j++) {
-            const GroupEntry &e = es[tile_entry(es, n_entries, t, lane)];
+            const GroupEntry &e = es[tile_entry(es, begin, t, lane)];
             const int nt = (t - e.tile_begin) / e.mtiles;
             // MMA shape: 128 rows; columns = this tile's filters (normal) or the member's pixels (swapped),
             // rounded up to 16; bf16 x bf16 -> fp32, both operands K-major
@@ -267,8 +263,8 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
         pdl_wait();  // residual reads and output writes must not pass the previous layers
         int j = 0;   // tiles of this CTA so far
         for (int t = (int)blockIdx.x; t < total_tiles; t += (int)gridDim.x, j++) {
-            const GroupEntry &e0 = es[tile_entry(es, n_entries, t, lane)];
-            const int local = t - e0.tile_begin, nt = local / e0.mtiles, mt = local % e0.mtiles;
+            const GroupEntry &e0 = es[tile_entry(es, begin, t, lane)];
+            const int local = t - e0.tile_begin, nt = local / e0.mtiles, mt = local - nt * e0.mtiles;
             // rows 64..127 of a pair's tile belong to the second member (a warp lies on one side)
             const bool second_half = e0.pair && quad >= 2;
             const GroupEntry &e = second_half ? (&e0)[1] : e0;
@@ -279,12 +275,13 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
             const uint32_t tacc = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * G_ACC_COLS);
             if (!e.swap) {
                 // ---- normal tile: rows are output pixels, columns are filters
-                const int n0 = (mt / e.tiles_hw) * e.bn, h0 = ((mt % e.tiles_hw) / e.tiles_w) * e.bh, w0 = (mt % e.tiles_w) * e.bw;
+                const int tn = mt / e.tiles_hw, mhw = mt - tn * e.tiles_hw, th = mhw / e.tiles_w, tw = mhw - th * e.tiles_w;
+                const int n0 = tn * e.bn, h0 = th * e.bh, w0 = tw * e.bw;
                 const int f0 = nt * e0.bn_tile;
                 // offset of the four rows this lane finishes (lr + 8 i), in vectors of 8 channels; ~0: outside the tensor
                 uint32_t off[4];
                 {
-                    const int dn = row / (e.bh * e.bw), dhh = (row / e.bw) % e.bh, dww = row % e.bw;
+                    const int dl = row / e.bw, dww = row - dl * e.bw, dn = dl / e.bh, dhh = dl - dn * e.bh;
                     const int n = n0 + dn, h = h0 + dhh, w = w0 + dww;
                     const bool valid = row < e.pix_rows && n < e.N && h < e.Ho && w < e.Wo;
                     const uint32_t mine = valid ? (uint32_t)(((size_t)((size_t)n * e.Ho + h) * e.Wo + w) * (size_t)(ldk >> 3)) + (uint32_t)(f0 >> 3) : 0xffffffffu;
@@ -294,33 +291,51 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
                 const int cend = min((int)e0.bn_tile, K - f0);    // filters of this tile, a multiple of 8 (<= 0: none of this member's)
                 const int cpad = min((int)e0.bn_tile, ldk - f0);  // ... and the end of the pixel's padding, written as zeros
                 const float lo = act == ACT_RELU ? 0.f : __int_as_float(0xff800000);  // ReLU as a maximum; no activation: -infinity
-                auto load_bn = [&](int c0, float2 *sc, float2 *sh) {
-                    const int f = f0 + min(c0 + 8 * lc, max(cend, 8) - 8);
-#pragma unroll
-                    for (int q = 0; q < 4; q++) {
-                        sc[q] = __ldg(reinterpret_cast<const float2 *>(e.scale + f) + q);
-                        sh[q] = __ldg(reinterpret_cast<const float2 *>(e.shift + f) + q);
-                    }
-                };
+                // Folded batch norm of a block's 32 filters: a lane loads one filter's, and the warp meets in the padding of its
+                // staging rows (4 floats a row: scales in rows 0..7, shifts in 8..15).
+                float *bnp = stage + (lane >> 2) * G_EPI_PITCH + 32 + (lane & 3);
+                auto load_bn = [&](int c0) { const int f = f0 + min(c0 + lane, max(cend, 1) - 1); return make_float2(__ldg(e.scale + f), __ldg(e.shift + f)); };
+                auto put_bn = [&](float2 b) { bnp[0] = b.x; bnp[8 * G_EPI_PITCH] = b.y; };
                 auto load_res = [&](int c0, int i) -> uint4 {
                     return (c0 + 8 * lc < cend && off[i] != 0xffffffffu) ? ld_act(reinterpret_cast<const uint4 *>(res) + off[i] + (uint32_t)((c0 >> 3) + lc)) : make_uint4(0u, 0u, 0u, 0u);
                 };
-                float2 sc[4], sh[4];
                 uint4 rv[4];
                 if (half * 32 < cend) {
-                    load_bn(half * 32, sc, sh);
                     if (res) {
 #pragma unroll
                         for (int i = 0; i < 4; i++) rv[i] = load_res(half * 32, i);
                     }
+                    put_bn(load_bn(half * 32));
                 }
                 if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[buf], (j >> 1) & 1, abort_flag))) break;
                 tc_fence_after();
 #pragma unroll 1
                 for (int c0 = half * 32; c0 < cpad; c0 += 64) {
+                    // The next block's residual and batch norm, asked for a whole block ahead into registers of their own.  All at
+                    // one place and all used at one place: loads in flight share scoreboards, and a use between two of them waits
+                    // for both (the first 16 rows of a block with a residual: 1350 -> 670 clocks; what is left of the residual's
+                    // latency is the first block's of a tile.  4 queries x 16 images of 224x224: 1 %).
+                    uint4 rn[4];
+                    float2 bn = make_float2(0.f, 0.f);
+                    const bool more = c0 + 64 < cend;
+                    if (more) {
+                        bn = load_bn(c0 + 64);
+                        if (res) {
+#pragma unroll
+                            for (int i = 0; i < 4; i++) rn[i] = load_res(c0 + 64, i);
+                        }
+                    }
                     uint32_t v[32];
                     tmem_ld32(tacc + c0, v);
                     const int c = c0 + 8 * lc;  // this lane's 8 filters
+                    __syncwarp();
+                    float2 sc[4], sh[4];
+#pragma unroll
+                    for (int q = 0; q < 2; q++) {
+                        const float4 a = *reinterpret_cast<const float4 *>(stage + (2 * lc + q) * G_EPI_PITCH + 32), b = *reinterpret_cast<const float4 *>(stage + (8 + 2 * lc + q) * G_EPI_PITCH + 32);
+                        sc[2 * q] = make_float2(a.x, a.y); sc[2 * q + 1] = make_float2(a.z, a.w);
+                        sh[2 * q] = make_float2(b.x, b.y); sh[2 * q + 1] = make_float2(b.z, b.w);
+                    }
                     tmem_ld_wait();
 #pragma unroll
                     for (int hr = 0; hr < 2; hr++) {
@@ -343,7 +358,6 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
                                 const uint32_t r4[4] = {rv[i].x, rv[i].y, rv[i].z, rv[i].w};
 #pragma unroll
                                 for (int q = 0; q < 4; q++) o[q] = __fadd2_rn(o[q], make_float2(__uint_as_float(r4[q] << 16), __uint_as_float(r4[q] & 0xffff0000u)));
-                                rv[i] = load_res(c0 + 64, i);  // the next block's, used after its tensor-memory load
                             }
                             if (act == ACT_HSWISH) {
 #pragma unroll
@@ -360,7 +374,13 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
                             if (c < cpad && off[i] != 0xffffffffu) reinterpret_cast<uint4 *>(y)[off[i] + (uint32_t)(c >> 3)] = out;
                         }
                     }
-                    if (c0 + 64 < cend) load_bn(c0 + 64, sc, sh);
+                    if (more) {
+                        put_bn(bn);  // (everybody has this block's in registers: two warp barriers since)
+                        if (res) {
+#pragma unroll
+                            for (int i = 0; i < 4; i++) rv[i] = rn[i];
+                        }
+                    }
                 }
             } else {
                 // ---- swapped tile: this thread owns filter `f`, columns are the member's output pixels
