@@ -314,8 +314,9 @@ sgs_status_t sgs_subnet_cost(const sgs_supernet_t *net, const sgs_subnet_cfg_t *
  * 16-byte aligned; kernels larger than 1x1 at stride 2 need at least 2x2 pixels), 1 = CUDA-core kernel, 2 = tensor cores or
  * SGS_EUNSUPPORTED.  weight_policy 0 = no L2 hint, 1 = evict-last for weight tiles with filter <
  * cache_k and channel < cache_c (default replacement for the rest), 2 = all weights evict-first.
- * Asynchronous on `cuda_stream`.  The tensor-core path may split the reduction over a cluster of CTAs, whose partial sums
- * stay in shared memory: no device memory is allocated.
+ * Asynchronous on `cuda_stream`; everything passed in, weights and parameters included, may be what earlier work on the
+ * stream writes.  The tensor-core path may split the reduction over a cluster of CTAs, whose partial sums stay in shared
+ * memory: no device memory is allocated.
  */
 typedef struct {
     int N, H, W, C, K;      /* input dims, sliced channels C, sliced filters K */

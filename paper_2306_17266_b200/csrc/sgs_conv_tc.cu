@@ -165,8 +165,9 @@ __global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_con
             if (c0 < hint_c) tma_load_3d_hint_if(on, sb, &p.tmW, fb, c0, tapw, f0, pol);
             else tma_load_3d_if(on, sb, &p.tmW, fb, c0, tapw, f0);
         };
-        // Weights do not depend on the previous layer: fill the first stages' weight halves before
-        // waiting for it, so that their latency overlaps the previous layer's tail.
+        // Stored weights do not depend on the previous layer: fill the first stages' weight halves before waiting for it, so
+        // that their latency overlaps the previous layer's tail.  A caller's weights may be what the previous kernel writes.
+        if (!p.early_weights) pdl_wait();
         {
             int cc2 = cc, r2 = r, sx2 = sx;
             const int pre = min(n_it, stages);
@@ -259,16 +260,17 @@ __global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_con
             const int n = n0 + dn, h = h0 + dhh, w = w0 + dww;
             row_m[et] = et < rows && n < p.N && h < p.Ho && w < p.Wo ? (int)(((size_t)n * p.Ho + h) * p.Wo + w) : -1;
         }
+        if (!p.early_weights) pdl_wait();
 #pragma unroll
         for (int j = 0; j < 8; j++) {
             const int f = min(fc, p.K - 8) + j;
             float a, b;
             if (I8) {
-                a = __int_as_float(__ldg(p.q_mult + f));
-                b = __int_as_float(min(max(__ldg(p.q_shift + f), 0), 31));  // (0..31 by contract)
-                bias[I8 ? j : 0] = __ldg(p.q_bias + f);
+                a = __int_as_float(ld_act(p.q_mult + f));
+                b = __int_as_float(min(max(ld_act(p.q_shift + f), 0), 31));  // (0..31 by contract)
+                bias[I8 ? j : 0] = ld_act(p.q_bias + f);
                 q_narrow = q_narrow && __float_as_int(b) >= 2 && bias[I8 ? j : 0] > -(1 << 28) && bias[I8 ? j : 0] < (1 << 28);
-            } else { a = __ldg(p.scale + f); b = __ldg(p.shift + f); }
+            } else { a = ld_act(p.scale + f); b = ld_act(p.shift + f); }
             if (j & 1) { sc[j >> 1].y = a; sh[j >> 1].y = b; } else { sc[j >> 1].x = a; sh[j >> 1].x = b; }
         }
         asm volatile("bar.sync 1, %0;" ::"n"(TC_EPI) : "memory");
@@ -789,6 +791,7 @@ cudaError_t tc_conv_launch(const TcConvPlan &pl, const ConvArgs &a, cudaStream_t
     prm.status = g_dev[dev].status;
     prm.cacheK = a.cacheK; prm.cacheC = a.cacheC; prm.weight_policy = a.weight_policy;
     prm.cache_tbl = a.cache_tbl; prm.layer = a.layer;
+    prm.early_weights = a.early_weights;
     if (pl.i8) {
         if (!a.q_mult || !a.q_shift || !a.q_bias || pl.bn_tile > 128) return cudaErrorInvalidValue;
         prm.q_mult = a.q_mult; prm.q_shift = a.q_shift; prm.q_bias = a.q_bias;
@@ -894,6 +897,7 @@ extern "C" sgs_status_t sgs_conv2d_sliced_static(const sgs_conv_desc_t *d, const
     prm.status = &sc->status;
     prm.cacheK = a.cacheK; prm.cacheC = a.cacheC; prm.weight_policy = a.weight_policy;
     prm.cache_tbl = nullptr; prm.layer = 0;
+    prm.early_weights = 0;
     const cudaError_t e = plan->bn_tile == 64 ? launch_variant<64, false>(*plan, prm, st) : launch_variant<128, false>(*plan, prm, st);
     return e == cudaSuccess ? SGS_OK : SGS_ECUDA;
 }

@@ -15,9 +15,10 @@ namespace sgs {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// Loads of activations in kernels that start before the previous kernel has finished.  The read-only path (__ldg, or a
-// const __restrict__ pointer) is for data that nothing writes while the kernel exists, and the compiler may move such a
-// load above pdl_wait(); these stay behind it.
+// Loads, in kernels that start before the previous kernel has finished, of what that kernel may still be writing:
+// activations, and weights and parameters that are the caller's.  The read-only path (__ldg, or a const __restrict__
+// pointer) is for data that nothing writes while the kernel exists, and the compiler may move such a load above pdl_wait();
+// these stay behind it.
 __device__ __forceinline__ uint4 ld_act(const uint4 *p) {
     uint4 v;
     asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
@@ -36,6 +37,11 @@ __device__ __forceinline__ uint2 ld_act(const uint2 *p) {
 __device__ __forceinline__ float ld_act(const float *p) {
     float v;
     asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ int ld_act(const int *p) {
+    int v;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
 }
 __device__ __forceinline__ unsigned short ld_act(const unsigned short *p) {

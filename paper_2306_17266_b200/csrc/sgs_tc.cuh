@@ -32,6 +32,7 @@ struct TcParams {
     int cacheK, cacheC, weight_policy;
     const int *cache_tbl;    // optional device table overriding the three values above (see ConvArgs)
     int layer;
+    int early_weights;       // 1: weights and epilogue parameters may be read before the previous kernel has finished (see ConvArgs)
     // int8 layers (8-bit operands, int32 accumulator): per-filter requantisation parameters and the integer epilogue
     //   v = rshift_round(acc * q_mult[f], 31 + q_shift[f]) + q_bias[f] + rshift_round((res - q_zr) * q_res_mult, 31 + q_res_shift) + q_zy
     const int *q_mult, *q_shift, *q_bias;
