@@ -404,6 +404,7 @@ sgs_status_t sgs_conv2d_sliced_i8(const sgs_conv_i8_desc_t *desc, const void *d_
  *   SGS_AUX_SE_GATE   y[n][c] = hsigmoid(b2[c] + sum_{j<K} w2[c][j] relu(b1[j] + sum_{i<C} w[j][i] x[n][i])), c < C;
  *                     x [N][C] fp32 pooled vectors, w [>=K][ld], w2 [>=C][ld2] dtype, y [N][C] fp32
  *   SGS_AUX_SE_SCALE  y[n][h][w][c] = x[n][h][w][c] * g[n][c]; x, y [N][H][W][C] dtype, g = `w` [N][C] fp32
+ * Everything passed in, weights included, may be what earlier work on the stream writes.
  * n_members >= 1 independent problems desc[m] / args[m].  grouped = 0: each runs in the kernel a single query
  * uses; grouped = 1: all of them (same kind and dtype SGS_BF16) run in ONE launch of the kernel a wave uses, whose
  * per-member records this call uploads to a temporary device table (it allocates and synchronises the stream).

@@ -775,7 +775,7 @@ SmallEntry small_entry(const sgs_supernet *net, const Plan *plan, const Op &op, 
     case OP_LINEAR: {
         const StoredLayer &L = net->layers[op.layer];
         e.x = sl.vec[op.vin]; e.y = op.vout < 0 ? d_logits : (void *)sl.vec[op.vout];
-        e.w = L.w; e.bias = L.shift;
+        e.w = L.w; e.bias = L.shift; e.early_weights = 1;
         e.N = op.N; e.C = op.C; e.K = op.K; e.ld = L.C; e.act = op.act;
         break;
     }
@@ -863,7 +863,7 @@ sgs_status_t launch_op(sgs_supernet *net, Plan *plan, Op &op, const void *d_inpu
     case OP_LINEAR: {
         const StoredLayer &L = net->layers[op.layer];
         float *y = op.vout < 0 ? static_cast<float *>(d_logits) : sl.vec[op.vout];
-        CU(launch_linear<T>(sl.vec[op.vin], (const T *)L.w, L.shift, y, op.N, op.C, op.K, L.C, op.act, st));
+        CU(launch_linear<T>(sl.vec[op.vin], (const T *)L.w, L.shift, y, op.N, op.C, op.K, L.C, op.act, 1, st));
         net->kernel_launches++;
         break;
     }
@@ -2727,8 +2727,8 @@ sgs_status_t sgs_aux_op(int n, const sgs_aux_desc_t *desc, const sgs_aux_args_t 
             ce = bf ? launch_gap<B>((const B *)e.x, (float *)e.y, d.N, d.H * d.W, d.C, st) : launch_gap<float>((const float *)e.x, (float *)e.y, d.N, d.H * d.W, d.C, st);
             break;
         case SGS_AUX_LINEAR:
-            ce = bf ? launch_linear<B>((const float *)e.x, (const B *)e.w, e.bias, (float *)e.y, d.N, d.C, d.K, d.ld, d.act, st)
-                    : launch_linear<float>((const float *)e.x, (const float *)e.w, e.bias, (float *)e.y, d.N, d.C, d.K, d.ld, d.act, st);
+            ce = bf ? launch_linear<B>((const float *)e.x, (const B *)e.w, e.bias, (float *)e.y, d.N, d.C, d.K, d.ld, d.act, 0, st)
+                    : launch_linear<float>((const float *)e.x, (const float *)e.w, e.bias, (float *)e.y, d.N, d.C, d.K, d.ld, d.act, 0, st);
             break;
         case SGS_AUX_SE_GATE:
             ce = bf ? launch_se_gate<B>((const float *)e.x, (const B *)e.w, e.bias, (const B *)e.w2, e.bias2, (float *)e.y, d.N, d.C, d.K, d.ld, d.ld2, st)

@@ -173,7 +173,7 @@ cudaError_t launch_se_gate(const float *g, const T *w1, const float *b1, const T
 template <typename T> cudaError_t launch_scale(const T *x, const float *gate, T *y, int N, int HW, int C, cudaStream_t st);
 template <typename T>
 cudaError_t launch_linear(const float *v, const T *w, const float *bias, float *y, int N, int C, int K, int ld, int act,
-                          cudaStream_t st);
+                          int early_weights, cudaStream_t st);
 cudaError_t launch_relayout_conv(const float *src, void *dst, int K, int C, int Cp, int R, int S, int bf16, cudaStream_t st);  // dst [K][R][S][Cp], zero beyond C
 cudaError_t launch_relayout_dw(const float *src, void *dst, int K, int R, int S, int bf16, cudaStream_t st);
 cudaError_t launch_convert(const float *src, void *dst, size_t n, int bf16, cudaStream_t st);
@@ -196,7 +196,8 @@ struct alignas(16) SmallEntry {
     const void *w2;      // SE gate: second FC weights [C][ld2] bf16 (first FC: w [K][ld], K = squeeze width)
     const float *bias2;  // SE gate: second FC bias [C]
     int ld2;
-    int pad_[7];
+    int early_weights;   // linear: as in ConvArgs
+    int pad_[6];
 };
 static_assert(sizeof(SmallEntry) == 128, "record size");
 // kind: OP_MAXPOOL (3x3 stride 2, C % 8 == 0), OP_GAP (C % 8 == 0), OP_LINEAR (C % 8 == 0, ld % 8 == 0),

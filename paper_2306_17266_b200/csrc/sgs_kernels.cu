@@ -185,10 +185,8 @@ template cudaError_t launch_gap<__nv_bfloat16>(const __nv_bfloat16 *, float *, i
 // One block per image; warps stride over outputs and reduce with shuffles.
 // ---------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(1024) se_gate_kernel(const float *g, const T *__restrict__ w1,
-                                                      const float *__restrict__ b1, const T *__restrict__ w2,
-                                                      const float *__restrict__ b2, float *gate, int mid,
-                                                      int sq, int w1_ld, int w2_ld) {
+__global__ void __launch_bounds__(1024) se_gate_kernel(const float *g, const T *w1, const float *b1, const T *w2,
+                                                      const float *b2, float *gate, int mid, int sq, int w1_ld, int w2_ld) {
     pdl_launch_dependents();
     pdl_wait();
     extern __shared__ float sm[];
@@ -198,18 +196,18 @@ __global__ void __launch_bounds__(1024) se_gate_kernel(const float *g, const T *
     __syncthreads();
     for (int j = warp; j < sq; j += nw) {
         float s = 0.f;
-        for (int c = lane; c < mid; c += 32) s = fmaf(to_f<T>(w1[(size_t)j * w1_ld + c]), gs[c], s);
+        for (int c = lane; c < mid; c += 32) s = fmaf(to_f<T>(ld_act(w1 + (size_t)j * w1_ld + c)), gs[c], s);
 #pragma unroll
         for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) zs[j] = fmaxf(s + b1[j], 0.f);
+        if (lane == 0) zs[j] = fmaxf(s + ld_act(b1 + j), 0.f);
     }
     __syncthreads();
     for (int c = warp; c < mid; c += nw) {
         float s = 0.f;
-        for (int j = lane; j < sq; j += 32) s = fmaf(to_f<T>(w2[(size_t)c * w2_ld + j]), zs[j], s);
+        for (int j = lane; j < sq; j += 32) s = fmaf(to_f<T>(ld_act(w2 + (size_t)c * w2_ld + j)), zs[j], s);
 #pragma unroll
         for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) gate[(size_t)n * mid + c] = fminf(fmaxf(s + b2[c] + 3.f, 0.f), 6.f) / 6.f;
+        if (lane == 0) gate[(size_t)n * mid + c] = fminf(fmaxf(s + ld_act(b2 + c) + 3.f, 0.f), 6.f) / 6.f;
     }
 }
 template <typename T>
@@ -275,8 +273,7 @@ template cudaError_t launch_scale<__nv_bfloat16>(const __nv_bfloat16 *, const fl
 // One warp per (n, j).
 // ---------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(256) linear_kernel(const float *v, const T *__restrict__ w,
-                                                     const float *__restrict__ bias, float *y, int N,
+__global__ void __launch_bounds__(256) linear_kernel(const float *v, const T *w, const float *bias, float *y, int N,
                                                      int C, int K, int ld, int act) {
     pdl_launch_dependents();
     pdl_wait();
@@ -284,10 +281,10 @@ __global__ void __launch_bounds__(256) linear_kernel(const float *v, const T *__
     if (warp >= N * K) return;
     int n = warp / K, j = warp % K;
     float s = 0.f;
-    for (int c = lane; c < C; c += 32) s = fmaf(to_f<T>(w[(size_t)j * ld + c]), ld_act(v + (size_t)n * C + c), s);
+    for (int c = lane; c < C; c += 32) s = fmaf(to_f<T>(ld_act(w + (size_t)j * ld + c)), ld_act(v + (size_t)n * C + c), s);
 #pragma unroll
     for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) y[(size_t)n * K + j] = apply_act(s + bias[j], act);
+    if (lane == 0) y[(size_t)n * K + j] = apply_act(s + ld_act(bias + j), act);
 }
 // ---------------------------------------------------------------------------------------------
 // Record-driven bf16 kernels (see SmallEntry): each body works on one member; the `single` kernels get
@@ -573,7 +570,8 @@ template <int KIND, int K, int ST> __global__ void __launch_bounds__(256) small_
 // of a weight row is loaded once for all of them, every piece of an input vector once for JB outputs.  What bounds it is
 // the latency of a chain of such loads (the weights of a classifier, 2 to 4 MB, lie in L2) and, with many rows, the loads of
 // the input vectors from L1: with JB = 1 a wave of 32 spent 22 - 27 us here, every warp reading 64 KB of inputs for one
-// weight row.  The first two pieces of the weight rows are requested before the wait for the previous layer.
+// weight row.  The first two pieces of stored weight rows are requested before the wait for the previous layer (a caller's
+// weights may be that layer's output).
 // Per output the arithmetic and its order do not depend on JB or on the rows that share the warp.
 constexpr int LIN_ROWS = 8;
 template <int JB, bool GROUP>
@@ -608,9 +606,10 @@ __global__ void __launch_bounds__(256) linear_rows_kernel(const SmallEntry e1, c
     auto load_w = [&](int c, uint4 *q) {
 #pragma unroll
         for (int u = 0; u < JB; u++)
-            q[u] = c < cmax ? __ldg(reinterpret_cast<const uint4 *>(w + (size_t)min(j0 + u, K - 1) * ld + c)) : make_uint4(0u, 0u, 0u, 0u);
+            q[u] = c < cmax ? ld_act(reinterpret_cast<const uint4 *>(w + (size_t)min(j0 + u, K - 1) * ld + c)) : make_uint4(0u, 0u, 0u, 0u);
     };
     uint4 wa[JB], wb[JB];
+    if (!e0.early_weights) pdl_wait();
     load_w(lane * 8, wa);
     load_w(lane * 8 + 256, wb);
     pdl_wait();
@@ -636,7 +635,7 @@ __global__ void __launch_bounds__(256) linear_rows_kernel(const SmallEntry e1, c
 #pragma unroll
     for (int u = 0; u < JB; u++) {
         if (j0 + u >= K) break;
-        const float bias = __ldg(e0.bias + j0 + u);
+        const float bias = ld_act(e0.bias + j0 + u);
 #pragma unroll
         for (int r = 0; r < LIN_ROWS; r++) {
             if (r >= nr) break;
@@ -666,20 +665,20 @@ static cudaError_t launch_linear_rows(const SmallEntry *h, const SmallEntry *d, 
 
 template <typename T>
 cudaError_t launch_linear(const float *v, const T *w, const float *bias, float *y, int N, int C, int K, int ld, int act,
-                          cudaStream_t st) {
+                          int early_weights, cudaStream_t st) {
     long long warps = (long long)N * K;
     if (warps <= 0) return cudaSuccess;
     if (sizeof(T) == 2 && C % 8 == 0 && ld % 8 == 0 && ((reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(v)) & 15) == 0 && N <= 65535) {
         SmallEntry e = {};
-        e.x = v; e.y = y; e.w = w; e.bias = bias; e.N = N; e.C = C; e.K = K; e.ld = ld; e.act = act;
+        e.x = v; e.y = y; e.w = w; e.bias = bias; e.N = N; e.C = C; e.K = K; e.ld = ld; e.act = act; e.early_weights = early_weights;
         return launch_linear_rows(&e, nullptr, 1, st);
     }
     int blocks = (int)((warps * 32 + 255) / 256);
     SGS_LAUNCH((linear_kernel<T>), dim3(blocks), dim3(256), 0, st, v, w, bias, y, N, C, K, ld, act);
     return cudaGetLastError();
 }
-template cudaError_t launch_linear<float>(const float *, const float *, const float *, float *, int, int, int, int, int, cudaStream_t);
-template cudaError_t launch_linear<__nv_bfloat16>(const float *, const __nv_bfloat16 *, const float *, float *, int, int, int, int, int, cudaStream_t);
+template cudaError_t launch_linear<float>(const float *, const float *, const float *, float *, int, int, int, int, int, int, cudaStream_t);
+template cudaError_t launch_linear<__nv_bfloat16>(const float *, const __nv_bfloat16 *, const float *, float *, int, int, int, int, int, int, cudaStream_t);
 
 bool small_supported(int kind, const SmallEntry &e) {
     auto al = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };

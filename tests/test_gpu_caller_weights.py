@@ -104,3 +104,26 @@ def test_int8_weights():
                                                    torch.cuda.current_stream().cuda_stream)
     first, second = layer(xs[0], b, w, C, 512, 1, 1, K, 1), layer(x, w, None, K, C, 1, H, H, 0)
     _check(lambda i: first(xs[i], w), lambda y: second(x, y), lambda: torch.zeros(1, H, H, K, device="cuda", dtype=torch.uint8))
+
+
+# (rows, inputs): one and many rows of the vectorised kernel, the scalar kernel
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("N,C", [(1, 512), (16, 512), (2, 508)])
+def test_linear_weights(N, C, dtype):
+    K = 1024
+    w, produce = _matrix_producer(K, 512, dtype, impl=0 if dtype == torch.bfloat16 else 1)
+    v, b = _rand(N, C, seed=5), torch.zeros(K, device="cuda")
+    d = sgs.AuxDesc(kind=sgs.binding.SGS_AUX_LINEAR, dtype=sgs.SGS_BF16 if dtype == torch.bfloat16 else sgs.SGS_F32, N=N, H=1, W=1, C=C, K=K, ld=512, act=0)
+    _check(produce, lambda y: sgs.aux_op([d], [sgs.AuxArgs(x=v.data_ptr(), y=y.data_ptr(), w=w.data_ptr(), bias=b.data_ptr())], False,
+                                         torch.cuda.current_stream().cuda_stream), lambda: torch.zeros(N, K, device="cuda"))
+
+
+def test_squeeze_excite_gate_weights():
+    mid, sq = 480, 120
+    w1, produce = _matrix_producer(sq, mid, torch.bfloat16)
+    w2, g = (_rand(mid, sq, seed=6) * 0.1).bfloat16(), _rand(3, mid, seed=7)
+    b1, b2 = torch.zeros(sq, device="cuda"), torch.zeros(mid, device="cuda")
+    d = sgs.AuxDesc(kind=sgs.binding.SGS_AUX_SE_GATE, dtype=sgs.SGS_BF16, N=3, H=1, W=1, C=mid, K=sq, ld=mid, ld2=sq)
+    _check(produce, lambda y: sgs.aux_op([d], [sgs.AuxArgs(x=g.data_ptr(), y=y.data_ptr(), w=w1.data_ptr(), bias=b1.data_ptr(), w2=w2.data_ptr(),
+                                                           bias2=b2.data_ptr())], False, torch.cuda.current_stream().cuda_stream),
+           lambda: torch.zeros(3, mid, device="cuda"))
