@@ -270,14 +270,14 @@ __global__ void __launch_bounds__(THREADS) conv_simt_kernel(const ConvArgs a) {
             if (res) rv = *reinterpret_cast<const float4 *>(res + oi);
             const float r4[4] = {rv.x, rv.y, rv.z, rv.w};
 #pragma unroll
-            for (int j = 0; j < 4; j++) out[j] = simt_act(v[j] * __ldg(a.scale + f + j) + __ldg(a.shift + f + j) + r4[j], a.act);
+            for (int j = 0; j < 4; j++) out[j] = simt_act(v[j] * ld_act(a.scale + f + j) + ld_act(a.shift + f + j) + r4[j], a.act);
             *reinterpret_cast<float4 *>(y + oi) = make_float4(out[0], out[1], out[2], out[3]);
             return;
         }
 #pragma unroll
         for (int j = 0; j < 4; j++) {
             if (f + j >= a.K) return;
-            float t = v[j] * __ldg(a.scale + f + j) + __ldg(a.shift + f + j);
+            float t = v[j] * ld_act(a.scale + f + j) + ld_act(a.shift + f + j);
             if (res) t += simt_f(res[oi + j]);
             t = simt_act(t, a.act);
             if constexpr (std::is_same<T, float>::value) y[oi + j] = t; else y[oi + j] = __float2bfloat16_rn(t);

@@ -57,7 +57,7 @@ __device__ __forceinline__ void dw_body(const ConvArgs &a, const int n, unsigned
         const int part = (threadIdx.x & 7) * 8;  // 8 channels of a tap
         for (int tap = threadIdx.x >> 3; tap < K * K; tap += DW_WARPS * 4) {
             uint4 v = make_uint4(0, 0, 0, 0);
-            if (cb * 64 + part < a.K) v = __ldg(reinterpret_cast<const uint4 *>(w + (size_t)((tap / K) * a.R + tap % K) * a.Kmax + part));
+            if (cb * 64 + part < a.K) v = ld_act(reinterpret_cast<const uint4 *>(w + (size_t)((tap / K) * a.R + tap % K) * a.Kmax + part));
             const float2 f0 = dw_unpack(v.x), f1 = dw_unpack(v.y), f2 = dw_unpack(v.z), f3 = dw_unpack(v.w);
             float4 *d = reinterpret_cast<float4 *>(wsm + tap * 64 + part);
             d[0] = make_float4(f0.x, f0.y, f1.x, f1.y);
@@ -68,7 +68,7 @@ __device__ __forceinline__ void dw_body(const ConvArgs &a, const int n, unsigned
     const int wt = (unit % strips) * TW, ho_begin = (unit / strips) * seg, ho_end = min(a.Ho, ho_begin + seg);
     if (ho_begin >= a.Ho) return;
     const int c = cb * 64 + 2 * lane, cc = min(c, a.K - 2);
-    const float2 sc = __ldg(reinterpret_cast<const float2 *>(a.scale + cc)), sh = __ldg(reinterpret_cast<const float2 *>(a.shift + cc));
+    const float2 sc = ld_act(reinterpret_cast<const float2 *>(a.scale + cc)), sh = ld_act(reinterpret_cast<const float2 *>(a.shift + cc));
     const bool hswish = a.act == ACT_HSWISH;
     const float lo = a.act == ACT_RELU ? 0.f : __int_as_float(0xff800000);  // ReLU as a maximum; no activation: -infinity
 
@@ -103,7 +103,7 @@ __device__ __forceinline__ void dw_body(const ConvArgs &a, const int n, unsigned
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    pdl_wait();  // (the weights above do not depend on the previous layer)
+    pdl_wait();  // (stored weights, read above, do not depend on the previous layer)
     copy_rows(S::WIN);
     const unsigned char *xlane = ring + lane * 4;
     const float2 *wlane = reinterpret_cast<const float2 *>(wsm) + lane;

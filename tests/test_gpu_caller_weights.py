@@ -106,6 +106,21 @@ def test_int8_weights():
     _check(lambda i: first(xs[i], w), lambda y: second(x, y), lambda: torch.zeros(1, H, H, K, device="cuda", dtype=torch.uint8))
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_cuda_core_weights(dtype):
+    K, C, H = 256, 128, 9
+    w, produce = _matrix_producer(K, C, dtype, impl=1)
+    x, one, zero = _rand(1, H, H, C, seed=5).to(dtype), torch.ones(K, device="cuda"), torch.zeros(K, device="cuda")
+    _check(produce, lambda y: _conv(x, w.view(K, 1, 1, C), one, zero, y, impl=1), lambda: torch.zeros(1, H, H, K, device="cuda", dtype=dtype))
+
+
+def test_depthwise_weights():
+    K, H = 512, 14
+    w, produce = _matrix_producer(25, K, torch.bfloat16)
+    x, one, zero = _rand(2, H, H, K, seed=5).bfloat16(), torch.ones(K, device="cuda"), torch.zeros(K, device="cuda")
+    _check(produce, lambda y: _conv(x, w.view(5, 5, K), one, zero, y, depthwise=True), lambda: torch.zeros(2, H, H, K, device="cuda", dtype=torch.bfloat16))
+
+
 # (rows, inputs): one and many rows of the vectorised kernel, the scalar kernel
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("N,C", [(1, 512), (16, 512), (2, 508)])
