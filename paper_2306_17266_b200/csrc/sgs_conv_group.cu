@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
                 }
                 const int cend = min((int)e0.bn_tile, K - f0);    // filters of this tile, a multiple of 8 (<= 0: none of this member's)
                 const int cpad = min((int)e0.bn_tile, ldk - f0);  // ... and the end of the pixel's padding, written as zeros
-                const float lo = act == ACT_RELU ? 0.f : __int_as_float(0xff800000);  // ReLU as a maximum; no activation: -infinity
+                const float lo = act == ACT_RELU ? 0.f : __int_as_float(0x7fc00000);  // ReLU as a maximum; no activation: the maximum with NaN is the other operand, a NaN stays one
                 // Folded batch norm of a block's 32 filters: a lane loads one filter's, and the warp meets in the padding of its
                 // staging rows (4 floats a row: scales in rows 0..7, shifts in 8..15).
                 float *bnp = stage + (lane >> 2) * G_EPI_PITCH + 32 + (lane & 3);

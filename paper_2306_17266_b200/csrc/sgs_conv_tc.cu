@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_con
     }
     if (splits > 1) cluster_sync_all();  // (also after a wait that ran out)
     if (ok_epi && fc < p.ldy) {
-        const float lo = p.act == ACT_RELU ? 0.f : __int_as_float(0xff800000);  // ReLU as a maximum; no activation: -infinity
+        const float lo = p.act == ACT_RELU ? 0.f : __int_as_float(0x7fc00000);  // ReLU as a maximum; no activation: the maximum with NaN is the other operand, a NaN stays one
         // One output: 8 filters of pixel m, o = accumulator (int32 bits in 8-bit layers).
         auto store_output = [&](const float *o, const uint4 rq, int m) {
             if (I8) {

@@ -70,7 +70,7 @@ __device__ __forceinline__ void dw_body(const ConvArgs &a, const int n, unsigned
     const int c = cb * 64 + 2 * lane, cc = min(c, a.K - 2);
     const float2 sc = ld_act(reinterpret_cast<const float2 *>(a.scale + cc)), sh = ld_act(reinterpret_cast<const float2 *>(a.shift + cc));
     const bool hswish = a.act == ACT_HSWISH;
-    const float lo = a.act == ACT_RELU ? 0.f : __int_as_float(0xff800000);  // ReLU as a maximum; no activation: -infinity
+    const float lo = a.act == ACT_RELU ? 0.f : __int_as_float(0x7fc00000);  // ReLU as a maximum; no activation: the maximum with NaN is the other operand, a NaN stays one
 
     const int wi0 = wt * ST - P;
     const int mine = c < a.K ? min(TW, a.Wo - wt) : 0;  // output columns this lane stores
