@@ -2647,7 +2647,7 @@ sgs_status_t sgs_conv2d_sliced(const sgs_conv_desc_t *d, const void *d_x, const 
     }
     if (d->impl == 2) return SGS_EUNSUPPORTED;
     e = d->dtype == SGS_BF16 ? launch_conv_plain<__nv_bfloat16>(a, st) : launch_conv_plain<float>(a, st);
-    return e == cudaSuccess ? SGS_OK : SGS_ECUDA;
+    return e == cudaSuccess ? SGS_OK : e == cudaErrorNotSupported ? SGS_EUNSUPPORTED : SGS_ECUDA;
 }
 
 // One sliced convolution layer with 8-bit operands on the tensor cores (see sgs.h).

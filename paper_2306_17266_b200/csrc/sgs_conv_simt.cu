@@ -334,6 +334,7 @@ cudaError_t launch_shape(const ConvArgs &a, int splits, cudaStream_t st) {
 template <typename T> cudaError_t launch_conv_plain(const ConvArgs &a, cudaStream_t st) {
     const long long M = (long long)a.N * a.Ho * a.Wo;
     if (M <= 0 || a.K <= 0) return cudaSuccess;
+    if (!conv_index_fits(a)) return cudaErrorNotSupported;
     const int iters = (a.k * a.k * a.C + BK - 1) / BK;
     const bool vec = a.C % 4 == 0 && a.Cmax % 4 == 0 &&
                      ((reinterpret_cast<uintptr_t>(a.x) | reinterpret_cast<uintptr_t>(a.w) | reinterpret_cast<uintptr_t>(a.y) | reinterpret_cast<uintptr_t>(a.res)) & 15) == 0;

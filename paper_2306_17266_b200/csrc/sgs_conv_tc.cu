@@ -606,6 +606,7 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
     if (a.i8 && ((a.ldx ? a.ldx : a.C) % 16 || a.C % 8 || a.Cmax % 16 || a.throughput || a.win || (a.ldy && (a.ldy % 16 || a.ldy < a.K || a.ldy - a.K >= 16)) || (!a.ldy && a.K % 8)))
         return no("8-bit layers: pixels in multiples of 16 bytes, single launches");
     if (a.C < 8 || a.K < 8) return no("too few channels");
+    if (!conv_index_fits(a)) return no("more pixels or reduction steps than 32 bits number");
     if (a.k % 2 == 0 || a.k > a.R) return no("kernel size");
     if (a.stride != 1 && a.stride != 2) return no("stride");
     if (a.stride == 2 && a.k > 1 && (a.H < 2 || a.W < 2)) return no("a parity view of a one-pixel side would be empty");

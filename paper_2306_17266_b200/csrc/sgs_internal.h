@@ -78,6 +78,11 @@ struct ConvArgs {
     int no_split = 0;  // 1: one block per tile (the reduction is never split over a cluster)
 };
 
+// Pixels and reduction steps of the regular convolutions are numbered with 32 bits (a tile may reach past the last of either).
+inline bool conv_index_fits(const ConvArgs &a) {
+    return (double)a.N * a.Ho * a.Wo <= 2147483647.0 - 1024.0 && (double)a.k * a.k * a.C <= 2147483647.0 - 1024.0;
+}
+
 // ---- persistent SubNet kernel (sgs_subnet_kernel.cu) ------------------------------------------
 // One launch serves a whole stream of one-image queries of the MobileNetV3-shaped family: every block (one per
 // SM) takes the next unserved query and runs ALL layers of that query's SubNet by itself, from the image to the
