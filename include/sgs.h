@@ -312,7 +312,7 @@ sgs_status_t sgs_subnet_cost(const sgs_supernet_t *net, const sgs_subnet_cfg_t *
  *   d_scale, d_shift  [>= K] fp32
  * impl 0 = automatic (tensor cores when dtype is bf16, C, K, Cmax are multiples of 8 and pointers are
  * 16-byte aligned; kernels larger than 1x1 at stride 2 need at least 2x2 pixels), 1 = CUDA-core kernel, 2 = tensor cores or
- * SGS_EUNSUPPORTED.  Without `depthwise`, N*Ho*Wo and k*k*C have to stay below 2^31 - 1024 (else SGS_EUNSUPPORTED).  weight_policy 0 = no L2 hint, 1 = evict-last for weight tiles with filter <
+ * SGS_EUNSUPPORTED.  Without `depthwise`, N*Ho*Wo and k*k*C have to stay below 2^31 - 128 (else SGS_EUNSUPPORTED).  weight_policy 0 = no L2 hint, 1 = evict-last for weight tiles with filter <
  * cache_k and channel < cache_c (default replacement for the rest), 2 = all weights evict-first.
  * Asynchronous on `cuda_stream`; everything passed in, weights and parameters included, may be what earlier work on the
  * stream writes.  The tensor-core path may split the reduction over a cluster of CTAs, whose partial sums stay in shared

@@ -78,9 +78,9 @@ struct ConvArgs {
     int no_split = 0;  // 1: one block per tile (the reduction is never split over a cluster)
 };
 
-// Pixels and reduction steps of the regular convolutions are numbered with 32 bits (a tile may reach past the last of either).
+// Pixels and reduction steps of the regular convolutions are numbered with 32 bits; a tile (of 128 at most) may reach past the last.
 inline bool conv_index_fits(const ConvArgs &a) {
-    return (double)a.N * a.Ho * a.Wo <= 2147483647.0 - 1024.0 && (double)a.k * a.k * a.C <= 2147483647.0 - 1024.0;
+    return (double)a.N * a.Ho * a.Wo <= 2147483647.0 - 128.0 && (double)a.k * a.k * a.C <= 2147483647.0 - 128.0;
 }
 
 // ---- persistent SubNet kernel (sgs_subnet_kernel.cu) ------------------------------------------

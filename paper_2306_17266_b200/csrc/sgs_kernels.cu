@@ -143,7 +143,7 @@ __device__ __forceinline__ float2 bf2f(uint32_t u) { return make_float2(__uint_a
 __global__ void __launch_bounds__(256) gap_vec_kernel(const __nv_bfloat16 *x, float *g, int N, int HW, int C) {
     pdl_launch_dependents();
     pdl_wait();
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    const int warp = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
     const int cvecs = C >> 3;
     if (warp >= N * cvecs) return;
     const int n = warp / cvecs, cv = warp % cvecs;
@@ -168,9 +168,9 @@ __global__ void __launch_bounds__(256) gap_vec_kernel(const __nv_bfloat16 *x, fl
 
 template <typename T> cudaError_t launch_gap(const T *x, float *g, int N, int HW, int C, cudaStream_t st) {
     if (N <= 0 || C <= 0) return cudaSuccess;
-    if (sizeof(T) == 2 && C % 8 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0 && (reinterpret_cast<uintptr_t>(g) & 15) == 0) {
-        const int warps = N * (C / 8);
-        SGS_LAUNCH(gap_vec_kernel, dim3((warps * 32 + 255) / 256), dim3(256), 0, st, reinterpret_cast<const __nv_bfloat16 *>(x), g, N, HW, C);
+    const long long warps = (long long)N * (C / 8);
+    if (sizeof(T) == 2 && C % 8 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0 && (reinterpret_cast<uintptr_t>(g) & 15) == 0 && warps < 0x7fffffffll - 8) {
+        SGS_LAUNCH(gap_vec_kernel, dim3((unsigned)((warps + 7) / 8)), dim3(256), 0, st, reinterpret_cast<const __nv_bfloat16 *>(x), g, N, HW, C);
         return cudaGetLastError();
     }
     dim3 grid((C + 31) / 32, N), block(32, 8);
@@ -277,9 +277,10 @@ __global__ void __launch_bounds__(256) linear_kernel(const float *v, const T *w,
                                                      int C, int K, int ld, int act) {
     pdl_launch_dependents();
     pdl_wait();
-    int warp = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x % 32;
-    if (warp >= N * K) return;
-    int n = warp / K, j = warp % K;
+    const long long warp = (long long)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+    const int lane = threadIdx.x % 32;
+    if (warp >= (long long)N * K) return;
+    const int n = (int)(warp / K), j = (int)(warp % K);
     float s = 0.f;
     for (int c = lane; c < C; c += 32) s = fmaf(to_f<T>(ld_act(w + (size_t)j * ld + c)), ld_act(v + (size_t)n * C + c), s);
 #pragma unroll
@@ -298,11 +299,11 @@ __device__ __forceinline__ uint32_t bf2_max(uint32_t a, uint32_t b) {
 // 3x3 stride-2 max pool, padding 1: a thread owns 8 channels of one output pixel.
 __device__ __forceinline__ void maxpool_body(const SmallEntry &e, int bx, int nbx) {
     const int cv = e.C >> 3;
-    const int total = e.N * e.Ho * e.Wo * cv;
+    const int total = e.N * e.Ho * e.Wo * cv, step = nbx * blockDim.x;
     const __nv_bfloat16 *x = static_cast<const __nv_bfloat16 *>(e.x);
     __nv_bfloat16 *y = static_cast<__nv_bfloat16 *>(e.y);
-    for (int i = bx * blockDim.x + threadIdx.x; i < total; i += nbx * blockDim.x) {
-        const int c = i % cv, m = i / cv;
+    for (int left = total - (int)(bx * blockDim.x + threadIdx.x); left > 0; left -= step) {  // (total may be just below 2^31)
+        const int i = total - left, c = i % cv, m = i / cv;
         const int wo = m % e.Wo, ho = (m / e.Wo) % e.Ho, n = m / (e.Wo * e.Ho);
         uint4 best = make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);  // -inf pairs
 #pragma unroll
@@ -323,7 +324,7 @@ __device__ __forceinline__ void maxpool_body(const SmallEntry &e, int bx, int nb
 
 // Global average pool: one warp per 8-channel vector of one image (fixed shuffle tree).
 __device__ __forceinline__ void gap_body(const SmallEntry &e, int bx) {
-    const int warp = (bx * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    const int warp = (int)(bx * (blockDim.x >> 5) + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
     const int cvecs = e.C >> 3, HW = e.H * e.W;
     if (warp >= e.N * cvecs) return;
     const int n = warp / cvecs, cv = warp % cvecs;
@@ -348,12 +349,12 @@ __device__ __forceinline__ void gap_body(const SmallEntry &e, int bx) {
 
 // y[n][hw][c] = x[n][hw][c] * gate[n][c] (gate = e.w, fp32): a thread scales one 8-channel vector.
 __device__ __forceinline__ void scale_body(const SmallEntry &e, int bx, int nbx) {
-    const int cvecs = e.C >> 3, per_image = e.H * e.W * cvecs, total = e.N * per_image;
+    const int cvecs = e.C >> 3, per_image = e.H * e.W * cvecs, total = e.N * per_image, step = nbx * blockDim.x;
     const __nv_bfloat16 *x = static_cast<const __nv_bfloat16 *>(e.x);
     const float *gate = static_cast<const float *>(e.w);
     __nv_bfloat16 *y = static_cast<__nv_bfloat16 *>(e.y);
-    for (int i = bx * blockDim.x + threadIdx.x; i < total; i += nbx * blockDim.x) {
-        const int n = i / per_image, cv = i % cvecs;
+    for (int left = total - (int)(bx * blockDim.x + threadIdx.x); left > 0; left -= step) {  // (as in maxpool_body)
+        const int i = total - left, n = i / per_image, cv = i % cvecs;
         const uint4 v = ld_act(reinterpret_cast<const uint4 *>(x + (size_t)i * 8));
         const float4 g0 = ld_act(reinterpret_cast<const float4 *>(gate + (size_t)n * e.C + cv * 8));
         const float4 g1 = ld_act(reinterpret_cast<const float4 *>(gate + (size_t)n * e.C + cv * 8 + 4));
@@ -528,10 +529,11 @@ __device__ __forceinline__ void im2col_body(const SmallEntry &e, int bx) {
 // 3-channel image -> [N][Ho][Wo][8] with the image at (k, k) and zeros elsewhere (margins and channels 3..7):
 // the input of the window-view stem.  A thread writes one padded pixel (16 bytes).
 __device__ __forceinline__ void pad8_body(const SmallEntry &e, int bx, int nbx) {
-    const int total = e.N * e.Ho * e.Wo;
+    const int total = e.N * e.Ho * e.Wo, step = nbx * blockDim.x;
     const unsigned short *x = static_cast<const unsigned short *>(e.x);
     uint4 *y = static_cast<uint4 *>(e.y);
-    for (int i = bx * blockDim.x + threadIdx.x; i < total; i += nbx * blockDim.x) {
+    for (int left = total - (int)(bx * blockDim.x + threadIdx.x); left > 0; left -= step) {  // (as in maxpool_body)
+        const int i = total - left;
         const int wp = i % e.Wo, hp = (i / e.Wo) % e.Ho, n = i / (e.Wo * e.Ho);
         const int h = hp - e.k, w = wp - e.k;
         uint4 v = make_uint4(0u, 0u, 0u, 0u);
@@ -597,7 +599,7 @@ __global__ void __launch_bounds__(256) linear_rows_kernel(const SmallEntry e1, c
         cr[threadIdx.x] = (int)threadIdx.x < nr ? C : 0;
     }
     __syncthreads();
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31, j0 = warp * JB;
+    const int lane = threadIdx.x & 31, j0 = (int)blockIdx.x * (8 * JB) + (int)(threadIdx.x >> 5) * JB;
     if (j0 >= K) return;
     int cmax = 0;
 #pragma unroll
@@ -651,8 +653,8 @@ static cudaError_t launch_linear_rows(const SmallEntry *h, const SmallEntry *d, 
     const long long rows = (long long)n * h[0].N;
     const unsigned gy = (unsigned)((rows + LIN_ROWS - 1) / LIN_ROWS);
     const int jb = rows <= 2 ? 1 : 4;
-    const unsigned gx = (unsigned)(((h[0].K + jb - 1) / jb * 32ll + 255) / 256);
-    if (gy > 65535) return cudaErrorInvalidValue;
+    const unsigned gx = (unsigned)((((long long)h[0].K + jb - 1) / jb + 7) / 8);
+    if (gy > 65535 || h[0].K > 0x7fffffff - 64) return cudaErrorInvalidValue;  // (a block's last warps may lie past K)
     if (d) {
         if (jb == 1) SGS_LAUNCH((linear_rows_kernel<1, true>), dim3(gx, gy), dim3(256), 0, st, h[0], d, n);
         else SGS_LAUNCH((linear_rows_kernel<4, true>), dim3(gx, gy), dim3(256), 0, st, h[0], d, n);
@@ -673,8 +675,9 @@ cudaError_t launch_linear(const float *v, const T *w, const float *bias, float *
         e.x = v; e.y = y; e.w = w; e.bias = bias; e.N = N; e.C = C; e.K = K; e.ld = ld; e.act = act; e.early_weights = early_weights;
         return launch_linear_rows(&e, nullptr, 1, st);
     }
-    int blocks = (int)((warps * 32 + 255) / 256);
-    SGS_LAUNCH((linear_kernel<T>), dim3(blocks), dim3(256), 0, st, v, w, bias, y, N, C, K, ld, act);
+    const long long blocks = (warps + 7) / 8;
+    if (blocks > 0x7fffffffll) return cudaErrorInvalidValue;
+    SGS_LAUNCH((linear_kernel<T>), dim3((unsigned)blocks), dim3(256), 0, st, v, w, bias, y, N, C, K, ld, act);
     return cudaGetLastError();
 }
 template cudaError_t launch_linear<float>(const float *, const float *, const float *, float *, int, int, int, int, int, int, cudaStream_t);
@@ -685,7 +688,7 @@ bool small_supported(int kind, const SmallEntry &e) {
     if (!al(e.x) || !al(e.y)) return false;
     switch (kind) {
     case OP_MAXPOOL: return e.C % 8 == 0 && (long long)e.N * e.Ho * e.Wo * (e.C / 8) < (1ll << 31);
-    case OP_GAP: return e.C % 8 == 0;
+    case OP_GAP: return e.C % 8 == 0 && (long long)e.N * (e.C / 8) < 0x7fffffffll - 8;
     case OP_SCALE: return e.C % 8 == 0 && al(e.w) && (long long)e.N * e.H * e.W * (e.C / 8) < (1ll << 31);
     case OP_SE_GATE: return e.w2 != nullptr;
     case OP_SE: return e.w2 != nullptr && al(e.w) && al(e.w2) && se_supported(e.N, e.H * e.W, e.C, e.K, e.ld, e.ld2, 1);
@@ -701,7 +704,7 @@ bool small_supported(int kind, const SmallEntry &e) {
 static long long small_blocks(int kind, const SmallEntry &e) {
     switch (kind) {
     case OP_MAXPOOL: return ((long long)e.N * e.Ho * e.Wo * (e.C / 8) + 255) / 256;
-    case OP_GAP: return ((long long)e.N * (e.C / 8) * 32 + 255) / 256;
+    case OP_GAP: return ((long long)e.N * (e.C / 8) + 7) / 8;
     case OP_SCALE: return ((long long)e.N * e.H * e.W * (e.C / 8) + 255) / 256;
     case OP_PAD8: return ((long long)e.N * e.Ho * e.Wo + 255) / 256;
     default: return (long long)e.N * e.Ho;  // patch matrix: one block per output row
