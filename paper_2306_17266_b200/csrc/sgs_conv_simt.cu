@@ -312,14 +312,9 @@ cudaError_t launch_shape(const ConvArgs &a, int splits, cudaStream_t st) {
     using S = SimtShape<T, TM, TN, VEC>;
     auto kernel = conv_simt_kernel<T, TM, TN, VEC>;
     if (S::SMEM > 48 * 1024) {
-        static bool set[64] = {};  // (per device; setting it twice is harmless)
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
+        static DeviceBits done;
+        const cudaError_t e = smem_limit_once(kernel, S::SMEM, done);
         if (e != cudaSuccess) return e;
-        if (dev < 0 || dev >= 64 || !set[dev]) {
-            if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM)) != cudaSuccess) return e;
-            if (dev >= 0 && dev < 64) set[dev] = true;
-        }
     }
     const int M = a.N * a.Ho * a.Wo;
     const dim3 grid((unsigned)((M + S::BM - 1) / S::BM), (unsigned)((a.K + S::BN - 1) / S::BN), (unsigned)splits);
@@ -330,7 +325,7 @@ cudaError_t launch_shape(const ConvArgs &a, int splits, cudaStream_t st) {
 
 // Tile and split: the one with the shortest estimated time.  A step of a tile costs its multiply-adds at 128 a clock
 // (packed operands leave about a quarter of that to loads and addresses) but never less than the latency of one step of
-// the pipeline; a launch has as many rounds as its blocks need on 148 SMs.
+// the pipeline; a launch has as many rounds as its blocks need on the device's SMs.
 template <typename T> cudaError_t launch_conv_plain(const ConvArgs &a, cudaStream_t st) {
     const long long M = (long long)a.N * a.Ho * a.Wo;
     if (M <= 0 || a.K <= 0) return cudaSuccess;
@@ -338,6 +333,7 @@ template <typename T> cudaError_t launch_conv_plain(const ConvArgs &a, cudaStrea
     const int iters = (a.k * a.k * a.C + BK - 1) / BK;
     const bool vec = a.C % 4 == 0 && a.Cmax % 4 == 0 &&
                      ((reinterpret_cast<uintptr_t>(a.x) | reinterpret_cast<uintptr_t>(a.w) | reinterpret_cast<uintptr_t>(a.y) | reinterpret_cast<uintptr_t>(a.res)) & 15) == 0;
+    const long long sms = sm_count();
     static const int shapes[4][2] = {{8, 8}, {4, 8}, {4, 4}, {4, 2}};
     int best = 1, best_s = 1;
     double best_t = 1e30;
@@ -347,7 +343,7 @@ template <typename T> cudaError_t launch_conv_plain(const ConvArgs &a, cudaStrea
         if ((M + bm - 1) / bm > 0x7fffffffll || (a.K + bn - 1) / bn > 65535) continue;
         for (int s = 1; s <= 8 && s <= iters; s *= 2) {
             const double step = std::max(bm * bn * BK / 128.0 * 1.3, 350.0);
-            const double rounds = (double)((tiles * s + 147) / 148);
+            const double rounds = (double)((tiles * s + sms - 1) / sms);
             const double t = rounds * ((double)((iters + s - 1) / s) * step + 1500.0 + 12.0 * (bm * bn / 64)) + (s > 1 ? 1500.0 : 0.0);
             if (t < best_t) { best_t = t; best = i; best_s = s; }
         }

@@ -491,7 +491,6 @@ bool encode_map(CUtensorMap *m, const void *base, int rank, const uint64_t *dims
 
 struct DeviceScratch {
     int *status = nullptr;
-    int sms = 0;
     bool attrs_set = false;
 };
 DeviceScratch g_dev[64];
@@ -692,13 +691,7 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
     const int mtiles = p.tiles_w * p.tiles_h * tiles_n;
 
     // filter tile: 128 wide unless the layer is narrow or too few CTAs would stream the weights
-    int sms = 148;
-    {
-        std::lock_guard<std::mutex> lk(g_mu);
-        DeviceScratch &ds = g_dev[device];
-        if (!ds.sms) cudaDeviceGetAttribute(&ds.sms, cudaDevAttrMultiProcessorCount, device);
-        if (ds.sms > 0) sms = ds.sms;
-    }
+    const int sms = sm_count();
     p.cchunks = (a.C + (int)CH - 1) / (int)CH;
     p.iters = a.k * plan->kw * p.cchunks;
     // Filter tile: 128 wide where the tiles then still occupy every SM (half the pixel copies per filter), else 64.
@@ -888,9 +881,7 @@ extern "C" sgs_status_t sgs_conv2d_sliced_static(const sgs_conv_desc_t *d, const
     std::shared_ptr<TcConvPlan> plan = tc_conv_prepare(a, dev, nullptr);  // host memory only
     if (!plan) return SGS_EUNSUPPORTED;
     TcParams prm = plan->prm;
-    int sms = 148;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (!d->split_k_off && contract_scratch_bytes(prm, (long long)a.N * a.Ho * a.Wo, (int)plan->grid.x, sms) > SGS_STATIC_SCRATCH_BYTES) return SGS_ENOMEM;
+    if (!d->split_k_off && contract_scratch_bytes(prm, (long long)a.N * a.Ho * a.Wo, (int)plan->grid.x, sm_count()) > SGS_STATIC_SCRATCH_BYTES) return SGS_ENOMEM;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     prm.scale = a.scale; prm.shift = a.shift;
     prm.res = static_cast<const __nv_bfloat16 *>(a.res);

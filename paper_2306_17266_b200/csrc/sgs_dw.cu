@@ -209,14 +209,17 @@ cudaError_t launch_shape(const ConvArgs &a, int kmin, int kmax, int ch, const ch
     // fills the device a few times (a ragged last round is short then); what a segment costs is its weights and k - 1 rows
     // that its neighbour reads too.
     const long long warps = columns * a.N * members;
-    const int nseg = (int)std::max(1ll, std::min<long long>((148 * 64 + warps - 1) / warps, (a.Ho + 1) / 2));
+    const int nseg = (int)std::max(1ll, std::min<long long>((sm_count() * 64ll + warps - 1) / warps, (a.Ho + 1) / 2));
     const int seg = ((a.Ho + nseg - 1) / nseg + 1) & ~1;
     int smem = 0;
     for (int k = kmin; k <= kmax; k += 2) smem = std::max(smem, block_bytes<ST, WIDE>(k));
     const int most = std::max({block_bytes<ST, WIDE>(3), block_bytes<ST, WIDE>(5), block_bytes<ST, WIDE>(7)});
-    const DwKernel kern = kmin != kmax ? dw_mixed_kernel<ST, WIDE> : kmin == 3 ? dw_kernel<3, ST, WIDE> : kmin == 5 ? dw_kernel<5, ST, WIDE> : dw_kernel<7, ST, WIDE>;
+    static const DwKernel kernels[4] = {dw_mixed_kernel<ST, WIDE>, dw_kernel<3, ST, WIDE>, dw_kernel<5, ST, WIDE>, dw_kernel<7, ST, WIDE>};
+    static DeviceBits done[4];
+    const int which = kmin != kmax ? 0 : (kmin - 1) / 2;
+    const DwKernel kern = kernels[which];
     if (smem + (int)sizeof(ConvArgs) > 47 * 1024) {  // (the static record counts too)
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most);  // (one value for all callers: threads may meet here)
+        const cudaError_t e = smem_limit_once(kern, most, done[which]);
         if (e != cudaSuccess) return e;
     }
     const long long units = (long long)((a.Wo + tw - 1) / tw) * ((a.Ho + seg - 1) / seg);

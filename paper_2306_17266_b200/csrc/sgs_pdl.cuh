@@ -1,9 +1,10 @@
-// Programmatic dependent launch: device-side controls and the host-side launch helper.
+// Programmatic dependent launch: device-side controls and the host-side launch helpers.
 #pragma once
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <utility>
 
 namespace sgs {
@@ -75,6 +76,31 @@ cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
         cfg.numAttrs = 2;
     }
     return cudaLaunchKernelEx(&cfg, kernel, P(std::forward<A>(args))...);
+}
+
+// Raises the dynamic shared-memory limit of `kernel` on the current device, the first time it is asked to.  `done`: one per
+// kernel, a bit per device; host threads that meet here set the same value twice.
+typedef std::atomic<unsigned long long> DeviceBits;
+template <typename Kernel> cudaError_t smem_limit_once(Kernel kernel, int bytes, DeviceBits &done) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = dev >= 0 && dev < 64 ? 1ull << dev : 0ull;
+    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+    return e;
+}
+
+// SMs of the current device (148, a B200's, where it cannot be asked).
+inline int sm_count() {
+    static std::atomic<int> known[64];
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
+    if ((n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 148;
+    known[dev].store(n, std::memory_order_relaxed);
+    return n;
 }
 
 }  // namespace sgs

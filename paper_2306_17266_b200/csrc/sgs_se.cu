@@ -197,14 +197,6 @@ size_t se_smem_bytes(int HW, int C, int sq, size_t elem) {
 }
 constexpr size_t SE_SMEM_MAX = 160 * 1024;  // (a pixel share of about 130 KB: maps of up to 1 MB; larger ones take separate launches)
 
-template <typename K> cudaError_t se_limit(K kernel, bool *set) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess || (dev >= 0 && dev < 64 && set[dev])) return e;
-    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SE_SMEM_MAX)) == cudaSuccess && dev >= 0 && dev < 64) set[dev] = true;
-    return e;
-}
-
 }  // namespace
 
 bool se_supported(int N, int HW, int C, int sq, int ld, int ld2, int bf16) {
@@ -221,19 +213,19 @@ cudaError_t launch_se(const SmallEntry *h, const SmallEntry *d, int n, int bf16,
         nimg = std::max(nimg, h[i].N);
     }
     const dim3 grid((unsigned)(nimg * SE_BLOCKS), (unsigned)n);
-    static bool set[3][64] = {};
+    static DeviceBits done[3];
     cudaError_t e;
     if (d) {
         if (!bf16) return cudaErrorInvalidValue;
-        if ((e = se_limit(se_members_kernel, set[0])) != cudaSuccess) return e;
+        if ((e = smem_limit_once(se_members_kernel, (int)SE_SMEM_MAX, done[0])) != cudaSuccess) return e;
         return launch_pdl(se_members_kernel, grid, dim3(SE_THREADS), smem, st, 1u, d);
     }
     if (n != 1) return cudaErrorInvalidValue;
     if (bf16) {
-        if ((e = se_limit(se_single_kernel<__nv_bfloat16>, set[1])) != cudaSuccess) return e;
+        if ((e = smem_limit_once(se_single_kernel<__nv_bfloat16>, (int)SE_SMEM_MAX, done[1])) != cudaSuccess) return e;
         return launch_pdl(se_single_kernel<__nv_bfloat16>, grid, dim3(SE_THREADS), smem, st, 1u, *h);
     }
-    if ((e = se_limit(se_single_kernel<float>, set[2])) != cudaSuccess) return e;
+    if ((e = smem_limit_once(se_single_kernel<float>, (int)SE_SMEM_MAX, done[2])) != cudaSuccess) return e;
     return launch_pdl(se_single_kernel<float>, grid, dim3(SE_THREADS), smem, st, 1u, *h);
 }
 
