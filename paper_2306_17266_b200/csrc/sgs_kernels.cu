@@ -577,7 +577,7 @@ template <int KIND, int K, int ST> __global__ void __launch_bounds__(256) small_
 // Per output the arithmetic and its order do not depend on JB or on the rows that share the warp.
 constexpr int LIN_ROWS = 8;
 template <int JB, bool GROUP>
-__global__ void __launch_bounds__(256) linear_rows_kernel(const SmallEntry e1, const SmallEntry *__restrict__ tbl, int n_members) {
+__global__ void __launch_bounds__(256) linear_rows_kernel(const SmallEntry e1, const SmallEntry *__restrict__ tbl, int n_members, int row_begin) {
     __shared__ SmallEntry first;
     __shared__ const float *xr[LIN_ROWS];
     __shared__ float *yr[LIN_ROWS];
@@ -589,7 +589,7 @@ __global__ void __launch_bounds__(256) linear_rows_kernel(const SmallEntry e1, c
     }
     const SmallEntry &e0 = GROUP ? first : e1;
     const int N = e0.N, K = e0.K, ld = e0.ld;
-    const int r0 = blockIdx.y * LIN_ROWS, nr = min(LIN_ROWS, (GROUP ? n_members : 1) * N - r0);
+    const int r0 = row_begin + (int)blockIdx.y * LIN_ROWS, nr = min(LIN_ROWS, (GROUP ? n_members : 1) * N - r0);
     if ((int)threadIdx.x < LIN_ROWS) {
         const int r = min(r0 + (int)threadIdx.x, r0 + nr - 1), m = r / N, n = r % N;
         const SmallEntry *e = GROUP ? tbl + m : nullptr;
@@ -599,7 +599,7 @@ __global__ void __launch_bounds__(256) linear_rows_kernel(const SmallEntry e1, c
         cr[threadIdx.x] = (int)threadIdx.x < nr ? C : 0;
     }
     __syncthreads();
-    const int lane = threadIdx.x & 31, j0 = (int)blockIdx.x * (8 * JB) + (int)(threadIdx.x >> 5) * JB;
+    const int lane = threadIdx.x & 31, j0 = (int)blockIdx.x * (8 * JB) + (int)(threadIdx.x >> 5) * JB;  // (8 warps a block)
     if (j0 >= K) return;
     int cmax = 0;
 #pragma unroll
@@ -651,16 +651,19 @@ __global__ void __launch_bounds__(256) linear_rows_kernel(const SmallEntry e1, c
 // rows = images over all members.  One or two rows: a warp per output (a classifier then fills the GPU); more: 4 outputs.
 static cudaError_t launch_linear_rows(const SmallEntry *h, const SmallEntry *d, int n, cudaStream_t st) {
     const long long rows = (long long)n * h[0].N;
-    const unsigned gy = (unsigned)((rows + LIN_ROWS - 1) / LIN_ROWS);
     const int jb = rows <= 2 ? 1 : 4;
     const unsigned gx = (unsigned)((((long long)h[0].K + jb - 1) / jb + 7) / 8);
-    if (gy > 65535 || h[0].K > 0x7fffffff - 64) return cudaErrorInvalidValue;  // (a block's last warps may lie past K)
-    if (d) {
-        if (jb == 1) SGS_LAUNCH((linear_rows_kernel<1, true>), dim3(gx, gy), dim3(256), 0, st, h[0], d, n);
-        else SGS_LAUNCH((linear_rows_kernel<4, true>), dim3(gx, gy), dim3(256), 0, st, h[0], d, n);
-    } else {
-        if (jb == 1) SGS_LAUNCH((linear_rows_kernel<1, false>), dim3(gx, gy), dim3(256), 0, st, h[0], d, n);
-        else SGS_LAUNCH((linear_rows_kernel<4, false>), dim3(gx, gy), dim3(256), 0, st, h[0], d, n);
+    if (h[0].K > 0x7fffffff - 64 || rows > 0x7fffffff - 64) return cudaErrorInvalidValue;  // (a block's last warps and rows may lie past the end)
+    constexpr int PART = 65535 * LIN_ROWS;  // rows that one grid numbers
+    for (int r0 = 0; r0 < rows; r0 += std::min<long long>(PART, rows - r0)) {
+        const dim3 grid(gx, (unsigned)((std::min<long long>(PART, rows - r0) + LIN_ROWS - 1) / LIN_ROWS));
+        if (d) {
+            if (jb == 1) SGS_LAUNCH((linear_rows_kernel<1, true>), grid, dim3(256), 0, st, h[0], d, n, r0);
+            else SGS_LAUNCH((linear_rows_kernel<4, true>), grid, dim3(256), 0, st, h[0], d, n, r0);
+        } else {
+            if (jb == 1) SGS_LAUNCH((linear_rows_kernel<1, false>), grid, dim3(256), 0, st, h[0], d, n, r0);
+            else SGS_LAUNCH((linear_rows_kernel<4, false>), grid, dim3(256), 0, st, h[0], d, n, r0);
+        }
     }
     return cudaGetLastError();
 }

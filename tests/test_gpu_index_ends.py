@@ -54,3 +54,18 @@ def test_average_pool_of_two_to_the_26_vectors(grouped):
     _run(sgs.AuxDesc(kind=SGS_AUX_AVGPOOL, dtype=sgs.SGS_BF16, N=N, H=2, W=1, C=C), sgs.AuxArgs(x=x.data_ptr(), y=y.data_ptr()), grouped)
     want = x[:, :, 0, 0].float().mean(1)
     assert torch.equal(y, want[:, None].expand(N, C))
+
+
+def test_linear_of_more_rows_than_one_grid_numbers():
+    # two members of 300 000 images each: 75 000 groups of rows
+    N, C, K = 300_000, 8, 10
+    w, bias = torch.randn(K, C, device="cuda").bfloat16(), torch.randn(K, device="cuda")
+    xs = [torch.randn(N, C, device="cuda") for _ in range(2)]
+    ys = [torch.full((N, K), 77.0, device="cuda") for _ in range(2)]
+    d = sgs.AuxDesc(kind=SGS_AUX_LINEAR, dtype=sgs.SGS_BF16, N=N, H=1, W=1, C=C, K=K, ld=C)
+    sgs.aux_op([d, d], [sgs.AuxArgs(x=x.data_ptr(), y=y.data_ptr(), w=w.data_ptr(), bias=bias.data_ptr()) for x, y in zip(xs, ys)], True,
+               torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    for x, y in zip(xs, ys):
+        ref = x.double() @ w.double().T + bias.double()
+        assert (y.double() - ref).abs().max() <= 1e-6 * ref.abs().max()  # (fp32 sums of 8 terms)
