@@ -392,6 +392,7 @@ struct Builder {
     int N;
     size_t max_elems = 0;
     bool padded = false;  // activation tensors keep pixels at a multiple of 16 channels (see ConvArgs::ldx)
+    bool split_se = false;  // squeeze-excite blocks as three ops whatever their size
 
     void note(size_t elems) { max_elems = std::max(max_elems, elems); }
     int phys(int channels) const { return padded ? (channels + 15) / 16 * 16 : channels; }
@@ -493,7 +494,7 @@ struct Builder {
         g.alg_bytes = 2.0 * mid * g.K * net->elem();
         plan->flops += g.flops;
         plan->weight_bytes += g.alg_bytes;
-        if (se_supported(N, h * w, mid, g.K, net->layers[g.layer].C, net->layers[g.layer2].C, net->dtype == SGS_BF16)) {
+        if (!split_se && se_supported(N, h * w, mid, g.K, net->layers[g.layer].C, net->layers[g.layer2].C, net->dtype == SGS_BF16)) {
             g.type = OP_SE; g.in = g.out = buf; g.H = h; g.W = w;
             g.alg_bytes += 2.0 * N * h * w * mid * net->elem();
             plan->ops.push_back(g);
@@ -515,11 +516,12 @@ struct Builder {
     }
 };
 
-sgs_status_t build_plan(sgs_supernet *net, const sgs_subnet_cfg_t *cfg, int batch, int res, Plan *plan) {
+sgs_status_t build_plan(sgs_supernet *net, const sgs_subnet_cfg_t *cfg, int batch, int res, Plan *plan, bool split_se = false) {
     const FamilyDef &d = net->def;
     plan->batch = batch; plan->res = res;
     plan->slices = slices_for(net, cfg);
     Builder B{net, plan, batch};
+    B.split_se = split_se;
     // ResNet-shaped family on bf16 handles: every convolution runs on the tensor cores (all channel counts are multiples of
     // 8, every stride-2 layer sees at least 2x2 pixels, and single queries have the patch-matrix stem), so the activation
     // tensors can be padded to 16-channel pixels: the copy unit moves rows that start or end inside a 32-byte sector at a
@@ -706,7 +708,8 @@ long long op_key(const Plan &p, size_t oi) {
 }
 
 // The largest SubNet runs every op any SubNet runs, in the same relative order (depth keeps the first
-// blocks of a stage), so the position of an op in its op list orders the ops of all SubNets.
+// blocks of a stage), so the position of an op in its op list orders the ops of all SubNets.  A squeeze-excite block has two
+// forms, chosen by its size (the members of one wave may differ in it): three ops, then the one op that stands for them.
 sgs_status_t ensure_ranks(sgs_supernet *net) {
     if (!net->op_rank.empty()) return SGS_OK;
     sgs_subnet_cfg_t c;
@@ -718,16 +721,22 @@ sgs_status_t ensure_ranks(sgs_supernet *net) {
         for (int b = 0; b < SGS_MAX_BLOCKS; b++) { c.expand[s][b] = net->family == SGS_MBV3 ? 6.0f : 0.35f; c.kernel[s][b] = 7; }
     }
     c.width[0] = 1.0f;
-    // (the stem has two forms, patch matrix + GEMM and padded copy + window view: both are ranked)
+    // (the stem has two forms too, patch matrix + GEMM and padded copy + window view, never in one wave: the same ranks)
     const int mode = net->throughput_mode;
+    std::unordered_map<long long, int> rank;
     for (int m : {0, 2}) {
         net->throughput_mode = m;
         Plan p;
-        sgs_status_t st = build_plan(net, &c, 1, 64, &p);
-        if (st != SGS_OK) { net->throughput_mode = mode; return st; }
-        for (size_t i = 0; i < p.ops.size(); i++) net->op_rank.emplace(op_key(p, i), (int)i);
+        sgs_status_t st = build_plan(net, &c, 1, 64, &p, true);
+        net->throughput_mode = mode;
+        if (st != SGS_OK) return st;
+        int next = 0;
+        for (size_t i = 0; i < p.ops.size(); i++) {
+            rank.emplace(op_key(p, i), next++);
+            if (p.ops[i].type == OP_SCALE) rank.emplace(((long long)OP_SE << 32) | (unsigned)p.ops[i - 1].layer, next++);  // (behind its gate)
+        }
     }
-    net->throughput_mode = mode;
+    net->op_rank.swap(rank);
     return SGS_OK;
 }
 
