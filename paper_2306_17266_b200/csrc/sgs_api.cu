@@ -2551,6 +2551,7 @@ sgs_status_t sgs_set_option(sgs_supernet_t *net, const char *name, long long val
         fold_profile(net);
         for (auto &kv : net->plans) destroy_plan_resources(kv.second.get());
         net->plans.clear();
+        net->op_rank.clear();  // (the stem's form depends on these options)
         return SGS_OK;
     }
     if (n == "profile") {

@@ -39,3 +39,15 @@ def test_streams(res):
                         sgs.StreamOpts(cache_enabled=1, window_q=4, wave=wave, concurrency=2 if wave else 1, persistent=persistent), st.cuda_stream)
         runs[wave, persistent] = y.cpu().numpy()
     assert np.isfinite(runs[0, 0]).all() and gu.rel_err(runs[4, 0], runs[0, 0]) <= 2e-2 and gu.rel_err(runs[0, 1], runs[0, 0]) <= 2e-2
+
+
+def test_plans_made_under_another_convolution_option():
+    # the order of a wave's layers is worked out once: also when the first plans of a handle were made without tensor cores
+    net = sgs.SuperNet(wl.RESNET, wl.make_blob(wl.RESNET, seed=0, bf16_weights=True), sgs.SGS_BF16)
+    cfg, x = wl.extreme_cfg(wl.RESNET, False), wl.make_inputs(1, 1, 64, seed=1, bf16=True)[0]
+    net.set_option("conv_impl", 1)
+    plain = gu.gpu_forward(net, cfg, x, True)
+    net.set_option("conv_impl", 0)
+    tc = gu.gpu_forward(net, cfg, x, True)
+    net.close()
+    assert gu.rel_err(tc, plain) <= 2e-2
