@@ -135,6 +135,21 @@ struct DeviceGuard {
     ~DeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
 };
 
+// CUDA events of one call, destroyed on every way out of it.
+struct EventList {
+    std::vector<cudaEvent_t> all;
+    ~EventList() {
+        for (cudaEvent_t e : all) cudaEventDestroy(e);
+    }
+    cudaError_t make(cudaEvent_t *e) {
+        all.push_back(nullptr);
+        const cudaError_t r = cudaEventCreate(&all.back());
+        if (r != cudaSuccess) all.pop_back();
+        else *e = all.back();
+        return r;
+    }
+};
+
 struct CacheState {
     bool enabled = false;
     int window_q = 4;
@@ -245,6 +260,17 @@ struct sgs_supernet {
 };
 
 namespace {
+
+// What a stream call leaves behind on every way out, errors and exceptions included: no work in flight (the next call writes
+// the same pinned tables and staging buffers), and the tile choice of single queries.
+struct StreamScope {
+    sgs_supernet *net;
+    bool in_flight = false;
+    ~StreamScope() {
+        if (in_flight) cudaDeviceSynchronize();
+        net->throughput_mode = 0;
+    }
+};
 
 sgs_status_t fail(const sgs_supernet *n, sgs_status_t st, const std::string &msg) {
     if (n) n->err = msg;
@@ -606,6 +632,7 @@ void release_slot_buffers(sgs_supernet *net, sgs_supernet::Slot &sl, bool act, b
 }
 
 sgs_status_t ensure_slots(sgs_supernet *net, int n_slots) {
+    net->slots.reserve((size_t)std::max(n_slots, 0));
     while ((int)net->slots.size() < n_slots) {
         sgs_supernet::Slot sl;
         if (!net->slots.empty()) {
@@ -722,13 +749,16 @@ sgs_status_t ensure_ranks(sgs_supernet *net) {
     }
     c.width[0] = 1.0f;
     // (the stem has two forms too, patch matrix + GEMM and padded copy + window view, never in one wave: the same ranks)
-    const int mode = net->throughput_mode;
+    struct RestoreMode {
+        sgs_supernet *net;
+        int mode;
+        ~RestoreMode() { net->throughput_mode = mode; }
+    } restore{net, net->throughput_mode};
     std::unordered_map<long long, int> rank;
     for (int m : {0, 2}) {
         net->throughput_mode = m;
         Plan p;
         sgs_status_t st = build_plan(net, &c, 1, 64, &p, true);
-        net->throughput_mode = mode;
         if (st != SGS_OK) return st;
         int next = 0;
         for (size_t i = 0; i < p.ops.size(); i++) {
@@ -992,7 +1022,13 @@ sgs_status_t run_query(sgs_supernet *net, const sgs_subnet_cfg_t *cfg, const voi
         cudaGraph_t g = nullptr;
         CU(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
         long long before = net->kernel_launches;
-        rc = run_plan(net, plan, d_input, d_logits, st, 1, n_ops - 1);
+        try {
+            rc = run_plan(net, plan, d_input, d_logits, st, 1, n_ops - 1);
+        } catch (...) {
+            cudaStreamEndCapture(st, &g);
+            if (g) cudaGraphDestroy(g);
+            throw;
+        }
         plan->launches = (int)(net->kernel_launches - before) + 2;
         net->kernel_launches = before;
         cudaError_t e = cudaStreamEndCapture(st, &g);
@@ -1168,7 +1204,7 @@ void cache_reset(sgs_supernet *net, bool enabled, size_t budget, int window_q) {
 extern "C" {
 
 sgs_status_t sgs_supernet_load(const sgs_arch_desc_t *arch, const void *host_blob, size_t nbytes,
-                               sgs_dtype_t compute_dtype, int device, sgs_supernet_t **out) {
+                               sgs_dtype_t compute_dtype, int device, sgs_supernet_t **out) try {
     if (!arch || !host_blob || !out || nbytes < 32 || nbytes % 4) return SGS_EINVAL;
     if (compute_dtype != SGS_F32 && compute_dtype != SGS_BF16) return SGS_EINVAL;
     if (arch->family < SGS_TINY || arch->family > SGS_MBV3) return SGS_EINVAL;
@@ -1181,8 +1217,9 @@ sgs_status_t sgs_supernet_load(const sgs_arch_desc_t *arch, const void *host_blo
     const uint32_t *words = static_cast<const uint32_t *>(host_blob);
     if (words[0] != BLOB_MAGIC || words[1] != 1u || (int)words[2] != arch->family) return SGS_EINVAL;
 
-    std::unique_ptr<sgs_supernet> holder(new (std::nothrow) sgs_supernet);
+    std::unique_ptr<sgs_supernet, void (*)(sgs_supernet *)> holder(new (std::nothrow) sgs_supernet, sgs_supernet_free);
     if (!holder) return SGS_ENOMEM;
+    holder->device = device;
     sgs_supernet *net = holder.get();
     net->family = arch->family; net->device = device; net->dtype = compute_dtype;
     net->def = family_def(arch->family);
@@ -1225,12 +1262,18 @@ sgs_status_t sgs_supernet_load(const sgs_arch_desc_t *arch, const void *host_blo
     if (pos != total_words) return SGS_EINVAL;
 
     sgs_status_t st;
-    float *stage = nullptr;
-    if ((st = dev_alloc(net, (void **)&stage, nbytes)) != SGS_OK) return st;
-    auto cleanup_stage = [&]() { dev_free(net, stage, nbytes); };
-    if ((st = dev_alloc(net, (void **)&net->weight_arena, arena)) != SGS_OK) { cleanup_stage(); sgs_supernet_free(holder.release()); return st; }
+    struct Stage {
+        sgs_supernet *net;
+        size_t bytes;
+        float *p = nullptr;
+        void release() { dev_free(net, p, bytes); p = nullptr; }
+        ~Stage() { release(); }
+    } stage_mem{net, nbytes};
+    if ((st = dev_alloc(net, (void **)&stage_mem.p, nbytes)) != SGS_OK) return st;
+    float *const stage = stage_mem.p;
+    if ((st = dev_alloc(net, (void **)&net->weight_arena, arena)) != SGS_OK) return st;
     net->weight_arena_bytes = arena;
-    if ((st = dev_alloc(net, (void **)&net->param_arena, params * 4)) != SGS_OK) { cleanup_stage(); sgs_supernet_free(holder.release()); return st; }
+    if ((st = dev_alloc(net, (void **)&net->param_arena, params * 4)) != SGS_OK) return st;
     net->param_arena_bytes = params * 4;
     cudaError_t e = cudaMemcpy(stage, host_blob, nbytes, cudaMemcpyHostToDevice);
     size_t aoff = 0, poff = 0;
@@ -1271,8 +1314,8 @@ sgs_status_t sgs_supernet_load(const sgs_arch_desc_t *arch, const void *host_blo
         }
     }
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    cleanup_stage();
-    if (e != cudaSuccess) { sgs_supernet_free(holder.release()); return e == cudaErrorMemoryAllocation ? SGS_ENOMEM : SGS_ECUDA; }
+    stage_mem.release();
+    if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? SGS_ENOMEM : SGS_ECUDA;
 
     int v = 0;
     if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, device) == cudaSuccess && v > 0) net->sms = v;
@@ -1285,19 +1328,13 @@ sgs_status_t sgs_supernet_load(const sgs_arch_desc_t *arch, const void *host_blo
                   cudaMemset(net->cache_tbl, 0, n * sizeof(int)) == cudaSuccess &&
                   cudaMallocHost((void **)&net->tbl_ring, 16 * n * sizeof(int)) == cudaSuccess;
         for (int i = 0; i < 16 && ok; i++) ok = cudaEventCreateWithFlags(&net->tbl_ring_ev[i], cudaEventDisableTiming) == cudaSuccess;
-        if (!ok) {
-            sgs_supernet_free(holder.release());
-            return SGS_ENOMEM;
-        }
+        if (!ok) return SGS_ENOMEM;
     }
-    if (compute_dtype == SGS_BF16 && tc_available() && tc_conv_init(device) != cudaSuccess) {
-        sgs_supernet_free(holder.release());
-        return SGS_ECUDA;
-    }
+    if (compute_dtype == SGS_BF16 && tc_available() && tc_conv_init(device) != cudaSuccess) return SGS_ECUDA;
     cache_reset(net, false, 0, 4);
     *out = holder.release();
     return SGS_OK;
-}
+} SGS_NO_THROW
 
 void sgs_supernet_free(sgs_supernet_t *net) {
     if (!net) return;
@@ -1339,23 +1376,23 @@ void sgs_supernet_free(sgs_supernet_t *net) {
     delete net;
 }
 
-sgs_status_t sgs_subnet_validate(const sgs_supernet_t *net, const sgs_subnet_cfg_t *cfg) {
+sgs_status_t sgs_subnet_validate(const sgs_supernet_t *net, const sgs_subnet_cfg_t *cfg) try {
     if (!net || !cfg) return SGS_EINVAL;
     return cfg_valid(net, cfg) ? SGS_OK : fail(net, SGS_ECONFIG, "SubNet config outside the elastic sets of this SuperNet");
-}
+} SGS_NO_THROW
 
 int sgs_num_layers(const sgs_supernet_t *net) { return net ? (int)net->layers.size() : 0; }
 
-sgs_status_t sgs_subnet_encode(const sgs_supernet_t *net, const sgs_subnet_cfg_t *cfg, int *out) {
+sgs_status_t sgs_subnet_encode(const sgs_supernet_t *net, const sgs_subnet_cfg_t *cfg, int *out) try {
     if (!net || !cfg || !out) return SGS_EINVAL;
     if (!cfg_valid(net, cfg)) return fail(net, SGS_ECONFIG, "SubNet config outside the elastic sets of this SuperNet");
     std::vector<int> e = encoding_of(slices_for(net, cfg));
     std::memcpy(out, e.data(), e.size() * sizeof(int));
     return SGS_OK;
-}
+} SGS_NO_THROW
 
 sgs_status_t sgs_subnet_cost(const sgs_supernet_t *cnet, const sgs_subnet_cfg_t *cfg, int batch, int res, double *flops,
-                             double *weight_bytes, double *activation_bytes) {
+                             double *weight_bytes, double *activation_bytes) try {
     sgs_supernet *net = const_cast<sgs_supernet *>(cnet);
     if (!net || !cfg || batch <= 0 || res <= 0) return SGS_EINVAL;
     if (!cfg_valid(net, cfg)) return fail(net, SGS_ECONFIG, "SubNet config outside the elastic sets of this SuperNet");
@@ -1366,10 +1403,10 @@ sgs_status_t sgs_subnet_cost(const sgs_supernet_t *cnet, const sgs_subnet_cfg_t 
     if (weight_bytes) *weight_bytes = p.weight_bytes;
     if (activation_bytes) *activation_bytes = p.act_bytes;
     return SGS_OK;
-}
+} SGS_NO_THROW
 
 sgs_status_t sgs_subnet_run(sgs_supernet_t *net, const sgs_subnet_cfg_t *cfg, const void *d_input, int batch, int res,
-                            void *d_logits, void *cuda_stream) {
+                            void *d_logits, void *cuda_stream) try {
     if (!net) return SGS_EINVAL;
     if (!cfg || !d_input || !d_logits || batch <= 0 || res < 8 || res > 1024) return fail(net, SGS_EINVAL, "bad argument");
     DeviceGuard guard(net->device);
@@ -1379,7 +1416,7 @@ sgs_status_t sgs_subnet_run(sgs_supernet_t *net, const sgs_subnet_cfg_t *cfg, co
     if (rc != SGS_OK) return rc;
     if (net->cache.enabled) cache_observe(net, plan->enc);
     return SGS_OK;
-}
+} SGS_NO_THROW
 
 // ------------------------------------------------------------------------------------------
 // Wave execution of a stream.  `G` consecutive queries form a wave; the wave walks the op list of the
@@ -1388,6 +1425,7 @@ sgs_status_t sgs_subnet_run(sgs_supernet_t *net, const sgs_subnet_cfg_t *cfg, co
 // types are launched per member.  Up to `W` waves are in flight on their own streams.
 // ------------------------------------------------------------------------------------------
 static sgs_status_t ensure_waves(sgs_supernet *net, int W) {
+    net->waves.reserve((size_t)W);
     while ((int)net->waves.size() < W) {
         sgs_supernet::WaveCtx w;
         CU(cudaStreamCreateWithFlags(&w.st, cudaStreamNonBlocking));
@@ -1399,12 +1437,13 @@ static sgs_status_t ensure_waves(sgs_supernet *net, int W) {
 
 static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subnet_cfg_t *cfgs, const void *inputs, int batch,
                               int res, void *logits, const sgs_stream_opts_t &o, sgs_stream_stats_t *stats, cudaStream_t st,
-                              bool host_buffers) {
+                              bool host_buffers, StreamScope &scope) {
     const int G = std::min(o.wave, TC_GROUP_MAX_ENTRIES);
     // per-launch timing (option "profile") wants the launches of one wave at a time
     const int W = net->profile ? 1 : std::max(1, std::min(o.concurrency ? o.concurrency : 2, 8));
     struct ProfRec { cudaEvent_t e0, e1; int cls; double bytes, flops; int layer, members, tiles; };
     std::vector<ProfRec> prof;
+    EventList events;
     sgs_status_t rc = ensure_slots(net, G * W);
     if (rc != SGS_OK) return rc;
     if ((rc = ensure_waves(net, W)) != SGS_OK) return rc;
@@ -1427,16 +1466,17 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
     std::vector<cudaEvent_t> ev;  // per wave: start and end on the wave's stream
     if (o.record_latency) {
         ev.resize(2 * (size_t)n_waves);
-        for (auto &e : ev) CU(cudaEventCreate(&e));
+        for (auto &e : ev) CU(events.make(&e));
     }
     cudaEvent_t e0, e1;
-    CU(cudaEventCreate(&e0));
-    CU(cudaEventCreate(&e1));
+    CU(events.make(&e0));
+    CU(events.make(&e1));
     const long long launches0 = net->kernel_launches;
     const int hits0 = net->plan_hits, miss0 = net->plan_misses;
     double flops = 0, wbytes = 0, miss_bytes = 0, hit = 0;
     int updates = 0;
     CU(cudaEventRecord(e0, st));
+    scope.in_flight = true;
     for (int w = 0; w < W; w++) { CU(cudaStreamWaitEvent(net->waves[w].st, e0, 0)); net->waves[w].busy = false; }
     const auto host_t0 = std::chrono::steady_clock::now();
     std::vector<Plan *> plans((size_t)G);
@@ -1703,8 +1743,8 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
         auto prof_begin = [&](int cls, double bytes, double fl, int layer, int members, int tiles) -> sgs_status_t {
             if (!net->profile) return SGS_OK;
             ProfRec r{nullptr, nullptr, cls, bytes, fl, layer, members, tiles};
-            CU(cudaEventCreate(&r.e0));
-            CU(cudaEventCreate(&r.e1));
+            CU(events.make(&r.e0));
+            CU(events.make(&r.e1));
             CU(cudaEventRecord(r.e0, ws));
             prof.push_back(r);
             return SGS_OK;
@@ -1795,6 +1835,7 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
     if (rc == SGS_OK && (ce != cudaSuccess || se != cudaSuccess))
         rc = fail(net, SGS_ECUDA, std::string("stream: ") + cudaGetErrorString(se != cudaSuccess ? se : ce));
     if (rc != SGS_OK) cudaDeviceSynchronize();
+    scope.in_flight = false;
     for (ProfRec &r : prof) {
         float ms = 0;
         if (rc == SGS_OK && r.e1 && cudaEventElapsedTime(&ms, r.e0, r.e1) == cudaSuccess) {
@@ -1806,8 +1847,6 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
                 net->prof_trace.push_back(tr);
             }
         }
-        if (r.e0) cudaEventDestroy(r.e0);
-        if (r.e1) cudaEventDestroy(r.e1);
     }
     if (rc == SGS_OK && tc_conv_status()) rc = fail(net, SGS_ETIMEOUT, "a bounded device-side wait ran out in the tensor-core kernel");
     if (rc == SGS_OK && stats) {
@@ -1843,10 +1882,6 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
         stats->plan_misses = net->plan_misses - miss0;
         stats->cache_updates = updates;
     }
-    for (auto &e : ev) cudaEventDestroy(e);
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    net->throughput_mode = 0;
     return rc;
 }
 
@@ -1856,7 +1891,7 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
 // The plan of a config as the op list the kernel interprets (one record per layer; the patch-matrix / padding ops
 // that the layer-by-layer paths put in front of the stem are dropped, the kernel convolves the image directly).
 static sgs_status_t build_pq_ops(sgs_supernet *net, Plan *plan) {
-    plan->pq.clear();
+    std::vector<PqOp> list;  // (the plan gets it when it is complete)
     const int stem_li = net->idx("stem");
     auto mult8 = [](int v) { return v > 0 && v % 8 == 0; };
     for (const Op &op : plan->ops) {
@@ -1905,12 +1940,12 @@ static sgs_status_t build_pq_ops(sgs_supernet *net, Plan *plan) {
             if (fused) {
                 PqOp g = q;
                 g.type = PQ_GAP; g.in = op.in; g.vout = 0; g.H = op.H; g.W = op.W; g.C = op.C;
-                plan->pq.push_back(g);
+                list.push_back(g);
             }
             q.type = PQ_SE_GATE; q.vin = fused ? 0 : op.vin; q.vout = fused ? 1 : op.vout; q.C = op.C; q.K = op.K;
             q.w = L1.w; q.ld = L1.C; q.shift = L1.shift; q.w2 = L2.w; q.ld2 = L2.C; q.bias2 = L2.shift;
             if (fused) {
-                plan->pq.push_back(q);
+                list.push_back(q);
                 std::memset(&q, 0, sizeof q);
                 q.res = q.vout = -1; q.cache_off = -1;
                 q.type = PQ_SCALE; q.in = op.in; q.out = op.out; q.vin = 1; q.H = op.H; q.W = op.W; q.C = op.C;
@@ -1930,14 +1965,15 @@ static sgs_status_t build_pq_ops(sgs_supernet *net, Plan *plan) {
         default: return fail(net, SGS_EUNSUPPORTED, "persistent kernel: layer type");
         }
         if (q.vin > 1 || q.vout > 1 || q.in > 3 || q.out > 3 || q.res > 3) return fail(net, SGS_EUNSUPPORTED, "persistent kernel: buffer id");
-        plan->pq.push_back(q);
+        list.push_back(q);
     }
+    plan->pq.swap(list);
     return SGS_OK;
 }
 
 static sgs_status_t persistent_impl(sgs_supernet_t *net, int n_queries, const sgs_subnet_cfg_t *cfgs, const void *inputs, int res,
                                     void *logits, const sgs_stream_opts_t &o, sgs_stream_stats_t *stats, cudaStream_t st,
-                                    bool host_buffers) {
+                                    bool host_buffers, StreamScope &scope) {
     if (net->family != SGS_MBV3 || net->dtype != SGS_BF16 || !tc_available())
         return fail(net, SGS_EUNSUPPORTED, "persistent execution serves bf16 handles of the MobileNetV3-shaped family on a tensor-core device");
     net->throughput_mode = 0;
@@ -2070,10 +2106,12 @@ static sgs_status_t persistent_impl(sgs_supernet_t *net, int n_queries, const sg
         if (h_bytes) std::memcpy(net->pq_h_tbl + ops_bytes + q_bytes, held.data(), h_bytes);
     }
 
+    EventList events;
     cudaEvent_t e0, e1;
-    CU(cudaEventCreate(&e0));
-    CU(cudaEventCreate(&e1));
+    CU(events.make(&e0));
+    CU(events.make(&e1));
     sgs_status_t rc = SGS_OK;
+    scope.in_flight = true;
     cudaError_t ce = cudaEventRecord(e0, st);
     if (ce == cudaSuccess && host_buffers && n_queries) ce = cudaMemcpyAsync(net->pq_stage_in, inputs, in_bytes * (size_t)n_queries, cudaMemcpyHostToDevice, st);
     if (ce == cudaSuccess && tbl_need) ce = cudaMemcpyAsync(net->pq_d_tbl, net->pq_h_tbl, tbl_need, cudaMemcpyHostToDevice, st);
@@ -2097,6 +2135,7 @@ static sgs_status_t persistent_impl(sgs_supernet_t *net, int n_queries, const sg
     if (ce == cudaSuccess && host_buffers && n_queries) ce = cudaMemcpyAsync(logits, net->pq_stage_out, out_bytes * (size_t)n_queries, cudaMemcpyDeviceToHost, st);
     if (ce == cudaSuccess) ce = cudaEventRecord(e1, st);
     cudaError_t se = cudaStreamSynchronize(st);
+    scope.in_flight = false;
     if (ce != cudaSuccess || se != cudaSuccess) rc = fail(net, SGS_ECUDA, std::string("persistent stream: ") + cudaGetErrorString(se != cudaSuccess ? se : ce));
     if (rc == SGS_OK && tc_conv_status()) rc = fail(net, SGS_ETIMEOUT, "a bounded device-side wait ran out in the persistent SubNet kernel");
     if (rc == SGS_OK && stats) {
@@ -2118,8 +2157,6 @@ static sgs_status_t persistent_impl(sgs_supernet_t *net, int n_queries, const sg
         stats->plan_misses = net->plan_misses - miss0;
         stats->cache_updates = updates;
     }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
     return rc;
 }
 
@@ -2131,6 +2168,7 @@ static sgs_status_t stream_impl(sgs_supernet_t *net, int n_queries, const sgs_su
         return fail(net, SGS_EINVAL, "bad argument");
     DeviceGuard guard(net->device);
     if (!guard.ok) return fail(net, SGS_ECUDA, "cudaSetDevice failed");
+    StreamScope scope{net};
     sgs_stream_opts_t o;
     if (opts) o = *opts;
     else { o.cache_enabled = 1; o.window_q = 4; o.cache_budget_bytes = 0; o.use_graphs = 1; o.record_latency = 1; o.weights_evict_first = 0; o.concurrency = 1; o.wave = 0; o.policy = 0; o.persistent = 0; }
@@ -2147,10 +2185,10 @@ static sgs_status_t stream_impl(sgs_supernet_t *net, int n_queries, const sgs_su
     net->cache.evict_first_when_off = (!o.cache_enabled && o.weights_evict_first) ? 1 : 0;
     if (o.persistent) {
         if (batch != 1) return fail(net, SGS_EINVAL, "persistent execution takes one image per query");
-        return persistent_impl(net, n_queries, cfgs, inputs, res, logits, o, stats, st, host_buffers);
+        return persistent_impl(net, n_queries, cfgs, inputs, res, logits, o, stats, st, host_buffers, scope);
     }
     if (o.wave > 0 && n_queries > 0 && net->dtype == SGS_BF16 && tc_available() && !net->force_plain)
-        return wave_impl(net, n_queries, cfgs, inputs, batch, res, logits, o, stats, st, host_buffers);
+        return wave_impl(net, n_queries, cfgs, inputs, batch, res, logits, o, stats, st, host_buffers, scope);
     // queries in flight at once: each runs in its own slot; per-kernel profiling wants them one by one
     const int S = net->profile ? 1 : std::max(1, std::min(o.concurrency ? o.concurrency : 1, std::max(1, n_queries)));
     {
@@ -2176,20 +2214,22 @@ static sgs_status_t stream_impl(sgs_supernet_t *net, int n_queries, const sgs_su
             if (!sl.stage_out) { sgs_status_t rc = dev_alloc(net, (void **)&sl.stage_out, net->stage_out_bytes); if (rc != SGS_OK) return rc; }
         }
     }
+    EventList events;
     std::vector<cudaEvent_t> ev;  // per query: start and end on the query's stream
     if (o.record_latency) {
         ev.resize(2 * (size_t)n_queries);
-        for (auto &e : ev) CU(cudaEventCreate(&e));
+        for (auto &e : ev) CU(events.make(&e));
     }
     cudaEvent_t e0, e1;
-    CU(cudaEventCreate(&e0));
-    CU(cudaEventCreate(&e1));
+    CU(events.make(&e0));
+    CU(events.make(&e1));
     const long long launches0 = net->kernel_launches;
     const int hits0 = net->plan_hits, miss0 = net->plan_misses;
     double flops = 0, wbytes = 0, miss_bytes = 0, hit = 0;
     int updates = 0;
     sgs_status_t rc = SGS_OK;
     CU(cudaEventRecord(e0, st));
+    scope.in_flight = true;
     const auto host_t0 = std::chrono::steady_clock::now();
     for (int sidx = 1; sidx < S; sidx++) CU(cudaStreamWaitEvent(net->slots[sidx].st, e0, 0));  // fork
     for (int t = 0; t < n_queries && rc == SGS_OK; t++) {
@@ -2253,6 +2293,7 @@ static sgs_status_t stream_impl(sgs_supernet_t *net, int n_queries, const sgs_su
     if (rc == SGS_OK && (ce != cudaSuccess || se != cudaSuccess))
         rc = fail(net, SGS_ECUDA, std::string("stream: ") + cudaGetErrorString(se != cudaSuccess ? se : ce));
     if (rc != SGS_OK) cudaDeviceSynchronize();  // leave no work of the other slots behind
+    scope.in_flight = false;
     if (rc == SGS_OK && tc_conv_status()) rc = fail(net, SGS_ETIMEOUT, "a bounded device-side wait ran out in the tensor-core kernel");
     if (rc == SGS_OK && stats) {
         std::memset(stats, 0, sizeof(*stats));
@@ -2281,33 +2322,29 @@ static sgs_status_t stream_impl(sgs_supernet_t *net, int n_queries, const sgs_su
         stats->plan_misses = net->plan_misses - miss0;
         stats->cache_updates = updates;
     }
-    for (auto &e : ev) cudaEventDestroy(e);
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    net->throughput_mode = 0;
     return rc;
 }
 
 sgs_status_t sgs_stream_run(sgs_supernet_t *net, int n_queries, const sgs_subnet_cfg_t *cfgs, const void *d_inputs,
                             int batch_per_query, int res, void *d_logits, const sgs_stream_opts_t *opts,
-                            sgs_stream_stats_t *stats, void *cuda_stream) {
+                            sgs_stream_stats_t *stats, void *cuda_stream) try {
     return stream_impl(net, n_queries, cfgs, d_inputs, batch_per_query, res, d_logits, opts, stats, (cudaStream_t)cuda_stream, false);
-}
+} SGS_NO_THROW
 
 sgs_status_t sgs_stream_run_host(sgs_supernet_t *net, int n_queries, const sgs_subnet_cfg_t *cfgs, const void *h_inputs,
                                  int batch_per_query, int res, void *h_logits, const sgs_stream_opts_t *opts,
-                                 sgs_stream_stats_t *stats, void *cuda_stream) {
+                                 sgs_stream_stats_t *stats, void *cuda_stream) try {
     return stream_impl(net, n_queries, cfgs, h_inputs, batch_per_query, res, h_logits, opts, stats, (cudaStream_t)cuda_stream, true);
-}
+} SGS_NO_THROW
 
-sgs_status_t sgs_cache_configure(sgs_supernet_t *net, int enabled, size_t budget_bytes, int window_q) {
+sgs_status_t sgs_cache_configure(sgs_supernet_t *net, int enabled, size_t budget_bytes, int window_q) try {
     if (!net) return SGS_EINVAL;
     if (window_q < 1) return fail(net, SGS_EINVAL, "window_q must be >= 1");
     cache_reset(net, enabled != 0, budget_bytes, window_q);
     return SGS_OK;
-}
+} SGS_NO_THROW
 
-sgs_status_t sgs_cache_set_candidates(sgs_supernet_t *net, const sgs_subnet_cfg_t *cfgs, int n) {
+sgs_status_t sgs_cache_set_candidates(sgs_supernet_t *net, const sgs_subnet_cfg_t *cfgs, int n) try {
     if (!net || n < 0 || (n && !cfgs)) return SGS_EINVAL;
     std::vector<std::vector<int>> raw;
     for (int j = 0; j < n; j++) {
@@ -2318,16 +2355,16 @@ sgs_status_t sgs_cache_set_candidates(sgs_supernet_t *net, const sgs_subnet_cfg_
     clip_candidates(net);
     if (n == 0) net->cache.policy = 0;
     return SGS_OK;
-}
+} SGS_NO_THROW
 
-sgs_status_t sgs_cache_set_policy(sgs_supernet_t *net, int policy) {
+sgs_status_t sgs_cache_set_policy(sgs_supernet_t *net, int policy) try {
     if (!net) return SGS_EINVAL;
     if (policy != SGS_POLICY_INTERSECTION && policy != SGS_POLICY_AVGNET) return fail(net, SGS_EINVAL, "unknown cache policy");
     if (policy == SGS_POLICY_AVGNET && net->cache.cand_raw.empty())
         return fail(net, SGS_EINVAL, "the AvgNet policy needs a candidate set (sgs_cache_set_candidates)");
     net->cache.policy = policy;
     return SGS_OK;
-}
+} SGS_NO_THROW
 
 // ------------------------------------------------------------------------------------------
 // Scheduler object: Algorithm 1 (Section 3.3) over a latency table (Section 3.2)
@@ -2370,7 +2407,7 @@ int sched_select(const sgs_sched *s, int policy, double a_t, double l_t) {
 extern "C" {
 
 sgs_status_t sgs_sched_create(sgs_supernet_t *net, const sgs_subnet_cfg_t *subnets, const double *accuracy, int n_subnets,
-                              int window_q, sgs_sched_t **out) {
+                              int window_q, sgs_sched_t **out) try {
     if (!net || !out) return SGS_EINVAL;
     if (!subnets || !accuracy || n_subnets < 1 || window_q < 1) return fail(net, SGS_EINVAL, "bad argument");
     if (net->cache.cand_raw.empty()) return fail(net, SGS_EINVAL, "a scheduler needs a candidate set (sgs_cache_set_candidates)");
@@ -2388,7 +2425,7 @@ sgs_status_t sgs_sched_create(sgs_supernet_t *net, const sgs_subnet_cfg_t *subne
     cache_pin(net, -1);
     *out = s.release();
     return SGS_OK;
-}
+} SGS_NO_THROW
 
 void sgs_sched_free(sgs_sched_t *s) {
     if (!s) return;
@@ -2421,7 +2458,7 @@ sgs_status_t sgs_sched_get_table(const sgs_sched_t *s, double *latency) {
 }
 
 sgs_status_t sgs_sched_measure(sgs_sched_t *s, const void *d_input, int batch, int res, void *d_logits, int reps,
-                               size_t flush_bytes, void *cuda_stream) {
+                               size_t flush_bytes, void *cuda_stream) try {
     if (!s) return SGS_EINVAL;
     sgs_supernet *net = s->net;
     if (!d_input || !d_logits || batch <= 0 || res < 8 || res > 1024 || reps < 1 || reps > 1000) return fail(net, SGS_EINVAL, "bad argument");
@@ -2437,8 +2474,9 @@ sgs_status_t sgs_sched_measure(sgs_sched_t *s, const void *d_input, int batch, i
         if (rc != SGS_OK) return rc;
         s->flush_bytes = flush_bytes;
     }
+    EventList events;
     std::vector<cudaEvent_t> ev(2 * (size_t)reps);
-    for (auto &e : ev) CU(cudaEventCreate(&e));
+    for (auto &e : ev) CU(events.make(&e));
     sgs_status_t rc = SGS_OK;
     std::vector<float> ms((size_t)reps);
     for (int j = 0; j <= s->M && rc == SGS_OK; j++) {
@@ -2461,14 +2499,13 @@ sgs_status_t sgs_sched_measure(sgs_sched_t *s, const void *d_input, int batch, i
         }
     }
     cudaStreamSynchronize(st);
-    for (auto &e : ev) cudaEventDestroy(e);
     cache_pin(net, s->state < s->M ? s->state : -1);
     if (rc == SGS_OK && tc_conv_status()) return fail(net, SGS_ETIMEOUT, "a bounded wait ran out in a tensor-core kernel");
     return rc;
-}
+} SGS_NO_THROW
 
 sgs_status_t sgs_sched_step(sgs_sched_t *s, int n, const int *policy, const double *a_t, const double *l_t, int *subnet,
-                            int *cache_state) {
+                            int *cache_state) try {
     if (!s) return SGS_EINVAL;
     if (n < 0 || (n && (!policy || !a_t || !l_t || !subnet))) return fail(s->net, SGS_EINVAL, "bad argument");
     if ((int)s->net->cache.cand.size() != s->M) return fail(s->net, SGS_EINVAL, "the candidate set changed under the scheduler");
@@ -2488,7 +2525,7 @@ sgs_status_t sgs_sched_step(sgs_sched_t *s, int n, const int *policy, const doub
     }
     if (s->state != before || s->net->cache.policy != 2) cache_pin(s->net, s->state < s->M ? s->state : -1);
     return SGS_OK;
-}
+} SGS_NO_THROW
 
 sgs_status_t sgs_sched_subnet(const sgs_sched_t *s, int i, sgs_subnet_cfg_t *out) {
     if (!s || !out || i < 0 || i >= s->N) return SGS_EINVAL;
@@ -2516,7 +2553,7 @@ sgs_status_t sgs_cache_stats(const sgs_supernet_t *net, sgs_cache_stats_t *out) 
 }
 
 sgs_status_t sgs_profile_read(sgs_supernet_t *net, int kernel_class, long long *launches, double *total_ms,
-                              double *alg_bytes, double *flops) {
+                              double *alg_bytes, double *flops) try {
     if (!net || kernel_class < 0 || kernel_class > 3) return SGS_EINVAL;
     DeviceGuard guard(net->device);
     fold_profile(net);
@@ -2525,7 +2562,7 @@ sgs_status_t sgs_profile_read(sgs_supernet_t *net, int kernel_class, long long *
     if (alg_bytes) *alg_bytes = net->prof_bytes[kernel_class];
     if (flops) *flops = net->prof_flops[kernel_class];
     return SGS_OK;
-}
+} SGS_NO_THROW
 
 int sgs_profile_trace(sgs_supernet_t *net, sgs_launch_record_t *out, int cap) {
     if (!net || cap < 0 || (cap && !out)) return -1;
@@ -2540,7 +2577,7 @@ int sgs_layer_name(const sgs_supernet_t *net, int layer, char *out, int cap) {
     return (int)net->layers[(size_t)layer].name.size();
 }
 
-sgs_status_t sgs_set_option(sgs_supernet_t *net, const char *name, long long value) {
+sgs_status_t sgs_set_option(sgs_supernet_t *net, const char *name, long long value) try {
     if (!net || !name) return SGS_EINVAL;
     std::string n(name);
     if (n == "conv_impl" || n == "pad_channels") {
@@ -2596,9 +2633,9 @@ sgs_status_t sgs_set_option(sgs_supernet_t *net, const char *name, long long val
         return SGS_OK;
     }
     return fail(net, SGS_EINVAL, "unknown option " + n);
-}
+} SGS_NO_THROW
 
-long long sgs_get_counter(const sgs_supernet_t *net, const char *name) {
+long long sgs_get_counter(const sgs_supernet_t *net, const char *name) try {
     if (!net || !name) return -1;
     std::string n(name);
     if (n == "kernel_launches") return net->kernel_launches;
@@ -2617,13 +2654,13 @@ long long sgs_get_counter(const sgs_supernet_t *net, const char *name) {
         return c;
     }
     return -1;
-}
+} catch (...) { return -1; }
 
 const char *sgs_last_error(const sgs_supernet_t *net) { return net ? net->err.c_str() : "null handle"; }
 
 // Stand-alone sliced convolution.
 sgs_status_t sgs_conv2d_sliced(const sgs_conv_desc_t *d, const void *d_x, const void *d_w, const float *d_scale,
-                               const float *d_shift, const void *d_res, void *d_y, void *cuda_stream) {
+                               const float *d_shift, const void *d_res, void *d_y, void *cuda_stream) try {
     if (!d || !d_x || !d_w || !d_scale || !d_shift || !d_y) return SGS_EINVAL;
     if (d->N <= 0 || d->H <= 0 || d->W <= 0 || d->C <= 0 || d->K <= 0 || d->k <= 0 || (d->k & 1) == 0 || d->k > d->R ||
         ((d->R - d->k) & 1) || d->K > d->Kmax || (!d->depthwise && d->C > d->Cmax) || (d->stride != 1 && d->stride != 2) ||
@@ -2658,11 +2695,11 @@ sgs_status_t sgs_conv2d_sliced(const sgs_conv_desc_t *d, const void *d_x, const 
     if (d->impl == 2) return SGS_EUNSUPPORTED;
     e = d->dtype == SGS_BF16 ? launch_conv_plain<__nv_bfloat16>(a, st) : launch_conv_plain<float>(a, st);
     return e == cudaSuccess ? SGS_OK : e == cudaErrorNotSupported ? SGS_EUNSUPPORTED : SGS_ECUDA;
-}
+} SGS_NO_THROW
 
 // One sliced convolution layer with 8-bit operands on the tensor cores (see sgs.h).
 sgs_status_t sgs_conv2d_sliced_i8(const sgs_conv_i8_desc_t *d, const void *d_x, const void *d_w, const int32_t *d_mult,
-                                  const int32_t *d_shift, const int32_t *d_bias, const void *d_res, void *d_y, void *cuda_stream) {
+                                  const int32_t *d_shift, const int32_t *d_bias, const void *d_res, void *d_y, void *cuda_stream) try {
     if (!d || !d_x || !d_w || !d_mult || !d_shift || !d_bias || !d_y) return SGS_EINVAL;
     if (d->N <= 0 || d->H <= 0 || d->W <= 0 || d->C <= 0 || d->K <= 0 || d->k <= 0 || (d->k & 1) == 0 || d->k > d->R ||
         ((d->R - d->k) & 1) || d->K > d->Kmax || d->C > d->Cmax || (d->stride != 1 && d->stride != 2) || d->res_shift < 0 || d->res_shift > 31)
@@ -2687,10 +2724,10 @@ sgs_status_t sgs_conv2d_sliced_i8(const sgs_conv_i8_desc_t *d, const void *d_x, 
     std::shared_ptr<TcConvPlan> plan = tc_conv_prepare(a, dev, &why);
     if (!plan) return SGS_EUNSUPPORTED;
     return tc_conv_launch(*plan, a, (cudaStream_t)cuda_stream) == cudaSuccess ? SGS_OK : SGS_ECUDA;
-}
+} SGS_NO_THROW
 
 // Non-convolution layers on caller tensors (see sgs.h).  Mirrors the dispatch of launch_op / wave_impl.
-sgs_status_t sgs_aux_op(int n, const sgs_aux_desc_t *desc, const sgs_aux_args_t *args, int grouped, void *cuda_stream) {
+sgs_status_t sgs_aux_op(int n, const sgs_aux_desc_t *desc, const sgs_aux_args_t *args, int grouped, void *cuda_stream) try {
     if (n <= 0 || n > 65535 || !desc || !args) return SGS_EINVAL;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     std::vector<SmallEntry> es((size_t)n);
@@ -2752,7 +2789,7 @@ sgs_status_t sgs_aux_op(int n, const sgs_aux_desc_t *desc, const sgs_aux_args_t 
         if (ce != cudaSuccess) return SGS_ECUDA;
     }
     return SGS_OK;
-}
+} SGS_NO_THROW
 
 int sgs_device_status(void) { return tc_conv_status(); }
 

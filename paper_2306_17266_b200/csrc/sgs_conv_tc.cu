@@ -856,7 +856,7 @@ int *static_status_word(int device) {
 
 extern "C" sgs_status_t sgs_conv2d_sliced_static(const sgs_conv_desc_t *d, const void *d_x, const void *d_w,
                                                  const float *d_scale, const float *d_shift, const void *d_res, void *d_y,
-                                                 void *cuda_stream) {
+                                                 void *cuda_stream) try {
     using namespace sgs;
     if (!d || !d_x || !d_w || !d_scale || !d_shift || !d_y) return SGS_EINVAL;
     if (d->N <= 0 || d->H <= 0 || d->W <= 0 || d->C <= 0 || d->K <= 0 || d->k <= 0 || (d->k & 1) == 0 || d->k > d->R ||
@@ -892,4 +892,4 @@ extern "C" sgs_status_t sgs_conv2d_sliced_static(const sgs_conv_desc_t *d, const
     prm.early_weights = 0;
     const cudaError_t e = plan->bn_tile == 64 ? launch_variant<64, false>(*plan, prm, st) : launch_variant<128, false>(*plan, prm, st);
     return e == cudaSuccess ? SGS_OK : SGS_ECUDA;
-}
+} SGS_NO_THROW

@@ -14,6 +14,11 @@
 
 #include "sgs.h"
 
+// End of a C entry point whose body is a try block: nothing is thrown through the C interface (what the bodies throw is a
+// failed host allocation).
+#define SGS_NO_THROW \
+    catch (...) { return SGS_ENOMEM; }
+
 namespace sgs {
 
 enum LayerKind { KIND_CONV = 0, KIND_DW = 1, KIND_LINEAR = 2 };

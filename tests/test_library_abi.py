@@ -2,6 +2,8 @@
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -54,3 +56,24 @@ def test_convolutions_beyond_32_bit_indexes_are_refused(N, H, C, k, impl, dtype)
     d = sgs.ConvDesc(N=N, H=H, W=H, C=C, K=8, Kmax=8, Cmax=C, R=k, k=k, stride=1, act=0, dtype=dtype, impl=impl)
     p = 1 << 20  # (never read)
     assert sgs.lib().sgs_conv2d_sliced(ctypes.byref(d), p, p, p, p, None, p, None) == sgs.binding.SGS_EUNSUPPORTED
+
+
+def test_a_failed_host_allocation_is_a_status_without_a_gpu():
+    # 65535 members: 8 MB of records that the call cannot have, because the process may not grow
+    program = """
+import ctypes, resource
+import paper_2306_17266_b200 as sgs
+from paper_2306_17266_b200.binding import AuxArgs, AuxDesc
+n = 65535
+L, descs, args = sgs.lib(), (AuxDesc * n)(), (AuxArgs * n)()
+assert L.sgs_aux_op(1, descs, args, 0, None) == sgs.binding.SGS_EINVAL
+with open("/proc/self/statm") as f:
+    size = int(f.read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (size, resource.RLIM_INFINITY))
+st = L.sgs_aux_op(n, descs, args, 0, None)
+resource.setrlimit(resource.RLIMIT_AS, (resource.RLIM_INFINITY, resource.RLIM_INFINITY))
+print("status", st)
+"""
+    r = subprocess.run([sys.executable, "-c", program], capture_output=True, text=True, cwd=ROOT, timeout=300)
+    assert r.returncode == 0, (r.returncode, r.stderr[-1000:])
+    assert r.stdout.split() == ["status", str(sgs.binding.SGS_ENOMEM)]
