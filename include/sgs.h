@@ -194,7 +194,8 @@ sgs_status_t sgs_subnet_run(sgs_supernet_t *net, const sgs_subnet_cfg_t *cfg, co
  * d_logits + t*batch_per_query*n_classes floats.  With the cache enabled the SubGraph shared by the
  * last window_q queries (element-wise minimum of their layer encodings = their exact intersection,
  * Section 2.2, Appendix A.4) is marked resident for the following queries.
- * Synchronises the stream before filling `stats` (may be NULL).  `opts` NULL = cache on, window 4,
+ * Synchronises the stream before filling `stats` (may be NULL), so it refuses a stream under capture (SGS_EINVAL;
+ * sgs_subnet_run and the layer entry points can be captured after a first call outside the capture).  `opts` NULL = cache on, window 4,
  * graphs on, latency recorded, one query at a time.  Per-query latency is measured from the moment
  * the query's first operation starts on its slot's stream to its last operation's end.
  */

@@ -272,6 +272,12 @@ struct StreamScope {
     }
 };
 
+// Calls that synchronise the stream cannot be captured; they refuse before anything joins the capture.
+bool being_captured(cudaStream_t st) {
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(st, &s) == cudaSuccess && s != cudaStreamCaptureStatusNone;
+}
+
 sgs_status_t fail(const sgs_supernet *n, sgs_status_t st, const std::string &msg) {
     if (n) n->err = msg;
     return st;
@@ -2168,6 +2174,7 @@ static sgs_status_t stream_impl(sgs_supernet_t *net, int n_queries, const sgs_su
         return fail(net, SGS_EINVAL, "bad argument");
     DeviceGuard guard(net->device);
     if (!guard.ok) return fail(net, SGS_ECUDA, "cudaSetDevice failed");
+    if (being_captured(st)) return fail(net, SGS_EINVAL, "the stream is being captured, and this call synchronises it");
     StreamScope scope{net};
     sgs_stream_opts_t o;
     if (opts) o = *opts;
@@ -2466,6 +2473,7 @@ sgs_status_t sgs_sched_measure(sgs_sched_t *s, const void *d_input, int batch, i
     DeviceGuard guard(net->device);
     if (!guard.ok) return fail(net, SGS_ECUDA, "cudaSetDevice failed");
     cudaStream_t st = (cudaStream_t)cuda_stream;
+    if (being_captured(st)) return fail(net, SGS_EINVAL, "the stream is being captured, and this call synchronises it");
     if (flush_bytes > s->flush_bytes) {
         CU(cudaStreamSynchronize(st));
         dev_free(net, s->flush, s->flush_bytes);
@@ -2752,6 +2760,7 @@ sgs_status_t sgs_aux_op(int n, const sgs_aux_desc_t *desc, const sgs_aux_args_t 
         if (grouped && (kind != kind0 || d.dtype != SGS_BF16 || d.dtype != desc[0].dtype || !small_supported(kind, e))) return SGS_EUNSUPPORTED;
     }
     if (grouped) {
+        if (being_captured(st)) return SGS_EINVAL;
         SmallEntry *d_tbl = nullptr;
         if (cudaMalloc((void **)&d_tbl, (size_t)n * sizeof(SmallEntry)) != cudaSuccess) return SGS_ENOMEM;
         cudaError_t e = cudaMemcpyAsync(d_tbl, es.data(), (size_t)n * sizeof(SmallEntry), cudaMemcpyHostToDevice, st);
