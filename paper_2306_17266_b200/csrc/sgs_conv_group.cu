@@ -45,11 +45,11 @@ struct __align__(16) GroupEntry {
     int mtiles;              // pixel tiles of this member (tile = filter tile * mtiles + pixel tile)
     int N, Ho, Wo, K, C;
     int R, tap0;             // stored kernel size; tap index of the cropped kernel's first tap
-    int tiles_w, tiles_hw, cchunks, iters, layer;
+    int tiles_w, tiles_hw, cchunks, layer;
     short bw, bh, bn;        // pixel box
     short bn_tile;           // MMA columns of a full tile
     short pix_rows;          // rows of the pixel box (bw * bh * bn)
-    short pad0_;
+    short pad0_[3];
     unsigned char k, stride, p, act, swap, kw;  // k x kw taps
     // Two members with at most 64 output pixels each can share a tile: the first ("pair") owns the tile's
     // geometry, filters and weight map and takes MMA rows 0..63, the entry after it ("second") takes rows
@@ -74,16 +74,14 @@ __device__ __forceinline__ int tile_entry(const GroupEntry *es, const int *begin
 
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap *m) { asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory"); }
 
-
 // Kernel parameters.  The tensor maps travel in the parameter block (the TMA unit reads them from
 // there); the per-member records travel in a device table.
 template <int NMAPS> struct GroupParams {
     const GroupEntry *entries;
-    const void *unused_;
     int *status;
     int n_entries, total_tiles;
     int n_stages, stage_bytes;  // operand ring of this launch
-    int pad_[6];
+    int pad_[8];  // (tensor maps lie at multiples of 64 bytes)
     CUtensorMap maps[NMAPS];
 };
 static_assert(sizeof(GroupParams<TC_GROUP_MAPS_LARGE>) <= 32764, "kernel parameter block");
@@ -488,7 +486,7 @@ void GroupLaunch::add(void *host_entry, const TcConvPlan &pl, const ConvArgs &a)
     }
     e.R = p.R; e.tap0 = p.o * p.R + p.o;
     e.tiles_w = p.tiles_w; e.tiles_hw = p.tiles_w * p.tiles_h;
-    e.cchunks = p.cchunks; e.iters = p.iters; e.layer = a.layer;
+    e.cchunks = p.cchunks; e.layer = a.layer;
     e.bw = (short)p.bw; e.bh = (short)p.bh; e.bn = (short)p.bn;
     e.pix_rows = (short)(p.bw * p.bh * p.bn);
     e.swap = (unsigned char)pl.swap;
@@ -531,7 +529,6 @@ cudaError_t GroupLaunch::launch(size_t window_max, int sms, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     impl->prm.status = tc_status_word(dev);
     if (!impl->prm.status) return cudaErrorInitializationError;
-    impl->prm.unused_ = nullptr;
     // stage = 16 KB for the row-side operand + room for the widest column-side operand of the launch
     const int col_rows = impl->col_rows <= 64 ? 64 : impl->col_rows <= 128 ? 128 : 256;
     impl->prm.stage_bytes = G_X_BYTES + col_rows * CHUNK_C * 2;
