@@ -183,7 +183,7 @@ sgs_status_t sgs_subnet_validate(const sgs_supernet_t *net, const sgs_subnet_cfg
  *   d_logits  device pointer, [batch][n_classes] fp32, caller-owned, written
  * Asynchronous on `cuda_stream`.  Invalid config -> SGS_ECONFIG before anything is launched.
  * No sliced copy of any weight is made; the only device memory that may grow is the activation
- * workspace (and the split-reduction scratch) on the first use of a larger (batch, res).
+ * workspace, on the first use of a larger (batch, res).
  */
 sgs_status_t sgs_subnet_run(sgs_supernet_t *net, const sgs_subnet_cfg_t *cfg, const void *d_input, int batch,
                             int res, void *d_logits, void *cuda_stream);

@@ -228,7 +228,7 @@ def conv2d_sliced(desc: ConvDesc, d_x: int, d_w: int, d_scale: int, d_shift: int
 
 def conv2d_sliced_static(desc: ConvDesc, d_x: int, d_w: int, d_scale: int, d_shift: int, d_res: int, d_y: int,
                          stream: int = 0):
-    """The sliced convolution without any device allocation (fixed scratch inside the library)."""
+    """The sliced convolution for callers that may not allocate: tensor cores only, status word inside the library image."""
     st = lib().sgs_conv2d_sliced_static(ctypes.byref(desc), d_x, d_w, d_scale, d_shift, d_res or None, d_y, stream)
     if st != SGS_OK:
         raise SgsError(st, "sgs_conv2d_sliced_static")

@@ -187,7 +187,7 @@ struct sgs_supernet {
     void *stem_win_w = nullptr;
     // Workspaces of the queries in flight.  Queries of a stream are independent, so up to
     // `concurrency` of them run at the same time, each in its own slot (own activation buffers, own
-    // scratch, own CUDA stream); slot 0 runs on the caller's stream.
+    // CUDA stream); slot 0 runs on the caller's stream.
     struct Slot {
         void *act[4] = {nullptr, nullptr, nullptr, nullptr};
         float *vec[3] = {nullptr, nullptr, nullptr};
@@ -630,13 +630,13 @@ sgs_status_t build_plan(sgs_supernet *net, const sgs_subnet_cfg_t *cfg, int batc
     return SGS_OK;
 }
 
-// Makes sure `n_slots` slots exist, each with buffers for the sizes in use.
-// Frees the activation / vector / split-reduction buffers of a slot (the sizes are the handle's current ones).
+// Frees the activation / vector buffers of a slot (the sizes are the handle's current ones).
 void release_slot_buffers(sgs_supernet *net, sgs_supernet::Slot &sl, bool act, bool vec) {
     for (int i = 0; i < 4 && act; i++) { dev_free(net, sl.act[i], net->act_elems * net->elem() + 256); sl.act[i] = nullptr; }
     for (int i = 0; i < 3 && vec; i++) { dev_free(net, sl.vec[i], net->vec_elems * 4); sl.vec[i] = nullptr; }
 }
 
+// Makes sure `n_slots` slots exist, each with buffers for the sizes in use.
 sgs_status_t ensure_slots(sgs_supernet *net, int n_slots) {
     net->slots.reserve((size_t)std::max(n_slots, 0));
     while ((int)net->slots.size() < n_slots) {

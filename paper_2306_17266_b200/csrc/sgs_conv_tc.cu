@@ -510,9 +510,9 @@ int *tc_status_word(int device) {
     return g_dev[device].status;
 }
 
-int *static_status_word(int device);  // status word inside the fixed scratch array (below); nullptr before its set-up
+int *static_status_word(int device);  // status word inside the library image (below); nullptr before its set-up
 
-// Both status words of the current device (the allocated one and the one inside the fixed scratch array of the
+// Both status words of the current device (the allocated one and the one inside the library image of the
 // allocation-free entry point); a word of another device is readable only while that device is current.
 int tc_conv_status() {
     std::lock_guard<std::mutex> lk(g_mu);

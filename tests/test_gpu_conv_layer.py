@@ -49,7 +49,7 @@ def run_case(N, H, W, Cmax, C, Kmax, K, R, k, stride, act, use_res, impl, seed=0
                         impl=impl, depthwise=int(depthwise), cache_k=K // 2, cache_c=C // 2, weight_policy=policy,
                         split_k_off=split_off)
     outs = []
-    for _ in range(2):  # twice: the split-K counters must come back clean, and the result must repeat
+    for _ in range(2):  # twice: the result must repeat (also that of a reduction split over a cluster)
         sgs.conv2d_sliced(desc, dev["x"].data_ptr(), dev["w"].data_ptr(), dev["scale"].data_ptr(), dev["shift"].data_ptr(),
                           dev["res"].data_ptr() if use_res else 0, dy.data_ptr(), torch.cuda.current_stream().cuda_stream)
         torch.cuda.synchronize()
@@ -104,7 +104,7 @@ def test_shapes_the_tensor_core_kernel_refuses():
         run_case(1, 8, 8, 16, 12, 16, 12, 3, 3, 1, 1, False, impl=2)
     assert e.value.status == sgs.binding.SGS_EUNSUPPORTED
     run_case(1, 8, 8, 16, 12, 16, 12, 3, 3, 1, 1, False, impl=0)
-    run_case(1, 9, 9, 16, 16, 16, 16, 3, 3, 2, 1, False, impl=0)  # odd input, stride 2 -> falls back
+    run_case(1, 9, 9, 16, 16, 16, 16, 3, 3, 2, 1, False, impl=0)  # odd input, stride 2: parity views of different sizes
 
 
 @pytest.mark.parametrize("k,stride", [(3, 1), (5, 1), (7, 1), (3, 2), (5, 2), (7, 2)])
@@ -115,9 +115,8 @@ def test_depthwise(k, stride):
 
 @pytest.mark.parametrize("k", [3, 5, 7])
 def test_depthwise_walking_kernel(k):
-    # stride-1 launches of 48 M outputs and more walk down the image behind a shared-memory ring of input rows; the
-    # library option makes every stride-1 shape take that kernel: ragged column tiles, maps shorter than the ring, more
-    # rows than a 56-row segment (two segments with their halo rows), channel counts off the 128-channel block
+    # warps walk down strips of columns behind rings of input rows: ragged strips, maps shorter than the ring, rows split into
+    # segments with their halo rows, channel counts off the 64-channel block; the option "dw_walk" is accepted without effect
     from tests import gpu_util as gu
     from paper_2306_17266_b200 import workload as wl
     _, _, net = gu.nets(wl.TINY, True)

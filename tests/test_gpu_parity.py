@@ -99,8 +99,8 @@ def test_no_sliced_weight_copy_is_made():
     base = gnet.get_counter("device_bytes")
     for c in wl.uniform_stream(wl.RESNET, 8, seed=32):
         gu.gpu_forward(gnet, c, x, True)
-    # only the split-reduction scratch may have grown, never by as much as the smallest sliced layer set
-    assert gnet.get_counter("device_bytes") - base < 4 << 20
+    # the workspaces of the largest SubNet serve all; a split reduction takes no scratch
+    assert gnet.get_counter("device_bytes") == base
 
 
 def test_stream_run_matches_single_queries_and_counts_bytes():

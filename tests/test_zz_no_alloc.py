@@ -2,11 +2,12 @@
 
 Some callers of the library cannot allocate device memory when they call it: they own all device
 memory through a pool of their own, or they cannot afford the device-wide synchronisation an
-allocation implies.  For them the library offers a variant whose
-split-reduction scratch is a fixed array inside the library image.  This file checks, through the C
+allocation implies.  For them the library offers a variant that keeps its status word inside the library
+image (a split reduction meets in shared memory and needs no scratch).  This file checks, through the C
 interface, that the variant returns what the ordinary entry point returns (within the layer tests'
 tolerance, 1e-2 * max|ref|), on two calls in a row, that free device memory does not change across
-its calls, and that it refuses work beyond its fixed scratch.
+its calls, and that it refuses the work its declaration refuses (split reductions whose partial
+tiles, written out, would exceed SGS_STATIC_SCRATCH_BYTES).
 
 Collected last on purpose (file name), so a run that stops at the first failure has already run every
 other test.  It needs nothing from the other tests and passes in a fresh process as well.
@@ -21,8 +22,8 @@ from tests.test_gpu_conv_layer import make_case
 pytestmark = pytest.mark.gpu
 
 # N, H, W, Cmax, C, Kmax, K, R, k, stride, act, residual
-SPLIT_CASE = (1, 7, 7, 720, 720, 720, 720, 3, 3, 1, 1, True)    # reduction split over several CTAs: uses the scratch
-PLAIN_CASE = (16, 14, 14, 360, 256, 1024, 824, 1, 1, 1, 1, True)  # fills the GPU unsplit: no scratch
+SPLIT_CASE = (1, 7, 7, 720, 720, 720, 720, 3, 3, 1, 1, True)    # reduction split over a cluster of CTAs
+PLAIN_CASE = (16, 14, 14, 360, 256, 1024, 824, 1, 1, 1, 1, True)  # fills the GPU unsplit
 
 
 def _desc(case):
@@ -48,20 +49,20 @@ def test_static_variant_matches_the_allocating_entry_point_twice(case):
     sgs.conv2d_sliced_static(desc, *args, outs[0].data_ptr(), stream)  # the first call on a device does the one-time set-up
     torch.cuda.synchronize()
     free_before = torch.cuda.mem_get_info()[0]
-    for i in (1, 2):  # the second call meets the array as the first one left it
+    for i in (1, 2):  # the second call meets the status word as the first one left it
         sgs.conv2d_sliced_static(desc, *args, outs[i].data_ptr(), stream)
         torch.cuda.synchronize()
         # no device memory was taken (the outputs were allocated before the measurement started)
         assert torch.cuda.mem_get_info()[0] == free_before
         got = outs[i].float().cpu().numpy()
-        assert sgs.device_status() == 0  # also reads the status word that lives inside the fixed array
+        assert sgs.device_status() == 0  # also reads the status word inside the library image
         assert np.all(np.isfinite(got))
         assert np.abs(got - want).max() <= tol
         assert np.abs(got - ref).max() <= tol
 
 
 def test_static_variant_rejects_what_it_cannot_hold():
-    # 128 pixels x 9216 filters split three ways: 13.5 MiB of fp32 partial sums, more than the fixed
+    # 128 pixels x 9216 filters split three ways: 13.5 MiB of fp32 partial sums, more than the declared
     # 8 MiB: refused, nothing launched
     big = (2, 8, 8, 128, 128, 9216, 9216, 3, 3, 1, 0, False)
     N, H, W, Cmax, C, Kmax, K, R, k, stride, act, _ = big
