@@ -8,7 +8,7 @@
 // conflict-free 4-byte read, unpacked once and used for all its taps in both rows; a weight is one 8-byte read (fp32, of the
 // block) and used for 2 TW outputs.  Warps meet only once, when the block's weights are in place.
 //
-// What bounds it: instruction issue (2.3 of 4 a cycle; half of them the packed multiply-adds and the unpacking of inputs,
+// What bounds it: instruction issue (2.2 of 4 a cycle; half of them the packed multiply-adds and the unpacking of inputs,
 // both at the rate of their pipes half the time).  Measured on 64x56x56x480, 5x5, stride 1, h-swish: 177 us against 228 us
 // of the kernel that it replaces, which kept weights in shared memory too but read 16 bytes of them for 4 packed
 // multiply-adds.  Slower forms of this one: a ring shared by the block (a barrier a step) 194 us; weights in registers
