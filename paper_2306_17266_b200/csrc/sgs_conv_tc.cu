@@ -83,7 +83,7 @@ __device__ __noinline__ void requantise_wide(const TcParams &p, QuantWide &t, ui
         if (p.res) {
             const uint32_t rb = ((j < 4 ? rq.x : rq.y) >> (8 * (j & 3))) & 0xffu;
             const int r8 = p.q_flags & 4 ? (int)(signed char)rb : (int)rb;
-            v += rshift_round((long long)(r8 - p.q_zr) * (long long)p.q_res_mult, 31 + p.q_res_shift);
+            v += rshift_round(((long long)r8 - p.q_zr) * (long long)p.q_res_mult, 31 + p.q_res_shift);
         }
         v += p.q_zy;
         t.acc[j] = (int)(v < -2147483647ll ? -2147483647ll : (v > 2147483647ll ? 2147483647ll : v));
@@ -236,7 +236,8 @@ __global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_con
     int bias[I8 ? 8 : 1];
     // 8-bit layers: the requantised sums of this thread's filters fit 32 bits (shifts of 33 and more, which every scale below
     // a quarter has, and terms within 2^28); 64-bit arithmetic otherwise.
-    bool q_narrow = I8 && abs(p.q_zy) < (1 << 28) && abs(p.q_zr) < (1 << 28) && p.q_res_shift >= 0;
+    // (unsigned: the magnitude of the lowest integer is 2^31)
+    bool q_narrow = I8 && (unsigned)abs(p.q_zy) < (1u << 28) && (unsigned)abs(p.q_zr) < (1u << 28) && p.q_res_shift >= 0;
     auto load_residual = [&](int i0) {
 #pragma unroll
         for (int i = 0; i < BATCH; i++) {

@@ -70,10 +70,21 @@ def test_split_reduction_and_narrow_tiles(N, H, W, C, K, k, stride, residual):
     _close(y, ref.contiguous())
 
 
+# the ends of the 32-bit zero points: sums that only 64 bits hold
+@pytest.mark.parametrize("zy", [-2 ** 31, -2 ** 28, 2 ** 28, 2 ** 31 - 1])
+@pytest.mark.parametrize("relu", [False, True])
+def test_int8_zero_point_ranges(zy, relu):
+    _requantise(2, 4, False, False, 72, zy=zy, relu=relu)
+
+
 # shifts on both sides of what 32-bit requantisation takes, biases that only 64-bit sums hold, the widest shift
 @pytest.mark.parametrize("shift_lo,shift_hi,big_bias,residual,K", [(0, 2, False, True, 176), (2, 3, False, True, 176), (1, 4, True, False, 72),
                                                                    (2, 4, True, True, 136), (31, 32, False, False, 40)])
 def test_int8_requantisation_ranges(shift_lo, shift_hi, big_bias, residual, K):
+    _requantise(shift_lo, shift_hi, big_bias, residual, K)
+
+
+def _requantise(shift_lo, shift_hi, big_bias, residual, K, zy=100, relu=False):
     rng = np.random.default_rng(shift_lo + K)
     N, H, C = 2, 9, 64
     w = rng.integers(-2, 3, (K, C, 1, 1)).astype(np.int8)
@@ -84,12 +95,12 @@ def test_int8_requantisation_ranges(shift_lo, shift_hi, big_bias, residual, K):
     if big_bias:
         bias[::3] = rng.choice([-2 ** 31, -2 ** 29, 2 ** 29, 2 ** 31 - 1], bias[::3].shape).astype(np.int32)
     res = rng.integers(0, 256, (N, H, H, K)).astype(np.uint8) if residual else None
-    ref = oracle.layer_conv_i8(w, x, C, K, 1, 1, mult, shift, bias, zx=0, zy=100, relu=False, res=res, zr=128, res_mult=1932735283, res_shift=1,
+    ref = oracle.layer_conv_i8(w, x, C, K, 1, 1, mult, shift, bias, zx=0, zy=zy, relu=relu, res=res, zr=128, res_mult=1932735283, res_shift=1,
                                y_signed=False)
     dx, dw, dm, ds, db = (torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (x, w.transpose(0, 2, 3, 1), mult, shift, bias))
     dr = torch.from_numpy(res).cuda() if residual else None
     dy = torch.empty(ref.shape, dtype=torch.uint8, device="cuda")
-    desc = sgs.ConvI8Desc(N=N, H=H, W=H, C=C, K=K, Kmax=K, Cmax=C, R=1, k=1, stride=1, relu=0, zy=100, zr=128, res_mult=1932735283, res_shift=1)
+    desc = sgs.ConvI8Desc(N=N, H=H, W=H, C=C, K=K, Kmax=K, Cmax=C, R=1, k=1, stride=1, relu=int(relu), zy=zy, zr=128, res_mult=1932735283, res_shift=1)
     sgs.conv2d_sliced_i8(desc, dx.data_ptr(), dw.data_ptr(), dm.data_ptr(), ds.data_ptr(), db.data_ptr(), dr.data_ptr() if residual else 0,
                          dy.data_ptr(), _stream())
     torch.cuda.synchronize()
