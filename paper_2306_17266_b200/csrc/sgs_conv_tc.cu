@@ -166,11 +166,11 @@ __global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_con
             else tma_load_3d_if(on, sb, &p.tmW, fb, c0, tapw, f0);
         };
         // Stored weights do not depend on the previous layer: fill the first stages' weight halves before waiting for it, so
-        // that their latency overlaps the previous layer's tail.  A caller's weights may be what the previous kernel writes.
-        if (!p.early_weights) pdl_wait();
+        // that their latency overlaps the previous layer's tail.  A caller's weights may be what the previous kernel writes:
+        // they go with the pixels, stage by stage.
+        const int pre = p.early_weights ? min(n_it, stages) : 0;
         {
             int cc2 = cc, r2 = r, sx2 = sx;
-            const int pre = min(n_it, stages);
             for (int i = 0; i < pre; i++) {
                 load_weights(i, cc2 * CH, (p.o + r2) * p.R + (p.o + sx2));
                 if (++cc2 == p.cchunks) { cc2 = 0; if (++sx2 == p.k) { sx2 = 0; ++r2; } }
@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_con
             const int c0 = cc * CH;
             const uint32_t sa = ring + (uint32_t)(s * STAGE_BYTES), fb = full0 + (uint32_t)(s * 8);
             const int dh = r - p.p, dw = sx - p.p;
-            if (i >= stages) load_weights(s, c0, (p.o + r) * p.R + (p.o + sx));
+            if (i >= pre) load_weights(s, c0, (p.o + r) * p.R + (p.o + sx));
             if (p.stride == 1) {
                 tma_load_4d_if(on, sa, &p.tmA[0], fb, c0, w0 + dw, h0 + dh, n0);
             } else {
