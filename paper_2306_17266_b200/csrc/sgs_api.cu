@@ -275,7 +275,11 @@ struct StreamScope {
 // Calls that synchronise the stream cannot be captured; they refuse before anything joins the capture.
 bool being_captured(cudaStream_t st) {
     cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
-    return cudaStreamIsCapturing(st, &s) == cudaSuccess && s != cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &s) != cudaSuccess) {  // (the legacy stream while another stream is captured)
+        cudaGetLastError();
+        return false;
+    }
+    return s != cudaStreamCaptureStatusNone;
 }
 
 sgs_status_t fail(const sgs_supernet *n, sgs_status_t st, const std::string &msg) {
