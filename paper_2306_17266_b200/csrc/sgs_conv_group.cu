@@ -23,7 +23,7 @@ namespace {
 
 constexpr int G_MAX_STAGES = 8;
 constexpr int G_X_BYTES = 128 * CHUNK_C * 2;  // operand on the MMA's row side: 128 rows
-constexpr int G_RING_BYTES = 192 * 1024;      // operand ring: 8 stages of 16 + 8 KB (tiles of at most 64 columns), 6 of 16 + 16 KB, or 4 of 16 + 32 KB (256-column tiles)
+constexpr int G_RING_BYTES = 192 * 1024;      // operand ring: 4 stages of 16 + 32 KB (256-column tiles) to 8 of 16 + 8 KB
 constexpr int G_ACC_COLS = 256;                   // tensor-memory columns of one accumulator buffer
 constexpr int G_EPI_WARPS = 8;                    // two per tensor-memory lane quadrant
 constexpr int G_EPI_PITCH = 36;                   // floats per staged row of 32 columns: 8 consecutive rows lie in 8 different groups of 4 banks
@@ -33,7 +33,7 @@ constexpr int G_THREADS = 64 + 32 * G_EPI_WARPS + 32;  // weight producer, MMA w
 constexpr int G_PIX_WARP = 2 + G_EPI_WARPS;
 
 // One member (query) of a grouped launch.
-//   normal  : MMA rows = a box of <= 128 output pixels, MMA columns = bn_tile (64 / 128 / 256) filters
+//   normal  : MMA rows = a box of <= 128 output pixels, MMA columns = bn_tile filters (a multiple of 16, at most 256)
 //   swapped : MMA rows = 128 filters, MMA columns = ALL output pixels of the member (<= 256, padded to 16)
 struct __align__(16) GroupEntry {
     const float *scale, *shift;
@@ -433,7 +433,7 @@ static int views_of(const TcParams &p) { return (p.stride == 2 && p.k > 1) ? 4 :
 struct GroupLaunch::Impl {
     GroupParams<TC_GROUP_MAPS_LARGE> prm;  // host image of the parameter block (the small variant is a prefix)
     int n_maps = 0;
-    int col_rows = 0;   // most rows any member's column-side operand has (64, 128 or 256: sizes the stages)
+    int col_rows = 0;   // most rows any member's column-side operand has (sizes the stages)
     const void *win_base = nullptr;  // largest cached filter prefix among the members' stored layers
     size_t win_bytes = 0;
 };
@@ -530,9 +530,8 @@ cudaError_t GroupLaunch::launch(size_t window_max, int sms, cudaStream_t st) {
     impl->prm.status = tc_status_word(dev);
     if (!impl->prm.status) return cudaErrorInitializationError;
     // stage = 16 KB for the row-side operand + room for the widest column-side operand of the launch
-    const int col_rows = impl->col_rows <= 64 ? 64 : impl->col_rows <= 128 ? 128 : 256;
-    impl->prm.stage_bytes = G_X_BYTES + col_rows * CHUNK_C * 2;
-    impl->prm.n_stages = G_RING_BYTES / impl->prm.stage_bytes;  // 8, 6 or 4
+    impl->prm.stage_bytes = G_X_BYTES + (impl->col_rows + 15) / 16 * 16 * CHUNK_C * 2;
+    impl->prm.n_stages = std::min(G_MAX_STAGES, G_RING_BYTES / impl->prm.stage_bytes);  // 4 (256 columns) to 8
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)std::min(impl->prm.total_tiles, std::max(1, sms)));
     cfg.blockDim = dim3(G_THREADS);

@@ -711,10 +711,12 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
         max_splits = p.iters >= 32 ? std::min(4, p.iters / 8) : 1;
     }
     if (a.throughput == 2) {
-        // grouped launch: no split; filter tile = the narrowest of 64 / 128 / 256 that holds the layer
-        // (256 at most), or 128 filters on the MMA's row side when swapped
+        // grouped launch: no split; as few filter tiles as 256 columns allow, all of about the same width and no wider than
+        // that (a box row that holds no filter costs the copy unit what a filter costs: 4 queries x 16 images of 224x224 with
+        // tiles of 64, 128 or 256 filters 15060 us, with these 14850), or 128 filters on the MMA's row side when swapped
         max_splits = 1;
-        BN = swap ? 128 : a.K <= 64 ? 64 : a.K <= 128 ? 128 : 256;
+        const int nt = (a.K + 255) / 256;
+        BN = swap ? 128 : ((a.K + nt - 1) / nt + 15) / 16 * 16;
     }
     if (a.no_split) max_splits = 1;
     plan->bn_tile = BN;
