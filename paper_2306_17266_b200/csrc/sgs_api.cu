@@ -195,8 +195,12 @@ struct sgs_supernet {
         float *stage_out = nullptr;
         cudaStream_t st = nullptr;  // internal stream (slots >= 1)
         cudaEvent_t ev = nullptr;
+        int chunk_index = 0, chunk_slots = 0;  // position among the slots whose activation buffers are one allocation
     };
     std::vector<Slot> slots;
+    // Activation buffers of slots that were made together are one allocation, slot by slot at a fixed distance, so that a tensor
+    // map can show the same buffer of all of them (the slot is a coordinate; see ConvArgs::slot).
+    std::vector<std::pair<void *, size_t>> act_chunks;
     // Wave execution (many queries advance through the layers together, one grouped launch per layer):
     // each wave in flight has its own stream, launch-table buffers and staging buffers.
     struct WaveCtx {
@@ -634,32 +638,63 @@ sgs_status_t build_plan(sgs_supernet *net, const sgs_subnet_cfg_t *cfg, int batc
     return SGS_OK;
 }
 
-// Frees the activation / vector buffers of a slot (the sizes are the handle's current ones).
-void release_slot_buffers(sgs_supernet *net, sgs_supernet::Slot &sl, bool act, bool vec) {
-    for (int i = 0; i < 4 && act; i++) { dev_free(net, sl.act[i], net->act_elems * net->elem() + 256); sl.act[i] = nullptr; }
-    for (int i = 0; i < 3 && vec; i++) { dev_free(net, sl.vec[i], net->vec_elems * 4); sl.vec[i] = nullptr; }
+size_t act_buffer_bytes(const sgs_supernet *net) { return (net->act_elems * net->elem() + 256 + 255) / 256 * 256; }
+
+// Frees the vector buffers of a slot (the size is the handle's current one).
+void release_slot_vectors(sgs_supernet *net, sgs_supernet::Slot &sl) {
+    for (int i = 0; i < 3; i++) { dev_free(net, sl.vec[i], net->vec_elems * 4); sl.vec[i] = nullptr; }
+}
+// Frees the activation buffers of all slots.
+void release_activations(sgs_supernet *net) {
+    for (auto &c : net->act_chunks) dev_free(net, c.first, c.second);
+    net->act_chunks.clear();
+    for (auto &sl : net->slots) {
+        for (void *&p : sl.act) p = nullptr;
+        sl.chunk_index = sl.chunk_slots = 0;
+    }
+}
+// Gives the slots [first, end) activation buffers of the current size, in one allocation.
+sgs_status_t allocate_activations(sgs_supernet *net, std::vector<sgs_supernet::Slot> &slots, size_t first) {
+    const size_t n = slots.size() - first, each = act_buffer_bytes(net);
+    if (!net->act_elems || !n) return SGS_OK;
+    void *base = nullptr;
+    net->act_chunks.reserve(net->act_chunks.size() + 1);
+    sgs_status_t st = dev_alloc(net, &base, n * 4 * each);
+    if (st != SGS_OK) return st;
+    net->act_chunks.emplace_back(base, n * 4 * each);
+    for (size_t i = 0; i < n; i++) {
+        sgs_supernet::Slot &sl = slots[first + i];
+        sl.chunk_index = (int)i; sl.chunk_slots = (int)n;
+        for (int j = 0; j < 4; j++) sl.act[j] = static_cast<char *>(base) + (4 * i + j) * each;
+    }
+    return SGS_OK;
 }
 
 // Makes sure `n_slots` slots exist, each with buffers for the sizes in use.
 sgs_status_t ensure_slots(sgs_supernet *net, int n_slots) {
-    net->slots.reserve((size_t)std::max(n_slots, 0));
-    while ((int)net->slots.size() < n_slots) {
-        sgs_supernet::Slot sl;
-        if (!net->slots.empty()) {
-            CU(cudaStreamCreateWithFlags(&sl.st, cudaStreamNonBlocking));
-            CU(cudaEventCreateWithFlags(&sl.ev, cudaEventDisableTiming));
-        }
-        sgs_status_t st = SGS_OK;
-        for (int i = 0; i < 4 && net->act_elems && st == SGS_OK; i++) st = dev_alloc(net, &sl.act[i], net->act_elems * net->elem() + 256);
+    if ((int)net->slots.size() >= n_slots) return SGS_OK;
+    net->slots.reserve((size_t)n_slots);
+    std::vector<sgs_supernet::Slot> fresh;
+    fresh.reserve((size_t)n_slots - net->slots.size());
+    sgs_status_t st = SGS_OK;
+    while (st == SGS_OK && (int)(net->slots.size() + fresh.size()) < n_slots) {
+        fresh.emplace_back();
+        sgs_supernet::Slot &sl = fresh.back();
+        if (net->slots.size() + fresh.size() > 1 && (cudaStreamCreateWithFlags(&sl.st, cudaStreamNonBlocking) != cudaSuccess ||
+                                                     cudaEventCreateWithFlags(&sl.ev, cudaEventDisableTiming) != cudaSuccess))
+            st = fail(net, SGS_ECUDA, "stream of a slot");
         for (int i = 0; i < 3 && net->vec_elems && st == SGS_OK; i++) st = dev_alloc(net, (void **)&sl.vec[i], net->vec_elems * 4);
-        if (st != SGS_OK) {  // nothing of a half-built slot stays behind
-            release_slot_buffers(net, sl, true, true);
+    }
+    if (st == SGS_OK) st = allocate_activations(net, fresh, 0);
+    if (st != SGS_OK) {  // nothing of half-built slots stays behind
+        for (auto &sl : fresh) {
+            release_slot_vectors(net, sl);
             if (sl.st) cudaStreamDestroy(sl.st);
             if (sl.ev) cudaEventDestroy(sl.ev);
-            return st;
         }
-        net->slots.push_back(sl);
+        return st;
     }
+    net->slots.insert(net->slots.end(), fresh.begin(), fresh.end());
     return SGS_OK;
 }
 
@@ -671,13 +706,10 @@ sgs_status_t ensure_workspace(sgs_supernet *net, size_t act_elems, int batch) {
     if (act_elems > net->act_elems) {
         drop_graphs(net);
         for (auto &kv : net->plans) kv.second->prepared = false;
-        for (auto &sl : net->slots) release_slot_buffers(net, sl, true, false);
+        release_activations(net);
         net->act_elems = act_elems;
-        sgs_status_t st = SGS_OK;
-        for (auto &sl : net->slots)
-            for (int i = 0; i < 4 && st == SGS_OK; i++) st = dev_alloc(net, &sl.act[i], act_elems * net->elem() + 256);
+        sgs_status_t st = allocate_activations(net, net->slots, 0);
         if (st != SGS_OK) {
-            for (auto &sl : net->slots) release_slot_buffers(net, sl, true, false);
             net->act_elems = 0;
             return st;
         }
@@ -685,13 +717,13 @@ sgs_status_t ensure_workspace(sgs_supernet *net, size_t act_elems, int batch) {
     size_t vneed = (size_t)batch * 2048;
     if (vneed > net->vec_elems) {
         drop_graphs(net);
-        for (auto &sl : net->slots) release_slot_buffers(net, sl, false, true);
+        for (auto &sl : net->slots) release_slot_vectors(net, sl);
         net->vec_elems = vneed;
         sgs_status_t st = SGS_OK;
         for (auto &sl : net->slots)
             for (int i = 0; i < 3 && st == SGS_OK; i++) st = dev_alloc(net, (void **)&sl.vec[i], vneed * 4);
         if (st != SGS_OK) {
-            for (auto &sl : net->slots) release_slot_buffers(net, sl, false, true);
+            for (auto &sl : net->slots) release_slot_vectors(net, sl);
             net->vec_elems = 0;
             return st;
         }
@@ -708,6 +740,8 @@ sgs_status_t choose_impls(sgs_supernet *net, Plan *plan) {
         op.conv.x = op.in >= 0 ? sl.act[op.in] : nullptr;
         op.conv.y = sl.act[op.out];
         op.conv.res = op.res >= 0 ? sl.act[op.res] : nullptr;
+        op.conv.layer = op.layer;
+        op.conv.slot = sl.chunk_index; op.conv.slots = sl.chunk_slots; op.conv.slot_bytes = 4 * act_buffer_bytes(net);
         op.impl = 0;
         op.tc.reset();
         op.conv.throughput = plan->throughput;
@@ -1357,8 +1391,8 @@ void sgs_supernet_free(sgs_supernet_t *net) {
     cudaFree(net->param_arena);
     cudaFree(net->stem_gemm_w);
     cudaFree(net->stem_win_w);
+    for (auto &c : net->act_chunks) cudaFree(c.first);
     for (auto &sl : net->slots) {
-        for (int i = 0; i < 4; i++) cudaFree(sl.act[i]);
         for (int i = 0; i < 3; i++) cudaFree(sl.vec[i]);
         cudaFree(sl.stage_in);
         cudaFree(sl.stage_out);
@@ -1554,11 +1588,10 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
         // persisting L2 lines of SubGraphs that are no longer cached go back to normal replacement
         if (net->cache.enabled && net->cache_mech != 0 && net->cache.epoch != epoch_at_issue) cudaCtxResetPersistingL2Cache();
         const int box_policy = !net->cache.enabled ? (net->cache.evict_first_when_off ? 2 : 0) : (net->cache_mech == 1 ? 3 : 1);
-        auto set_box = [&](ConvArgs &a, int member, int layer) {
-            a.weight_policy = box_policy; a.cacheK = a.cacheC = 0;
+        auto add_member = [&](GroupLaunch *g, char *entry, const Op &op, int member) {
             const std::vector<int> &G = *boxes[(size_t)member];
-            if ((box_policy == 1 || box_policy == 3) && !G.empty()) { a.cacheK = G[3 * (size_t)layer]; a.cacheC = G[3 * (size_t)layer + 1]; }
-            else if (box_policy == 1 || box_policy == 3) a.weight_policy = 0;
+            const bool boxed = (box_policy == 1 || box_policy == 3) && !G.empty();
+            g->add(entry, *op.tc, op.conv, boxed || box_policy == 2 ? box_policy : 0, boxed ? G[3 * (size_t)op.layer] : 0, boxed ? G[3 * (size_t)op.layer + 1] : 0);
         };
         // merge the members' op lists by rank
         for (auto &b : buckets) b.clear();
@@ -1603,21 +1636,23 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
             {
                 const Op &o0 = plans[b[0].first]->ops[(size_t)b[0].second];
                 if (o0.type == OP_CONV && o0.impl == 1 && (long long)o0.conv.N * o0.conv.Ho * o0.conv.Wo <= 64 && b.size() > 2) {
-                    auto opof = [&](const std::pair<int, int> &mo) -> const Op & { return plans[mo.first]->ops[(size_t)mo.second]; };
-                    std::stable_sort(order.begin(), order.end(), [&](const std::pair<int, int> &x, const std::pair<int, int> &y) {
-                        const ConvArgs &cx_ = opof(x).conv, &cy_ = opof(y).conv;
-                        return cx_.K != cy_.K ? cx_.K > cy_.K : cx_.C > cy_.C;
-                    });
+                    struct Item { int K, C; std::pair<int, int> mo; };
+                    std::vector<Item> items;
+                    for (const auto &mo : order) {
+                        const ConvArgs &a = plans[mo.first]->ops[(size_t)mo.second].conv;
+                        items.push_back({a.K, a.C, mo});
+                    }
+                    std::stable_sort(items.begin(), items.end(), [](const Item &x, const Item &y) { return x.K != y.K ? x.K > y.K : x.C > y.C; });
                     std::vector<std::pair<int, int>> placed;
-                    std::vector<char> used_m(order.size(), 0);
-                    for (size_t i = 0; i < order.size(); i++) {
+                    std::vector<char> used_m(items.size(), 0);
+                    for (size_t i = 0; i < items.size(); i++) {
                         if (used_m[i]) continue;
                         used_m[i] = 1;
-                        placed.push_back(order[i]);
-                        for (size_t j = i + 1; j < order.size(); j++) {
-                            if (used_m[j] || opof(order[j]).conv.C > opof(order[i]).conv.C) continue;
+                        placed.push_back(items[i].mo);
+                        for (size_t j = i + 1; j < items.size(); j++) {
+                            if (used_m[j] || items[j].C > items[i].C) continue;
                             used_m[j] = 1;
-                            placed.push_back(order[j]);
+                            placed.push_back(items[j].mo);
                             break;
                         }
                     }
@@ -1629,10 +1664,7 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
                 const Op &op = pl->ops[(size_t)mo.second];
                 if (op.type != OP_CONV || op.impl != 1) continue;  // launched per member below
                 if (!g || !g->fits(*op.tc)) { g = next_group(); launches.push_back({r, g, -1, 0, 0}); }
-                ConvArgs a = op.conv;
-                a.layer = op.layer;
-                set_box(a, mo.first, op.layer);
-                g->add(cx.h_tbl + off, *op.tc, a);
+                add_member(g, cx.h_tbl + off, op, mo.first);
                 off += TC_GROUP_ENTRY_BYTES;
             }
             // Two consecutive convolution layers that do not depend on each other (a block's projection
@@ -1649,29 +1681,26 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
                         return true;
                     };
                     const auto &b2 = buckets[(size_t)r2];
-                    bool ok = all_tc(b) && all_tc(b2) && g->members() + (int)b2.size() <= TC_GROUP_MAX_ENTRIES;
+                    bool ok = g->members() + (int)b2.size() <= TC_GROUP_MAX_ENTRIES;
+                    size_t i1 = 0;  // (both buckets list their members in ascending order)
                     for (const auto &m2 : b2) {
-                        if (!ok) break;
-                        const Op &o2 = plans[m2.first]->ops[(size_t)m2.second];
-                        for (const auto &m1 : b) {
-                            if (m1.first != m2.first) continue;
-                            const Op &o1 = plans[m1.first]->ops[(size_t)m1.second];
-                            // same member: no read-after-write, write-after-read or write-after-write between them
-                            if (o2.in == o1.out || o2.res == o1.out || o2.out == o1.out || o2.out == o1.in || (o1.res >= 0 && o2.out == o1.res)) ok = false;
-                        }
+                        while (ok && i1 < b.size() && b[i1].first < m2.first) i1++;
+                        if (!ok || i1 >= b.size()) break;
+                        if (b[i1].first != m2.first) continue;
+                        const Op &o1 = plans[m2.first]->ops[(size_t)b[i1].second], &o2 = plans[m2.first]->ops[(size_t)m2.second];
+                        // same member: no read-after-write, write-after-read or write-after-write between them
+                        ok = !(o2.in == o1.out || o2.res == o1.out || o2.out == o1.out || o2.out == o1.in || (o1.res >= 0 && o2.out == o1.res));
                     }
+                    ok = ok && all_tc(b) && all_tc(b2);
                     if (ok) {
-                        // (fits() also bounds the tensor maps; checked entry by entry, undone as a whole is not
-                        // possible, so test the worst case first: 5 maps per member)
-                        ok = g->members() + (int)b2.size() <= TC_GROUP_MAX_ENTRIES && g->maps() + 5 * (int)b2.size() <= TC_GROUP_MAPS_LARGE;
+                        int need = g->maps();
+                        for (const auto &mo : b2) need += g->maps_for(*plans[mo.first]->ops[(size_t)mo.second].tc);
+                        ok = need <= TC_GROUP_MAPS_LARGE;
                     }
                     if (ok) {
                         for (const auto &mo : b2) {
                             const Op &op = plans[mo.first]->ops[(size_t)mo.second];
-                            ConvArgs a = op.conv;
-                            a.layer = op.layer;
-                            set_box(a, mo.first, op.layer);
-                            g->add(cx.h_tbl + off, *op.tc, a);
+                            add_member(g, cx.h_tbl + off, op, mo.first);
                             off += TC_GROUP_ENTRY_BYTES;
                         }
                         launches.back().rank2 = r2;
@@ -1769,6 +1798,7 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
         };
         auto bucket_cost = [&](int rank, bool tc, double *bytes, double *fl) {
             *bytes = 0; *fl = 0;
+            if (!net->profile) return;
             for (const auto &mo : buckets[(size_t)rank]) {
                 const Op &op = plans[mo.first]->ops[(size_t)mo.second];
                 if ((op.type == OP_CONV && op.impl == 1) != tc) continue;

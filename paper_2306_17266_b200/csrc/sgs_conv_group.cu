@@ -5,9 +5,9 @@
 // form one list of tiles; persistent CTAs (one per SM) walk that list with a fixed stride.
 //
 // Per CTA: warp 0 = weight producer, warp 10 = activation producer, warp 1 = MMA issuer, warps 2..9 =
-// epilogue.  The shared-memory ring of operand stages runs on across tiles, and the fp32 accumulator in tensor memory
-// is double buffered (2 x 256 columns), so the epilogue of a tile (tensor memory -> folded batch norm -> residual ->
-// activation -> bf16 NHWC) overlaps the loads and MMAs of the tiles that follow.
+// epilogue, warp 11 = residual loads and output stores.  The shared-memory ring of operand stages runs on across tiles, and
+// the fp32 accumulator in tensor memory is double buffered (2 x 256 columns), so the epilogue of a tile (tensor memory ->
+// folded batch norm -> residual -> activation -> bf16 NHWC) overlaps the loads and MMAs of the tiles that follow.
 //
 // The arithmetic of one tile is that of conv_tc_kernel (sgs_conv_tc.cu): implicit GEMM with
 // 128 output pixels x up to 256 filters, 64 channels per stage, slicing through the tensor maps'
@@ -23,14 +23,16 @@ namespace {
 
 constexpr int G_MAX_STAGES = 8;
 constexpr int G_X_BYTES = 128 * CHUNK_C * 2;  // operand on the MMA's row side: 128 rows
-constexpr int G_RING_BYTES = 192 * 1024;      // operand ring: 4 stages of 16 + 32 KB (256-column tiles) to 8 of 16 + 8 KB
-constexpr int G_ACC_COLS = 256;                   // tensor-memory columns of one accumulator buffer
-constexpr int G_EPI_WARPS = 8;                    // two per tensor-memory lane quadrant
-constexpr int G_EPI_PITCH = 36;                   // floats per staged row of 32 columns: 8 consecutive rows lie in 8 different groups of 4 banks
-constexpr int G_EPI_FLOATS = 16 * G_EPI_PITCH;    // a warp's staging area: 16 rows
-constexpr int G_SMEM_BYTES = 1024 + G_RING_BYTES + G_EPI_WARPS * G_EPI_FLOATS * 4;
-constexpr int G_THREADS = 64 + 32 * G_EPI_WARPS + 32;  // weight producer, MMA warp, epilogue warps, pixel producer
-constexpr int G_PIX_WARP = 2 + G_EPI_WARPS;
+constexpr int G_ACC_COLS = 256;               // tensor-memory columns of one accumulator buffer
+constexpr int G_EPI_WARPS = 8;                // two per tensor-memory lane quadrant
+constexpr int G_BUF_BYTES = 128 * 128;        // one block of an output tile: 128 pixels x 64 filters, bf16
+constexpr int G_MAX_BUFS = 6;
+constexpr int G_RECORDS = 128;                // tiles of a CTA whose records are worked out ahead
+constexpr int G_POOL_BYTES = 208 * 1024;      // operand stages and output blocks together (GroupLaunch::launch divides it)
+constexpr int G_BN_FLOATS = 128;              // folded batch norm of a warp's block: 64 scales, 64 shifts
+constexpr int G_SMEM_BYTES = 1024 + G_POOL_BYTES + G_EPI_WARPS * G_BN_FLOATS * 4;
+constexpr int G_THREADS = 64 + 32 * G_EPI_WARPS + 64;  // weight producer, MMA warp, epilogue warps, pixel producer, output warp
+constexpr int G_PIX_WARP = 2 + G_EPI_WARPS, G_OUT_WARP = G_PIX_WARP + 1;
 
 // One member (query) of a grouped launch.
 //   normal  : MMA rows = a box of <= 128 output pixels, MMA columns = bn_tile filters (a multiple of 16, at most 256)
@@ -43,13 +45,16 @@ struct __align__(16) GroupEntry {
                              // larger than 1x1: the parity views; else 1) and the sliced weight view
     int tile_begin;          // index of this member's first tile in the launch's tile list
     int mtiles;              // pixel tiles of this member (tile = filter tile * mtiles + pixel tile)
-    int N, Ho, Wo, K, C;
+    int K, C;
+    int slot_h, slot_n;      // added to the pixel coordinates: the member's place in maps that show several slots
+    int pad1_;
     int R, tap0;             // stored kernel size; tap index of the cropped kernel's first tap
     int tiles_w, tiles_hw, cchunks, layer;
     short bw, bh, bn;        // pixel box
     short bn_tile;           // MMA columns of a full tile
     short pix_rows;          // rows of the pixel box (bw * bh * bn)
-    short pad0_[3];
+    short map_y, map_r;      // output and residual views (not of swapped members)
+    short can_pair;          // (host) one tile of at most 64 pixels, square kernel: may share a tile, see below
     unsigned char k, stride, p, act, swap, kw;  // k x kw taps
     // Two members with at most 64 output pixels each can share a tile: the first ("pair") owns the tile's
     // geometry, filters and weight map and takes MMA rows 0..63, the entry after it ("second") takes rows
@@ -63,16 +68,67 @@ struct __align__(16) GroupEntry {
 };
 static_assert(sizeof(GroupEntry) == TC_GROUP_ENTRY_BYTES, "entry size");
 
-// Index of the entry that owns tile t's geometry (the first member of a pair); the whole warp calls it.  begin[]: the entries'
-// first tiles, sorted, INT_MAX beyond the last (an array of its own: read out of the 128-byte records, the 32 lanes' words
-// would lie in one bank).
-__device__ __forceinline__ int tile_entry(const GroupEntry *es, const int *begin, int t, int lane) {
-    const unsigned b0 = __ballot_sync(0xffffffffu, begin[lane] <= t), b1 = __ballot_sync(0xffffffffu, begin[lane + 32] <= t);
-    const int i = __popc(b0) + __popc(b1) - 1;
-    return es[i].second ? i - 1 : i;
+// A tile of the launch's list: x = entry that owns its geometry (the first member of a pair) in the low 8 bits, first filter
+// above; y, z, w = first column, row and image of its pixels.  begin[]: the entries' first tiles, sorted, INT_MAX beyond the
+// last (an array of its own: read out of the 128-byte records, the lanes' words would lie in one bank).
+__device__ __forceinline__ int4 tile_record(const GroupEntry *es, const int *begin, int t) {
+    int i = 0;
+#pragma unroll
+    for (int step = TC_GROUP_MAX_ENTRIES / 2; step; step >>= 1)
+        if (begin[i + step] <= t) i += step;
+    if (es[i].second) i--;
+    const GroupEntry &e = es[i];
+    const int lt = t - e.tile_begin, nt = lt / e.mtiles;
+    if (e.swap) return make_int4(i | nt * 128 << 8, 0, e.slot_h, e.slot_n);
+    const int mt = lt - nt * e.mtiles, n = mt / e.tiles_hw, mhw = mt - n * e.tiles_hw, h = mhw / e.tiles_w;
+    return make_int4(i | nt * e.bn_tile << 8, (mhw - h * e.tiles_w) * e.bw, h * e.bh + e.slot_h, n * e.bn + e.slot_n);
 }
+static_assert(TC_GROUP_MAX_ENTRIES <= 256 && (TC_GROUP_MAX_ENTRIES & (TC_GROUP_MAX_ENTRIES - 1)) == 0, "entry index");
+
+// First filter, within its tile, of a tile's last block of 64: where another tile follows, the block ends with the tile (and
+// repeats some filters of the one before it); a layer's last block may reach beyond the tensor, the copy unit clips it.
+__device__ __forceinline__ int last_block(const GroupEntry &e, int f0) { return f0 + e.bn_tile < e.ldk ? e.bn_tile - 64 : 256; }
 
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap *m) { asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory"); }
+
+// 64 filters of a lane's pixel: accumulator v -> folded batch norm (bn: 64 scales, 64 shifts, the same in all lanes) -> residual
+// (RES: in the pixel's row of the block's buffer) -> activation -> bf16, into that row.  Filters from `left` on are zeros.
+template <bool RES, bool HS>
+__device__ __forceinline__ void finish_block(const uint32_t *v, const float *bn, uint32_t row, uint32_t swz, int left, __nv_bfloat162 lo) {
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+        uint4 rv[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) rv[q] = RES ? lds128(row + (((uint32_t)(4 * h + q) ^ swz) << 4)) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const int c = 32 * h + 8 * q;
+            float2 o[4];
+#pragma unroll
+            for (int i = 0; i < 2; i++) {
+                const float4 sc = *reinterpret_cast<const float4 *>(bn + c + 4 * i), sh = *reinterpret_cast<const float4 *>(bn + 64 + c + 4 * i);
+                const uint32_t *vi = v + c + 4 * i;
+                o[2 * i] = __ffma2_rn(make_float2(__uint_as_float(vi[0]), __uint_as_float(vi[1])), make_float2(sc.x, sc.y), make_float2(sh.x, sh.y));
+                o[2 * i + 1] = __ffma2_rn(make_float2(__uint_as_float(vi[2]), __uint_as_float(vi[3])), make_float2(sc.z, sc.w), make_float2(sh.z, sh.w));
+            }
+            if (RES) {
+                const uint32_t r4[4] = {rv[q].x, rv[q].y, rv[q].z, rv[q].w};
+#pragma unroll
+                for (int i = 0; i < 4; i++) o[i] = __fadd2_rn(o[i], make_float2(__uint_as_float(r4[i] << 16), __uint_as_float(r4[i] & 0xffff0000u)));
+            }
+            uint4 out;
+            __nv_bfloat162 *ob = reinterpret_cast<__nv_bfloat162 *>(&out);
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                if (HS) { o[i].x = act_fn(o[i].x, ACT_HSWISH); o[i].y = act_fn(o[i].y, ACT_HSWISH); }
+                ob[i] = __float22bfloat162_rn(o[i]);
+                if (!HS) ob[i] = __hmax2(ob[i], lo);  // (of the rounded values: rounding keeps the order, zero stays zero)
+            }
+            if (c >= left) out = make_uint4(0u, 0u, 0u, 0u);
+            sts128(row + (((uint32_t)(4 * h + q) ^ swz) << 4), out);
+        }
+    }
+}
 
 // Kernel parameters.  The tensor maps travel in the parameter block (the TMA unit reads them from
 // there); the per-member records travel in a device table.
@@ -81,7 +137,8 @@ template <int NMAPS> struct GroupParams {
     int *status;
     int n_entries, total_tiles;
     int n_stages, stage_bytes;  // operand ring of this launch
-    int pad_[8];  // (tensor maps lie at multiples of 64 bytes)
+    int n_bufs;                 // blocks of output in flight: 1, or an even number (the two epilogue halves have their own)
+    int pad_[7];  // (tensor maps lie at multiples of 64 bytes)
     CUtensorMap maps[NMAPS];
 };
 static_assert(sizeof(GroupParams<TC_GROUP_MAPS_LARGE>) <= 32764, "kernel parameter block");
@@ -94,7 +151,9 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
     extern __shared__ uint8_t smem_raw[];
     __shared__ GroupEntry es[TC_GROUP_MAX_ENTRIES];
     __shared__ int begin[TC_GROUP_MAX_ENTRIES];
+    __shared__ int4 recs[G_RECORDS];
     __shared__ __align__(8) uint64_t full_bar[G_MAX_STAGES], empty_bar[G_MAX_STAGES], acc_full[2], acc_empty[2];
+    __shared__ __align__(8) uint64_t buf_ready[G_MAX_BUFS], buf_done[G_MAX_BUFS];
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s;
 
@@ -110,6 +169,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
     if (threadIdx.x == 0) {
         for (int s = 0; s < G_MAX_STAGES; s++) { mbar_init(&full_bar[s], 2); mbar_init(&empty_bar[s], 1); }  // (full: both producers arrive)
         for (int b = 0; b < 2; b++) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], G_EPI_WARPS); }
+        for (int b = 0; b < G_MAX_BUFS; b++) { mbar_init(&buf_ready[b], 1); mbar_init(&buf_done[b], G_EPI_WARPS / 2); }
         abort_s = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -117,12 +177,21 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    // The CTA's tiles, a thread each: look-up and divisions cost a role that does them tile by tile some 700 clocks.
+    for (int i = threadIdx.x, t = blockIdx.x + i * gridDim.x; i < G_RECORDS && t < total_tiles; i += blockDim.x, t += blockDim.x * gridDim.x)
+        recs[i] = tile_record(es, begin, t);
+    __syncthreads();
+    auto record = [&](int i) -> int4 { return i < G_RECORDS ? recs[i] : tile_record(es, begin, (int)(blockIdx.x + i * gridDim.x)); };  // of the CTA's i-th tile
+    const int n_tiles = (total_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
     const uint32_t tmem_base = tmem_base_s;
-    const int n_stages = P.n_stages, stage_bytes = P.stage_bytes;
-    pdl_launch_dependents();
+    const int n_stages = P.n_stages, stage_bytes = P.stage_bytes, n_bufs = P.n_bufs, n_bars = n_bufs > 1 ? n_bufs : G_MAX_BUFS;
+
+    // Launches with one output buffer (long reductions, no residual): the CTA's last tile puts its blocks where the operands were,
+    // which nobody needs any more when its accumulator is complete; no block waits for another's store there.
+    const bool tail_in_ring = n_bufs == 1;
 
     // The three issuing warps run their loops converged; the elected lane issues (see sgs_tc.cuh).
-    const uint32_t ring = smem_u32(smem), full0 = smem_u32(full_bar), empty0 = smem_u32(empty_bar);
+    const uint32_t ring = smem_u32(smem), bufs = ring + (uint32_t)(n_stages * stage_bytes), full0 = smem_u32(full_bar), empty0 = smem_u32(empty_bar);
     if (warp == 0) {
         // ------------------------------------------------------------------ weight producer
         // Weights do not depend on the previous layer, so this warp never waits for it: it runs ahead
@@ -132,11 +201,11 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
         int s = 0;
         uint32_t phase = 0;
         bool wrapped = false, ok = true;
-        for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x) {
-            const GroupEntry &e = es[tile_entry(es, begin, t, lane)];
-            const int nt = (t - e.tile_begin) / e.mtiles;
+        for (int j = 0; j < n_tiles && ok; j++) {
+            const int4 rec = record(j);
+            const GroupEntry &e = es[rec.x & 255];
             const int wrows = e.swap ? 128 : e.bn_tile;  // rows of the weight box
-            const int f0 = (int)uniform((uint32_t)(nt * wrows));
+            const int f0 = (int)uniform((uint32_t)(rec.x >> 8));
             const uint32_t w_bytes = uniform((uint32_t)(wrows * CHUNK_C * 2));
             const uint32_t dst0 = uniform(ring + (e.swap ? 0u : (uint32_t)G_X_BYTES));
             const CUtensorMap *map_w = &P.maps[uniform((uint32_t)e.map_w)];
@@ -158,11 +227,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
                     }
                 }
             }
-            const int tn = t + (int)gridDim.x;
-            if (ok && tn < total_tiles) {
-                const int en = tile_entry(es, begin, tn, lane);
-                if (on) prefetch_tensormap(&P.maps[es[en].map_w]);
-            }
+            if (ok && on && j + 1 < n_tiles) prefetch_tensormap(&P.maps[es[record(j + 1).x & 255].map_w]);
             __syncwarp();
         }
     } else if (warp == G_PIX_WARP) {
@@ -171,15 +236,17 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
         int s = 0;
         uint32_t phase = 0;
         bool wrapped = false, ok = true;
+        if (on) prefetch_tensormap(&P.maps[es[recs[0].x & 255].map_a]);
+        __syncwarp();
         pdl_wait();  // activations (and the buffers this layer overwrites) belong to the previous layers until here
-        for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x) {
-            const GroupEntry &e = es[tile_entry(es, begin, t, lane)];
-            const int lt = t - e.tile_begin, mt = lt - lt / e.mtiles * e.mtiles;
-            const int tn_ = mt / e.tiles_hw, mhw = mt - tn_ * e.tiles_hw, th_ = mhw / e.tiles_w, tw_ = mhw - th_ * e.tiles_w;
-            const int n0 = (int)uniform((uint32_t)(tn_ * e.bn)), h0 = (int)uniform((uint32_t)(th_ * e.bh)), w0 = (int)uniform((uint32_t)(tw_ * e.bw));
+        for (int j = 0; j < n_tiles && ok; j++) {
+            const int4 rec = record(j);
+            const GroupEntry &e = es[rec.x & 255];
+            const int n0 = (int)uniform((uint32_t)rec.w), h0 = (int)uniform((uint32_t)rec.z), w0 = (int)uniform((uint32_t)rec.y);
             const bool pair = uniform(e.pair) != 0;
             const uint32_t pix_bytes = uniform((uint32_t)(e.pix_rows * CHUNK_C * 2) + (pair ? (uint32_t)((&e)[1].pix_rows * CHUNK_C * 2) : 0u));
             const uint32_t dst0 = uniform(ring + (e.swap ? (uint32_t)G_X_BYTES : 0u));
+            const int dh2 = (int)uniform((uint32_t)(pair ? (&e)[1].slot_h - e.slot_h : 0)), dn2 = (int)uniform((uint32_t)(pair ? (&e)[1].slot_n - e.slot_n : 0));
             const int map_a = (int)uniform((uint32_t)e.map_a), map_a2 = (int)uniform((uint32_t)(pair ? (&e)[1].map_a : e.map_a));
             const int k = (int)uniform(e.k), kw = (int)uniform(e.kw), cchunks = (int)uniform((uint32_t)e.cchunks), pad = (int)uniform(e.p), stride = (int)uniform(e.stride);
             for (int r = 0; r < k && ok; r++) {
@@ -194,30 +261,29 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
                         mbar_expect_tx_if(on, fb, pix_bytes);
                         tma_load_4d_if(on, sb, &P.maps[map_a + view], fb, c0, cw, ch, n0);
                         // (a pair is a single tile of one layer: same tap offsets and parity view, box origin 0)
-                        if (pair) tma_load_4d_if(on, sb + 64 * CHUNK_C * 2, &P.maps[map_a2 + view], fb, c0, cw, ch, n0);
+                        if (pair) tma_load_4d_if(on, sb + 64 * CHUNK_C * 2, &P.maps[map_a2 + view], fb, c0, cw, ch + dh2, n0 + dn2);
                         if (++s == n_stages) { s = 0; phase ^= 1; wrapped = true; }
                     }
                 }
             }
-            const int tn = t + (int)gridDim.x;
-            if (ok && tn < total_tiles) {
-                const int en = tile_entry(es, begin, tn, lane);
-                if (on) prefetch_tensormap(&P.maps[es[en].map_a]);
-            }
+            if (ok && on && j + 1 < n_tiles) prefetch_tensormap(&P.maps[es[record(j + 1).x & 255].map_a]);
             __syncwarp();
         }
+        // The next launch's CTAs come when this one's have asked for their last operands.  Told earlier, they (and those of the
+        // launch after) sat on SMs that other waves could have used: 190 of 908 us of SM time a wave with four in flight, 71 now.
+        pdl_launch_dependents();
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
         const uint32_t on = elect_one(), acc_base = uniform(tmem_base);
-        int s = 0, j = 0;
+        int s = 0;
         uint32_t phase = 0;
         bool ok = true;
-        for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x, j++) {
-            const GroupEntry &e = es[tile_entry(es, begin, t, lane)];
-            const int nt = (t - e.tile_begin) / e.mtiles;
+        for (int j = 0; j < n_tiles && ok; j++) {
+            const int4 rec = record(j);
+            const GroupEntry &e = es[rec.x & 255];
             // MMA shape: 128 rows; columns = this tile's filters (normal) or the member's pixels (swapped),
             // rounded up to 16; bf16 x bf16 -> fp32, both operands K-major
-            const int n_mma = e.swap ? e.bn_tile : min((int)e.bn_tile, (e.K - nt * e.bn_tile + 15) & ~15);
+            const int n_mma = e.swap ? e.bn_tile : min((int)e.bn_tile, (e.K - (rec.x >> 8) + 15) & ~15);
             const uint32_t idesc = uniform((1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n_mma >> 3) << 17) | ((uint32_t)(TILE_M >> 4) << 24));
             const int buf = j & 1;
             const int cchunks = (int)uniform((uint32_t)e.cchunks), iters = (int)uniform((uint32_t)(e.k * e.kw)) * cchunks;
@@ -242,154 +308,184 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
                 if (++s == n_stages) { s = 0; phase ^= 1; }
             }
         }
+    } else if (warp == G_OUT_WARP) {
+        // ------------------------------------------------------------------ residual loads and output stores
+        // Blocks (128 pixels x 64 filters) of the CTA's tiles are numbered through; block g lies in buffer g % n_bufs and has the
+        // barriers g % n_bars (an even number: a half of the epilogue sees every phase of its own barriers).  For each
+        // this warp makes the buffer ready (fetches the residual into it, or only says that it is free) and, when the epilogue
+        // has put the results in the residual's place, stores it.
+        const uint32_t on = elect_one();
+        const int lag = n_bufs >= 4 ? 1 : 0;  // stores that may still be reading their buffer when the next one is made ready
+        {
+            const GroupEntry &e = es[recs[0].x & 255];
+            if (lane < 2 && !e.swap) {  // (a map's first use waits for its fetch)
+                if (lane == 0 || e.pair) prefetch_tensormap(&P.maps[(&e)[lane].map_y]);
+                if (e.res && (lane == 0 || e.pair)) prefetch_tensormap(&P.maps[(&e)[lane].map_r]);
+            }
+            __syncwarp();
+        }
+        pdl_wait();  // residual reads and output writes must not pass the previous layers
+        struct Box { const GroupEntry *e; int f0, blocks, last, w0, h0, n0; };
+        auto box_of = [&](int j) -> Box {
+            Box x;
+            const int4 rec = record(j);
+            x.e = &es[rec.x & 255];
+            const GroupEntry &e = *x.e;
+            x.f0 = (int)uniform((uint32_t)(rec.x >> 8));
+            x.blocks = e.swap ? 0 : (int)uniform((uint32_t)((min((int)e.bn_tile, e.ldk - x.f0) + 63) >> 6));
+            x.last = (int)uniform((uint32_t)last_block(e, x.f0));
+            x.w0 = (int)uniform((uint32_t)rec.y); x.h0 = (int)uniform((uint32_t)rec.z); x.n0 = (int)uniform((uint32_t)rec.w);
+            return x;
+        };
+        // cursor of the buffers made ready: block r_b of tile r_j goes to buffer r_buf
+        int r_j = 0, r_b = 0, r_buf = 0;
+        Box r_x = box_of(0);  // (every CTA has a tile)
+        auto make_ready = [&]() {
+            while (r_j < n_tiles && r_b >= r_x.blocks) {
+                r_b = 0;
+                if (++r_j < n_tiles) r_x = box_of(r_j);
+            }
+            if (r_j >= n_tiles || (r_j == n_tiles - 1 && tail_in_ring)) return;
+            const GroupEntry &e = *r_x.e;
+            const uint32_t bar = smem_u32(&buf_ready[r_buf]), dst = bufs + (n_bufs == 1 ? 0u : (uint32_t)(r_buf * G_BUF_BYTES));
+            const int c = r_x.f0 + min(64 * r_b, r_x.last);
+            if (uniform(e.res != nullptr)) {
+                const bool pair = uniform(e.pair) != 0 && c < (int)uniform((uint32_t)(&e)[1].ldk);
+                mbar_expect_tx_if(on, bar, uniform((uint32_t)(e.pix_rows * 128) + (pair ? (uint32_t)((&e)[1].pix_rows * 128) : 0u)));
+                tma_load_4d_if(on, dst, &P.maps[uniform((uint32_t)e.map_r)], bar, c, r_x.w0, r_x.h0, r_x.n0);
+                if (pair) tma_load_4d_if(on, dst + 64 * 128, &P.maps[uniform((uint32_t)(&e)[1].map_r)], bar, c, 0, (int)uniform((uint32_t)(&e)[1].slot_h), (int)uniform((uint32_t)(&e)[1].slot_n));
+            } else if (on) mbar_arrive(&buf_ready[r_buf]);
+            __syncwarp();
+            r_b++;
+            if (++r_buf == n_bars) r_buf = 0;
+        };
+        for (int i = 0; i < n_bufs; i++) make_ready();
+        int buf = 0, stored = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (int j = 0; j < n_tiles && ok; j++) {
+            const Box x = box_of(j);
+            const GroupEntry &e = *x.e;
+            const bool pair = uniform(e.pair) != 0;
+            const CUtensorMap *map = &P.maps[uniform((uint32_t)e.map_y)], *map2 = &P.maps[uniform((uint32_t)(pair ? (&e)[1].map_y : e.map_y))];
+            const int ldk2 = (int)uniform((uint32_t)(pair ? (&e)[1].ldk : 0)), h2 = (int)uniform((uint32_t)(pair ? (&e)[1].slot_h : 0)), n2 = (int)uniform((uint32_t)(pair ? (&e)[1].slot_n : 0));
+            for (int b = 0; b < x.blocks; b++) {
+                if (!(ok = __all_sync(0xffffffffu, mbar_wait(&buf_done[buf], phase, abort_flag)))) break;
+                const uint32_t src = tail_in_ring && j == n_tiles - 1 ? ring + (uint32_t)(b * G_BUF_BYTES) : bufs + (n_bufs == 1 ? 0u : (uint32_t)(buf * G_BUF_BYTES));
+                const int c = x.f0 + min(64 * b, x.last);
+                tma_store_4d_if(on, map, src, c, x.w0, x.h0, x.n0);
+                if (c < ldk2) tma_store_4d_if(on, map2, src + 64 * 128, c, 0, h2, n2);
+                bulk_commit();
+                if (!tail_in_ring || j + 1 < n_tiles) {
+                    if (lag) bulk_wait_read<1>();
+                    else bulk_wait_read<0>();
+                    if (stored++ >= lag) make_ready();
+                }
+                if (++buf == n_bars) { buf = 0; phase ^= 1; }
+            }
+        }
+        bulk_wait_read<0>();  // (what they write is visible when the grid has ended)
     } else {
         // ------------------------------------------------------------------ epilogue (warps 2..9)
         // All eight warps work on every tile: a warp takes its tensor-memory lane quadrant (warp % 4) and every other block
-        // of 32 columns; the accumulator is double buffered, so the main loop of the next tile runs meanwhile.
+        // of 64 filters; the accumulator is double buffered, so the main loop of the next tile runs meanwhile.
         //
-        // What bounds it: the memory pipe, then issue slots.  When a lane stored its own pixel row, 16 bytes at a time, a
-        // warp's store touched 32 lines and a 128 x 256 tile took 10.8k clocks (20k with a residual) against 512 clocks of
-        // tensor time per 64 channels - most launches were bound by that.  So each block goes through a few KB of shared
-        // memory private to the warp (fp32, 16 rows at a time): afterwards four neighbouring lanes own 32 neighbouring
-        // filters of a pixel, residual reads and output writes are runs of 64 bytes, and a lane keeps the folded batch norm
-        // of its 8 filters in registers for all of the block's rows.
+        // What bounds it: the memory pipe and issue slots.  A lane owns a pixel; its 64 filters lie in eight 16-byte pieces of
+        // a 128-byte row of the block's buffer, in the copy unit's 128-byte swizzle (eight neighbouring lanes touch the eight
+        // different groups of banks).  The residual was brought there by the copy unit, the results take its place and the
+        // copy unit stores them: no address arithmetic, no masks, no partial lines.  (Loads and stores by the lanes
+        // themselves, through a transposition in shared memory, took 456 instructions per 32 x 32 outputs, this takes about 130:
+        // a 56x56 1x1 layer with a residual, 64 images, 67 us then, 50 now; waves of 4 queries x 16 images 14850 -> 14160 us.)
+        // What is left of it is latency: 0.6 us a block without and 0.8 with a residual, one warp of a half per scheduler.
         const int quad = warp & 3;                // tensor-memory lane quadrant this warp may read
-        const int half = (warp - 2) >> 2;         // which of every two column blocks
+        const int half = (warp - 2) >> 2;         // which of every two blocks
         const int row_all = quad * 32 + lane;     // accumulator row: output pixel (normal) or filter (swapped)
-        const int lr = lane >> 2, lc = lane & 3;  // in the staged form: row within 8, 8-filter chunk within 32
-        float *stage = reinterpret_cast<float *>(smem + G_RING_BYTES) + (warp - 2) * G_EPI_FLOATS;
-        pdl_wait();  // residual reads and output writes must not pass the previous layers
-        int j = 0;   // tiles of this CTA so far
-        for (int t = (int)blockIdx.x; t < total_tiles; t += (int)gridDim.x, j++) {
-            const GroupEntry &e0 = es[tile_entry(es, begin, t, lane)];
-            const int local = t - e0.tile_begin, nt = local / e0.mtiles, mt = local - nt * e0.mtiles;
+        float *bn_s = reinterpret_cast<float *>(smem + G_POOL_BYTES) + (warp - 2) * G_BN_FLOATS;
+        const uint32_t row_addr = bufs + (uint32_t)(row_all * 128), swz = (uint32_t)(row_all & 7);
+        pdl_wait();  // (swapped tiles read the residual and write the output themselves)
+        struct Tile { const GroupEntry *e0, *e; int f0, cend, blocks, last, first; };
+        auto tile_of = [&](int j, int g) -> Tile {  // g: number of the tile's first block
+            Tile x;
+            const int4 rec = record(j);
+            x.e0 = &es[rec.x & 255];
             // rows 64..127 of a pair's tile belong to the second member (a warp lies on one side)
-            const bool second_half = e0.pair && quad >= 2;
-            const GroupEntry &e = second_half ? (&e0)[1] : e0;
-            const int row = second_half ? row_all - 64 : row_all;
-            const int K = e.K, ldk = e.ldk, act = e.act, buf = j & 1;
+            x.e = x.e0->pair && quad >= 2 ? x.e0 + 1 : x.e0;
+            x.f0 = rec.x >> 8;
+            x.blocks = x.cend = x.last = 0;
+            if (!x.e0->swap) {
+                x.cend = min((int)x.e0->bn_tile, x.e->K - x.f0);  // filters of this tile, a multiple of 8 (<= 0: none of this member's)
+                x.blocks = (min((int)x.e0->bn_tile, x.e0->ldk - x.f0) + 63) >> 6;  // (up to the end of the pixel's padding)
+                x.last = last_block(*x.e0, x.f0);
+            }
+            x.first = (g ^ half) & 1;  // this warp's blocks: those whose number has its half's parity
+            return x;
+        };
+        // Folded batch norm of a block's 64 filters, two per lane, asked for a block ahead.
+        float2 bn_sc = make_float2(0.f, 0.f), bn_sh = bn_sc;
+        auto load_bn = [&](const Tile &x, int b) {
+            if (b >= x.blocks) return;
+            const int f = x.f0 + max(min(min(64 * b, x.last) + 2 * lane, x.cend - 2), 0);
+            bn_sc = __ldg(reinterpret_cast<const float2 *>(x.e->scale + min(f, x.e->K - 2)));
+            bn_sh = __ldg(reinterpret_cast<const float2 *>(x.e->shift + min(f, x.e->K - 2)));
+        };
+        int g0 = 0, buf = half;   // number of the tile's first block; barriers of this warp's next block
+        uint32_t phase = 0;
+        Tile cur = tile_of(0, 0);
+        load_bn(cur, cur.first);
+        for (int j = 0; j < n_tiles; j++) {
+            const GroupEntry &e = *cur.e;
+            const int K = e.K, ldk = e.ldk, act = e.act, abuf = j & 1;
             const __nv_bfloat16 *res = e.res;
             __nv_bfloat16 *y = e.y;
-            const uint32_t tacc = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * G_ACC_COLS);
-            if (!e.swap) {
+            const uint32_t tacc = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(abuf * G_ACC_COLS);
+            Tile next = cur;
+            next.blocks = 0;
+            if (j + 1 < n_tiles) next = tile_of(j + 1, g0 + cur.blocks);
+            if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[abuf], (j >> 1) & 1, abort_flag))) break;
+            tc_fence_after();
+            if (!cur.e0->swap) {
                 // ---- normal tile: rows are output pixels, columns are filters
-                const int tn = mt / e.tiles_hw, mhw = mt - tn * e.tiles_hw, th = mhw / e.tiles_w, tw = mhw - th * e.tiles_w;
-                const int n0 = tn * e.bn, h0 = th * e.bh, w0 = tw * e.bw;
-                const int f0 = nt * e0.bn_tile;
-                // offset of the four rows this lane finishes (lr + 8 i), in vectors of 8 channels; ~0: outside the tensor
-                uint32_t off[4];
-                {
-                    const int dl = row / e.bw, dww = row - dl * e.bw, dn = dl / e.bh, dhh = dl - dn * e.bh;
-                    const int n = n0 + dn, h = h0 + dhh, w = w0 + dww;
-                    const bool valid = row < e.pix_rows && n < e.N && h < e.Ho && w < e.Wo;
-                    const uint32_t mine = valid ? (uint32_t)(((size_t)((size_t)n * e.Ho + h) * e.Wo + w) * (size_t)(ldk >> 3)) + (uint32_t)(f0 >> 3) : 0xffffffffu;
-#pragma unroll
-                    for (int i = 0; i < 4; i++) off[i] = __shfl_sync(0xffffffffu, mine, lr + 8 * i);
-                }
-                const int cend = min((int)e0.bn_tile, K - f0);    // filters of this tile, a multiple of 8 (<= 0: none of this member's)
-                const int cpad = min((int)e0.bn_tile, ldk - f0);  // ... and the end of the pixel's padding, written as zeros
-                const float lo = act == ACT_RELU ? 0.f : __int_as_float(0x7fc00000);  // ReLU as a maximum; no activation: the maximum with NaN is the other operand, a NaN stays one
-                // Folded batch norm of a block's 32 filters: a lane loads one filter's, and the warp meets in the padding of its
-                // staging rows (4 floats a row: scales in rows 0..7, shifts in 8..15).
-                float *bnp = stage + (lane >> 2) * G_EPI_PITCH + 32 + (lane & 3);
-                auto load_bn = [&](int c0) { const int f = f0 + min(c0 + lane, max(cend, 1) - 1); return make_float2(__ldg(e.scale + f), __ldg(e.shift + f)); };
-                auto put_bn = [&](float2 b) { bnp[0] = b.x; bnp[8 * G_EPI_PITCH] = b.y; };
-                auto load_res = [&](int c0, int i) -> uint4 {
-                    return (c0 + 8 * lc < cend && off[i] != 0xffffffffu) ? ld_act(reinterpret_cast<const uint4 *>(res) + off[i] + (uint32_t)((c0 >> 3) + lc)) : make_uint4(0u, 0u, 0u, 0u);
-                };
-                uint4 rv[4];
-                if (half * 32 < cend) {
-                    if (res) {
-#pragma unroll
-                        for (int i = 0; i < 4; i++) rv[i] = load_res(half * 32, i);
-                    }
-                    put_bn(load_bn(half * 32));
-                }
-                if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[buf], (j >> 1) & 1, abort_flag))) break;
-                tc_fence_after();
+                const __nv_bfloat162 lo = __bfloat162bfloat162(__ushort_as_bfloat16(act == ACT_RELU ? 0 : 0x7fff));  // ReLU as a maximum; no activation: the maximum with NaN is the other operand, a NaN stays one
+                bool ok = true;
+                if (cur.first >= cur.blocks) load_bn(next, next.first);
 #pragma unroll 1
-                for (int c0 = half * 32; c0 < cpad; c0 += 64) {
-                    // The next block's residual and batch norm, asked for a whole block ahead into registers of their own.  All at
-                    // one place and all used at one place: loads in flight share scoreboards, and a use between two of them waits
-                    // for both (the first 16 rows of a block with a residual: 1350 -> 670 clocks; what is left of the residual's
-                    // latency is the first block's of a tile.  4 queries x 16 images of 224x224: 1 %).
-                    uint4 rn[4];
-                    float2 bn = make_float2(0.f, 0.f);
-                    const bool more = c0 + 64 < cend;
-                    if (more) {
-                        bn = load_bn(c0 + 64);
-                        if (res) {
-#pragma unroll
-                            for (int i = 0; i < 4; i++) rn[i] = load_res(c0 + 64, i);
-                        }
-                    }
-                    uint32_t v[32];
-                    tmem_ld32(tacc + c0, v);
-                    const int c = c0 + 8 * lc;  // this lane's 8 filters
+                for (int b = cur.first; b < cur.blocks; b += 2) {
                     __syncwarp();
-                    float2 sc[4], sh[4];
-#pragma unroll
-                    for (int q = 0; q < 2; q++) {
-                        const float4 a = *reinterpret_cast<const float4 *>(stage + (2 * lc + q) * G_EPI_PITCH + 32), b = *reinterpret_cast<const float4 *>(stage + (8 + 2 * lc + q) * G_EPI_PITCH + 32);
-                        sc[2 * q] = make_float2(a.x, a.y); sc[2 * q + 1] = make_float2(a.z, a.w);
-                        sh[2 * q] = make_float2(b.x, b.y); sh[2 * q + 1] = make_float2(b.z, b.w);
-                    }
+                    *reinterpret_cast<float2 *>(bn_s + 2 * lane) = bn_sc;
+                    *reinterpret_cast<float2 *>(bn_s + 64 + 2 * lane) = bn_sh;
+                    __syncwarp();
+                    if (b + 2 < cur.blocks) load_bn(cur, b + 2);
+                    else load_bn(next, next.first);
+                    const int c0 = min(64 * b, cur.last);
+                    uint32_t v[64];
+                    tmem_ld32(tacc + (uint32_t)c0, v);
+                    tmem_ld32(tacc + (uint32_t)(c0 + 32), v + 32);
+                    uint32_t row = row_addr + (n_bufs == 1 ? 0u : (uint32_t)(buf * G_BUF_BYTES));
+                    if (tail_in_ring && j + 1 == n_tiles) row = ring + (uint32_t)(b * G_BUF_BYTES + row_all * 128);
+                    else if (!(ok = __all_sync(0xffffffffu, mbar_wait(&buf_ready[buf], phase, abort_flag)))) break;
                     tmem_ld_wait();
-#pragma unroll
-                    for (int hr = 0; hr < 2; hr++) {
-                        __syncwarp();
-                        if ((lane >> 4) == hr) {
-#pragma unroll
-                            for (int g = 0; g < 8; g++)
-                                *reinterpret_cast<uint4 *>(stage + (lane & 15) * G_EPI_PITCH + 4 * g) = make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
-                        }
-                        __syncwarp();
-#pragma unroll
-                        for (int i2 = 0; i2 < 2; i2++) {
-                            const int i = hr * 2 + i2;
-                            const float4 qa = *reinterpret_cast<const float4 *>(stage + (lr + 8 * i2) * G_EPI_PITCH + 8 * lc);
-                            const float4 qb = *reinterpret_cast<const float4 *>(stage + (lr + 8 * i2) * G_EPI_PITCH + 8 * lc + 4);
-                            float2 o[4] = {make_float2(qa.x, qa.y), make_float2(qa.z, qa.w), make_float2(qb.x, qb.y), make_float2(qb.z, qb.w)};
-#pragma unroll
-                            for (int q = 0; q < 4; q++) o[q] = __ffma2_rn(o[q], sc[q], sh[q]);
-                            if (res) {
-                                const uint32_t r4[4] = {rv[i].x, rv[i].y, rv[i].z, rv[i].w};
-#pragma unroll
-                                for (int q = 0; q < 4; q++) o[q] = __fadd2_rn(o[q], make_float2(__uint_as_float(r4[q] << 16), __uint_as_float(r4[q] & 0xffff0000u)));
-                            }
-                            if (act == ACT_HSWISH) {
-#pragma unroll
-                                for (int q = 0; q < 4; q++) { o[q].x = act_fn(o[q].x, ACT_HSWISH); o[q].y = act_fn(o[q].y, ACT_HSWISH); }
-                            } else {
-#pragma unroll
-                                for (int q = 0; q < 4; q++) { o[q].x = fmaxf(o[q].x, lo); o[q].y = fmaxf(o[q].y, lo); }
-                            }
-                            uint4 out;
-                            __nv_bfloat162 *ob = reinterpret_cast<__nv_bfloat162 *>(&out);
-#pragma unroll
-                            for (int q = 0; q < 4; q++) ob[q] = __float22bfloat162_rn(o[q]);
-                            if (c >= cend) out = make_uint4(0u, 0u, 0u, 0u);  // (the pixel's padding)
-                            if (c < cpad && off[i] != 0xffffffffu) reinterpret_cast<uint4 *>(y)[off[i] + (uint32_t)(c >> 3)] = out;
-                        }
+                    const int left = cur.cend - c0;  // filters of the block (beyond: the pixel's padding, zeros)
+                    if (res) {
+                        if (act == ACT_HSWISH) finish_block<true, true>(v, bn_s, row, swz, left, lo);
+                        else finish_block<true, false>(v, bn_s, row, swz, left, lo);
+                    } else {
+                        if (act == ACT_HSWISH) finish_block<false, true>(v, bn_s, row, swz, left, lo);
+                        else finish_block<false, false>(v, bn_s, row, swz, left, lo);
                     }
-                    if (more) {
-                        put_bn(bn);  // (everybody has this block's in registers: two warp barriers since)
-                        if (res) {
-#pragma unroll
-                            for (int i = 0; i < 4; i++) rv[i] = rn[i];
-                        }
-                    }
+                    fence_async_smem();  // the results are visible to the copy unit
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&buf_done[buf]);
+                    if ((buf += 2) >= n_bars) { buf = half; phase ^= 1; }
                 }
+                if (!ok) break;
             } else {
                 // ---- swapped tile: this thread owns filter `f`, columns are the member's output pixels
-                const int f = nt * 128 + row;
+                const int f = cur.f0 + row_all;
                 const bool fvalid = f < K, fpad = f >= K && f < ldk;
                 const int cend = e.pix_rows;  // == N * Ho * Wo: the pixel tile is the whole member
                 float sc = 0.f, sh = 0.f;
                 if (fvalid) { sc = __ldg(e.scale + f); sh = __ldg(e.shift + f); }
                 const unsigned short *resu = reinterpret_cast<const unsigned short *>(res);
-                if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[buf], (j >> 1) & 1, abort_flag))) break;
-                tc_fence_after();
 #pragma unroll 1
                 for (int c0 = half * 16; c0 < cend; c0 += 32) {  // (at most 32 pixels: one block of 16 per warp)
                     uint32_t v[16];
@@ -405,11 +501,14 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
                                 y[(size_t)(c0 + q) * ldk + f] = __float2bfloat16_rn(fvalid ? act_fn(__uint_as_float(v[q]) * sc + sh + __uint_as_float((uint32_t)rv[q] << 16), act) : 0.f);
                     }
                 }
+                load_bn(next, next.first);
             }
             // hand the accumulator buffer back to the MMA warp
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&acc_empty[buf]);
+            if (lane == 0) mbar_arrive(&acc_empty[abuf]);
+            g0 += cur.blocks;
+            cur = next;
         }
     }
     // ---------------------------------------------------------------------- teardown
@@ -433,6 +532,10 @@ static int views_of(const TcParams &p) { return (p.stride == 2 && p.k > 1) ? 4 :
 struct GroupLaunch::Impl {
     GroupParams<TC_GROUP_MAPS_LARGE> prm;  // host image of the parameter block (the small variant is a prefix)
     int n_maps = 0;
+    unsigned ids[TC_GROUP_MAPS_LARGE];  // the maps' numbers (TcConvPlan), 0: never shared
+    int ids_n[TC_GROUP_MAPS_LARGE];     // maps that lie there together
+    int iters = 0;      // longest reduction among the members, in stages
+    bool res = false;   // any member with a residual
     int col_rows = 0;   // most rows any member's column-side operand has (sizes the stages)
     const void *win_base = nullptr;  // largest cached filter prefix among the members' stored layers
     size_t win_bytes = 0;
@@ -444,6 +547,8 @@ GroupLaunch::~GroupLaunch() { delete impl; }
 void GroupLaunch::reset(const void *d_entries) {
     impl->n_maps = 0;
     impl->col_rows = 0;
+    impl->iters = 0;
+    impl->res = false;
     impl->win_base = nullptr;
     impl->win_bytes = 0;
     impl->prm.entries = static_cast<const GroupEntry *>(d_entries);
@@ -453,53 +558,78 @@ void GroupLaunch::reset(const void *d_entries) {
 int GroupLaunch::members() const { return impl->prm.n_entries; }
 int GroupLaunch::maps() const { return impl->n_maps; }
 int GroupLaunch::tiles() const { return impl->prm.total_tiles; }
+int GroupLaunch::maps_for(const TcConvPlan &pl) const { return pl.g_maps; }
 
 bool GroupLaunch::fits(const TcConvPlan &pl) const {
-    return impl->prm.n_entries < TC_GROUP_MAX_ENTRIES && impl->n_maps + views_of(pl.prm) + 1 <= TC_GROUP_MAPS_LARGE;
+    return impl->prm.n_entries < TC_GROUP_MAX_ENTRIES && impl->n_maps + pl.g_maps <= TC_GROUP_MAPS_LARGE;
 }
 
-void GroupLaunch::add(void *host_entry, const TcConvPlan &pl, const ConvArgs &a) {
+void tc_group_entry(TcConvPlan &pl, const ConvArgs &a) {
     const TcParams &p = pl.prm;
     GroupEntry e;
     std::memset(&e, 0, sizeof e);
-    const int views = views_of(p);
-    e.map_a = impl->n_maps;
-    std::memcpy(&impl->prm.maps[impl->n_maps], p.tmA, (size_t)views * sizeof(CUtensorMap));
-    impl->n_maps += views;
-    e.map_w = impl->n_maps;
-    std::memcpy(&impl->prm.maps[impl->n_maps], &p.tmW, sizeof(CUtensorMap));
-    impl->n_maps += 1;
     e.scale = a.scale; e.shift = a.shift;
     e.res = static_cast<const __nv_bfloat16 *>(a.res);
     e.y = static_cast<__nv_bfloat16 *>(a.y);
-    e.tile_begin = impl->prm.total_tiles;
     e.mtiles = (int)pl.grid.x;
-    e.N = p.N; e.Ho = p.Ho; e.Wo = p.Wo; e.K = p.K; e.C = p.C;
+    e.K = p.K; e.C = p.C;
+    e.slot_h = pl.slot_h; e.slot_n = pl.slot_n;
     e.ldk = a.ldy ? a.ldy : p.K;
-    // weight_policy 1: per-tile hints from the box; 2: all evict-first; 3: the box only feeds the launch's window
-    e.cacheK = a.weight_policy == 2 ? -1 : a.weight_policy == 1 ? a.cacheK : 0;
-    e.cacheC = a.weight_policy == 1 ? a.cacheC : 0;
-    if ((a.weight_policy == 1 || a.weight_policy == 3) && a.cacheK > 0) {
-        // the launch's access-policy window (optional mechanism): the filters [0, cacheK) of this stored layer, whole rows
-        const size_t bytes = (size_t)a.cacheK * a.R * a.R * a.Cmax * 2;
-        if (bytes > impl->win_bytes) { impl->win_base = a.w; impl->win_bytes = bytes; }
-    }
     e.R = p.R; e.tap0 = p.o * p.R + p.o;
     e.tiles_w = p.tiles_w; e.tiles_hw = p.tiles_w * p.tiles_h;
-    e.cchunks = p.cchunks; e.layer = a.layer;
+    e.cchunks = p.cchunks; e.layer = 0;
     e.bw = (short)p.bw; e.bh = (short)p.bh; e.bn = (short)p.bn;
     e.pix_rows = (short)(p.bw * p.bh * p.bn);
     e.swap = (unsigned char)pl.swap;
     e.bn_tile = (short)(pl.swap ? (e.pix_rows + 15) / 16 * 16 : pl.bn_tile);
     e.k = (unsigned char)p.k; e.kw = (unsigned char)pl.kw; e.stride = (unsigned char)p.stride; e.p = (unsigned char)p.p; e.act = (unsigned char)p.act;
-    impl->col_rows = std::max(impl->col_rows, (int)(pl.swap ? e.pix_rows : e.bn_tile));
+    e.can_pair = !pl.swap && !a.win && e.mtiles == 1 && e.pix_rows <= 64;
+    std::memcpy(pl.entry, &e, sizeof e);
+    pl.g_iters = p.iters;
+    pl.g_col_rows = pl.swap ? e.pix_rows : e.bn_tile;
+    pl.g_tiles = e.mtiles * (int)pl.grid.y;
+    pl.g_views = (unsigned char)views_of(p);
+    pl.g_maps = (unsigned char)(pl.g_views + 1 + (pl.swap ? 0 : pl.has_res ? 2 : 1));
+}
+
+void GroupLaunch::add(void *host_entry, const TcConvPlan &pl, const ConvArgs &a, int policy, int cacheK, int cacheC) {
+    GroupEntry e;
+    std::memcpy(&e, pl.entry, sizeof e);
+    // Members whose maps are the same ones share them (weights: the same slice; activations: the same channel pitch, see
+    // ConvArgs::slot): fewer of them fit a smaller parameter block, which every launch copies.
+    auto add_maps = [&](const CUtensorMap *m, int n, unsigned id) {
+        for (int i = 0; i < impl->n_maps && id; i++)
+            if (impl->ids[i] == id && impl->ids_n[i] == n) return i;
+        const int at = impl->n_maps;
+        std::memcpy(&impl->prm.maps[at], m, (size_t)n * sizeof(CUtensorMap));
+        for (int i = 0; i < n; i++) { impl->ids[at + i] = i ? 0 : id; impl->ids_n[at + i] = n; }
+        impl->n_maps += n;
+        return at;
+    };
+    e.map_a = add_maps(pl.prm.tmA, pl.g_views, pl.id_a);
+    e.map_w = add_maps(&pl.prm.tmW, 1, pl.id_w);
+    if (!e.swap) {
+        e.map_y = (short)add_maps(&pl.tmY, 1, pl.id_y);
+        if (e.res) { e.map_r = (short)add_maps(&pl.tmR, 1, pl.id_r); impl->res = true; }
+    }
+    impl->iters = std::max(impl->iters, pl.g_iters);
+    impl->col_rows = std::max(impl->col_rows, pl.g_col_rows);
+    e.tile_begin = impl->prm.total_tiles;
+    e.layer = a.layer;
+    // policy 1: per-tile hints from the box; 2: all evict-first; 3: the box only feeds the launch's window
+    e.cacheK = policy == 2 ? -1 : policy == 1 ? cacheK : 0;
+    e.cacheC = policy == 1 ? cacheC : 0;
+    if ((policy == 1 || policy == 3) && cacheK > 0) {
+        // the launch's access-policy window (optional mechanism): the filters [0, cacheK) of this stored layer, whole rows
+        const size_t bytes = (size_t)cacheK * a.R * a.R * a.Cmax * 2;
+        if (bytes > impl->win_bytes) { impl->win_base = a.w; impl->win_bytes = bytes; }
+    }
     impl->prm.n_entries++;
     // Pairing: this member and the previous one of the launch each fit the lower / upper half of a tile's 128
     // rows, run the same stored layer, and one's slice contains the other's (filters and channels): they
     // share the larger one's tiles and weight copies.
-    auto half = [](const GroupEntry &g) { return !g.swap && g.mtiles == 1 && g.pix_rows <= 64 && g.kw == g.k; };
     GroupEntry *prev = impl->prm.n_entries >= 2 ? static_cast<GroupEntry *>(host_entry) - 1 : nullptr;
-    if (prev && !a.win && half(e) && half(*prev) && !prev->pair && !prev->second && prev->layer == e.layer && prev->k == e.k &&
+    if (prev && e.can_pair && prev->can_pair && !prev->pair && !prev->second && prev->layer == e.layer && prev->k == e.k &&
         prev->stride == e.stride && prev->act == e.act && ((prev->K >= e.K && prev->C >= e.C) || (e.K >= prev->K && e.C >= prev->C))) {
         GroupEntry first = *prev, second = e;
         if (!(prev->K >= e.K && prev->C >= e.C)) { first = e; second = *prev; }
@@ -513,13 +643,21 @@ void GroupLaunch::add(void *host_entry, const TcConvPlan &pl, const ConvArgs &a)
         return;
     }
     std::memcpy(host_entry, &e, sizeof e);
-    impl->prm.total_tiles += e.mtiles * (int)pl.grid.y;
+    impl->prm.total_tiles += pl.g_tiles;
 }
 
+// Kernel variants by the tensor maps they have room for: a launch passes the whole parameter block.
+typedef void (*GroupKernel)(void);
+template <int N> static GroupKernel group_variant() { return reinterpret_cast<GroupKernel>(conv_group_kernel<N>); }
+static const struct { int maps; GroupKernel kernel; } GROUP_VARIANTS[] = {
+    {64, group_variant<64>()}, {TC_GROUP_MAPS_LARGE, group_variant<TC_GROUP_MAPS_LARGE>()}};
+
 cudaError_t tc_group_init(int) {
-    cudaError_t e = cudaFuncSetAttribute(conv_group_kernel<TC_GROUP_MAPS_SMALL>, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM_BYTES);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(conv_group_kernel<TC_GROUP_MAPS_LARGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM_BYTES);
+    for (const auto &v : GROUP_VARIANTS) {
+        const cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(v.kernel), cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM_BYTES);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t GroupLaunch::launch(size_t window_max, int sms, cudaStream_t st) {
@@ -529,9 +667,14 @@ cudaError_t GroupLaunch::launch(size_t window_max, int sms, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     impl->prm.status = tc_status_word(dev);
     if (!impl->prm.status) return cudaErrorInitializationError;
-    // stage = 16 KB for the row-side operand + room for the widest column-side operand of the launch
+    // Shared memory: stages of 16 KB for the row-side operand + room for the widest column-side operand of the launch, and
+    // buffers for blocks of output.  A residual has to be asked for early: with short reductions it gets most of the room (1 or 2
+    // stages a tile, 6 buffers: 56x56 1x1 layers of a wave of 32 wait 0.9 us a tile for it, 1.3 with 4).  Long reductions without
+    // one live on operands in flight (7x7 3x3 layers of 63 - 72 stages of 46 KB: 50 us with 4 stages, 65 with 3).
     impl->prm.stage_bytes = G_X_BYTES + (impl->col_rows + 15) / 16 * 16 * CHUNK_C * 2;
-    impl->prm.n_stages = std::min(G_MAX_STAGES, G_RING_BYTES / impl->prm.stage_bytes);  // 4 (256 columns) to 8
+    auto stages_with = [&](int bufs) { return std::min(G_MAX_STAGES, (G_POOL_BYTES - bufs * G_BUF_BYTES) / impl->prm.stage_bytes); };
+    impl->prm.n_bufs = impl->res && impl->iters <= 2 ? 6 : impl->res || impl->iters < 12 ? 4 : 1;
+    impl->prm.n_stages = stages_with(impl->prm.n_bufs);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)std::min(impl->prm.total_tiles, std::max(1, sms)));
     cfg.blockDim = dim3(G_THREADS);
@@ -554,13 +697,11 @@ cudaError_t GroupLaunch::launch(size_t window_max, int sms, cudaStream_t st) {
         attr[1].val.accessPolicyWindow.missProp = cudaAccessPropertyNormal;
         cfg.numAttrs = 2;
     }
-    if (impl->n_maps <= TC_GROUP_MAPS_SMALL) {
-        // the small parameter block is a prefix of the large one (same header, fewer maps)
-        void *args[1] = {&impl->prm};
-        return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(conv_group_kernel<TC_GROUP_MAPS_SMALL>), args);
-    }
+    // (a smaller parameter block is a prefix of the largest one: same header, fewer maps)
     void *args[1] = {&impl->prm};
-    return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(conv_group_kernel<TC_GROUP_MAPS_LARGE>), args);
+    for (const auto &v : GROUP_VARIANTS)
+        if (impl->n_maps <= v.maps) return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(v.kernel), args);
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace sgs

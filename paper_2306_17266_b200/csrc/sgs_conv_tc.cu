@@ -461,11 +461,13 @@ struct MapKeyHash {
         return (size_t)h;
     }
 };
-std::unordered_map<MapKey, CUtensorMap, MapKeyHash> g_map_cache;
+struct KnownMap { CUtensorMap map; unsigned id; };
+std::unordered_map<MapKey, KnownMap, MapKeyHash> g_map_cache;
 std::mutex g_map_mu;
 
 bool encode_map(CUtensorMap *m, const void *base, int rank, const uint64_t *dims, const uint64_t *strides_bytes,
-                const uint32_t *box, bool bytes = false) {
+                const uint32_t *box, bool bytes = false, unsigned *id = nullptr) {
+    if (id) *id = 0;
     MapKey key;
     std::memset(&key, 0, sizeof key);
     key.v[0] = reinterpret_cast<uint64_t>(base);
@@ -475,7 +477,7 @@ bool encode_map(CUtensorMap *m, const void *base, int rank, const uint64_t *dims
     {
         std::lock_guard<std::mutex> lk(g_map_mu);
         auto it = g_map_cache.find(key);
-        if (it != g_map_cache.end()) { *m = it->second; return true; }
+        if (it != g_map_cache.end()) { *m = it->second.map; if (id) *id = it->second.id; return true; }
     }
     cuuint64_t gd[5], gs[4];
     cuuint32_t bx[5], es[5];
@@ -486,7 +488,10 @@ bool encode_map(CUtensorMap *m, const void *base, int rank, const uint64_t *dims
                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return false;
     std::lock_guard<std::mutex> lk(g_map_mu);
-    if (g_map_cache.size() < (1u << 20)) g_map_cache.emplace(key, *m);  // (128 bytes each; bounded)
+    if (g_map_cache.size() < (1u << 20)) {  // (bounded)
+        auto r = g_map_cache.emplace(key, KnownMap{*m, (unsigned)g_map_cache.size() + 1u});
+        if (id) *id = r.first->second.id;
+    }
     return true;
 }
 
@@ -634,6 +639,11 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
     const uint64_t C = (uint64_t)(a.ldx ? a.ldx : a.C), eb = a.i8 ? 1 : 2;
     const uint32_t CH = a.i8 ? 2 * CHUNK_C : CHUNK_C;  // channels per stage (128 bytes)
     const bool b8 = a.i8 != 0;
+    // Maps over all slots: the slot is the row of a flat layer's matrix of pixels, else the image (members of one image).
+    const bool shared = a.throughput == 2 && a.slots > 0 && a.slot_bytes % 16 == 0 && (flat || a.N == 1);
+    const size_t back = shared ? (size_t)a.slot * a.slot_bytes : 0;
+    auto first_slot = [&](const void *q) { return static_cast<const void *>(static_cast<const char *>(q) - back); };
+    if (shared) (flat ? plan->slot_h : plan->slot_n) = a.slot;
     plan->i8 = a.i8;
     // Grouped launches (throughput == 2) run a layer with very few output pixels "swapped": the filters
     // take the 128-row side of the MMA and ALL pixels of the member form the other operand (one pixel
@@ -650,8 +660,9 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
         p.bw = swap ? (int)M : a.throughput == 2 ? (int)std::min<uint64_t>(M, TILE_M) : TILE_M; p.bh = 1; p.bn = 1;
         p.N = 1; p.Ho = 1; p.Wo = (int)M;
         uint64_t dims[4] = {C, M, 1, 1}, str[3] = {C * eb, M * C * eb, M * C * eb};
+        if (shared) { dims[2] = (uint64_t)a.slots; str[1] = a.slot_bytes; str[2] = a.slot_bytes * dims[2]; }
         uint32_t box[4] = {CH, (uint32_t)p.bw, 1, 1};
-        if (!encode_map(&p.tmA[0], a.x, 4, dims, str, box, b8)) return no("activation tensor map");
+        if (!encode_map(&p.tmA[0], first_slot(a.x), 4, dims, str, box, b8, &plan->id_a)) return no("activation tensor map");
     } else {
         if (swap) { p.bw = a.Wo; p.bh = a.Ho; p.bn = a.N; }
         else choose_box(a.N, a.Ho, a.Wo, &p.bw, &p.bh, &p.bn);
@@ -661,10 +672,11 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
             uint32_t wbox[4] = {CHUNK_C, (uint32_t)p.bw, (uint32_t)p.bh, (uint32_t)p.bn};
             const uint64_t px = 8 * eb, st = (uint64_t)a.stride;
             for (int ph = 0; ph < a.stride; ph++) {
-                const char *base = static_cast<const char *>(a.x) + (size_t)ph * a.W * px;
+                const char *base = static_cast<const char *>(first_slot(a.x)) + (size_t)ph * a.W * px;
                 uint64_t dims[4] = {CHUNK_C, (uint64_t)a.Wo, (uint64_t)(a.H - ph + a.stride - 1) / st, (uint64_t)a.N};
                 uint64_t str[3] = {st * px, st * (uint64_t)a.W * px, (uint64_t)a.H * a.W * px};
-                if (!encode_map(&p.tmA[ph * 2], base, 4, dims, str, wbox)) return no("window tensor map");
+                if (shared) { dims[3] = (uint64_t)a.slots; str[2] = a.slot_bytes; }
+                if (!encode_map(&p.tmA[ph * 2], base, 4, dims, str, wbox, false, ph ? nullptr : &plan->id_a)) return no("window tensor map");
             }
         }
         uint32_t box[4] = {CH, (uint32_t)p.bw, (uint32_t)p.bh, (uint32_t)p.bn};
@@ -673,16 +685,18 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
         } else if (a.stride == 1) {
             uint64_t dims[4] = {C, (uint64_t)a.W, (uint64_t)a.H, (uint64_t)a.N};
             uint64_t str[3] = {C * eb, (uint64_t)a.W * C * eb, (uint64_t)a.H * a.W * C * eb};
-            if (!encode_map(&p.tmA[0], a.x, 4, dims, str, box, b8)) return no("activation tensor map");
+            if (shared) { dims[3] = (uint64_t)a.slots; str[2] = a.slot_bytes; }
+            if (!encode_map(&p.tmA[0], first_slot(a.x), 4, dims, str, box, b8, &plan->id_a)) return no("activation tensor map");
         } else {
             // (odd sizes: the views of odd rows / columns are one shorter; what lies beyond is zero fill like any border)
             const int views = a.k > 1 ? 2 : 1;  // a 1x1 kernel reads even rows and columns only
             for (int ph = 0; ph < views; ph++)
                 for (int pw = 0; pw < views; pw++) {
-                    const char *base = static_cast<const char *>(a.x) + ((size_t)ph * a.W + pw) * C * eb;
+                    const char *base = static_cast<const char *>(first_slot(a.x)) + ((size_t)ph * a.W + pw) * C * eb;
                     uint64_t dims[4] = {C, (uint64_t)(a.W - pw + 1) / 2, (uint64_t)(a.H - ph + 1) / 2, (uint64_t)a.N};
                     uint64_t str[3] = {2 * C * eb, 2 * (uint64_t)a.W * C * eb, (uint64_t)a.H * a.W * C * eb};
-                    if (!encode_map(&p.tmA[ph * 2 + pw], base, 4, dims, str, box, b8)) return no("activation tensor map");
+                    if (shared) { dims[3] = (uint64_t)a.slots; str[2] = a.slot_bytes; }
+                    if (!encode_map(&p.tmA[ph * 2 + pw], base, 4, dims, str, box, b8, ph + pw ? nullptr : &plan->id_a)) return no("activation tensor map");
                 }
         }
     }
@@ -727,7 +741,18 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
         uint64_t dims[3] = {Cw, taps, (uint64_t)a.K};
         uint64_t str[2] = {(uint64_t)a.Cmax * eb, taps * a.Cmax * eb};
         uint32_t box[3] = {CH, 1, (uint32_t)BN};
-        if (!encode_map(&p.tmW, a.w, 3, dims, str, box, b8)) return no("weight tensor map");
+        if (!encode_map(&p.tmW, a.w, 3, dims, str, box, b8, &plan->id_w)) return no("weight tensor map");
+    }
+    if (a.throughput == 2 && !swap) {
+        const uint64_t ldk = (uint64_t)(a.ldy ? a.ldy : a.K);
+        uint64_t dims[4] = {ldk, (uint64_t)p.Wo, (uint64_t)p.Ho, (uint64_t)p.N};
+        uint64_t str[3] = {ldk * eb, dims[1] * ldk * eb, dims[1] * dims[2] * ldk * eb};
+        uint32_t box[4] = {CHUNK_C, (uint32_t)p.bw, (uint32_t)p.bh, (uint32_t)p.bn};
+        if (shared && flat) { dims[2] = (uint64_t)a.slots; str[1] = a.slot_bytes; str[2] = a.slot_bytes * dims[2]; }
+        else if (shared) { dims[3] = (uint64_t)a.slots; str[2] = a.slot_bytes; }
+        if (!encode_map(&plan->tmY, first_slot(a.y), 4, dims, str, box, false, &plan->id_y)) return no("output tensor map");
+        plan->has_res = a.res != nullptr;
+        if (a.res && !encode_map(&plan->tmR, first_slot(a.res), 4, dims, str, box, false, &plan->id_r)) return no("residual tensor map");
     }
     const int ntiles = (a.K + BN - 1) / BN;
     // split the K loop when the tiles alone cannot fill the machine
@@ -742,6 +767,7 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
     const int steps = (p.iters + splits - 1) / splits, room = (long long)ctas * splits > sms ? 98304 : TC_RING_MAX;
     p.stages = std::max(BN == 128 ? 3 : 2, std::min({steps, room / tc_stage_bytes(BN), TC_MAX_STAGES}));
     plan->grid = dim3((unsigned)mtiles, (unsigned)ntiles, (unsigned)splits);
+    if (a.throughput == 2) tc_group_entry(*plan, a);
     return plan;
 }
 

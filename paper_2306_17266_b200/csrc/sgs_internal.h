@@ -80,6 +80,10 @@ struct ConvArgs {
                          // 2: member of a grouped launch (128-filter tiles, reduction never split)
     int early_weights = 0;  // 1: the weights belong to a loaded SuperNet, so a kernel may read them before the previous kernel of
                             // the stream has finished; 0: they are the caller's and may come from that kernel
+    // Members of a grouped launch whose x, y and res are the same buffers of different slots, slot_bytes apart, share tensor maps that
+    // show all `slots` of them; this member is slot number `slot` (slots = 0: maps of its own).
+    int slot = 0, slots = 0;
+    size_t slot_bytes = 0;
     int no_split = 0;  // 1: one block per tile (the reduction is never split over a cluster)
 };
 
@@ -252,7 +256,7 @@ cudaError_t tc_expire_wait(unsigned limit_us, cudaStream_t st);  // a kernel who
 // ConvArgs::throughput == 2 (128-filter tiles, reduction never split).
 constexpr int TC_GROUP_ENTRY_BYTES = 128;
 constexpr int TC_GROUP_MAX_ENTRIES = 64;
-constexpr int TC_GROUP_MAPS_SMALL = 64, TC_GROUP_MAPS_LARGE = 248;  // tensor maps per launch (two kernel variants)
+constexpr int TC_GROUP_MAPS_LARGE = 248;  // tensor maps per launch
 class GroupLaunch {
 public:
     GroupLaunch();
@@ -262,10 +266,13 @@ public:
     void reset(const void *d_entries);       // start a launch whose member records will live at d_entries
     bool fits(const TcConvPlan &p) const;   // room for one more member (records and tensor maps)?
     // Adds a member: writes its record to host_entry (the host image of the next device record).
-    void add(void *host_entry, const TcConvPlan &p, const ConvArgs &a);
+    // Its weight loads take the hints of `policy` (0 none; 1 the box of the first cacheK filters x cacheC channels evict-last; 2 all
+    // evict-first; 3 the box only feeds the launch's window).
+    void add(void *host_entry, const TcConvPlan &p, const ConvArgs &a, int policy, int cacheK, int cacheC);
     int members() const;
     int maps() const;                       // tensor maps used so far
     int tiles() const;
+    int maps_for(const TcConvPlan &p) const;  // tensor maps a member takes
     // window_max > 0: also mark the launch's cached filter prefix with an access-policy window of at most that many bytes
     cudaError_t launch(size_t window_max, int sms, cudaStream_t st);
 private:
@@ -273,6 +280,7 @@ private:
     Impl *impl;
 };
 cudaError_t tc_group_init(int device);
+void tc_group_entry(TcConvPlan &p, const ConvArgs &a);  // fills the plan's record for grouped launches
 
 cudaError_t subnet_kernel_init(int device);
 size_t subnet_kernel_smem();  // dynamic shared memory of a block

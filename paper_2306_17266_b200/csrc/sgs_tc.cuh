@@ -122,6 +122,27 @@ __device__ __forceinline__ void tma_load_3d_hint_if(uint32_t on, uint32_t dst, c
         ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "l"(policy), "r"(on)
         : "memory");
 }
+__device__ __forceinline__ void tma_store_4d_if(uint32_t on, const CUtensorMap *map, uint32_t src, int c0, int c1, int c2, int c3) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %6, 0;\n\t"
+        "@q cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];\n\t}"
+        ::"l"(map), "r"(src), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(on)
+        : "memory");
+}
+// Groups of bulk stores: commit() closes one, wait_read<N> waits until all but the last N have read their shared memory,
+// wait_all until everything is written.
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory"); }
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ uint4 lds128(uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ void sts128(uint32_t addr, uint4 v) {
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w));  // (no clobber: a lane's own row)
+}
 template <bool I8>
 __device__ __forceinline__ void umma_if(uint32_t on, uint32_t tmem_d, uint64_t desc_a, uint64_t desc_b, uint32_t idesc, uint32_t accumulate) {
     if (I8)
@@ -226,11 +247,21 @@ __device__ __forceinline__ void finish_store(float *o, const __nv_bfloat16 *res,
 __host__ __device__ __forceinline__ long long rshift_round(long long v, int s) { return (v + (1ll << (s - 1))) >> s; }
 
 struct TcConvPlan {
+    // Member of a grouped launch: its record but for what depends on the launch, which of its maps are the same ones as other
+    // members' (0: not known), the reduction in stages, rows of its column-side operand, activation views.  All that a wave's
+    // tables need of a plan lies here together: a wave reads some two thousand of them.
+    alignas(64) unsigned char entry[TC_GROUP_ENTRY_BYTES] = {};
+    unsigned id_a = 0, id_w = 0, id_y = 0, id_r = 0;
+    int g_iters = 0, g_col_rows = 0, g_tiles = 0;
+    unsigned char g_views = 0, g_maps = 0;
     TcParams prm;
     int i8 = 0;          // 8-bit operands: 128 channels per stage, 32 per MMA
     dim3 grid;
     int bn_tile = 128;   // filters per tile
     int swap = 0;        // grouped launches only: filters on the MMA's row side, all pixels on the column side
+    int slot_h = 0, slot_n = 0;  // where this member lies in maps that show several slots
+    CUtensorMap tmY, tmR;  // grouped launches, not swapped: output and residual as boxes of 64 filters x the tile's pixels
+    int has_res = 0;
     int kw = 1;          // taps along x (k for square kernels, 1 for the window view of a stem)
 };
 
