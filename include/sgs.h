@@ -110,8 +110,8 @@ typedef struct {
                            SGS_POLICY_AVGNET (1): Algorithm 1 - the candidate SubGraph (sgs_cache_set_candidates)
                            nearest to the running average of the last window_q SubNets' encodings */
     int persistent;     /* 1 (bf16 handles of the MobileNetV3-shaped family, one image per query): the whole stream
-                           is ONE launch of a persistent kernel; every SM takes the next unserved query and runs all
-                           layers of its SubNet by itself out of a private scratch area, pointwise convolutions on the
+                           is ONE launch of a persistent kernel; every SM, or team of 2 to 16 SMs where queries are
+                           few, takes the next unserved query and runs all layers of its SubNet by itself out of a private scratch area, pointwise convolutions on the
                            tensor cores (Section 3.1: one query per pass of the accelerator; Section 4.2: what is needed
                            again stays on chip).  wave, concurrency and use_graphs are ignored; every query starts and
                            ends with the launch (its recorded latency).  With the cache enabled one SubGraph is chosen for the launch,
@@ -461,7 +461,8 @@ sgs_status_t sgs_debug_expire_wait(unsigned limit_us, void *cuda_stream);
  * prefix of the launch's stored layer, persisting; the persisting-L2 carve-out of the process is sized to the cache
  * budget), 2 = both; "dw_walk" is accepted and has no effect (there is one depthwise
  * kernel); "persistent_held_kb" n = shared memory per SM that persistent
- * execution spends on the cached SubGraph's first pointwise layers (default 16, 0 = none); "nvtx" 1 = an NVTX range named after the stored layer around
+ * execution spends on the cached SubGraph's first pointwise layers (default 16, 0 = none); "persistent_team" n = SMs that serve a
+ * query of persistent execution together (1, 2, 4, 8, 16; default 0 = chosen by the number and size of a call's queries); "nvtx" 1 = an NVTX range named after the stored layer around
  * every launch (for timeline tools); "fail_alloc_after" n = the handle's device allocations fail from
  * the (n+1)-th on with SGS_ENOMEM (fault injection on the host, -1 = off); "drop_plans" forgets every cached plan (measuring what a never-seen config costs); "profile" see
  * sgs_profile_read; "stage_group" 0..4 is accepted

@@ -243,6 +243,7 @@ struct sgs_supernet {
     size_t pq_stage_in_bytes = 0, pq_stage_out_bytes = 0;
     size_t persist_limit_set = 0;  // cudaLimitPersistingL2CacheSize as last set by this handle
     int nvtx = 0;  // 1: NVTX ranges named after the stored layer around every launch
+    int persistent_team = 0;  // persistent execution: blocks that serve a query together (0: chosen by the call)
     int persistent_held_kb = 16;  // persistent execution: shared memory per SM for the cached SubGraph's first layers (0: none)
     long long fail_alloc_after = -1;  // < 0: off; else device allocations left before they start failing (test aid)
     int cache_mech = 0;    // how grouped launches keep the cached SubGraph in L2: 0 per-tile hints, 1 access-policy window of the launch, 2 both
@@ -2011,6 +2012,23 @@ static sgs_status_t build_pq_ops(sgs_supernet *net, Plan *plan) {
     return SGS_OK;
 }
 
+// Blocks per query (a cluster: 1, 2, 4, 8 or 16) and how many such teams the device holds.  A query takes work / team + overhead, where
+// the overhead (some 100 layers, each with a barrier, the fill of its pipelines and a last round of tiles) does not shrink, and
+// larger clusters leave SMs unused (148, 148, 132, 120 and 112 of 148).  Measured (B200, 224x224, ms a call; 1 / 2 / 4 / 8 / 16
+// blocks): 8 queries 3.45 / 1.96 / 1.21 / 0.87 / 1.11, 33: 3.97 / 2.23 / 1.42 / 2.07 / 3.09, 74: 4.22 / 2.37 / 3.21 / 3.98, 148: 4.33 /
+// 4.42 / 5.52, 333: 9.99 / 9.17 / 11.67.  With more queries than teams they come one after the other, dealt as teams get free.
+static void choose_team(const sgs_supernet *net, int n, double flops, int *team, int *clusters) {
+    const double work = n > 0 ? flops / n * 6.2e-12 : 0, overhead = 0.35e-3;  // seconds on one SM: 3.4 ms for 0.55 GFLOP
+    double best = 0;
+    for (int t : {1, 2, 4, 8, 16}) {
+        if (net->persistent_team && t != net->persistent_team) continue;
+        const int c = t == 1 ? std::max(1, net->sms) : subnet_kernel_clusters(t);
+        if (c <= 0) continue;
+        const double rounds = n <= c ? 1.0 : std::max(1.75, 0.8 * n / c + 0.4), time = (work / t + overhead) * rounds;
+        if (best == 0 || time < best) { best = time; *team = t; *clusters = std::min(c, std::max(1, net->sms)); }
+    }
+}
+
 static sgs_status_t persistent_impl(sgs_supernet_t *net, int n_queries, const sgs_subnet_cfg_t *cfgs, const void *inputs, int res,
                                     void *logits, const sgs_stream_opts_t &o, sgs_stream_stats_t *stats, cudaStream_t st,
                                     bool host_buffers, StreamScope &scope) {
@@ -2023,7 +2041,7 @@ static sgs_status_t persistent_impl(sgs_supernet_t *net, int n_queries, const sg
     // plans and op lists (one list per distinct config of the call)
     std::vector<Plan *> plans((size_t)n_queries);
     std::unordered_map<Plan *, int> begin;
-    std::vector<PqOp> ops;
+    size_t n_ops = 0;
     std::vector<PqQuery> qs((size_t)n_queries);
     size_t act_elems = 0;
     double flops = 0, wbytes = 0, miss_bytes = 0, hit = 0;
@@ -2041,7 +2059,6 @@ static sgs_status_t persistent_impl(sgs_supernet_t *net, int n_queries, const sg
     // boxes in shared memory, front layers first, as far as the buffer reaches.  One launch has one choice; the
     // accounting below is against what is actually held.
     std::vector<PqHeld> held;
-    std::unordered_map<const void *, size_t> held_of;  // stored weights -> entry
     unsigned held_bytes = 0;
     if (net->cache.enabled && net->persistent_held_kb > 0 && n_queries > 0) {
         const int first = std::min(n_queries, net->cache.window_q);
@@ -2060,7 +2077,6 @@ static sgs_status_t persistent_impl(sgs_supernet_t *net, int n_queries, const sg
             PqHeld h;
             std::memset(&h, 0, sizeof h);
             h.w = L.w; h.ld = L.Cp; h.rows = rows; h.chunks = chunks; h.C = C; h.off = held_bytes;
-            held_of.emplace(L.w, held.size());
             held.push_back(h);
             held_bytes += (unsigned)bytes;
             kept[3 * li] = rows; kept[3 * li + 1] = C; kept[3 * li + 2] = 1;
@@ -2072,17 +2088,8 @@ static sgs_status_t persistent_impl(sgs_supernet_t *net, int n_queries, const sg
     }
     for (int t = 0; t < n_queries; t++) {
         Plan *pl = plans[(size_t)t];
-        auto it = begin.find(pl);
-        if (it == begin.end()) {
-            it = begin.emplace(pl, (int)ops.size()).first;
-            for (PqOp q : pl->pq) {
-                if (q.type == PQ_PW) {
-                    auto h = held_of.find(q.w);
-                    if (h != held_of.end()) { const PqHeld &e = held[h->second]; q.cache_off = e.off; q.cache_rows = e.rows; q.ld2 = e.C; }
-                }
-                ops.push_back(q);
-            }
-        }
+        auto it = begin.emplace(pl, (int)n_ops).first;
+        if (it->second == (int)n_ops) n_ops += pl->pq.size();
         PqQuery &q = qs[(size_t)t];
         std::memset(&q, 0, sizeof q);
         q.op_begin = it->second; q.op_count = (int)pl->pq.size();
@@ -2090,7 +2097,9 @@ static sgs_status_t persistent_impl(sgs_supernet_t *net, int n_queries, const sg
         flops += pl->flops; wbytes += qa.weight_bytes; miss_bytes += qa.miss_bytes; hit += qa.hit_ratio;
     }
     // device resources: scratch of the blocks, tables, counter, staging for host buffers
-    const int blocks_max = std::max(1, net->sms) * subnet_kernel_blocks_per_sm();
+    int team = 1, clusters = std::max(1, net->sms);
+    choose_team(net, n_queries, flops, &team, &clusters);
+    const int blocks_max = std::max(1, net->sms);  // (a team has one scratch area)
     const size_t act_bytes = (act_elems * net->elem() + 255) / 256 * 256, slot_bytes = 4 * act_bytes;
     if (net->pq_scratch_bytes < slot_bytes * blocks_max) {
         CU(cudaStreamSynchronize(st));
@@ -2099,7 +2108,7 @@ static sgs_status_t persistent_impl(sgs_supernet_t *net, int n_queries, const sg
         if (rc != SGS_OK) return rc;
         net->pq_scratch_bytes = slot_bytes * blocks_max;
     }
-    const size_t ops_bytes = ops.size() * sizeof(PqOp), q_bytes = qs.size() * sizeof(PqQuery), h_bytes = held.size() * sizeof(PqHeld);
+    const size_t ops_bytes = n_ops * sizeof(PqOp), q_bytes = qs.size() * sizeof(PqQuery), h_bytes = held.size() * sizeof(PqHeld);
     const size_t tbl_need = ops_bytes + q_bytes + h_bytes;
     if (net->pq_tbl_bytes < tbl_need) {
         CU(cudaStreamSynchronize(st));
@@ -2139,9 +2148,25 @@ static sgs_status_t persistent_impl(sgs_supernet_t *net, int n_queries, const sg
         qs[(size_t)t].x = din + (size_t)t * in_bytes;
         qs[(size_t)t].logits = reinterpret_cast<float *>(dout + (size_t)t * out_bytes);
     }
+    {   // the longest queries first, so that the last ones to be taken are short
+        std::vector<int> order((size_t)n_queries);
+        for (int t = 0; t < n_queries; t++) order[(size_t)t] = t;
+        std::stable_sort(order.begin(), order.end(), [&](int i, int j) { return plans[(size_t)i]->flops > plans[(size_t)j]->flops; });
+        std::vector<PqQuery> sorted;
+        sorted.reserve(qs.size());
+        for (int t : order) sorted.push_back(qs[(size_t)t]);
+        qs.swap(sorted);
+    }
     CU(cudaStreamSynchronize(st));  // the pinned table image may still be the source of an earlier call's copy
     if (tbl_need) {
-        std::memcpy(net->pq_h_tbl, ops.data(), ops_bytes);
+        for (const auto &kv : begin) {
+            const std::vector<PqOp> &list = kv.first->pq;
+            PqOp *dst = reinterpret_cast<PqOp *>(net->pq_h_tbl) + kv.second;
+            std::memcpy(dst, list.data(), list.size() * sizeof(PqOp));
+            for (size_t i = 0; i < list.size() && !held.empty(); i++)
+                for (const PqHeld &e : held)
+                    if (list[i].type == PQ_PW && list[i].w == e.w) { dst[i].cache_off = e.off; dst[i].cache_rows = e.rows; dst[i].ld2 = e.C; }
+        }
         std::memcpy(net->pq_h_tbl + ops_bytes, qs.data(), q_bytes);
         if (h_bytes) std::memcpy(net->pq_h_tbl + ops_bytes + q_bytes, held.data(), h_bytes);
     }
@@ -2169,7 +2194,7 @@ static sgs_status_t persistent_impl(sgs_supernet_t *net, int n_queries, const sg
         p.slot_bytes = slot_bytes; p.act_bytes = act_bytes;
         p.status = tc_status_word(net->device);
         LayerRange range(net, -1, "persistent SubNet kernel");
-        ce = subnet_kernel_launch(p, std::min(blocks_max, n_queries), st);
+        ce = subnet_kernel_launch(p, std::min(clusters, n_queries), team, st);
         net->kernel_launches++;
     }
     if (ce == cudaSuccess && host_buffers && n_queries) ce = cudaMemcpyAsync(logits, net->pq_stage_out, out_bytes * (size_t)n_queries, cudaMemcpyDeviceToHost, st);
@@ -2641,6 +2666,11 @@ sgs_status_t sgs_set_option(sgs_supernet_t *net, const char *name, long long val
             for (int i = 0; i < 4; i++) { net->prof_ms[i] = net->prof_bytes[i] = net->prof_flops[i] = 0; net->prof_launches[i] = 0; }
             net->prof_trace.clear();
         }
+        return SGS_OK;
+    }
+    if (n == "persistent_team") {
+        if (!in_set((int)value, {0, 1, 2, 4, 8, 16})) return fail(net, SGS_EINVAL, "persistent_team is 0, 1, 2, 4, 8 or 16");
+        net->persistent_team = (int)value;
         return SGS_OK;
     }
     if (n == "persistent_held_kb") {

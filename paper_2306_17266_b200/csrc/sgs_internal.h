@@ -283,9 +283,8 @@ cudaError_t tc_group_init(int device);
 void tc_group_entry(TcConvPlan &p, const ConvArgs &a);  // fills the plan's record for grouped launches
 
 cudaError_t subnet_kernel_init(int device);
-size_t subnet_kernel_smem();  // dynamic shared memory of a block
-int subnet_kernel_blocks_per_sm();
-cudaError_t subnet_kernel_launch(const PqParams &p, int blocks, cudaStream_t st);
+int subnet_kernel_clusters(int team);  // clusters of `team` blocks the device holds at a time (0: none)
+cudaError_t subnet_kernel_launch(const PqParams &p, int clusters, int team, cudaStream_t st);  // `team` blocks serve a query together
 size_t subnet_kernel_held_max();  // largest weight buffer a block can keep
 
 }  // namespace sgs

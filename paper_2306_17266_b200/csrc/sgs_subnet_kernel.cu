@@ -4,7 +4,10 @@
 // (Section 3.1, Section 4.2 "Persistent Buffer").  On this GPU a one-image MobileNetV3-sized SubNet is far too
 // small to fill the machine layer by layer: a wave of 32 such queries needs about a hundred dependent launches of
 // 10 - 20 us each.  Here the whole stream is ONE launch instead.  Every block (one per SM, 512 threads) takes the
-// next unserved query from a counter and runs all layers of that query's SubNet by itself, image to logits:
+// next unserved query from a counter and runs all layers of that query's SubNet by itself, image to logits.  With fewer queries
+// than SMs a query is served by a team of 2 to 16 blocks, a cluster: every layer's tiles, rows, pixels or outputs are dealt to
+// them, pooled vectors and gates go to all through distributed shared memory, and a cluster barrier ends a layer (8 queries:
+// 3.45 ms with a block each, 0.87 with 8; the choice is the host's, choose_team in sgs_api.cu).
 //   * pointwise (1x1) convolutions on the tensor cores: tcgen05.mma with the fp32 accumulator in tensor memory
 //     (two 256-column buffers, so the epilogue of one tile overlaps the MMAs of the next); the operands are
 //     brought into 128-byte-swizzled shared-memory tiles by the block's own threads with 16-byte asynchronous
@@ -12,15 +15,15 @@
 //     small and too many to be worth a tensor map each;
 //   * depthwise convolutions, the 3-channel stem, pooling, the squeeze-excite gate and the linear layers on the
 //     CUDA cores, with 16-byte accesses;
-//   * activations in a private scratch area of the block in global memory (written and read back by the same
-//     SM, so they stay in L1 / L2); pooled vectors and gates in shared memory.
+//   * activations in a private scratch area of the team in global memory (a query's fit L2); pooled vectors and gates in
+//     shared memory.
 //   * optionally a weight buffer in shared memory, filled once per block at the start of the launch with the
 //     cached SubGraph's boxes of the first pointwise layers (the first filters x first channels of their stored
 //     rows) and read in place by the MMAs of every query the block serves; filters and channels of a query's
 //     slice beyond the box are streamed through the ring as usual (the SubGraph-stationary dataflow of
 //     Section 4.3: what the queries share is fetched once, the rest per query).
-// Nothing waits on another block, so the kernel needs no co-scheduling guarantee; its only waits are on its own
-// copies and MMAs, and they are bounded like those of the other tensor-core kernels.
+// Nothing waits on a block of another team, so the kernel needs no co-scheduling guarantee beyond the cluster's own; a block's
+// other waits are on its copies and MMAs, and they are bounded like those of the other tensor-core kernels.
 // Slicing is the same as everywhere else in the library: the first K' filters and C' channels of the stored rows,
 // the centre k x k taps of a stored depthwise filter; no sliced copy of a weight exists.
 
@@ -33,7 +36,6 @@ namespace {
 using bf16 = __nv_bfloat16;
 
 constexpr int PQ_THREADS = 512;
-constexpr int PQ_BLOCKS_PER_SM = 1;          // (measured: two blocks of 256 threads per SM with 96-filter tiles serve 28k queries/s, one of 512 serves 42k)
 constexpr int PQ_WARPS = PQ_THREADS / 32;
 constexpr int PQ_ROWS = PQ_THREADS / 8;      // rows of 128 bytes one round of 16-byte copies covers
 constexpr int PQ_MAX_K = 1024;               // widest pointwise layer (folded batch norm staged in shared memory)
@@ -43,7 +45,26 @@ constexpr int PQ_LAG = 2;                    // copies run this many stages ahea
 constexpr int PQ_VEC = 1280;                 // longest fp32 vector held in shared memory (the head's width)
 constexpr int PQ_ACC_COLS = 256;             // tensor-memory columns of one accumulator buffer
 constexpr int PQ_HELD_MAX = 56 * 1024;       // largest weight buffer (dynamic shared memory beyond the ring)
+constexpr int PQ_MAX_CLUSTER = 16;
 constexpr unsigned long long PQ_WAIT_NS = 2000000000ull;
+
+// A query's blocks: `n` of them (a cluster), this one is number `rank`.  Every layer is split over them; what one block wrote the
+// others may read after sync().
+struct Team {
+    int rank, n;
+    __device__ __forceinline__ void sync() const {
+        if (n == 1) __syncthreads();
+        else asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+    }
+};
+// Address of this block's shared-memory location p in block `rank` of the cluster.
+__device__ __forceinline__ uint32_t in_block(const void *p, int rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_block(uint32_t addr, float v) { asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory"); }
+__device__ __forceinline__ void st_block(uint32_t addr, int v) { asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
 
 // Completed phases of the block's barriers since the kernel started (the same in every thread; only ever
 // indexed with constants, so they live in registers).
@@ -88,13 +109,17 @@ __device__ __forceinline__ float dot8w(uint4 wv, float4 x0, float4 x1, float s) 
 struct PwShape {
     int M, C, K, n_tiles, BN, cchunks, m_tiles, stage_bytes, S;
 };
-__device__ __forceinline__ PwShape pw_shape(const PqOp &op) {
+// Filter tiles: as few as PQ_MAX_BN allows, more where the pixel tiles alone leave blocks of the team idle (a 7x7 map is one
+// pixel tile).
+__device__ __forceinline__ PwShape pw_shape(const PqOp &op, const Team &team) {
     PwShape s;
     s.M = op.Ho * op.Wo; s.C = op.C; s.K = op.K;
-    s.n_tiles = (s.K + PQ_MAX_BN - 1) / PQ_MAX_BN;
-    s.BN = (((s.K + s.n_tiles - 1) / s.n_tiles) + 15) & ~15;  // MMA width: a multiple of 16, at most PQ_MAX_BN
-    s.cchunks = (s.C + 63) >> 6;
     s.m_tiles = (s.M + 127) >> 7;
+    s.n_tiles = (s.K + PQ_MAX_BN - 1) / PQ_MAX_BN;
+    if (s.n_tiles * s.m_tiles < team.n) s.n_tiles = min((s.K + 15) >> 4, (team.n + s.m_tiles - 1) / s.m_tiles);
+    s.BN = (((s.K + s.n_tiles - 1) / s.n_tiles) + 15) & ~15;  // MMA width: a multiple of 16, at most PQ_MAX_BN
+    s.n_tiles = (s.K + s.BN - 1) / s.BN;  // (the rounding may leave the last one empty)
+    s.cchunks = (s.C + 63) >> 6;
     s.stage_bytes = A_STAGE_BYTES + s.BN * 128;
     s.S = min(4, PQ_RING_BYTES / s.stage_bytes);
     return s;
@@ -168,11 +193,12 @@ __device__ __forceinline__ bool pw_epilogue(const PqOp &op, const PwShape &s, co
 // Returns false when a wait ran out (the caller leaves at its next block barrier).
 __device__ __forceinline__ bool pq_pointwise(const PqOp &op, const bf16 *x, const bf16 *res, bf16 *y, uint8_t *ring, float *bn,
                                              uint32_t held_u32, uint64_t *free_bar, uint64_t *acc_bar, uint32_t tmem_base, PipeState &ps,
-                                             volatile int *abort_flag) {
+                                             volatile int *abort_flag, const Team &team) {
     const int tid = threadIdx.x;
-    const PwShape s = pw_shape(op);
+    const PwShape s = pw_shape(op, team);
     const int S = s.S;
-    const int total = s.n_tiles * s.m_tiles * s.cchunks;
+    const int tiles = s.n_tiles * s.m_tiles, mine = tiles > team.rank ? (tiles - team.rank + team.n - 1) / team.n : 0;  // tile = rank + i * n
+    const int total = mine * s.cchunks;
     // instruction descriptor: fp32 accumulator, bf16 x bf16, both K-major, N = BN, M = 128
     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(s.BN >> 3) << 17) | ((uint32_t)(TILE_M >> 4) << 24);
     const uint32_t ring_u32 = smem_u32(ring);
@@ -193,8 +219,9 @@ __device__ __forceinline__ bool pq_pointwise(const PqOp &op, const bf16 *x, cons
     auto chunk_held = [&](int ch) { return hK > 0 && min(s.C, (ch + 1) * 64) <= op.ld2; };
 
     bool ok = true;
-    int p_chunk = 0, p_mt = 0, p_nt = 0, p_stage = 0;  // next iteration to copy
-    int c_chunk = 0, c_mt = 0, c_nt = 0, c_stage = 0;  // next iteration to multiply
+    int p_chunk = 0, p_nt = team.rank / s.m_tiles, p_mt = team.rank - p_nt * s.m_tiles, p_stage = 0;  // next iteration to copy
+    int c_chunk = 0, c_nt = p_nt, c_mt = p_mt, c_stage = 0;                                            // next iteration to multiply
+    auto next_tile = [&](int &mt, int &nt) { for (mt += team.n; mt >= s.m_tiles; mt -= s.m_tiles) ++nt; };
     int e_mt = -1, e_nt = 0;                           // finished tile whose epilogue is still to run
     uint32_t e_buf = 0;
     for (int i = 0; i < total + PQ_LAG; i++) {
@@ -237,7 +264,7 @@ __device__ __forceinline__ bool pq_pointwise(const PqOp &op, const bf16 *x, cons
                 e_mt = c_mt; e_nt = c_nt; e_buf = buf;
             }
             if (++c_stage == S) c_stage = 0;
-            if (++c_chunk == s.cchunks) { c_chunk = 0; if (++c_mt == s.m_tiles) { c_mt = 0; ++c_nt; } }
+            if (++c_chunk == s.cchunks) { c_chunk = 0; next_tile(c_mt, c_nt); }
         }
         if (i < total) {
             // the stage was last read by the MMAs of iteration i - S, issued in the previous step
@@ -258,7 +285,7 @@ __device__ __forceinline__ bool pq_pointwise(const PqOp &op, const bf16 *x, cons
                 cp16_ca(sb + (uint32_t)(row * 128) + piece, v ? w + (size_t)f * op.ld + c0 : w, v);
             }
             if (++p_stage == S) p_stage = 0;
-            if (++p_chunk == s.cchunks) { p_chunk = 0; if (++p_mt == s.m_tiles) { p_mt = 0; ++p_nt; } }
+            if (++p_chunk == s.cchunks) { p_chunk = 0; next_tile(p_mt, p_nt); }
         }
         cp_commit();  // (an empty group in the drain steps keeps the group count in step with i)
     }
@@ -279,7 +306,7 @@ __device__ __forceinline__ bool pq_pointwise(const PqOp &op, const bf16 *x, cons
 // L1: slower as well.)
 // ---------------------------------------------------------------------------------------------
 template <int K, int ST>
-__device__ __noinline__ void pq_depthwise(const PqOp &op, const bf16 *x, bf16 *y) {
+__device__ __noinline__ void pq_depthwise(const PqOp &op, const bf16 *x, bf16 *y, const Team team) {
     constexpr int TW = (ST == 2 && K > 3) ? 2 : 4;  // (the wide stride-2 windows would not fit the register budget of 512 threads)
     constexpr int NCOL = (TW - 1) * ST + K, P = (K - 1) / 2;
     constexpr int RU = K == 7 ? 1 : K;  // filter rows unrolled together (all 7 rows of the widest filter at once would spill)
@@ -287,7 +314,8 @@ __device__ __noinline__ void pq_depthwise(const PqOp &op, const bf16 *x, bf16 *y
     const int per_row = groups * wblocks, total = per_row * op.Ho;
     const int o = (op.R - K) / 2;
     const bf16 *__restrict__ w = static_cast<const bf16 *>(op.w);
-    for (int it = threadIdx.x; it < total; it += PQ_THREADS) {
+    const int end = (int)((long long)total * (team.rank + 1) / team.n);  // (a run of rows each)
+    for (int it = (int)((long long)total * team.rank / team.n) + threadIdx.x; it < end; it += PQ_THREADS) {
         const int ho = it / per_row, idx = it - ho * per_row;
         const int cg = idx % groups, wb = idx / groups;
         const int c0 = cg * 8, wo0 = wb * TW;
@@ -343,7 +371,7 @@ __device__ __noinline__ void pq_depthwise(const PqOp &op, const bf16 *x, bf16 *y
 
 // Stem: 3-channel image, k x k taps (k <= 3 here), stride `stride`, direct on the CUDA cores; a thread owns one
 // output pixel and produces the filters eight at a time.  wsm: k * k * 3 * K floats of shared memory.
-__device__ __noinline__ void pq_stem(const PqOp &op, const bf16 *img, bf16 *y, float *wsm) {
+__device__ __noinline__ void pq_stem(const PqOp &op, const bf16 *img, bf16 *y, float *wsm, const Team team) {
     const int k = op.k, K = op.K, taps = k * k * 3, o = (op.R - k) / 2, P = (k - 1) / 2;
     const bf16 *w = static_cast<const bf16 *>(op.w);
     for (int i = threadIdx.x; i < taps * K; i += PQ_THREADS) {
@@ -352,7 +380,7 @@ __device__ __noinline__ void pq_stem(const PqOp &op, const bf16 *img, bf16 *y, f
     }
     __syncthreads();
     const int npx = op.Ho * op.Wo;
-    for (int px = threadIdx.x; px < npx; px += PQ_THREADS) {
+    for (int px = team.rank * PQ_THREADS + threadIdx.x; px < npx; px += team.n * PQ_THREADS) {
         const int ho = px / op.Wo, wo = px - ho * op.Wo;
         float in[27];
 #pragma unroll
@@ -392,36 +420,50 @@ __device__ __noinline__ void pq_stem(const PqOp &op, const bf16 *img, bf16 *y, f
     }
 }
 
-// Global average pool into a shared-memory vector: a warp per 8-channel vector.
-__device__ __forceinline__ void pq_gap(const PqOp &op, const bf16 *x, float *out) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, cvecs = op.C >> 3, HW = op.H * op.W;
-    const float inv = 1.f / (float)HW;
-    for (int cv = warp; cv < cvecs; cv += PQ_WARPS) {
+// Global average pool into a shared-memory vector of every block of the team.  Neighbouring threads take neighbouring channels of a
+// pixel; a block sums its share of the pixels (thread by thread, then over the threads), the blocks' sums meet in part[rank][C].
+// All sums have a fixed order for a given team size.
+__device__ __forceinline__ void pq_gap(const PqOp &op, const bf16 *x, float *out, float *buf, float *part, const Team &team) {
+    const int cvecs = op.C >> 3, HW = op.H * op.W, lanes = PQ_THREADS / cvecs;  // (C <= PQ_VEC: at least 3 pixels at a time)
+    const int pl = threadIdx.x / cvecs, cv = threadIdx.x - pl * cvecs;
+    const int end = HW * (team.rank + 1) / team.n;
+    if (pl < lanes) {
         const bf16 *base = x + cv * 8;
         float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int i = lane; i < HW; i += 32) {
+        for (int i = HW * team.rank / team.n + pl; i < end; i += lanes) {
             const uint4 v = *reinterpret_cast<const uint4 *>(base + (size_t)i * op.C);
             const float2 a = unpack2(v.x), b = unpack2(v.y), c = unpack2(v.z), d = unpack2(v.w);
             acc[0] += a.x; acc[1] += a.y; acc[2] += b.x; acc[3] += b.y; acc[4] += c.x; acc[5] += c.y; acc[6] += d.x; acc[7] += d.y;
         }
-#pragma unroll
-        for (int j = 0; j < 8; j++) {
-#pragma unroll
-            for (int o = 16; o; o >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
-        }
-        if (lane == 0) {
-#pragma unroll
-            for (int j = 0; j < 8; j++) out[cv * 8 + j] = acc[j] * inv;
-        }
+        float4 *dst = reinterpret_cast<float4 *>(buf + (size_t)pl * op.C + cv * 8);
+        dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+        dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+    }
+    __syncthreads();
+    const float inv = 1.f / (float)HW;
+    for (int c = threadIdx.x; c < op.C; c += PQ_THREADS) {
+        float t = 0.f;
+        for (int i = 0; i < lanes; i++) t += buf[(size_t)i * op.C + c];
+        if (team.n == 1) out[c] = t * inv;
+        else
+            for (int r = 0; r < team.n; r++) st_block(in_block(part + (size_t)team.rank * PQ_VEC + c, r), t);
+    }
+    if (team.n == 1) return;
+    team.sync();
+    for (int c = threadIdx.x; c < op.C; c += PQ_THREADS) {
+        float t = 0.f;
+        for (int r = 0; r < team.n; r++) t += part[(size_t)r * PQ_VEC + c];
+        out[c] = t * inv;
     }
 }
 
 // y[j] = f(bias[j] + sum_c w[j][c] * v[c]) for j < K: a warp takes JB outputs at a time and has the 16-byte weight
-// loads of all of them in flight together.  HS: hard sigmoid (the squeeze-excite gate) instead of `act`.
-template <int JB, bool HS>
-__device__ __noinline__ void pq_matvec(const bf16 *w, int ld, const float *bias, const float *v, float *y, int C, int K, int act) {
+// loads of all of them in flight together; the outputs are dealt to the team's warps.  HS: hard sigmoid (the squeeze-excite gate)
+// instead of `act`.  SH: y is in shared memory, and every block of the team gets every output.
+template <int JB, bool HS, bool SH>
+__device__ __noinline__ void pq_matvec(const bf16 *w, int ld, const float *bias, const float *v, float *y, int C, int K, int act, const Team team) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int j0 = warp * JB; j0 < K; j0 += PQ_WARPS * JB) {
+    for (int j0 = (team.rank * PQ_WARPS + warp) * JB; j0 < K; j0 += team.n * PQ_WARPS * JB) {
         float s[JB];
 #pragma unroll
         for (int u = 0; u < JB; u++) s[u] = 0.f;
@@ -438,18 +480,19 @@ __device__ __noinline__ void pq_matvec(const bf16 *w, int ld, const float *bias,
         for (int u = 0; u < JB; u++) {
 #pragma unroll
             for (int o = 16; o; o >>= 1) s[u] += __shfl_xor_sync(0xffffffffu, s[u], o);
-            if (lane == 0 && j0 + u < K) {
-                const float t = s[u] + __ldg(bias + j0 + u);
-                y[j0 + u] = HS ? fminf(fmaxf(t + 3.f, 0.f), 6.f) / 6.f : act_fn(t, act);
+            if (j0 + u < K && lane < (SH ? team.n : 1)) {
+                const float t = s[u] + __ldg(bias + j0 + u), o = HS ? fminf(fmaxf(t + 3.f, 0.f), 6.f) / 6.f : act_fn(t, act);
+                if (SH && team.n > 1) st_block(in_block(y + j0 + u, lane), o);
+                else y[j0 + u] = o;
             }
         }
     }
 }
 
 // In-place squeeze-excite scale: x[p][c] *= gate[c].
-__device__ __forceinline__ void pq_scale(const PqOp &op, bf16 *x, const float *gate) {
+__device__ __forceinline__ void pq_scale(const PqOp &op, bf16 *x, const float *gate, const Team &team) {
     const int cvecs = op.C >> 3, total = op.H * op.W * cvecs;
-    for (int i = threadIdx.x; i < total; i += PQ_THREADS) {
+    for (int i = team.rank * PQ_THREADS + threadIdx.x; i < total; i += team.n * PQ_THREADS) {
         const int cv = i % cvecs;
         const uint4 v = *reinterpret_cast<const uint4 *>(x + (size_t)i * 8);
         const float4 g0 = *reinterpret_cast<const float4 *>(gate + cv * 8), g1 = *reinterpret_cast<const float4 *>(gate + cv * 8 + 4);
@@ -464,18 +507,21 @@ __device__ __forceinline__ void pq_scale(const PqOp &op, bf16 *x, const float *g
     }
 }
 
-__global__ void __launch_bounds__(PQ_THREADS, PQ_BLOCKS_PER_SM) subnet_kernel(const PqParams p) {
+__global__ void __launch_bounds__(PQ_THREADS, 1) subnet_kernel(const PqParams p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *ring = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     __shared__ __align__(16) float vec_s[3][PQ_VEC];
     __shared__ __align__(16) float bn_s[2 * PQ_MAX_K];
-    __shared__ __align__(16) PqOp op_s;
+    __shared__ __align__(16) PqOp op_s[2];  // this layer's record and the next one's
     __shared__ __align__(16) PqQuery q_s;
     __shared__ __align__(8) uint64_t free_bar[4], acc_bar[2];
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s, next_s;
     volatile int *abort_flag = &abort_s;
     const int tid = threadIdx.x, warp = tid >> 5;
+    Team team;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(team.rank));
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(team.n));
 
     if (tid == 0) {
         for (int s = 0; s < 4; s++) mbar_init(&free_bar[s], 1);
@@ -491,7 +537,7 @@ __global__ void __launch_bounds__(PQ_THREADS, PQ_BLOCKS_PER_SM) subnet_kernel(co
     const uint32_t tmem_base = tmem_base_s;
     PipeState ps;
     ps.use[0] = ps.use[1] = ps.use[2] = ps.use[3] = 0u; ps.acc[0] = ps.acc[1] = 0u; ps.tiles = 0u;
-    uint8_t *slot = p.scratch + (size_t)blockIdx.x * p.slot_bytes;
+    uint8_t *slot = p.scratch + (size_t)(blockIdx.x / team.n) * p.slot_bytes;
     bool ok = true;
     // the weight buffer: behind the ring, filled once
     const uint32_t held_u32 = p.n_held > 0 ? smem_u32(ring + PQ_RING_BYTES) : 0u;
@@ -513,77 +559,122 @@ __global__ void __launch_bounds__(PQ_THREADS, PQ_BLOCKS_PER_SM) subnet_kernel(co
         __syncthreads();
     }
 
+    // (in a team, a block whose wait ran out says so to all of them in front of a barrier, and all leave behind it)
+    team.sync();
     for (;;) {
-        if (tid == 0) next_s = atomicAdd(p.counter, 1);
-        __syncthreads();
+        if (team.rank == 0 && tid == 0) {
+            const int q = atomicAdd(p.counter, 1);
+            if (team.n == 1) next_s = q;
+            else
+                for (int r = 0; r < team.n; r++) st_block(in_block(&next_s, r), q);
+        }
+        team.sync();
         const int qi = next_s;
         if (qi >= p.n_queries || *abort_flag) break;
         if (tid < 2) reinterpret_cast<uint4 *>(&q_s)[tid] = __ldg(reinterpret_cast<const uint4 *>(p.queries + qi) + tid);
         __syncthreads();
         const int op_begin = q_s.op_begin, op_count = q_s.op_count;
+        auto fetch_op = [&](int oi) {
+            if (tid >= PQ_THREADS - 8 && oi < op_count) {
+                const int i = tid - (PQ_THREADS - 8);
+                reinterpret_cast<uint4 *>(&op_s[oi & 1])[i] = __ldg(reinterpret_cast<const uint4 *>(p.ops + op_begin + oi) + i);
+            }
+        };
+        fetch_op(0);
+        __syncthreads();
         for (int oi = 0; oi < op_count; oi++) {
-            __syncthreads();  // the previous layer is complete: its outputs are visible, its record is free
-            if (*abort_flag) break;
-            if (tid < 8) reinterpret_cast<uint4 *>(&op_s)[tid] = __ldg(reinterpret_cast<const uint4 *>(p.ops + op_begin + oi) + tid);
-            __syncthreads();
-            const PqOp &op = op_s;
+            const PqOp &op = op_s[oi & 1];
+            fetch_op(oi + 1);  // (its place held the layer before this one)
             const bf16 *x = op.in < 0 ? static_cast<const bf16 *>(q_s.x) : reinterpret_cast<const bf16 *>(slot + (size_t)op.in * p.act_bytes);
             bf16 *y = op.out < 0 ? nullptr : reinterpret_cast<bf16 *>(slot + (size_t)op.out * p.act_bytes);
             const bf16 *res = op.res < 0 ? nullptr : reinterpret_cast<const bf16 *>(slot + (size_t)op.res * p.act_bytes);
             switch (op.type) {
-            case PQ_STEM: pq_stem(op, x, y, reinterpret_cast<float *>(ring)); break;
-            case PQ_PW: ok = pq_pointwise(op, x, res, y, ring, bn_s, held_u32, free_bar, acc_bar, tmem_base, ps, abort_flag) && ok; break;
+            case PQ_STEM: pq_stem(op, x, y, reinterpret_cast<float *>(ring), team); break;
+            case PQ_PW: ok = pq_pointwise(op, x, res, y, ring, bn_s, held_u32, free_bar, acc_bar, tmem_base, ps, abort_flag, team) && ok; break;
             case PQ_DW:
                 if (op.stride == 1) {
-                    if (op.k == 3) pq_depthwise<3, 1>(op, x, y);
-                    else if (op.k == 5) pq_depthwise<5, 1>(op, x, y);
-                    else pq_depthwise<7, 1>(op, x, y);
+                    if (op.k == 3) pq_depthwise<3, 1>(op, x, y, team);
+                    else if (op.k == 5) pq_depthwise<5, 1>(op, x, y, team);
+                    else pq_depthwise<7, 1>(op, x, y, team);
                 } else {
-                    if (op.k == 3) pq_depthwise<3, 2>(op, x, y);
-                    else if (op.k == 5) pq_depthwise<5, 2>(op, x, y);
-                    else pq_depthwise<7, 2>(op, x, y);
+                    if (op.k == 3) pq_depthwise<3, 2>(op, x, y, team);
+                    else if (op.k == 5) pq_depthwise<5, 2>(op, x, y, team);
+                    else pq_depthwise<7, 2>(op, x, y, team);
                 }
                 break;
-            case PQ_GAP: pq_gap(op, x, vec_s[op.vout]); break;
+            case PQ_GAP: pq_gap(op, x, vec_s[op.vout], reinterpret_cast<float *>(ring), reinterpret_cast<float *>(ring) + PQ_THREADS * 8, team); break;
             case PQ_SE_GATE:
                 // first FC (ReLU) into the third vector, second FC (hard sigmoid) into the gate
-                pq_matvec<4, false>(static_cast<const bf16 *>(op.w), op.ld, op.shift, vec_s[op.vin], vec_s[2], op.C, op.K, ACT_RELU);
-                __syncthreads();
-                pq_matvec<8, true>(static_cast<const bf16 *>(op.w2), op.ld2, op.bias2, vec_s[2], vec_s[op.vout], op.K, op.C, 0);
+                pq_matvec<4, false, true>(static_cast<const bf16 *>(op.w), op.ld, op.shift, vec_s[op.vin], vec_s[2], op.C, op.K, ACT_RELU, team);
+                team.sync();
+                pq_matvec<8, true, true>(static_cast<const bf16 *>(op.w2), op.ld2, op.bias2, vec_s[2], vec_s[op.vout], op.K, op.C, 0, team);
                 break;
-            case PQ_SCALE: pq_scale(op, y, vec_s[op.vin]); break;
+            case PQ_SCALE: pq_scale(op, y, vec_s[op.vin], team); break;
             case PQ_LINEAR:
-                pq_matvec<8, false>(static_cast<const bf16 *>(op.w), op.ld, op.shift, vec_s[op.vin], op.vout < 0 ? q_s.logits : vec_s[op.vout], op.C, op.K, op.act);
+                if (op.vout < 0) pq_matvec<8, false, false>(static_cast<const bf16 *>(op.w), op.ld, op.shift, vec_s[op.vin], q_s.logits, op.C, op.K, op.act, team);
+                else pq_matvec<8, false, true>(static_cast<const bf16 *>(op.w), op.ld, op.shift, vec_s[op.vin], vec_s[op.vout], op.C, op.K, op.act, team);
                 break;
             default: break;
             }
+            if (team.n > 1 && tid == 0 && *abort_flag)
+                for (int r = 0; r < team.n; r++) st_block(in_block(&abort_s, r), 1);
+            team.sync();  // the layer is complete: its outputs are visible, its record is free
+            if (*abort_flag) break;
         }
-        __syncthreads();  // (also keeps next_s and q_s until every thread is done with them)
         if (*abort_flag) break;
     }
-    // (every thread left the loops after the same block barrier; the flag is only written inside waits)
+    // (every thread left the loops after the same barrier; the flag is only written inside waits and in front of barriers)
     tc_fence_before();
-    __syncthreads();
+    team.sync();  // (nobody leaves while another block may still write to its shared memory)
     if (warp == 0) tmem_dealloc(tmem_base, 2 * PQ_ACC_COLS);
     if (tid == 0 && (*abort_flag || !ok)) atomicExch(p.status, 1);
 }
 
 }  // namespace
 
-size_t subnet_kernel_smem() { return (size_t)PQ_RING_BYTES + 1024; }
 size_t subnet_kernel_held_max() { return (size_t)PQ_HELD_MAX; }
-int subnet_kernel_blocks_per_sm() { return PQ_BLOCKS_PER_SM; }
+
+static size_t subnet_kernel_smem() { return (size_t)PQ_RING_BYTES + 1024; }
 
 cudaError_t subnet_kernel_init(int device) {
     (void)device;
-    return cudaFuncSetAttribute(subnet_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(subnet_kernel_smem() + PQ_HELD_MAX));
+    const cudaError_t e = cudaFuncSetAttribute(subnet_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(subnet_kernel_smem() + PQ_HELD_MAX));
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(subnet_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
 }
 
-cudaError_t subnet_kernel_launch(const PqParams &p, int blocks, cudaStream_t st) {
-    if (blocks <= 0) return cudaSuccess;
-    if (p.held_bytes > (unsigned)PQ_HELD_MAX || (p.held_bytes & 1023u)) return cudaErrorInvalidValue;
-    subnet_kernel<<<blocks, PQ_THREADS, subnet_kernel_smem() + (p.n_held > 0 ? p.held_bytes : 0u), st>>>(p);
-    return cudaGetLastError();
+static void subnet_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &attr, int clusters, int team, unsigned held_bytes, cudaStream_t st) {
+    cfg = {};
+    cfg.gridDim = dim3((unsigned)(clusters * team));
+    cfg.blockDim = dim3(PQ_THREADS);
+    cfg.dynamicSmemBytes = subnet_kernel_smem() + held_bytes;
+    cfg.stream = st;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)team; attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+}
+
+// (a block has its SM to itself whatever its weight buffer: asked once per device and team, the question takes some 100 us)
+int subnet_kernel_clusters(int team) {
+    static std::atomic<int> known[64][PQ_MAX_CLUSTER + 1];  // answer + 1
+    int dev = 0, n = 0;
+    if (team < 1 || team > PQ_MAX_CLUSTER || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    if ((n = known[dev][team].load(std::memory_order_relaxed)) > 0) return n - 1;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    subnet_config(cfg, attr, 1, team, (unsigned)PQ_HELD_MAX, nullptr);
+    if (cudaOccupancyMaxActiveClusters(&n, subnet_kernel, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+    known[dev][team].store(n + 1, std::memory_order_relaxed);
+    return n;
+}
+
+cudaError_t subnet_kernel_launch(const PqParams &p, int clusters, int team, cudaStream_t st) {
+    if (clusters <= 0) return cudaSuccess;
+    if (team < 1 || team > PQ_MAX_CLUSTER || p.held_bytes > (unsigned)PQ_HELD_MAX || (p.held_bytes & 1023u)) return cudaErrorInvalidValue;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    subnet_config(cfg, attr, clusters, team, p.n_held > 0 ? p.held_bytes : 0u, st);
+    return cudaLaunchKernelEx(&cfg, subnet_kernel, p);
 }
 
 }  // namespace sgs
