@@ -179,12 +179,8 @@ struct sgs_supernet {
     size_t weight_arena_bytes = 0;
     float *param_arena = nullptr;  // folded scale / shift
     size_t param_arena_bytes = 0;
-    // bf16 handles: the stem's weights once more as a GEMM operand [K][stem_kkp] (rows = the stored
-    // (r, s, c) order, zero padded to a multiple of 8), used with the patch matrix of the input
-    void *stem_gemm_w = nullptr;
-    int stem_kkp = 0;
-    // ... and as [K][k][64] for the window view used by waves: per filter row an 8-pixel x 8-channel window
-    void *stem_win_w = nullptr;
+    // bf16 handles: the stem's weights once more, filter rows padded to whole 16-byte pieces (sgs_stem.cu)
+    void *stem_rows_w = nullptr;
     // Workspaces of the queries in flight.  Queries of a stream are independent, so up to
     // `concurrency` of them run at the same time, each in its own slot (own activation buffers, own
     // CUDA stream); slot 0 runs on the caller's stream.
@@ -466,53 +462,29 @@ struct Builder {
         H = a.Ho; W = a.Wo;
         plan->ops.push_back(op);
     }
-    // Stem (3 input channels): on bf16 handles with a filter count that is a multiple of 8 it runs on the
-    // tensor cores as patch matrix (tmp) x GEMM weights; otherwise as a direct convolution.
-    void stem(const std::string &name, int out, int tmp, int &H, int &W, int stride, int act) {
+    // Stem (3 input channels), and the max pool behind it: on bf16 handles with a filter count that is a multiple of 8 one launch on
+    // the tensor cores, otherwise a direct convolution (and a pool).
+    void stem(const std::string &name, int out, int tmp, int &H, int &W, int stride, int act, bool pool) {
         const int li = net->idx(name);
-        const StoredLayer &L = net->layers[li];
         const Slice &s = plan->slices[li];
-        const size_t first = plan->ops.size();
         const int Hin = H, Win = W;
-        conv(name, -1, out, -1, H, W, stride, act);
-        // (the patch-matrix kernel stages whole input rows with 16-byte loads: widths that are multiples of 8)
-        if (net->throughput_mode == 2 && net->stem_win_w && !net->force_plain && s.K % 8 == 0 && (s.k == 3 || s.k == 7)) {
-            // Waves: no patch matrix.  The image is copied once into an 8-channel buffer with a zero margin
-            // (16 bytes per pixel, so that pixels can be TMA rows); the 64 contiguous elements that start at
-            // padded pixel wo * stride are the 8-pixel window of output column wo, and the stem becomes a
-            // convolution over the k filter ROWS with 64 "channels" per row.
-            Op &cv = plan->ops[first];
-            const int P = (s.k - 1) / 2;
-            int Hp = std::max((H - 1) * stride + s.k, Hin + P), Wp = std::max((W - 1) * stride + 8, Win + P);
-            Hp += Hp & 1; Wp += Wp & 1;
-            Op pd;
-            pd.type = OP_PAD8; pd.layer = li; pd.in = -1; pd.out = tmp;
-            pd.N = N; pd.H = Hin; pd.W = Win; pd.C = 3; pd.K = P;
-            pd.conv.Ho = Hp; pd.conv.Wo = Wp;
-            pd.alg_bytes = ((double)N * Hin * Win * 3 + (double)N * Hp * Wp * 8) * net->elem();
-            cv.in = tmp;
-            ConvArgs &a = cv.conv;
-            a.w = net->stem_win_w;
-            a.H = Hp; a.W = Wp; a.C = 64; a.Cmax = 64; a.win = 1; a.ldx = 0;
-            note((size_t)N * Hp * Wp * 8);
-            plan->ops.insert(plan->ops.begin() + (long)first, pd);
+        conv(name, -1, pool ? tmp : out, -1, H, W, stride, act);
+        Op &cv = plan->ops.back();
+        const int Hp = (H - 1) / 2 + 1, Wp = (W - 1) / 2 + 1, C = phys(s.K);
+        if (net->stem_rows_w && !net->force_plain && s.k == net->layers[li].R && s.K % 8 == 0 && stem_supported(s.k, stride, pool, s.K, C, act, N, Hin, Win)) {
+            cv.type = OP_STEM; cv.out = out;
+            cv.N = N; cv.H = Hin; cv.W = Win; cv.C = 3; cv.K = s.K; cv.act = act;
+            if (pool) { H = Hp; W = Wp; }
+            note((size_t)N * H * W * C);
             return;
         }
-        if (!net->stem_gemm_w || net->force_plain || s.K % 8 || (s.k != 3 && s.k != 7) || Win % 8 || Win > 1024) return;
-        Op &cv = plan->ops[first];
-        const int KKp = net->stem_kkp;
-        Op im;
-        im.type = OP_IM2COL; im.layer = li; im.in = -1; im.out = tmp;
-        im.N = N; im.H = Hin; im.W = Win; im.C = 3; im.K = KKp;
-        im.conv = cv.conv;  // geometry (k, stride, output dims)
-        im.alg_bytes = ((double)N * Hin * Win * 3 + (double)N * H * W * KKp) * net->elem();
-        cv.in = tmp;
-        ConvArgs &a = cv.conv;
-        a.w = net->stem_gemm_w;
-        a.H = H; a.W = W; a.C = KKp; a.Cmax = KKp; a.R = 1; a.k = 1; a.stride = 1;
-        note((size_t)N * H * W * KKp);
-        plan->ops.insert(plan->ops.begin() + (long)first, im);
-        (void)L;
+        if (!pool) return;
+        Op op;
+        op.type = OP_MAXPOOL; op.in = tmp; op.out = out; op.N = N; op.H = H; op.W = W; op.C = C;
+        op.alg_bytes = ((double)N * H * W + (double)N * Hp * Wp) * s.K * net->elem();
+        plan->ops.push_back(op);
+        H = Hp; W = Wp;
+        note((size_t)N * H * W * C);
     }
     void linear(const std::string &name, int vin, int vout, int act, bool vin_padded = false) {
         int li = net->idx(name);
@@ -564,18 +536,17 @@ sgs_status_t build_plan(sgs_supernet *net, const sgs_subnet_cfg_t *cfg, int batc
     Builder B{net, plan, batch};
     B.split_se = split_se;
     // ResNet-shaped family on bf16 handles: every convolution runs on the tensor cores (all channel counts are multiples of
-    // 8, every stride-2 layer sees at least 2x2 pixels, and single queries have the patch-matrix stem), so the activation
+    // 8, every stride-2 layer sees at least 2x2 pixels), so the activation
     // tensors can be padded to 16-channel pixels: the copy unit moves rows that start or end inside a 32-byte sector at a
     // third of the rate (0.35 us per 24 KB stage of a query's small layers).  choose_impls refuses a padded plan otherwise.
-    const bool stem_tc = net->throughput_mode == 2 ? net->stem_win_w != nullptr : (net->stem_gemm_w != nullptr && res % 8 == 0 && res <= 1024);
-    B.padded = net->family == SGS_RESNET && stem_tc && net->dtype == SGS_BF16 && !net->force_plain &&
+    B.padded = net->family == SGS_RESNET && net->stem_rows_w && net->dtype == SGS_BF16 && !net->force_plain &&
                tc_available() && (res >= 64 || res % 32 == 0) && net->pad_channels;
     plan->padded = B.padded;
     int H = res, W = res;
     // activation buffers: X current tensor, T1/T2 temporaries, SC shortcut
     int X = 0, T1 = 1, T2 = 2, SC = 3;
     if (net->family == SGS_TINY) {
-        B.stem("stem", X, T1, H, W, 1, ACT_RELU);
+        B.stem("stem", X, T1, H, W, 1, ACT_RELU, false);
         for (int s = 0; s < 3; s++)
             for (int b = 0; b < cfg->depth[s]; b++) {
                 int st = b == 0 ? d.stride[s] : 1, shortcut = X;
@@ -589,16 +560,7 @@ sgs_status_t build_plan(sgs_supernet *net, const sgs_subnet_cfg_t *cfg, int batc
         B.gap(X, 0, H, W, C);
         B.linear("fc", 0, -1, ACT_NONE);
     } else if (net->family == SGS_RESNET) {
-        B.stem("stem", T1, T2, H, W, 2, ACT_RELU);
-        {
-            Op op;
-            op.type = OP_MAXPOOL; op.in = T1; op.out = X; op.N = batch; op.H = H; op.W = W; op.C = B.phys(plan->slices[net->idx("stem")].K);
-            int Hp = (H - 1) / 2 + 1, Wp = (W - 1) / 2 + 1;
-            op.alg_bytes = ((double)batch * H * W + (double)batch * Hp * Wp) * plan->slices[net->idx("stem")].K * net->elem();
-            plan->ops.push_back(op);
-            H = Hp; W = Wp;
-            B.note((size_t)batch * H * W * op.C);
-        }
+        B.stem("stem", X, T1, H, W, 2, ACT_RELU, true);
         for (int s = 0; s < 4; s++)
             for (int b = 0; b < cfg->depth[s]; b++) {
                 int st = b == 0 ? d.stride[s] : 1, shortcut = X;
@@ -613,7 +575,7 @@ sgs_status_t build_plan(sgs_supernet *net, const sgs_subnet_cfg_t *cfg, int batc
         B.gap(X, 0, H, W, C);
         B.linear("fc", 0, -1, ACT_NONE, B.padded);
     } else {
-        B.stem("stem", X, T1, H, W, 2, ACT_HSWISH);
+        B.stem("stem", X, T1, H, W, 2, ACT_HSWISH, false);
         { int h = H, w = W; B.conv("first.dw", X, T1, -1, h, w, 1, ACT_RELU); }
         { int h = H, w = W; B.conv("first.pw", T1, T2, X, h, w, 1, ACT_NONE); }
         std::swap(X, T2);
@@ -750,7 +712,6 @@ sgs_status_t choose_impls(sgs_supernet *net, Plan *plan) {
         if (net->dtype != SGS_BF16 || net->force_plain || !tc_available()) continue;
         std::string why;
         op.tc = tc_conv_prepare(op.conv, net->device, &why);
-        if (!op.tc && op.conv.win) return fail(net, SGS_EUNSUPPORTED, "window view of the stem: " + why);
         if (!op.tc && plan->padded) return fail(net, SGS_EUNSUPPORTED, "padded activation layout needs the tensor-core kernel: " + why);
         if (op.tc) op.impl = 1;
     }
@@ -793,22 +754,16 @@ sgs_status_t ensure_ranks(sgs_supernet *net) {
         for (int b = 0; b < SGS_MAX_BLOCKS; b++) { c.expand[s][b] = net->family == SGS_MBV3 ? 6.0f : 0.35f; c.kernel[s][b] = 7; }
     }
     c.width[0] = 1.0f;
-    // (the stem has two forms too, patch matrix + GEMM and padded copy + window view, never in one wave: the same ranks)
-    struct RestoreMode {
-        sgs_supernet *net;
-        int mode;
-        ~RestoreMode() { net->throughput_mode = mode; }
-    } restore{net, net->throughput_mode};
     std::unordered_map<long long, int> rank;
-    for (int m : {0, 2}) {
-        net->throughput_mode = m;
-        Plan p;
-        sgs_status_t st = build_plan(net, &c, 1, 64, &p, true);
-        if (st != SGS_OK) return st;
-        int next = 0;
-        for (size_t i = 0; i < p.ops.size(); i++) {
-            rank.emplace(op_key(p, i), next++);
-            if (p.ops[i].type == OP_SCALE) rank.emplace(((long long)OP_SE << 32) | (unsigned)p.ops[i - 1].layer, next++);  // (behind its gate)
+    Plan p;
+    sgs_status_t st = build_plan(net, &c, 1, 64, &p, true);
+    if (st != SGS_OK) return st;
+    int next = 0;
+    for (size_t i = 0; i < p.ops.size(); i++) {
+        rank.emplace(op_key(p, i), next++);
+        if (p.ops[i].type == OP_SCALE) rank.emplace(((long long)OP_SE << 32) | (unsigned)p.ops[i - 1].layer, next++);  // (behind its gate)
+        if (p.ops[i].type == OP_STEM) {  // a narrower stem (12 filters) is a direct convolution
+            rank.emplace(((long long)OP_CONV << 32) | (unsigned)p.ops[i].layer, next++);
         }
     }
     net->op_rank.swap(rank);
@@ -881,15 +836,15 @@ SmallEntry small_entry(const sgs_supernet *net, const Plan *plan, const Op &op, 
         e.N = op.N; e.H = op.H; e.W = op.W; e.C = op.C; e.K = op.K;
         break;
     }
-    case OP_PAD8:
+    case OP_STEM: {
+        const StoredLayer &L = net->layers[op.layer];
         e.x = d_input; e.y = sl.act[op.out];
-        e.N = op.N; e.H = op.H; e.W = op.W; e.C = 3; e.k = op.K; e.Ho = op.conv.Ho; e.Wo = op.conv.Wo;
+        e.w = net->stem_rows_w; e.w2 = L.scale; e.bias2 = L.shift;
+        e.N = op.N; e.H = op.H; e.W = op.W; e.C = 3; e.K = op.K; e.act = op.act;
+        e.ld = op.conv.ldy ? op.conv.ldy : op.K;
+        e.Ho = op.conv.Ho; e.Wo = op.conv.Wo; e.k = op.conv.k; e.stride = op.conv.stride;
         break;
-    case OP_IM2COL:
-        e.x = d_input; e.y = sl.act[op.out];
-        e.N = op.N; e.H = op.H; e.W = op.W; e.C = 3;
-        e.Ho = op.conv.Ho; e.Wo = op.conv.Wo; e.k = op.conv.k; e.stride = op.conv.stride; e.KKp = op.K;
-        break;
+    }
     default: break;
     }
     return e;
@@ -918,8 +873,7 @@ sgs_status_t launch_op(sgs_supernet *net, Plan *plan, Op &op, const void *d_inpu
         net->kernel_launches++;
         break;
     }
-    case OP_PAD8:
-    case OP_IM2COL: {
+    case OP_STEM: {
         SmallEntry e = small_entry(net, plan, op, d_input, d_logits);
         CU(launch_small(op.type, &e, nullptr, 1, st));
         net->kernel_launches++;
@@ -985,7 +939,7 @@ void fold_profile(sgs_supernet *net) {
         if (plan->prof_ev.size() != 2 * plan->ops.size()) continue;
         for (size_t oi = 0; oi < plan->ops.size(); oi++) {
             const Op &op = plan->ops[oi];
-            const int cls = op.type == OP_CONV ? (op.impl == 1 ? 0 : 1) : op.type == OP_DW ? 2 : 3;
+            const int cls = op.type == OP_STEM ? 0 : op.type == OP_CONV ? (op.impl == 1 ? 0 : 1) : op.type == OP_DW ? 2 : 3;
             float ms = 0;
             if (cudaEventElapsedTime(&ms, plan->prof_ev[2 * oi], plan->prof_ev[2 * oi + 1]) == cudaSuccess) {
                 net->prof_ms[cls] += ms; net->prof_bytes[cls] += op.alg_bytes; net->prof_flops[cls] += op.flops;
@@ -1349,13 +1303,9 @@ sgs_status_t sgs_supernet_load(const sgs_arch_desc_t *arch, const void *host_blo
     }
     if (e == cudaSuccess && bf && !net->layers.empty() && net->layers[0].kind == KIND_CONV && net->layers[0].C == 3) {
         const StoredLayer &L = net->layers[0];
-        const int KK = L.R * L.R * 3;
-        net->stem_kkp = (KK + 15) / 16 * 16;  // (rows of whole 32-byte sectors)
-        if (dev_alloc(net, &net->stem_gemm_w, (size_t)L.K * net->stem_kkp * 2) != SGS_OK) e = cudaErrorMemoryAllocation;
-        else e = launch_stem_gemm_weights(L.w, net->stem_gemm_w, L.K, KK, net->stem_kkp, 0);
-        if (e == cudaSuccess && L.R <= 8) {
-            if (dev_alloc(net, &net->stem_win_w, (size_t)L.K * L.R * 64 * 2) != SGS_OK) e = cudaErrorMemoryAllocation;
-            else e = launch_stem_window_weights(L.w, net->stem_win_w, L.K, L.R, 0);
+        if (L.R == 3 || L.R == 7) {
+            if (dev_alloc(net, &net->stem_rows_w, stem_rows_bytes(L.R)) != SGS_OK) e = cudaErrorMemoryAllocation;
+            else e = launch_stem_rows(L.w, net->stem_rows_w, L.K, L.R, 0);
         }
     }
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -1390,8 +1340,7 @@ void sgs_supernet_free(sgs_supernet_t *net) {
     net->prof_used.clear();
     cudaFree(net->weight_arena);
     cudaFree(net->param_arena);
-    cudaFree(net->stem_gemm_w);
-    cudaFree(net->stem_win_w);
+    cudaFree(net->stem_rows_w);
     for (auto &c : net->act_chunks) cudaFree(c.first);
     for (auto &sl : net->slots) {
         for (int i = 0; i < 3; i++) cudaFree(sl.vec[i]);
@@ -1713,7 +1662,7 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
             // member's op has the vectorised form; the remaining ops run member by member
             const Op &op0 = plans[b[0].first]->ops[(size_t)b[0].second];
             const int kind = op0.type;
-            bool grouped = kind == OP_MAXPOOL || kind == OP_GAP || kind == OP_LINEAR || kind == OP_IM2COL || kind == OP_SCALE || kind == OP_SE_GATE || kind == OP_PAD8 || kind == OP_SE;
+            bool grouped = kind == OP_MAXPOOL || kind == OP_GAP || kind == OP_LINEAR || kind == OP_STEM || kind == OP_SCALE || kind == OP_SE_GATE || kind == OP_SE;
             if (grouped) {
                 const size_t off0 = off;
                 for (const auto &mo : b) {
@@ -1802,7 +1751,7 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
             if (!net->profile) return;
             for (const auto &mo : buckets[(size_t)rank]) {
                 const Op &op = plans[mo.first]->ops[(size_t)mo.second];
-                if ((op.type == OP_CONV && op.impl == 1) != tc) continue;
+                if (((op.type == OP_CONV && op.impl == 1) || op.type == OP_STEM) != tc) continue;
                 *bytes += op.alg_bytes; *fl += op.flops;
             }
         };
@@ -1840,10 +1789,11 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
                 continue;
             }
             if (L.small_kind >= 0) {
-                bucket_cost(L.rank, false, &pb, &pf);
-                if ((rc = prof_begin(3, pb, pf, first_layer(L.rank), L.count, 0)) != SGS_OK) break;
-                CU(launch_small(L.small_kind, reinterpret_cast<const SmallEntry *>(cx.h_tbl + L.off),
-                                reinterpret_cast<const SmallEntry *>(cx.d_tbl + L.off), L.count, ws));
+                const bool stem = L.small_kind == OP_STEM;  // (a tensor-core convolution)
+                bucket_cost(L.rank, stem, &pb, &pf);
+                const SmallEntry *recs = reinterpret_cast<const SmallEntry *>(cx.h_tbl + L.off);
+                if ((rc = prof_begin(stem ? 0 : 3, pb, pf, first_layer(L.rank), L.count, stem ? (int)(stem_tiles(recs[0]) * L.count) : 0)) != SGS_OK) break;
+                CU(launch_small(L.small_kind, recs, reinterpret_cast<const SmallEntry *>(cx.d_tbl + L.off), L.count, ws));
                 if ((rc = prof_end()) != SGS_OK) break;
                 net->kernel_launches++;
                 continue;
@@ -1929,8 +1879,7 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
 // ---------------------------------------------------------------------------------------------
 // Persistent execution (sgs_stream_opts_t::persistent): the whole stream is one launch of the SubNet kernel.
 // ---------------------------------------------------------------------------------------------
-// The plan of a config as the op list the kernel interprets (one record per layer; the patch-matrix / padding ops
-// that the layer-by-layer paths put in front of the stem are dropped, the kernel convolves the image directly).
+// The plan of a config as the op list the kernel interprets (one record per layer).
 static sgs_status_t build_pq_ops(sgs_supernet *net, Plan *plan) {
     std::vector<PqOp> list;  // (the plan gets it when it is complete)
     const int stem_li = net->idx("stem");
@@ -1941,8 +1890,7 @@ static sgs_status_t build_pq_ops(sgs_supernet *net, Plan *plan) {
         q.in = q.out = q.res = q.vin = q.vout = -1;
         q.cache_off = -1;
         switch (op.type) {
-        case OP_IM2COL:
-        case OP_PAD8: continue;
+        case OP_STEM:
         case OP_CONV: {
             const StoredLayer &L = net->layers[op.layer];
             const Slice &s = plan->slices[op.layer];

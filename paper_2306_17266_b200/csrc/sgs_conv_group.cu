@@ -527,7 +527,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
 
 // Number of activation views a member needs: the four parity views only when a stride-2 kernel
 // reaches odd offsets, i.e. for kernels larger than 1x1.
-static int views_of(const TcParams &p) { return (p.stride == 2 && p.k > 1) ? 4 : 1; }  // (a stride-2 window view uses views 0 and 2 of 4)
+static int views_of(const TcParams &p) { return (p.stride == 2 && p.k > 1) ? 4 : 1; }
 
 struct GroupLaunch::Impl {
     GroupParams<TC_GROUP_MAPS_LARGE> prm;  // host image of the parameter block (the small variant is a prefix)
@@ -583,7 +583,7 @@ void tc_group_entry(TcConvPlan &pl, const ConvArgs &a) {
     e.swap = (unsigned char)pl.swap;
     e.bn_tile = (short)(pl.swap ? (e.pix_rows + 15) / 16 * 16 : pl.bn_tile);
     e.k = (unsigned char)p.k; e.kw = (unsigned char)pl.kw; e.stride = (unsigned char)p.stride; e.p = (unsigned char)p.p; e.act = (unsigned char)p.act;
-    e.can_pair = !pl.swap && !a.win && e.mtiles == 1 && e.pix_rows <= 64;
+    e.can_pair = !pl.swap && e.mtiles == 1 && e.pix_rows <= 64;
     std::memcpy(pl.entry, &e, sizeof e);
     pl.g_iters = p.iters;
     pl.g_col_rows = pl.swap ? e.pix_rows : e.bn_tile;

@@ -608,7 +608,7 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
     auto no = [&](const char *msg) { if (why) *why = msg; return std::shared_ptr<TcConvPlan>(); };
     if (!encode_fn()) return no("cuTensorMapEncodeTiled unavailable");
     if (a.C % 8 || a.K % 8 || a.Cmax % 8) return no("channel counts must be multiples of 8");
-    if (a.i8 && ((a.ldx ? a.ldx : a.C) % 16 || a.C % 8 || a.Cmax % 16 || a.throughput || a.win || (a.ldy && (a.ldy % 16 || a.ldy < a.K || a.ldy - a.K >= 16)) || (!a.ldy && a.K % 8)))
+    if (a.i8 && ((a.ldx ? a.ldx : a.C) % 16 || a.C % 8 || a.Cmax % 16 || a.throughput || (a.ldy && (a.ldy % 16 || a.ldy < a.K || a.ldy - a.K >= 16)) || (!a.ldy && a.K % 8)))
         return no("8-bit layers: pixels in multiples of 16 bytes, single launches");
     if (a.C < 8 || a.K < 8) return no("too few channels");
     if (!conv_index_fits(a)) return no("more pixels or reduction steps than 32 bits number");
@@ -627,11 +627,6 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
     p.N = a.N; p.Ho = a.Ho; p.Wo = a.Wo; p.K = a.K; p.C = a.C;
     p.k = a.k; p.stride = a.stride; p.R = a.R; p.o = (a.R - a.k) / 2; p.p = (a.k - 1) / 2;
     plan->kw = a.k;
-    if (a.win) {
-        // window view of a stem: taps = the k filter rows, no arithmetic padding (the margin is in the buffer)
-        if (a.throughput != 2 || a.C != CHUNK_C || a.Cmax != CHUNK_C) return no("window view");
-        plan->kw = 1; p.R = 1; p.o = 0; p.p = 0;
-    }
     p.act = a.act;
     const bool flat = a.k == 1 && a.stride == 1;
     // C = channels per pixel of x as stored (pitch and extent of the activation maps): with padded pixels the
@@ -666,23 +661,8 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
     } else {
         if (swap) { p.bw = a.Wo; p.bh = a.Ho; p.bn = a.N; }
         else choose_box(a.N, a.Ho, a.Wo, &p.bw, &p.bh, &p.bn);
-        if (a.win) {
-            // dim 0 = the 64-element window of output column wo (starts at padded pixel wo * stride), dim 1 = wo,
-            // dim 2 = input row (stride 2: rows of one parity), dim 3 = image
-            uint32_t wbox[4] = {CHUNK_C, (uint32_t)p.bw, (uint32_t)p.bh, (uint32_t)p.bn};
-            const uint64_t px = 8 * eb, st = (uint64_t)a.stride;
-            for (int ph = 0; ph < a.stride; ph++) {
-                const char *base = static_cast<const char *>(first_slot(a.x)) + (size_t)ph * a.W * px;
-                uint64_t dims[4] = {CHUNK_C, (uint64_t)a.Wo, (uint64_t)(a.H - ph + a.stride - 1) / st, (uint64_t)a.N};
-                uint64_t str[3] = {st * px, st * (uint64_t)a.W * px, (uint64_t)a.H * a.W * px};
-                if (shared) { dims[3] = (uint64_t)a.slots; str[2] = a.slot_bytes; }
-                if (!encode_map(&p.tmA[ph * 2], base, 4, dims, str, wbox, false, ph ? nullptr : &plan->id_a)) return no("window tensor map");
-            }
-        }
         uint32_t box[4] = {CH, (uint32_t)p.bw, (uint32_t)p.bh, (uint32_t)p.bn};
-        if (a.win) {
-            // (encoded above)
-        } else if (a.stride == 1) {
+        if (a.stride == 1) {
             uint64_t dims[4] = {C, (uint64_t)a.W, (uint64_t)a.H, (uint64_t)a.N};
             uint64_t str[3] = {C * eb, (uint64_t)a.W * C * eb, (uint64_t)a.H * a.W * C * eb};
             if (shared) { dims[3] = (uint64_t)a.slots; str[2] = a.slot_bytes; }
@@ -735,7 +715,7 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
     if (a.no_split) max_splits = 1;
     plan->bn_tile = BN;
     {
-        const uint64_t taps = a.win ? (uint64_t)a.k : (uint64_t)a.R * a.R;  // stored taps per filter
+        const uint64_t taps = (uint64_t)a.R * a.R;  // stored taps per filter
         // (padded pixels: the weight map shows the stored channels up to the pixel's pitch; they meet zeros)
         const uint64_t Cw = a.ldx ? std::min<uint64_t>((uint64_t)a.ldx, (uint64_t)a.Cmax) : (uint64_t)a.C;
         uint64_t dims[3] = {Cw, taps, (uint64_t)a.K};

@@ -63,11 +63,6 @@ struct ConvArgs {
     const int *q_mult = nullptr, *q_shift = nullptr, *q_bias = nullptr;  // ... with the integer epilogue of TcParams
     int q_zy = 0, q_zr = 0, q_res_mult = 0, q_res_shift = 0, q_flags = 0;
     int k = 1, stride = 1, act = 0;
-    // Window view of a 3-channel stem (grouped launches): x is the input padded to 8 channels with a zero
-    // margin, [N][H][W][8] with H, W the PADDED sizes; an "input channel" chunk is the 8-pixel x 8-channel
-    // window that starts at output column wo * stride (64 contiguous elements), the taps are the k filter ROWS
-    // only (C = Cmax = 64, R = 1), and the weights are [Kmax][k][64] with zeros where the window has no tap.
-    int win = 0;
     // SubGraph cache box of this layer: weight tiles with filter < cacheK and channel < cacheC are
     // loaded with an evict-last L2 policy; weight_policy 0 = none, 1 = use the box, 2 = all evict-first
     int cacheK = 0, cacheC = 0, weight_policy = 0;
@@ -142,7 +137,7 @@ struct PqParams {
     int *status;             // device status word: nonzero after a bounded wait ran out
 };
 
-enum OpType { OP_CONV, OP_DW, OP_MAXPOOL, OP_GAP, OP_SE_GATE, OP_SCALE, OP_LINEAR, OP_IM2COL, OP_PAD8, OP_SE };
+enum OpType { OP_CONV, OP_DW, OP_MAXPOOL, OP_GAP, OP_SE_GATE, OP_SCALE, OP_LINEAR, OP_STEM, OP_SE };
 
 struct TcConvPlan;  // tensor-core launch description (sgs_conv_tc.cu)
 
@@ -205,10 +200,10 @@ struct alignas(16) SmallEntry {
     const float *bias;   // linear: bias [K]
     int N, H, W, C;      // input dims (linear: C inputs; gap: H*W pixels)
     int K, ld, act;      // linear: outputs, row pitch of w, activation
-    int Ho, Wo;          // output dims (max pool, patch matrix)
-    int k, stride, KKp;  // patch matrix: kernel size, stride, padded row length
-    const void *w2;      // SE gate: second FC weights [C][ld2] bf16 (first FC: w [K][ld], K = squeeze width)
-    const float *bias2;  // SE gate: second FC bias [C]
+    int Ho, Wo;          // output dims (max pool; stem: of the convolution)
+    int k, stride, pad0_;  // stem: kernel size, stride
+    const void *w2;      // SE gate: second FC weights [C][ld2] bf16 (first FC: w [K][ld], K = squeeze width); stem: scale
+    const float *bias2;  // SE gate: second FC bias [C]; stem: shift
     int ld2;
     int early_weights;   // linear: as in ConvArgs
     int pad_[6];
@@ -216,8 +211,7 @@ struct alignas(16) SmallEntry {
 static_assert(sizeof(SmallEntry) == 128, "record size");
 // kind: OP_MAXPOOL (3x3 stride 2, C % 8 == 0), OP_GAP (C % 8 == 0), OP_LINEAR (C % 8 == 0, ld % 8 == 0),
 // OP_SCALE (SE scale, gate vector in w; C % 8 == 0), OP_SE_GATE (grouped launches only),
-// OP_IM2COL (3 input channels; k in {3, 7}; stride in {1, 2}), OP_PAD8 (3-channel image -> 8 channels with a
-// zero margin: k = margin left / top, Ho x Wo = padded size).  `h` is the host image of the `n` records
+// OP_STEM (sgs_stem.cu).  `h` is the host image of the `n` records
 // at device address `d` (it sizes the grid); with d == nullptr, n must be 1 and the record is passed by value.
 bool small_supported(int kind, const SmallEntry &e);
 cudaError_t launch_small(int kind, const SmallEntry *h, const SmallEntry *d, int n, cudaStream_t st);
@@ -233,10 +227,13 @@ constexpr int DW_ENTRY_BYTES = 256;
 bool dw_eligible(const ConvArgs &a);  // shapes and pointers the bf16 depthwise kernels (sgs_dw.cu) take
 cudaError_t launch_dw_single(const ConvArgs &a, cudaStream_t st);
 cudaError_t launch_dw_group(const char *h_tbl, const char *d_tbl, int members, cudaStream_t st);
-// Stem weights for the window view: dst[f][r][px * 8 + c] = src[f][r][px][c] (px < k, c < 3), else 0; dst [K][k][64].
-cudaError_t launch_stem_window_weights(const void *src, void *dst, int K, int k, cudaStream_t st);
-// Stem weights as a GEMM operand: dst[f][kk] = src[f][kk] for kk < KK (the stored [K][R][R][3] row), 0 up to KKp.
-cudaError_t launch_stem_gemm_weights(const void *src, void *dst, int K, int KK, int KKp, cudaStream_t st);
+// Stem (sgs_stem.cu): 7x7 stride 2 + ReLU + 3x3 stride-2 max pool, or 3x3 of stride 1 or 2, on a 3-channel bf16 image.  w = the
+// stored weights as launch_stem_rows writes them (stem_rows_bytes), K filters, ld channels per output pixel (zeros beyond K).
+bool stem_supported(int k, int stride, int pool, int K, int ld, int act, long long n, int H, int W);
+long long stem_tiles(const SmallEntry &e);  // of one record
+size_t stem_rows_bytes(int k);
+cudaError_t launch_stem_rows(const void *src, void *dst, int K, int k, cudaStream_t st);  // src [K][k][k][3]
+cudaError_t launch_stem(const SmallEntry *h, const SmallEntry *d, int n, cudaStream_t st);  // records as for launch_small
 
 // ---- tensor-core convolution (sgs_conv_tc.cu) -----------------------------------------------
 // Returns nullptr when the shape is not handled by the tensor-core kernel (caller falls back).

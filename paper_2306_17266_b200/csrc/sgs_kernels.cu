@@ -472,99 +472,23 @@ __global__ void __cluster_dims__(SE_SPLIT, 1, 1) __launch_bounds__(SE_THREADS) s
     }
 }
 
-// Patch matrix of a convolution with 3 input channels (the stems): row m = output pixel, column
-// kk = (r * k + s) * 3 + c holds x[n][ho*st + r - p][wo*st + s - p][c] (0 outside the image and for the
-// padding columns kk >= k*k*3).  With it the stem is a GEMM on the tensor cores like every other layer.
-// A block owns one output row of one image: it stages the k input rows in shared memory (16-byte
-// loads), then every thread assembles 8 consecutive columns of a patch row and writes them with one
-// 16-byte store, consecutive threads to consecutive addresses.
-constexpr int IM2COL_MAX_W = 1024;  // widest input row the shared-memory staging holds (7 rows x 3 channels)
-template <int K, int ST>
-__device__ __forceinline__ void im2col_body(const SmallEntry &e, int bx) {
-    constexpr int P = (K - 1) / 2, KK = K * K * 3;
-    constexpr int ROWLEN = (IM2COL_MAX_W + 2 * P) * 3;  // a staged row with P zero pixels on either side
-    // rows[r] = input row ho*ST + r - P, shifted right by P pixels and zero outside the image, so that the
-    // patch element (r, s, c) of output column wo is rows[r][(wo*ST + s) * 3 + c] without any bounds test
-    __shared__ __align__(16) unsigned short rows[K][ROWLEN];
-    if (bx >= e.N * e.Ho) return;
-    const int n = bx / e.Ho, ho = bx % e.Ho;
-    const int rowlen = e.W * 3;  // elements; a multiple of 8 (checked by the host)
-    const unsigned short *ximg = static_cast<const unsigned short *>(e.x) + (size_t)n * e.H * rowlen;
-    const int padded = rowlen + 2 * P * 3;
-#pragma unroll
-    for (int r = 0; r < K; r++) {
-        const int hi = ho * ST + r - P;
-        const bool rok = hi >= 0 && hi < e.H;
-        const unsigned short *src = ximg + (size_t)(rok ? hi : 0) * rowlen;
-        for (int i = threadIdx.x; i < padded; i += blockDim.x) {
-            const int j = i - P * 3;
-            rows[r][i] = (rok && j >= 0 && j < rowlen) ? ld_act(src + j) : (unsigned short)0;
-        }
-    }
-    __syncthreads();
-    // a thread keeps one group of 8 patch columns (their 8 offsets into `rows` stay in registers) and walks
-    // the output columns; neighbouring threads write neighbouring 16-byte pieces
-    const int gv = e.KKp >> 3;
-    const int lanes_w = blockDim.x / gv;  // output columns in flight per block
-    const int g = threadIdx.x % gv, wl = threadIdx.x / gv;
-    if (wl >= lanes_w) return;
-    int off[8];
-#pragma unroll
-    for (int q = 0; q < 8; q++) {
-        const int kk = g * 8 + q;
-        const int c = kk % 3, rs = kk / 3, s = rs % K, r = rs / K;
-        off[q] = kk < KK ? r * ROWLEN + s * 3 + c : -1;  // -1: padding column, always zero
-    }
-    uint4 *y = static_cast<uint4 *>(e.y) + ((size_t)n * e.Ho + ho) * e.Wo * gv;
-    const unsigned short *base = &rows[0][0];
-    for (int wo = wl; wo < e.Wo; wo += lanes_w) {
-        const unsigned short *p = base + wo * ST * 3;
-        unsigned short v[8];
-#pragma unroll
-        for (int q = 0; q < 8; q++) v[q] = off[q] >= 0 ? p[off[q]] : (unsigned short)0;
-        y[wo * gv + g] = make_uint4(v[0] | ((uint32_t)v[1] << 16), v[2] | ((uint32_t)v[3] << 16), v[4] | ((uint32_t)v[5] << 16), v[6] | ((uint32_t)v[7] << 16));
-    }
-}
-
-// 3-channel image -> [N][Ho][Wo][8] with the image at (k, k) and zeros elsewhere (margins and channels 3..7):
-// the input of the window-view stem.  A thread writes one padded pixel (16 bytes).
-__device__ __forceinline__ void pad8_body(const SmallEntry &e, int bx, int nbx) {
-    const int total = e.N * e.Ho * e.Wo, step = nbx * blockDim.x;
-    const unsigned short *x = static_cast<const unsigned short *>(e.x);
-    uint4 *y = static_cast<uint4 *>(e.y);
-    for (int left = total - (int)(bx * blockDim.x + threadIdx.x); left > 0; left -= step) {  // (as in maxpool_body)
-        const int i = total - left;
-        const int wp = i % e.Wo, hp = (i / e.Wo) % e.Ho, n = i / (e.Wo * e.Ho);
-        const int h = hp - e.k, w = wp - e.k;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (h >= 0 && h < e.H && w >= 0 && w < e.W) {
-            const unsigned short *p = x + (((size_t)n * e.H + h) * e.W + w) * 3;
-            v.x = ld_act(p) | ((uint32_t)ld_act(p + 1) << 16);
-            v.y = ld_act(p + 2);
-        }
-        y[i] = v;
-    }
-}
-
-template <int KIND, int K, int ST> __device__ __forceinline__ void small_body(const SmallEntry &e, int bx, int nbx) {
+template <int KIND> __device__ __forceinline__ void small_body(const SmallEntry &e, int bx, int nbx) {
     if constexpr (KIND == OP_MAXPOOL) maxpool_body(e, bx, nbx);
     else if constexpr (KIND == OP_GAP) gap_body(e, bx);
-    else if constexpr (KIND == OP_SCALE) scale_body(e, bx, nbx);
-    else if constexpr (KIND == OP_PAD8) pad8_body(e, bx, nbx);
-    else im2col_body<K, ST>(e, bx);
+    else scale_body(e, bx, nbx);
 }
-template <int KIND, int K, int ST> __global__ void __launch_bounds__(256) small_single_kernel(const SmallEntry e) {
+template <int KIND> __global__ void __launch_bounds__(256) small_single_kernel(const SmallEntry e) {
     pdl_launch_dependents();
     pdl_wait();
-    small_body<KIND, K, ST>(e, blockIdx.x, gridDim.x);
+    small_body<KIND>(e, blockIdx.x, gridDim.x);
 }
-template <int KIND, int K, int ST> __global__ void __launch_bounds__(256) small_group_kernel(const SmallEntry *__restrict__ tbl) {
+template <int KIND> __global__ void __launch_bounds__(256) small_group_kernel(const SmallEntry *__restrict__ tbl) {
     pdl_launch_dependents();
     pdl_wait();
     __shared__ SmallEntry e;
     if (threadIdx.x < 8) reinterpret_cast<uint4 *>(&e)[threadIdx.x] = __ldg(reinterpret_cast<const uint4 *>(tbl + blockIdx.y) + threadIdx.x);
     __syncthreads();
-    small_body<KIND, K, ST>(e, blockIdx.x, gridDim.x);
+    small_body<KIND>(e, blockIdx.x, gridDim.x);
 }
 
 // Sliced linear layer on fp32 vectors, bf16 weights, for the images of one query or of all members of a wave that use the
@@ -688,6 +612,7 @@ template cudaError_t launch_linear<__nv_bfloat16>(const float *, const __nv_bflo
 
 bool small_supported(int kind, const SmallEntry &e) {
     auto al = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+    if (kind == OP_STEM) return al(e.y) && al(e.w);  // (the image is read 2 bytes at a time)
     if (!al(e.x) || !al(e.y)) return false;
     switch (kind) {
     case OP_MAXPOOL: return e.C % 8 == 0 && (long long)e.N * e.Ho * e.Wo * (e.C / 8) < (1ll << 31);
@@ -695,10 +620,7 @@ bool small_supported(int kind, const SmallEntry &e) {
     case OP_SCALE: return e.C % 8 == 0 && al(e.w) && (long long)e.N * e.H * e.W * (e.C / 8) < (1ll << 31);
     case OP_SE_GATE: return e.w2 != nullptr;
     case OP_SE: return e.w2 != nullptr && al(e.w) && al(e.w2) && se_supported(e.N, e.H * e.W, e.C, e.K, e.ld, e.ld2, 1);
-    case OP_PAD8: return (long long)e.N * e.Ho * e.Wo < (1ll << 31);
     case OP_LINEAR: return e.C % 8 == 0 && e.ld % 8 == 0 && al(e.w);
-    case OP_IM2COL: return (e.k == 3 || e.k == 7) && (e.stride == 1 || e.stride == 2) && e.KKp % 8 == 0 && e.KKp >= e.k * e.k * 3 &&
-                           e.W % 8 == 0 && e.W <= IM2COL_MAX_W && (long long)e.N * e.Ho < (1ll << 31) && (long long)e.Wo * (e.KKp / 8) < (1ll << 31);
     default: return false;
     }
 }
@@ -709,15 +631,14 @@ static long long small_blocks(int kind, const SmallEntry &e) {
     case OP_MAXPOOL: return ((long long)e.N * e.Ho * e.Wo * (e.C / 8) + 255) / 256;
     case OP_GAP: return ((long long)e.N * (e.C / 8) + 7) / 8;
     case OP_SCALE: return ((long long)e.N * e.H * e.W * (e.C / 8) + 255) / 256;
-    case OP_PAD8: return ((long long)e.N * e.Ho * e.Wo + 255) / 256;
-    default: return (long long)e.N * e.Ho;  // patch matrix: one block per output row
+    default: return 1;
     }
 }
 
-template <int KIND, int K, int ST>
+template <int KIND>
 static cudaError_t launch_small_t(const SmallEntry *h, const SmallEntry *d, int n, unsigned bx, cudaStream_t st) {
-    if (d) SGS_LAUNCH((small_group_kernel<KIND, K, ST>), dim3(bx, (unsigned)n), dim3(256), 0, st, d);
-    else SGS_LAUNCH((small_single_kernel<KIND, K, ST>), dim3(bx), dim3(256), 0, st, *h);
+    if (d) SGS_LAUNCH(small_group_kernel<KIND>, dim3(bx, (unsigned)n), dim3(256), 0, st, d);
+    else SGS_LAUNCH(small_single_kernel<KIND>, dim3(bx), dim3(256), 0, st, *h);
     return cudaGetLastError();
 }
 
@@ -727,13 +648,13 @@ cudaError_t launch_small(int kind, const SmallEntry *h, const SmallEntry *d, int
     long long blocks = 1;
     for (int i = 0; i < n; i++) blocks = std::max(blocks, small_blocks(kind, h[i]));
     // the grid-stride kernels (max pool, SE scale) need not cover every element with a block of their own
-    if (kind == OP_MAXPOOL || kind == OP_SCALE || kind == OP_PAD8) blocks = std::min<long long>(blocks, 148 * 16);
+    if (kind == OP_MAXPOOL || kind == OP_SCALE) blocks = std::min<long long>(blocks, 148 * 16);
     const unsigned bx = (unsigned)blocks;
     switch (kind) {
-    case OP_MAXPOOL: return launch_small_t<OP_MAXPOOL, 0, 0>(h, d, n, bx, st);
-    case OP_GAP: return launch_small_t<OP_GAP, 0, 0>(h, d, n, bx, st);
-    case OP_SCALE: return launch_small_t<OP_SCALE, 0, 0>(h, d, n, bx, st);
-    case OP_PAD8: return launch_small_t<OP_PAD8, 0, 0>(h, d, n, bx, st);
+    case OP_MAXPOOL: return launch_small_t<OP_MAXPOOL>(h, d, n, bx, st);
+    case OP_GAP: return launch_small_t<OP_GAP>(h, d, n, bx, st);
+    case OP_SCALE: return launch_small_t<OP_SCALE>(h, d, n, bx, st);
+    case OP_STEM: return launch_stem(h, d, n, st);
     case OP_SE: return launch_se(h, d, n, 1, st);
     case OP_SE_GATE: {
         if (!d) return cudaErrorInvalidValue;
@@ -754,41 +675,8 @@ cudaError_t launch_small(int kind, const SmallEntry *h, const SmallEntry *d, int
         }
         return cudaSuccess;
     }
-    case OP_IM2COL: {
-        const int key = h[0].k * 10 + h[0].stride;
-        for (int i = 1; i < n; i++)
-            if (h[i].k * 10 + h[i].stride != key) return cudaErrorInvalidValue;
-        if (key == 72) return launch_small_t<OP_IM2COL, 7, 2>(h, d, n, bx, st);
-        if (key == 71) return launch_small_t<OP_IM2COL, 7, 1>(h, d, n, bx, st);
-        if (key == 32) return launch_small_t<OP_IM2COL, 3, 2>(h, d, n, bx, st);
-        if (key == 31) return launch_small_t<OP_IM2COL, 3, 1>(h, d, n, bx, st);
-        return cudaErrorInvalidValue;
-    }
     default: return cudaErrorInvalidValue;
     }
-}
-
-__global__ void stem_gemm_weights_kernel(const __nv_bfloat16 *__restrict__ src, __nv_bfloat16 *__restrict__ dst, int K, int KK, int KKp) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= K * KKp) return;
-    const int f = i / KKp, kk = i % KKp;
-    dst[i] = kk < KK ? src[(size_t)f * KK + kk] : __float2bfloat16_rn(0.f);
-}
-__global__ void stem_window_weights_kernel(const __nv_bfloat16 *__restrict__ src, __nv_bfloat16 *__restrict__ dst, int K, int k) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;  // dst index [f][r][px][c8]
-    if (i >= K * k * 64) return;
-    const int c = i % 8, px = (i / 8) % 8, r = (i / 64) % k, f = i / (64 * k);
-    dst[i] = (px < k && c < 3) ? src[(((size_t)f * k + r) * k + px) * 3 + c] : __float2bfloat16_rn(0.f);
-}
-cudaError_t launch_stem_window_weights(const void *src, void *dst, int K, int k, cudaStream_t st) {
-    const int total = K * k * 64;
-    stem_window_weights_kernel<<<(total + 255) / 256, 256, 0, st>>>(static_cast<const __nv_bfloat16 *>(src), static_cast<__nv_bfloat16 *>(dst), K, k);
-    return cudaGetLastError();
-}
-cudaError_t launch_stem_gemm_weights(const void *src, void *dst, int K, int KK, int KKp, cudaStream_t st) {
-    const int total = K * KKp;
-    stem_gemm_weights_kernel<<<(total + 255) / 256, 256, 0, st>>>(static_cast<const __nv_bfloat16 *>(src), static_cast<__nv_bfloat16 *>(dst), K, KK, KKp);
-    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------------------------
