@@ -532,8 +532,9 @@ static int views_of(const TcParams &p) { return (p.stride == 2 && p.k > 1) ? 4 :
 struct GroupLaunch::Impl {
     GroupParams<TC_GROUP_MAPS_LARGE> prm;  // host image of the parameter block (the small variant is a prefix)
     int n_maps = 0;
-    unsigned ids[TC_GROUP_MAPS_LARGE];  // the maps' numbers (TcConvPlan), 0: never shared
-    int ids_n[TC_GROUP_MAPS_LARGE];     // maps that lie there together
+    unsigned keys[TC_GROUP_MAPS_LARGE];  // which maps they are (number, views that lie there together)
+    unsigned char known[512];            // look-up by key: index + 1
+    static_assert(TC_GROUP_MAPS_LARGE < 255, "look-up");
     int iters = 0;      // longest reduction among the members, in stages
     bool res = false;   // any member with a residual
     int col_rows = 0;   // most rows any member's column-side operand has (sizes the stages)
@@ -549,6 +550,7 @@ void GroupLaunch::reset(const void *d_entries) {
     impl->col_rows = 0;
     impl->iters = 0;
     impl->res = false;
+    std::memset(impl->known, 0, sizeof impl->known);
     impl->win_base = nullptr;
     impl->win_bytes = 0;
     impl->prm.entries = static_cast<const GroupEntry *>(d_entries);
@@ -598,11 +600,13 @@ void GroupLaunch::add(void *host_entry, const TcConvPlan &pl, const ConvArgs &a,
     // Members whose maps are the same ones share them (weights: the same slice; activations: the same channel pitch, see
     // ConvArgs::slot): fewer of them fit a smaller parameter block, which every launch copies.
     auto add_maps = [&](const CUtensorMap *m, int n, unsigned id) {
-        for (int i = 0; i < impl->n_maps && id; i++)
-            if (impl->ids[i] == id && impl->ids_n[i] == n) return i;
+        const unsigned key = id * 8u + (unsigned)n;  // (a map alone and as the first of four views are two things)
+        unsigned h = key * 2654435761u >> 23;         // look-up table of 512
+        for (; id && impl->known[h]; h = (h + 1) & 511)
+            if (impl->keys[impl->known[h] - 1] == key) return impl->known[h] - 1;
         const int at = impl->n_maps;
         std::memcpy(&impl->prm.maps[at], m, (size_t)n * sizeof(CUtensorMap));
-        for (int i = 0; i < n; i++) { impl->ids[at + i] = i ? 0 : id; impl->ids_n[at + i] = n; }
+        if (id) { impl->known[h] = (unsigned char)(at + 1); impl->keys[at] = key; }
         impl->n_maps += n;
         return at;
     };
@@ -650,7 +654,7 @@ void GroupLaunch::add(void *host_entry, const TcConvPlan &pl, const ConvArgs &a,
 typedef void (*GroupKernel)(void);
 template <int N> static GroupKernel group_variant() { return reinterpret_cast<GroupKernel>(conv_group_kernel<N>); }
 static const struct { int maps; GroupKernel kernel; } GROUP_VARIANTS[] = {
-    {64, group_variant<64>()}, {TC_GROUP_MAPS_LARGE, group_variant<TC_GROUP_MAPS_LARGE>()}};
+    {40, group_variant<40>()}, {TC_GROUP_MAPS_LARGE, group_variant<TC_GROUP_MAPS_LARGE>()}};
 
 cudaError_t tc_group_init(int) {
     for (const auto &v : GROUP_VARIANTS) {
