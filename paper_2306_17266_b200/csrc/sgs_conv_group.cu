@@ -138,7 +138,11 @@ template <int NMAPS> struct GroupParams {
     int n_entries, total_tiles;
     int n_stages, stage_bytes;  // operand ring of this launch
     int n_bufs;                 // blocks of output in flight: 1, or an even number (the two epilogue halves have their own)
-    int pad_[7];  // (tensor maps lie at multiples of 64 bytes)
+    int layer;                  // of cache_tbl
+    const int *cache_tbl;       // device table of the cached SubGraph (see ConvArgs) in place of the entries' boxes, or nullptr
+    int pad_[4];
+    GroupEntry one;             // the only member's record where there is no table (entries == nullptr)
+    // (tensor maps lie at multiples of 64 bytes)
     CUtensorMap maps[NMAPS];
 };
 static_assert(sizeof(GroupParams<TC_GROUP_MAPS_LARGE>) <= 32764, "kernel parameter block");
@@ -163,9 +167,13 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
 
     // The table was uploaded before the first kernel of the stream segment, so it may be read before
     // the wait on the previous layer.
-    for (int i = threadIdx.x; i < n_entries * (int)(sizeof(GroupEntry) / 16); i += blockDim.x)
-        reinterpret_cast<uint4 *>(es)[i] = __ldg(reinterpret_cast<const uint4 *>(entries) + i);
-    for (int i = threadIdx.x; i < TC_GROUP_MAX_ENTRIES; i += blockDim.x) begin[i] = i < n_entries ? __ldg(&entries[i].tile_begin) : 0x7fffffff;
+    if (entries) {
+        for (int i = threadIdx.x; i < n_entries * (int)(sizeof(GroupEntry) / 16); i += blockDim.x)
+            reinterpret_cast<uint4 *>(es)[i] = __ldg(reinterpret_cast<const uint4 *>(entries) + i);
+    } else if (threadIdx.x < sizeof(GroupEntry) / 16) {
+        reinterpret_cast<uint4 *>(es)[threadIdx.x] = reinterpret_cast<const uint4 *>(&P.one)[threadIdx.x];
+    }
+    for (int i = threadIdx.x; i < TC_GROUP_MAX_ENTRIES; i += blockDim.x) begin[i] = i < n_entries ? (entries ? __ldg(&entries[i].tile_begin) : 0) : 0x7fffffff;
     if (threadIdx.x == 0) {
         for (int s = 0; s < G_MAX_STAGES; s++) { mbar_init(&full_bar[s], 2); mbar_init(&empty_bar[s], 1); }  // (full: both producers arrive)
         for (int b = 0; b < 2; b++) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], G_EPI_WARPS); }
@@ -198,6 +206,12 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
         // as far as the ring allows.
         const uint32_t on = elect_one();
         const uint64_t pol_keep = make_policy(1), pol_stream = make_policy(2);
+        int tblK = 0, tblC = 0;
+        if (P.cache_tbl) {
+            const int policy = (int)uniform((uint32_t)__ldg(P.cache_tbl));
+            tblK = policy == 2 ? -1 : policy == 1 ? (int)uniform((uint32_t)__ldg(P.cache_tbl + 1 + 2 * P.layer)) : 0;
+            tblC = policy == 1 ? (int)uniform((uint32_t)__ldg(P.cache_tbl + 2 + 2 * P.layer)) : 0;
+        }
         int s = 0;
         uint32_t phase = 0;
         bool wrapped = false, ok = true;
@@ -211,8 +225,8 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
             const CUtensorMap *map_w = &P.maps[uniform((uint32_t)e.map_w)];
             const int k = (int)uniform(e.k), kw = (int)uniform(e.kw), cchunks = (int)uniform((uint32_t)e.cchunks), R = (int)uniform((uint32_t)e.R);
             // channels below hint_c take a hint: the cached SubGraph's box (keep), or everything (stream)
-            const int cacheK = (int)uniform((uint32_t)e.cacheK);
-            const int hint_c = cacheK < 0 ? 0x7fffffff : f0 < cacheK ? (int)uniform((uint32_t)e.cacheC) : 0;
+            const int cacheK = P.cache_tbl ? tblK : (int)uniform((uint32_t)e.cacheK), cacheC = P.cache_tbl ? tblC : (int)uniform((uint32_t)e.cacheC);
+            const int hint_c = cacheK < 0 ? 0x7fffffff : f0 < cacheK ? cacheC : 0;
             const uint64_t pol = cacheK < 0 ? pol_stream : pol_keep;
             int tap_row = (int)uniform((uint32_t)e.tap0);
             for (int r = 0; r < k && ok; r++, tap_row += R) {
@@ -554,6 +568,8 @@ void GroupLaunch::reset(const void *d_entries) {
     impl->win_base = nullptr;
     impl->win_bytes = 0;
     impl->prm.entries = static_cast<const GroupEntry *>(d_entries);
+    impl->prm.cache_tbl = nullptr;
+    impl->prm.layer = 0;
     impl->prm.n_entries = 0;
     impl->prm.total_tiles = 0;
 }
@@ -662,6 +678,18 @@ cudaError_t tc_group_init(int) {
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
+}
+
+cudaError_t tc_group_launch_one(const TcConvPlan &pl, const ConvArgs &a, cudaStream_t st) {
+    static thread_local GroupLaunch g;
+    g.reset(nullptr);
+    return g.launch_one(pl, a, st);
+}
+cudaError_t GroupLaunch::launch_one(const TcConvPlan &pl, const ConvArgs &a, cudaStream_t st) {
+    add(&impl->prm.one, pl, a, a.weight_policy, a.cacheK, a.cacheC);
+    impl->prm.cache_tbl = a.cache_tbl;
+    impl->prm.layer = a.layer;
+    return launch(0, sm_count(), st);
 }
 
 cudaError_t GroupLaunch::launch(size_t window_max, int sms, cudaStream_t st) {

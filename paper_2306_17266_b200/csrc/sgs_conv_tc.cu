@@ -605,6 +605,19 @@ static void choose_box(int N, int Ho, int Wo, int *bw_, int *bh_, int *bn_) {
 }
 
 std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::string *why) {
+    // A layer of a single query with two and more tiles for every SM runs on the grouped kernel, as its only member: persistent
+    // blocks finish a tile while the next one's operands arrive.  One query of 16 images of 224x224: 595 us without, 565 from
+    // here, 560 from one tile per SM, which costs queries of 6 to 12 images 1 to 2 %.  (That kernel reads weights early: a
+    // caller's do not go there.)
+    if (!a.throughput && a.early_weights && !a.i8 && !a.no_split &&
+        ((double)a.N * a.Ho * a.Wo / TILE_M) * ((a.K + 255) / 256) >= 2.0 * sm_count()) {
+        ConvArgs g = a;
+        g.throughput = 2;
+        g.slots = 0;
+        auto plan = tc_conv_prepare(g, device, why);
+        if (plan && !plan->swap) { plan->grouped = 1; return plan; }
+    }
+
     auto no = [&](const char *msg) { if (why) *why = msg; return std::shared_ptr<TcConvPlan>(); };
     if (!encode_fn()) return no("cuTensorMapEncodeTiled unavailable");
     if (a.C % 8 || a.K % 8 || a.Cmax % 8) return no("channel counts must be multiples of 8");
@@ -787,6 +800,7 @@ cudaError_t tc_conv_launch(const TcConvPlan &pl, const ConvArgs &a, cudaStream_t
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if ((e = tc_conv_init(dev)) != cudaSuccess) return e;
+    if (pl.grouped) return tc_group_launch_one(pl, a, st);
     TcParams prm = pl.prm;
     prm.scale = a.scale; prm.shift = a.shift;
     prm.res = static_cast<const __nv_bfloat16 *>(a.res);

@@ -272,11 +272,14 @@ public:
     int maps_for(const TcConvPlan &p) const;  // tensor maps a member takes
     // window_max > 0: also mark the launch's cached filter prefix with an access-policy window of at most that many bytes
     cudaError_t launch(size_t window_max, int sms, cudaStream_t st);
+    // After reset(nullptr): a launch of one member, whose record travels with the parameters.
+    cudaError_t launch_one(const TcConvPlan &p, const ConvArgs &a, cudaStream_t st);
 private:
     struct Impl;
     Impl *impl;
 };
 cudaError_t tc_group_init(int device);
+cudaError_t tc_group_launch_one(const TcConvPlan &p, const ConvArgs &a, cudaStream_t st);
 void tc_group_entry(TcConvPlan &p, const ConvArgs &a);  // fills the plan's record for grouped launches
 
 cudaError_t subnet_kernel_init(int device);

@@ -37,3 +37,26 @@ def test_waves_at_tile_edges(family, res, batch, n, wave, conc):
         ref = onet.forward(cfgs[t], xs[t], oracle.BF16_STORE)
         assert gu.rel_err(got[t], ref) <= TOL_BF16, t
     assert sgs.device_status() == 0
+
+
+def test_single_query_of_many_images_equals_the_checker():
+    # 16 images of 224x224: the layers with two tiles for every SM run on the grouped kernel, the others on the latency kernel;
+    # with the cached SubGraph's hints on (their table is read by the kernel) and off
+    _, onet, gnet = gu.nets(wl.RESNET, True)
+    batch, res, n = 16, 224, 3
+    cfgs = wl.markov_stream(n, seed=3)
+    xs = wl.make_inputs(n, batch, res, seed=8, bf16=True)
+    d_in = gu.to_device(xs.reshape(n * batch, res, res, 3), True)
+    out = torch.zeros((2, n * batch, 1000), dtype=torch.float32, device="cuda")
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for i, cache in enumerate((0, 1)):
+        opts = sgs.StreamOpts(cache_enabled=cache, window_q=1, use_graphs=1, record_latency=0, concurrency=1, wave=0)
+        for _ in range(2):
+            gnet.stream_run(cfgs, d_in.data_ptr(), batch, res, out[i].data_ptr(), opts, stream.cuda_stream)
+    got = out.cpu().numpy()
+    np.testing.assert_array_equal(got[0], got[1])
+    for t, b in ((0, 0), (1, 7), (2, 15)):
+        ref = onet.forward(cfgs[t], xs[t][b:b + 1], oracle.BF16_STORE)
+        assert gu.rel_err(got[0][t * batch + b:t * batch + b + 1], ref) <= TOL_BF16
+    assert sgs.device_status() == 0
