@@ -715,6 +715,13 @@ sgs_status_t choose_impls(sgs_supernet *net, Plan *plan) {
         if (!op.tc && plan->padded) return fail(net, SGS_EUNSUPPORTED, "padded activation layout needs the tensor-core kernel: " + why);
         if (op.tc) op.impl = 1;
     }
+    // Single queries: a projection shortcut and the convolution after it both read the block's input and share a launch.
+    for (size_t i = 0; i + 1 < plan->ops.size(); i++) {
+        Op &a = plan->ops[i], &b = plan->ops[i + 1];
+        a.with_next = plan->throughput == 0 && a.type == OP_CONV && b.type == OP_CONV && a.impl == 1 && b.impl == 1 && a.in >= 0 && a.in == b.in &&
+                      a.res < 0 && b.res < 0 && a.out != b.out && a.out != a.in && b.out != b.in && tc_conv_pairs(*a.tc, *b.tc);
+        if (a.with_next) i++;
+    }
     plan->prepared = true;
     return SGS_OK;
 }
@@ -922,6 +929,15 @@ sgs_status_t run_ops(sgs_supernet *net, Plan *plan, const void *d_input, void *d
                 for (auto &e : plan->prof_ev) CU(cudaEventCreate(&e));
             }
             CU(cudaEventRecord(plan->prof_ev[2 * oi], st));
+        }
+        if (op.with_next && !net->profile && oi + 1 < last) {
+            Op &next = plan->ops[++oi];
+            ConvArgs a = op.conv, b = next.conv;
+            a.cache_tbl = b.cache_tbl = net->cache_tbl;
+            LayerRange range(net, op.layer, "two layers");
+            CU(tc_conv_launch_pair(*op.tc, a, *next.tc, b, st));
+            net->kernel_launches++;
+            continue;
         }
         sgs_status_t rc = launch_op<T>(net, plan, op, d_input, d_logits, st);
         if (rc != SGS_OK) return rc;

@@ -90,8 +90,14 @@ __device__ __noinline__ void requantise_wide(const TcParams &p, QuantWide &t, ui
     }
 }
 
+// Two layers that do not depend on each other (a block's projection shortcut and its first convolution) in one launch: blocks
+// below `first` along x are the first layer's tiles (filter tile * pixel tiles + pixel tile), the others the second's.
+struct TcPair {
+    TcParams p[2];
+    int first, mtiles[2];
+};
 template <int BN, bool I8>
-__global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_constant__ TcParams p) {
+__device__ __forceinline__ void conv_tc_body(const TcParams &p, int bx, int by) {
     // (a stage row is 128 bytes either way: 64 bf16 or 128 8-bit channels; an MMA takes 32 bytes of it)
     constexpr int CH = I8 ? 2 * CHUNK_C : CHUNK_C, KS = I8 ? 32 : 16;
     constexpr int B_STAGE_BYTES = BN * CHUNK_C * 2;
@@ -111,9 +117,9 @@ __global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_con
 
     // tile coordinates
     const int tiles_hw = p.tiles_w * p.tiles_h;
-    const int tn = blockIdx.x / tiles_hw, th = (blockIdx.x % tiles_hw) / p.tiles_w, tw = blockIdx.x % p.tiles_w;
+    const int tn = bx / tiles_hw, th = (bx % tiles_hw) / p.tiles_w, tw = bx % p.tiles_w;
     const int n0 = tn * p.bn, h0 = th * p.bh, w0 = tw * p.bw;
-    const int f0 = blockIdx.y * BN;
+    const int f0 = by * BN;
     // MMA shape: M = 128, N = this tile's filters rounded up to 16, bf16 x bf16 -> fp32, both K-major
     const int n_mma = min(BN, (p.K - f0 + 15) & ~15);
     // instruction descriptor: accumulator format (1 fp32, 2 int32) at bit 4, A / B formats at bits 7 / 10 (bf16 = 1;
@@ -425,6 +431,14 @@ __global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_con
         __syncthreads();
     }
     if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem_base, BN); }
+}
+
+template <int BN, bool I8>
+__global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(const __grid_constant__ TcParams p) { conv_tc_body<BN, I8>(p, blockIdx.x, blockIdx.y); }
+template <int BN>
+__global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_pair_kernel(const __grid_constant__ TcPair q) {
+    const int which = (int)blockIdx.x >= q.first, t = (int)blockIdx.x - (which ? q.first : 0), nt = t / q.mtiles[which];
+    conv_tc_body<BN, false>(q.p[which], t - nt * q.mtiles[which], nt);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -772,6 +786,8 @@ static cudaError_t set_limits() {
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(conv_tc_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(conv_tc_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(conv_tc_pair_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(conv_tc_pair_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(conv_tc_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess) return e;
     return cudaFuncSetAttribute(conv_tc_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
 }
@@ -795,12 +811,7 @@ cudaError_t tc_conv_init(int dev) {
     return cudaSuccess;
 }
 
-cudaError_t tc_conv_launch(const TcConvPlan &pl, const ConvArgs &a, cudaStream_t st) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if ((e = tc_conv_init(dev)) != cudaSuccess) return e;
-    if (pl.grouped) return tc_group_launch_one(pl, a, st);
+static TcParams launch_params(const TcConvPlan &pl, const ConvArgs &a, int dev) {
     TcParams prm = pl.prm;
     prm.scale = a.scale; prm.shift = a.shift;
     prm.res = static_cast<const __nv_bfloat16 *>(a.res);
@@ -809,6 +820,39 @@ cudaError_t tc_conv_launch(const TcConvPlan &pl, const ConvArgs &a, cudaStream_t
     prm.cacheK = a.cacheK; prm.cacheC = a.cacheC; prm.weight_policy = a.weight_policy;
     prm.cache_tbl = a.cache_tbl; prm.layer = a.layer;
     prm.early_weights = a.early_weights;
+    return prm;
+}
+
+// One launch instead of two saves a link of a query's chain (some 4 us) as long as the blocks of both layers are on the GPU at the
+// same time.  The tiles have one shape and the reductions one split (a property of the launch).
+bool tc_conv_pairs(const TcConvPlan &a, const TcConvPlan &b) {
+    const long long blocks = (long long)a.grid.x * a.grid.y * a.grid.z + (long long)b.grid.x * b.grid.y * b.grid.z;
+    return !a.i8 && !b.i8 && !a.grouped && !b.grouped && a.bn_tile == b.bn_tile && a.bn_tile <= 128 && a.prm.splits == b.prm.splits &&
+           blocks <= (std::max(a.prm.stages, b.prm.stages) * tc_stage_bytes(a.bn_tile) <= 98304 ? 2ll : 1ll) * sm_count();
+}
+cudaError_t tc_conv_launch_pair(const TcConvPlan &pa, const ConvArgs &a, const TcConvPlan &pb, const ConvArgs &b, cudaStream_t st) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if ((e = tc_conv_init(dev)) != cudaSuccess) return e;
+    TcPair q;
+    q.p[0] = launch_params(pa, a, dev);
+    q.p[1] = launch_params(pb, b, dev);
+    q.first = (int)(pa.grid.x * pa.grid.y);
+    q.mtiles[0] = (int)pa.grid.x; q.mtiles[1] = (int)pb.grid.x;
+    const dim3 grid((unsigned)q.first + pb.grid.x * pb.grid.y, 1, pa.grid.z);
+    const size_t smem = (size_t)(std::max(q.p[0].stages, q.p[1].stages) * tc_stage_bytes(pa.bn_tile) + 1024);
+    return pa.bn_tile == 64 ? launch_pdl(conv_tc_pair_kernel<64>, grid, dim3(TC_THREADS), smem, st, (unsigned)q.p[0].splits, q)
+                            : launch_pdl(conv_tc_pair_kernel<128>, grid, dim3(TC_THREADS), smem, st, (unsigned)q.p[0].splits, q);
+}
+
+cudaError_t tc_conv_launch(const TcConvPlan &pl, const ConvArgs &a, cudaStream_t st) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if ((e = tc_conv_init(dev)) != cudaSuccess) return e;
+    if (pl.grouped) return tc_group_launch_one(pl, a, st);
+    TcParams prm = launch_params(pl, a, dev);
     if (pl.i8) {
         if (!a.q_mult || !a.q_shift || !a.q_bias || pl.bn_tile > 128) return cudaErrorInvalidValue;
         prm.q_mult = a.q_mult; prm.q_shift = a.q_shift; prm.q_bias = a.q_bias;

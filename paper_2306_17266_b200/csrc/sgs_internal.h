@@ -152,6 +152,7 @@ struct Op {
     double alg_bytes = 0, flops = 0;  // algorithmic traffic (weights + input + output + residual) and useful FLOPs
     std::shared_ptr<TcConvPlan> tc;
     int rank = -1;                    // position of this op in the largest SubNet's op list (wave merging)
+    bool with_next = false;           // shares its launch with the next op (single queries)
 };
 
 struct Plan {
@@ -239,6 +240,8 @@ cudaError_t launch_stem(const SmallEntry *h, const SmallEntry *d, int n, cudaStr
 // Returns nullptr when the shape is not handled by the tensor-core kernel (caller falls back).
 std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::string *why);
 cudaError_t tc_conv_launch(const TcConvPlan &p, const ConvArgs &a, cudaStream_t st);
+bool tc_conv_pairs(const TcConvPlan &a, const TcConvPlan &b);  // may two layers that do not depend on each other share a launch?
+cudaError_t tc_conv_launch_pair(const TcConvPlan &pa, const ConvArgs &a, const TcConvPlan &pb, const ConvArgs &b, cudaStream_t st);
 cudaError_t tc_conv_init(int device);  // one-time device set-up; call outside stream capture
 bool tc_available();
 int tc_conv_status();  // nonzero once any tensor-core kernel reported a bounded wait running out
