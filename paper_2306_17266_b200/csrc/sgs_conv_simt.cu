@@ -17,9 +17,10 @@
 //    quarter-warp reads are in 8 different bank groups), filled by 16-byte asynchronous copies three steps ahead.
 //    Fragments are 4 consecutive reduction elements, and the packed FMA works on pairs of them (even and odd elements
 //    are summed apart), so nothing has to be transposed or duplicated.
-// Measured (B200): ResNet-shaped SubNet, fp32, 3 images of 160x160 (47 convolutions, 7.6 GFLOP): 5.92 -> 0.78 ms against
+// Measured (B200): ResNet-shaped SubNet, fp32, 3 images of 160x160 (47 convolutions, 7.6 GFLOP): 5.92 -> 0.72 ms against
 // the 64 x 64 tile of 4 x 4-output threads fed by scalar loads that it replaces; Tiny SubNet, one 32x32 image (17
-// convolutions): 286 -> 57 us.
+// convolutions): 286 -> 57 us.  (One group of 256 threads of 4 x 4 outputs on the 64 x 64 tile, no sums to meet: 5 to 20 % slower
+// on three images and more, the 8 x 8-output threads read half as much shared memory per multiply-add.)
 #include "sgs_internal.h"
 #include "sgs_pdl.cuh"
 
@@ -58,8 +59,9 @@ struct SimtShape {
     static constexpr int SMEM = (RING > RED ? RING : RED) * 4;       // bytes
 };
 
-template <typename T, int TM, int TN, int VEC>
-__global__ void __launch_bounds__(THREADS) conv_simt_kernel(const ConvArgs a) {
+// BLOCKS: of an SM, which the register allocation is to make room for (0: its own choice; told 1 it takes more than two have room for).
+template <typename T, int TM, int TN, int VEC, int BLOCKS>
+__global__ void __launch_bounds__(THREADS, BLOCKS) conv_simt_kernel(const ConvArgs a) {
     using S = SimtShape<T, TM, TN, VEC>;
     constexpr int BM = S::BM, BN = S::BN;
     constexpr bool ASYNC = VEC == 4 && std::is_same<T, float>::value;
@@ -198,6 +200,22 @@ __global__ void __launch_bounds__(THREADS) conv_simt_kernel(const ConvArgs a) {
         for (int i = 0; i < STAGES - 1 && i < n_it; i++) { load_regs(); step(c, tr, ts); store_regs(i); }
     }
 
+    // ---- the folded batch norm of the 4 filters this thread finishes (the same for all of its outputs), asked for ahead
+    constexpr int FQ = BN / 4;
+    static_assert(THREADS % FQ == 0, "a thread's outputs have the same filters");
+    float bn_sc[4] = {0.f, 0.f, 0.f, 0.f}, bn_sh[4] = {0.f, 0.f, 0.f, 0.f};
+    constexpr bool AHEAD = BLOCKS == 2;  // (in launches of many rounds other blocks fill the wait, and the loads are only more of them)
+    if (AHEAD && tid < BM * BN / 4) {
+        const int f = f0 + (tid % FQ) * 4;
+        if (a.K % 4 == 0 && ((reinterpret_cast<uintptr_t>(a.scale) | reinterpret_cast<uintptr_t>(a.shift)) & 15) == 0) {
+            const float4 s4 = ld_act(reinterpret_cast<const float4 *>(a.scale + min(f, a.K - 4))), h4 = ld_act(reinterpret_cast<const float4 *>(a.shift + min(f, a.K - 4)));
+            bn_sc[0] = s4.x; bn_sc[1] = s4.y; bn_sc[2] = s4.z; bn_sc[3] = s4.w;
+            bn_sh[0] = h4.x; bn_sh[1] = h4.y; bn_sh[2] = h4.z; bn_sh[3] = h4.w;
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; j++) { bn_sc[j] = ld_act(a.scale + min(f + j, a.K - 1)); bn_sh[j] = ld_act(a.shift + min(f + j, a.K - 1)); }
+        }
+    }
     // ---- arithmetic: thread (tm, tn) of k-group g owns pixels tm + 8 i and filters tn + 8 j
     const int g = tid / 64, tm = tid % 8, tn = (tid % 64) / 8;
     float2 acc[TM][TN];
@@ -270,14 +288,14 @@ __global__ void __launch_bounds__(THREADS) conv_simt_kernel(const ConvArgs a) {
             if (res) rv = *reinterpret_cast<const float4 *>(res + oi);
             const float r4[4] = {rv.x, rv.y, rv.z, rv.w};
 #pragma unroll
-            for (int j = 0; j < 4; j++) out[j] = simt_act(v[j] * ld_act(a.scale + f + j) + ld_act(a.shift + f + j) + r4[j], a.act);
+            for (int j = 0; j < 4; j++) out[j] = simt_act(AHEAD ? v[j] * bn_sc[j] + bn_sh[j] + r4[j] : v[j] * ld_act(a.scale + f + j) + ld_act(a.shift + f + j) + r4[j], a.act);
             *reinterpret_cast<float4 *>(y + oi) = make_float4(out[0], out[1], out[2], out[3]);
             return;
         }
 #pragma unroll
         for (int j = 0; j < 4; j++) {
             if (f + j >= a.K) return;
-            float t = v[j] * ld_act(a.scale + f + j) + ld_act(a.shift + f + j);
+            float t = AHEAD ? v[j] * bn_sc[j] + bn_sh[j] : v[j] * ld_act(a.scale + f + j) + ld_act(a.shift + f + j);
             if (res) t += simt_f(res[oi + j]);
             t = simt_act(t, a.act);
             if constexpr (std::is_same<T, float>::value) y[oi + j] = t; else y[oi + j] = __float2bfloat16_rn(t);
@@ -307,10 +325,10 @@ __global__ void __launch_bounds__(THREADS) conv_simt_kernel(const ConvArgs a) {
     cluster.sync();  // nobody leaves while another block may still read its sums
 }
 
-template <typename T, int TM, int TN, int VEC>
+template <typename T, int TM, int TN, int VEC, int BLOCKS = 0>
 cudaError_t launch_shape(const ConvArgs &a, int splits, cudaStream_t st) {
     using S = SimtShape<T, TM, TN, VEC>;
-    auto kernel = conv_simt_kernel<T, TM, TN, VEC>;
+    auto kernel = conv_simt_kernel<T, TM, TN, VEC, BLOCKS>;
     if (S::SMEM > 48 * 1024) {
         static DeviceBits done;
         const cudaError_t e = smem_limit_once(kernel, S::SMEM, done);
@@ -326,6 +344,11 @@ cudaError_t launch_shape(const ConvArgs &a, int splits, cudaStream_t st) {
 // Tile and split: the one with the shortest estimated time.  A step of a tile costs its multiply-adds at 128 a clock
 // (packed operands leave about a quarter of that to loads and addresses) but never less than the latency of one step of
 // the pipeline; a launch has as many rounds as its blocks need on the device's SMs.
+// The tiles of 32 x 32 and 32 x 16 have a second form with 128 registers a thread, of which an SM holds two blocks: for launches
+// that are one round with it, and 32 x 32 tiles with 12 steps or more.  In launches of many short blocks the compiler's own choice
+// (102 and 80 registers) is faster: 32 images of 64x64 of the Tiny SubNet 415 us, 511 with the second form.  ResNet-shaped
+// SubNets, two configs, us with one form and one block per SM in the estimate / now: one image of 160x160 499 / 422, two 659 / 562,
+// three 866 / 809, four 1000 / 996, one of 128x128 404 / 322, four of 192x192 1197 / 1083; 8 images of 64x64 of Tiny 154 / 137.
 template <typename T> cudaError_t launch_conv_plain(const ConvArgs &a, cudaStream_t st) {
     const long long M = (long long)a.N * a.Ho * a.Wo;
     if (M <= 0 || a.K <= 0) return cudaSuccess;
@@ -335,25 +358,29 @@ template <typename T> cudaError_t launch_conv_plain(const ConvArgs &a, cudaStrea
                      ((reinterpret_cast<uintptr_t>(a.x) | reinterpret_cast<uintptr_t>(a.w) | reinterpret_cast<uintptr_t>(a.y) | reinterpret_cast<uintptr_t>(a.res)) & 15) == 0;
     const long long sms = sm_count();
     static const int shapes[4][2] = {{8, 8}, {4, 8}, {4, 4}, {4, 2}};
+    static const double cost[4] = {1.3, 1.3, 1.4, 1.5};
     int best = 1, best_s = 1;
+    bool two = false;
     double best_t = 1e30;
     for (int i = vec ? 0 : 1; i < 4; i++) {  // (single-element copies: the 64 x 64 tile would not fit the registers)
         const int bm = 8 * shapes[i][0], bn = 8 * shapes[i][1];
         const long long tiles = ((M + bm - 1) / bm) * ((a.K + bn - 1) / bn);
         if ((M + bm - 1) / bm > 0x7fffffffll || (a.K + bn - 1) / bn > 65535) continue;
         for (int s = 1; s <= 8 && s <= iters; s *= 2) {
-            const double step = std::max(bm * bn * BK / 128.0 * 1.3, 350.0);
-            const double rounds = (double)((tiles * s + sms - 1) / sms);
+            const bool roomy = vec && i >= 2 && (tiles * s <= 2 * sms || (i == 2 && iters >= 12 * s));  // the form with many registers
+            const long long room = roomy ? 2 : 1, per_sm = std::min(room, (tiles * s + sms - 1) / sms);  // blocks an SM holds, and has
+            const double step = std::max((double)per_sm * bm * bn * BK / 128.0 * (roomy ? cost[i] : 1.3), roomy ? 550.0 : 350.0);
+            const double rounds = (double)((tiles * s + room * sms - 1) / (room * sms));
             const double t = rounds * ((double)((iters + s - 1) / s) * step + 1500.0 + 12.0 * (bm * bn / 64)) + (s > 1 ? 1500.0 : 0.0);
-            if (t < best_t) { best_t = t; best = i; best_s = s; }
+            if (t < best_t) { best_t = t; best = i; best_s = s; two = roomy; }
         }
     }
     if (vec) {
         switch (best) {
         case 0: return launch_shape<T, 8, 8, 4>(a, best_s, st);
         case 1: return launch_shape<T, 4, 8, 4>(a, best_s, st);
-        case 2: return launch_shape<T, 4, 4, 4>(a, best_s, st);
-        default: return launch_shape<T, 4, 2, 4>(a, best_s, st);
+        case 2: return two ? launch_shape<T, 4, 4, 4, 2>(a, best_s, st) : launch_shape<T, 4, 4, 4>(a, best_s, st);
+        default: return two ? launch_shape<T, 4, 2, 4, 2>(a, best_s, st) : launch_shape<T, 4, 2, 4>(a, best_s, st);
         }
     }
     switch (best) {
