@@ -804,7 +804,7 @@ sgs_status_t get_plan(sgs_supernet *net, const sgs_subnet_cfg_t *cfg, int batch,
     return SGS_OK;
 }
 
-// Argument record of a max pool, global average pool, linear or patch-matrix op (bf16 handles).
+// Argument record of a max pool, global average pool, linear or stem op (bf16 handles).
 SmallEntry small_entry(const sgs_supernet *net, const Plan *plan, const Op &op, const void *d_input, void *d_logits) {
     const sgs_supernet::Slot &sl = net->slots[plan->slot];
     SmallEntry e;
@@ -1674,7 +1674,7 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
                     }
                 }
             }
-            // max pool / average pool / linear / patch matrix: one launch over the members when every
+            // stem / average pool / linear / squeeze-excite: one launch over the members when every
             // member's op has the vectorised form; the remaining ops run member by member
             const Op &op0 = plans[b[0].first]->ops[(size_t)b[0].second];
             const int kind = op0.type;

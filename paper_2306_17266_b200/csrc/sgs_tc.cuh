@@ -263,7 +263,7 @@ struct TcConvPlan {
     CUtensorMap tmY, tmR;  // grouped launches, not swapped: output and residual as boxes of 64 filters x the tile's pixels
     int has_res = 0;
     int grouped = 0;     // this layer of a single query runs on the grouped kernel
-    int kw = 1;          // taps along x (k for square kernels, 1 for the window view of a stem)
+    int kw = 1;          // taps along x
 };
 
 }  // namespace sgs
