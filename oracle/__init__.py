@@ -67,6 +67,8 @@ def lib():
         L.orc_hit_ratio.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int]
         fw = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_void_p]
         L.orc_forward.argtypes = fw
+        L.orc_max_act_elems.restype = ctypes.c_size_t
+        L.orc_max_act_elems.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int]
         L.orc_forward_extracted.argtypes = fw
         L.orc_forward_unsliced.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_void_p]
         L.orc_layer_conv.argtypes = [ctypes.c_void_p] + [ctypes.c_int] * 4 + [ctypes.c_void_p] + [ctypes.c_int] * 7 + [ctypes.c_void_p]
@@ -125,6 +127,10 @@ class Net:
         if lib().orc_encode(self._h, ctypes.byref(cfg), _ptr(out)) < 0:
             raise ValueError("config outside the elastic sets")
         return out
+
+    def act_capacity(self, n: int, res: int) -> int:
+        """Elements each activation buffer of a forward pass holds."""
+        return int(lib().orc_max_act_elems(self._h, n, res))
 
     def _n_classes(self) -> int:
         return 10 if self.family == 0 else 1000

@@ -551,12 +551,12 @@ static void tap(int layer, const float *y, int N, int H, int W, int C) {
 /* ------------------------------------------------------------------------------------------ */
 /* Sliced forward pass                                                                          */
 /* ------------------------------------------------------------------------------------------ */
-static size_t max_act_elems(const orc_net *net, int N, int res) {
+size_t orc_max_act_elems(const orc_net *net, int N, int res) {
     /* generous bound: the largest activation of any of the three nets at this resolution */
-    size_t r = (size_t)res;
+    size_t r = (size_t)res, h = (r + 1) / 2; /* side of the map behind the stride-2 stem */
     if (net->family == ORC_TINY) return (size_t)N * r * r * 64;
-    if (net->family == ORC_RESNET) return (size_t)N * (r / 2) * (r / 2) * 64 * 4 + 1024;
-    return (size_t)N * (r / 2) * (r / 2) * 16 * 6 + 1024;
+    if (net->family == ORC_RESNET) return (size_t)N * (h * h * 64 * 4 + 1024);
+    return (size_t)N * (h * h * 16 * 6 + 1024);
 }
 
 static int conv_bn(const orc_net *net, int id, const orc_slice *sl, const float *x, int N, int H, int W, int st,
@@ -580,7 +580,7 @@ int orc_forward(const orc_net *net, const orc_cfg *cfg, const float *input, int 
     if (orc_validate(net, cfg)) return -1;
     orc_slice sl[ORC_MAX_LAYERS];
     slices_of(net, cfg, sl);
-    size_t cap = max_act_elems(net, N, res);
+    size_t cap = orc_max_act_elems(net, N, res);
     float *A = (float *)malloc(cap * sizeof(float)), *B = (float *)malloc(cap * sizeof(float));
     float *Cb = (float *)malloc(cap * sizeof(float)), *D = (float *)malloc(cap * sizeof(float));
     float *vec = (float *)malloc((size_t)N * 4096 * sizeof(float)), *vec2 = (float *)malloc((size_t)N * 4096 * sizeof(float));
@@ -746,7 +746,7 @@ static void dense_linear(const dense_layer *d, const float *v, int N, float *y) 
  * many blocks are present) is read from the layer table. */
 static int dense_forward(const orc_net *net, const dense_layer *d, const int *depth, const float *input, int N,
                          int res, int mode, float *logits) {
-    size_t cap = max_act_elems(net, N, res);
+    size_t cap = orc_max_act_elems(net, N, res);
     float *A = (float *)malloc(cap * sizeof(float)), *B = (float *)malloc(cap * sizeof(float));
     float *Cb = (float *)malloc(cap * sizeof(float)), *D = (float *)malloc(cap * sizeof(float));
     float *vec = (float *)malloc((size_t)N * 4096 * sizeof(float)), *vec2 = (float *)malloc((size_t)N * 4096 * sizeof(float));

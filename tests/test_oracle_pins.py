@@ -282,6 +282,53 @@ def _record_offsets(fam):
     return out
 
 
+def map_sizes(fam, enc, names, res):
+    """Elements of every map a forward pass of one image stores: stored layers in order, each behind its strides."""
+    half = lambda v: (v + 1) // 2  # (odd kernel, padding (k - 1) / 2, stride 2)
+    at = {name: i for i, name in enumerate(names)}
+    K = lambda name: int(enc[at[name]][0])
+    h, out = res, []
+    if fam != wl.TINY:
+        h = half(h)
+    out.append(h * h * K("stem"))
+    if fam == wl.RESNET:
+        h = half(h)  # max pool
+        out.append(h * h * K("stem"))
+    strides = {wl.TINY: (1, 2, 2), wl.RESNET: (1, 2, 2, 2), wl.MBV3: (2, 2, 2, 1, 2)}[fam]
+    for s, st in enumerate(strides):
+        for b in range(16):
+            leaves = [n for n in names if n.startswith(f"s{s}b{b}.") and K(n) and ".se" not in n]
+            if not leaves:
+                break
+            h_in, h = h, half(h) if b == 0 and st == 2 else h
+            before = ("expand",) if fam == wl.MBV3 else ("conv1",) if fam == wl.RESNET else ()  # (layers in front of the strided one)
+            out += [(h_in if n.endswith(before) else h) ** 2 * K(n) for n in leaves]
+    if fam == wl.MBV3:
+        out.append(h * h * K("head.conv"))
+    return out
+
+
+@pytest.mark.parametrize("fam", [wl.TINY, wl.RESNET, wl.MBV3])
+def test_activation_buffers_hold_every_map_at_odd_and_even_resolutions(nets, fam):
+    names = [r.name for r in wl.supernet_records(fam)]
+    net = nets[fam][1]
+    enc = net.encode(wl.extreme_cfg(fam, True))
+    for res in list(range(8, 72)) + [127, 223, 224, 225, 1023]:
+        for n in (1, 3):
+            assert n * max(map_sizes(fam, enc, names, res)) <= net.act_capacity(n, res), (res, n)
+
+
+@pytest.mark.parametrize("fam,res", [(wl.MBV3, 33), (wl.MBV3, 71), (wl.RESNET, 37), (wl.TINY, 27)])
+def test_odd_resolutions_match_library_restatement(nets, fam, res):
+    blob, net = nets[fam]
+    P = torch_ref.parse_blob(fam, blob)
+    x = wl.make_inputs(1, 2, res, seed=res)[0]
+    for c in (wl.extreme_cfg(fam, False), wl.extreme_cfg(fam, True)):
+        got, ref = net.forward(c, x), torch_ref.forward(fam, P, c, x)
+        assert np.abs(got - ref).max() <= 2e-4 * max(1.0, np.abs(ref).max())  # as at the even resolutions above
+        np.testing.assert_array_equal(net.forward(c, x, path="extracted"), got)
+
+
 def test_zeroed_complement_equals_slice_network(nets):
     # zero every stored weight outside a config's prefixes, then run the widest config of the same
     # depth: the logits equal the config's own
