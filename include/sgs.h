@@ -454,6 +454,12 @@ sgs_status_t sgs_measure_fma_peak(double *tflops, void *cuda_stream);
  * device status word exactly as the convolution kernels do, and returns normally; nothing faults or hangs. */
 sgs_status_t sgs_debug_expire_wait(unsigned limit_us, void *cuda_stream);
 
+/* The same for persistent execution with several SMs a query: one cluster of `team` (1, 2, 4, 8, 16) blocks goes through four empty
+ * layers with the SubNet kernel's layer barrier, and in the third one thread of one block waits in vain for limit_us.  All blocks
+ * have to leave behind the same barrier: d_left (device, `team` ints) receives the layers each of them has ended, 2 where the wait
+ * ran out.  Sets the device status word. */
+sgs_status_t sgs_debug_expire_team_wait(int team, int block, int thread, unsigned limit_us, int *d_left, void *cuda_stream);
+
 /* Library options by name (debug and measurement aids): "conv_impl" 0 = automatic, 1 = force the
  * CUDA-core kernels; "pad_channels" 1 (default) = waves of the ResNet-shaped family keep their activation tensors
  * at 16-channel pixels (zeros beyond the slice), 0 = dense pixels; "cache_mechanism" how grouped launches keep the cached SubGraph in L2: 0 (default) = an evict-last

@@ -2842,4 +2842,11 @@ sgs_status_t sgs_debug_expire_wait(unsigned limit_us, void *cuda_stream) {
     return tc_expire_wait(limit_us, (cudaStream_t)cuda_stream) == cudaSuccess ? SGS_OK : SGS_ECUDA;
 }
 
+sgs_status_t sgs_debug_expire_team_wait(int team, int block, int thread, unsigned limit_us, int *d_left, void *cuda_stream) {
+    if (!in_set(team, {1, 2, 4, 8, 16}) || block < 0 || block >= team || thread < 0 || thread >= SUBNET_THREADS || limit_us == 0 || limit_us > 1000000u || !d_left) return SGS_EINVAL;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || tc_conv_init(dev) != cudaSuccess) return SGS_ECUDA;
+    return subnet_team_expire(team, block, thread, limit_us, d_left, tc_status_word(dev), (cudaStream_t)cuda_stream) == cudaSuccess ? SGS_OK : SGS_ECUDA;
+}
+
 }  // extern "C"

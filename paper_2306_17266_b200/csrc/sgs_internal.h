@@ -289,5 +289,7 @@ cudaError_t subnet_kernel_init(int device);
 int subnet_kernel_clusters(int team);  // clusters of `team` blocks the device holds at a time (0: none)
 cudaError_t subnet_kernel_launch(const PqParams &p, int clusters, int team, cudaStream_t st);  // `team` blocks serve a query together
 size_t subnet_kernel_held_max();  // largest weight buffer a block can keep
+cudaError_t subnet_team_expire(int team, int block, int thread, unsigned limit_us, int *left, int *status, cudaStream_t st);  // test of the time-out path
+constexpr int SUBNET_THREADS = 512;  // of a block
 
 }  // namespace sgs

@@ -35,7 +35,7 @@ namespace {
 
 using bf16 = __nv_bfloat16;
 
-constexpr int PQ_THREADS = 512;
+constexpr int PQ_THREADS = SUBNET_THREADS;
 constexpr int PQ_WARPS = PQ_THREADS / 32;
 constexpr int PQ_ROWS = PQ_THREADS / 8;      // rows of 128 bytes one round of 16-byte copies covers
 constexpr int PQ_MAX_K = 1024;               // widest pointwise layer (folded batch norm staged in shared memory)
@@ -65,6 +65,15 @@ __device__ __forceinline__ uint32_t in_block(const void *p, int rank) {
 }
 __device__ __forceinline__ void st_block(uint32_t addr, float v) { asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory"); }
 __device__ __forceinline__ void st_block(uint32_t addr, int v) { asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
+// Ends a layer; false: all blocks of the team leave.  ok: false in a thread one of whose waits ran out (it has set its own block's
+// flag).  That thread itself tells every block, in front of the barrier, so all threads of all blocks read the same flag behind it: a
+// flag read in front of the barrier on behalf of other threads could still be raised by one of them, and a block would leave alone.
+__device__ __forceinline__ bool end_layer(const Team &team, int *abort_s, bool ok) {
+    if (team.n > 1 && !ok)
+        for (int r = 0; r < team.n; r++) st_block(in_block(abort_s, r), 1);
+    team.sync();
+    return *(volatile int *)abort_s == 0;
+}
 
 // Completed phases of the block's barriers since the kernel started (the same in every thread; only ever
 // indexed with constants, so they live in registers).
@@ -559,7 +568,6 @@ __global__ void __launch_bounds__(PQ_THREADS, 1) subnet_kernel(const PqParams p)
         __syncthreads();
     }
 
-    // (in a team, a block whose wait ran out says so to all of them in front of a barrier, and all leave behind it)
     team.sync();
     for (;;) {
         if (team.rank == 0 && tid == 0) {
@@ -616,10 +624,7 @@ __global__ void __launch_bounds__(PQ_THREADS, 1) subnet_kernel(const PqParams p)
                 break;
             default: break;
             }
-            if (team.n > 1 && tid == 0 && *abort_flag)
-                for (int r = 0; r < team.n; r++) st_block(in_block(&abort_s, r), 1);
-            team.sync();  // the layer is complete: its outputs are visible, its record is free
-            if (*abort_flag) break;
+            if (!end_layer(team, &abort_s, ok)) break;  // the layer is complete: its outputs are visible, its record is free
         }
         if (*abort_flag) break;
     }
@@ -628,6 +633,33 @@ __global__ void __launch_bounds__(PQ_THREADS, 1) subnet_kernel(const PqParams p)
     team.sync();  // (nobody leaves while another block may still write to its shared memory)
     if (warp == 0) tmem_dealloc(tmem_base, 2 * PQ_ACC_COLS);
     if (tid == 0 && (*abort_flag || !ok)) atomicExch(p.status, 1);
+}
+
+// The end of a layer when a wait runs out (test of the time-out path): in the third of four layers thread `thread` of block `block`
+// waits for a barrier that nothing arrives at, for limit_ns, while all other threads are through.  left[b]: layers block b has ended.
+__global__ void team_expire_kernel(int block, int thread, unsigned long long limit_ns, int *left, int *status) {
+    __shared__ __align__(8) uint64_t bar;
+    __shared__ int abort_s;
+    Team team;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(team.rank));
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(team.n));
+    if (threadIdx.x == 0) {
+        mbar_init(&bar, 1);
+        abort_s = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    team.sync();
+    bool ok = true;
+    int layer = 0;
+    do {
+        if (layer == 2 && team.rank == block && (int)threadIdx.x == thread) ok = mbar_wait(&bar, 0, &abort_s, limit_ns);
+    } while (end_layer(team, &abort_s, ok) && ++layer < 4);
+    team.sync();
+    if (threadIdx.x == 0) {
+        left[team.rank] = layer;
+        if (abort_s) atomicExch(status, 1);
+    }
 }
 
 }  // namespace
@@ -675,6 +707,16 @@ cudaError_t subnet_kernel_launch(const PqParams &p, int clusters, int team, cuda
     cudaLaunchAttribute attr;
     subnet_config(cfg, attr, clusters, team, p.n_held > 0 ? p.held_bytes : 0u, st);
     return cudaLaunchKernelEx(&cfg, subnet_kernel, p);
+}
+
+cudaError_t subnet_team_expire(int team, int block, int thread, unsigned limit_us, int *left, int *status, cudaStream_t st) {
+    cudaError_t e = cudaFuncSetAttribute(team_expire_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    subnet_config(cfg, attr, 1, team, 0u, st);
+    cfg.dynamicSmemBytes = 0;
+    return cudaLaunchKernelEx(&cfg, team_expire_kernel, block, thread, (unsigned long long)limit_us * 1000ull, left, status);
 }
 
 }  // namespace sgs

@@ -110,6 +110,27 @@ def test_a_wait_that_runs_out_is_reported_and_leaves_the_device_usable():
         assert gu.rel_err(got[t:t + 1], onet.forward(cfgs[t], xs[t], oracle.BF16_STORE)) <= 2e-2
 
 
+@pytest.mark.parametrize("team,block,thread", [(1, 0, 77), (2, 1, 0), (2, 0, 511), (4, 3, 77), (8, 5, 200), (16, 15, 33), (16, 0, 0)])
+def test_a_wait_that_runs_out_ends_every_block_of_a_team(team, block, thread):
+    # the wait of one thread runs out (limit 1 ms) long after the other threads of its block have come to the layer's end: all
+    # blocks of the cluster leave behind the third layer
+    left = torch.full((16,), -1, dtype=torch.int32, device="cuda")
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    assert sgs.device_status() == 0
+    try:
+        sgs.debug_expire_team_wait(team, block, thread, 1000, left.data_ptr(), stream.cuda_stream)
+        torch.cuda.synchronize()
+        assert left.tolist() == [2] * team + [-1] * (16 - team)
+        assert sgs.device_status() != 0
+    finally:
+        sgs.device_status_clear()
+    for bad in ((3, 0, 0, 1000), (4, 4, 0, 1000), (4, 0, 512, 1000), (4, 0, 0, 0)):
+        with pytest.raises(sgs.SgsError):
+            sgs.debug_expire_team_wait(*bad, left.data_ptr(), stream.cuda_stream)
+    assert sgs.device_status() == 0
+
+
 def test_device_allocation_failure_is_reported_and_survivable():
     # fault injection on the host: the handle's device allocations are made to fail while its workspaces have to grow
     # (a larger resolution, more wave slots).  The call must come back with SGS_ENOMEM, nothing may be left half
