@@ -436,43 +436,72 @@ template <class T> __device__ __noinline__ void pq_stem(const PqOp &op, const bf
     }
 }
 
-// Global average pool into a shared-memory vector of every block of the team.  Neighbouring threads take neighbouring channels of a
-// pixel; a block sums its share of the pixels (thread by thread, then over the threads), the blocks' sums meet in part[rank][C].
-// All sums have a fixed order for a given team size.
+// f(i) + ... + f(i + N - 1) as a binary tree.
+template <int N, class F> __device__ __forceinline__ float tree_sum(const F &f, int i = 0) {
+    if constexpr (N == 1) return f(i);
+    else {
+        const float a = tree_sum<N / 2>(f, i);
+        return a + tree_sum<N / 2>(f, i + N / 2);
+    }
+}
+template <class F> __device__ __forceinline__ float tree_sum_of(const F &f, int n) {  // n: 1, 2, 4, 8 or 16
+    return n == 16 ? tree_sum<16>(f) : n == 8 ? tree_sum<8>(f) : n == 4 ? tree_sum<4>(f) : n == 2 ? tree_sum<2>(f) : tree_sum<1>(f);
+}
+// Global average pool into a shared-memory vector of every block of the team.  The sum's order must not depend on the team, which is
+// chosen by how many queries a call has: the pixels are always cut into PQ_SHARES shares of `sub` threads each, a share is the sum of
+// its threads' in their order, and the shares are added in a binary tree.  A block of a team has 1, 2, 4 or 8 neighbouring shares, a
+// whole branch of that tree, and the branches meet in part[rank][C] of every block.  Neighbouring threads take neighbouring channels.
+// What the fixed order costs (224x224, device time; against as many threads a channel as the block has): 1000 queries of one block each
+// 20.3 -> 20.45 ms, 333 of two 8.80 -> 8.91; one pixel asked for after the other instead of four together: 20.6 and 8.98.
+constexpr int PQ_SHARES = 16;
+constexpr int PQ_RING_FLOATS = PQ_RING_BYTES / 4;
 template <class T>
-__device__ __forceinline__ void pq_gap(const PqOp &op, const bf16 *x, float *out, float *buf, float *part, const T &team) {
-    const int cvecs = op.C >> 3, HW = op.H * op.W, lanes = PQ_THREADS / cvecs;  // (C <= PQ_VEC: at least 3 pixels at a time)
-    const int pl = threadIdx.x / cvecs, cv = threadIdx.x - pl * cvecs;
-    const int end = HW * (team.rank + 1) / team.n;
-    if (pl < lanes) {
+__device__ __forceinline__ void pq_gap(const PqOp &op, const bf16 *x, float *out, float *buf, const T &team) {
+    const int C = op.C, cvecs = C >> 3, HW = op.H * op.W;
+    // threads of a share: 8 pixels each at least, and as many as the sums of all shares (Single), or of half of them beside part (Team), fit the ring
+    const int sub = max(1, min(HW / (8 * PQ_SHARES), PQ_RING_FLOATS / (PQ_SHARES * C) - 1));
+    const int own = PQ_SHARES / team.n, first = own * team.rank;  // (n divides PQ_SHARES)
+    float *part = buf + PQ_SHARES / 2 * sub * C;
+    for (int u = threadIdx.x; u < own * sub * cvecs; u += PQ_THREADS) {
+        const int k = u / cvecs, cv = u - k * cvecs, share = first + k / sub;
+        const int end = HW * (share + 1) / PQ_SHARES;  // (HW <= 512 * 512)
         const bf16 *base = x + cv * 8;
         float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int i = HW * team.rank / team.n + pl; i < end; i += lanes) {
-            const uint4 v = *reinterpret_cast<const uint4 *>(base + (size_t)i * op.C);
-            const float2 a = unpack2(v.x), b = unpack2(v.y), c = unpack2(v.z), d = unpack2(v.w);
-            acc[0] += a.x; acc[1] += a.y; acc[2] += b.x; acc[3] += b.y; acc[4] += c.x; acc[5] += c.y; acc[6] += d.x; acc[7] += d.y;
+        for (int i = HW * share / PQ_SHARES + k % sub; i < end; i += 4 * sub) {
+            uint4 v[4];  // (asked for together; beyond the share: zeros)
+#pragma unroll
+            for (int j = 0; j < 4; j++) v[j] = i + j * sub < end ? *reinterpret_cast<const uint4 *>(base + (size_t)(i + j * sub) * C) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                const float2 a = unpack2(v[j].x), b = unpack2(v[j].y), c = unpack2(v[j].z), d = unpack2(v[j].w);
+                acc[0] += a.x; acc[1] += a.y; acc[2] += b.x; acc[3] += b.y; acc[4] += c.x; acc[5] += c.y; acc[6] += d.x; acc[7] += d.y;
+            }
         }
-        float4 *dst = reinterpret_cast<float4 *>(buf + (size_t)pl * op.C + cv * 8);
+        float4 *dst = reinterpret_cast<float4 *>(buf + (size_t)k * C + cv * 8);
         dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
         dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
     }
     __syncthreads();
     const float inv = 1.f / (float)HW;
-    for (int c = threadIdx.x; c < op.C; c += PQ_THREADS) {
-        float t = 0.f;
-        for (int i = 0; i < lanes; i++) t += buf[(size_t)i * op.C + c];
+    for (int c = threadIdx.x; c < C; c += PQ_THREADS) {
+        auto share_sum = [&](int k) {
+            const float *q = buf + (size_t)(k * sub) * C + c;
+            float t = q[0];
+            for (int i = 1; i < sub; i++) t += q[(size_t)i * C];
+            return t;
+        };
+        const float t = tree_sum_of(share_sum, own);
         if (team.n == 1) out[c] = t * inv;
         else
-            for (int r = 0; r < team.n; r++) st_block(in_block(part + (size_t)team.rank * PQ_VEC + c, r), t);
+            for (int r = 0; r < team.n; r++) st_block(in_block(part + (size_t)team.rank * C + c, r), t);
     }
     if (team.n == 1) return;
     team.sync();
-    for (int c = threadIdx.x; c < op.C; c += PQ_THREADS) {
-        float t = 0.f;
-        for (int r = 0; r < team.n; r++) t += part[(size_t)r * PQ_VEC + c];
-        out[c] = t * inv;
-    }
+    for (int c = threadIdx.x; c < C; c += PQ_THREADS) out[c] = tree_sum_of([&](int r) { return part[(size_t)r * C + c]; }, team.n) * inv;
 }
+static_assert(PQ_SHARES == 16 && PQ_SHARES == PQ_MAX_CLUSTER, "tree_sum_of");
+static_assert(PQ_SHARES * PQ_VEC <= PQ_RING_FLOATS && (PQ_SHARES / 2 + PQ_SHARES) * PQ_VEC <= PQ_RING_FLOATS,
+              "with one thread a share the sums of a vector of PQ_VEC fit the ring; with more, sub + 1 <= PQ_RING_FLOATS / (PQ_SHARES * C) bounds both");
 
 // y[j] = f(bias[j] + sum_c w[j][c] * v[c]) for j < K: a warp takes JB outputs at a time and has the 16-byte weight
 // loads of all of them in flight together; the outputs are dealt to the team's warps.  HS: hard sigmoid (the squeeze-excite gate)
@@ -617,7 +646,7 @@ template <class T> __global__ void __launch_bounds__(PQ_THREADS, 1) subnet_kerne
                     else pq_depthwise<7, 2>(op, x, y, team);
                 }
                 break;
-            case PQ_GAP: pq_gap(op, x, vec_s[op.vout], reinterpret_cast<float *>(ring), reinterpret_cast<float *>(ring) + PQ_THREADS * 8, team); break;
+            case PQ_GAP: pq_gap(op, x, vec_s[op.vout], reinterpret_cast<float *>(ring), team); break;
             case PQ_SE_GATE:
                 // first FC (ReLU) into the third vector, second FC (hard sigmoid) into the gate
                 pq_matvec<4, false, true>(static_cast<const bf16 *>(op.w), op.ld, op.shift, vec_s[op.vin], vec_s[2], op.C, op.K, ACT_RELU, team);

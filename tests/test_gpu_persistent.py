@@ -167,3 +167,25 @@ def test_teams_of_blocks_agree_with_single_blocks(team, res, n):
     for t in (0, n - 2, n - 1):
         assert gu.rel_err(got[t:t + 1], onet.forward(cfgs[t], xs[t], oracle.BF16_STORE)) <= TOL_BF16, t
     assert sgs.device_status() == 0
+
+
+@pytest.mark.parametrize("res", [224, 72])
+def test_logits_do_not_depend_on_the_number_of_queries(res):
+    # a query alone, in calls of more and more queries (teams of 16 blocks down to one) and with every team asked for: the same
+    # bits.  224: pooled maps of 28, 14 and 7 pixels a side; 72: 9, 5 and 3, fewer pixels than shares.
+    _, _, gnet = gu.nets(wl.MBV3, True)
+    n = 170
+    cfgs = [wl.extreme_cfg(wl.MBV3, False), wl.extreme_cfg(wl.MBV3, True)] + wl.uniform_stream(wl.MBV3, n - 2, seed=12)
+    d_in = gu.to_device(wl.make_inputs(n, 1, res, seed=3, bf16=True).reshape(n, res, res, 3), True)
+    gnet.set_option("persistent_team", 1)
+    try:
+        ref, _ = _run(gnet, cfgs, d_in, res, cache=0)
+        for team in (2, 4, 8, 16):
+            gnet.set_option("persistent_team", team)
+            got, _ = _run(gnet, cfgs[:40], d_in, res, cache=0)
+            np.testing.assert_array_equal(got, ref[:40])
+    finally:
+        gnet.set_option("persistent_team", 0)
+    for m in (1, 2, 9, 33, 70, 140, 170):
+        got, _ = _run(gnet, cfgs[:m], d_in, res, cache=0)
+        np.testing.assert_array_equal(got, ref[:m])
