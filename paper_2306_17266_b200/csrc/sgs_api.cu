@@ -3,6 +3,7 @@
 #include "sgs_internal.h"
 
 #include <algorithm>
+#include <functional>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -1976,20 +1977,35 @@ static sgs_status_t build_pq_ops(sgs_supernet *net, Plan *plan) {
     return SGS_OK;
 }
 
-// Blocks per query (a cluster: 1, 2, 4, 8 or 16) and how many such teams the device holds.  A query takes work / team + overhead, where
-// the overhead (some 100 layers, each with a barrier, the fill of its pipelines and a last round of tiles) does not shrink, and
-// larger clusters leave SMs unused (148, 148, 132, 120 and 112 of 148).  Measured (B200, 224x224, ms a call; 1 / 2 / 4 / 8 / 16
-// blocks): 8 queries 3.45 / 1.96 / 1.21 / 0.87 / 1.11, 33: 3.97 / 2.23 / 1.42 / 2.07 / 3.09, 74: 4.22 / 2.37 / 3.21 / 3.98, 148: 4.33 /
-// 4.42 / 5.52, 333: 9.99 / 9.17 / 11.67.  With more queries than teams they come one after the other, dealt as teams get free.
-static void choose_team(const sgs_supernet *net, int n, double flops, int *team, int *clusters) {
-    const double work = n > 0 ? flops / n * 6.2e-12 : 0, overhead = 0.35e-3;  // seconds on one SM: 3.4 ms for 0.55 GFLOP
+// Blocks per query (a cluster: 1, 2, 4, 8 or 16) and how many such teams the device holds.  The queries come longest first and a team
+// takes the next one when it is free, so a call lasts as long as that schedule does with the times below; larger clusters leave SMs
+// unused (148, 148, 132, 120 and 112 of 148).  With more than four queries a team the overhead decides, and a block a query wins.
+// A query takes 0.5 ms + 5.2 ms per GFLOP / team: the first part (some 100 layers, each with a barrier, the fill of its pipelines and
+// a last round of tiles) is the same for all teams and for images of 32x32 to 384x384.  Measured (B200, ms a call; 1 / 2 / 4 / 8 / 16
+// blocks) at 224x224: 8 queries 3.05 / 1.96 / 1.21 / 0.87 / 1.06, 33: 3.56 / 2.27 / 1.42 / 2.06 / 2.98, 74: 3.74 / 2.40 / 3.13 / 3.86,
+// 148: 3.83 / 3.86 / 5.33, 222: 5.63 / 5.61; at 64x64: 8: 0.82 / 0.71 / 0.60 / 0.56 / 0.81, 74: 0.88 / 0.78 / 1.46, 148: 0.92 / 1.32,
+// 170: 1.30 / 1.77.  Over 680 calls of 1 to 600 queries of 32x32 to 384x384 the choice is 0.5 % slower than the best team on average
+// and 24 % at worst (34 queries, one more than there are teams of four); on sizes and configs that the two numbers were not fitted
+// to (154 calls, 48x48 to 240x240) 0.7 % and 16 %.
+static void choose_team(const sgs_supernet *net, const std::vector<double> &flops, int *team, int *clusters) {  // flops: of the queries, in the order in which they are taken
+    const int n = (int)flops.size();
+    const int sms = std::max(1, net->sms);
+    *team = 1; *clusters = sms;
+    if (!net->persistent_team && n > 4 * (sms / 2)) return;
     double best = 0;
+    std::vector<double> free_at;  // (a heap, earliest first)
     for (int t : {1, 2, 4, 8, 16}) {
         if (net->persistent_team && t != net->persistent_team) continue;
-        const int c = t == 1 ? std::max(1, net->sms) : subnet_kernel_clusters(t);
-        if (c <= 0) continue;
-        const double rounds = n <= c ? 1.0 : std::max(1.75, 0.8 * n / c + 0.4), time = (work / t + overhead) * rounds;
-        if (best == 0 || time < best) { best = time; *team = t; *clusters = std::min(c, std::max(1, net->sms)); }
+        const int c = t == 1 ? sms : std::min(subnet_kernel_clusters(t), sms);
+        if (c <= 0 || (t > 1 && !net->persistent_team && n > 4 * c)) continue;
+        double time = 0;
+        free_at.assign((size_t)c, 0.0);
+        for (int i = 0; i < n; i++) {
+            std::pop_heap(free_at.begin(), free_at.end(), std::greater<double>());
+            time = std::max(time, free_at.back() += 0.5e-3 + flops[(size_t)i] * 5.2e-12 / t);
+            std::push_heap(free_at.begin(), free_at.end(), std::greater<double>());
+        }
+        if (best == 0 || time < best) { best = time; *team = t; *clusters = c; }
     }
 }
 
@@ -2061,8 +2077,16 @@ static sgs_status_t persistent_impl(sgs_supernet_t *net, int n_queries, const sg
         flops += pl->flops; wbytes += qa.weight_bytes; miss_bytes += qa.miss_bytes; hit += qa.hit_ratio;
     }
     // device resources: scratch of the blocks, tables, counter, staging for host buffers
-    int team = 1, clusters = std::max(1, net->sms);
-    choose_team(net, n_queries, flops, &team, &clusters);
+    int team = 1, clusters = 1;
+    std::vector<int> order((size_t)n_queries);  // the longest queries first, so that the last ones to be taken are short
+    for (int t = 0; t < n_queries; t++) order[(size_t)t] = t;
+    std::stable_sort(order.begin(), order.end(), [&](int i, int j) { return plans[(size_t)i]->flops > plans[(size_t)j]->flops; });
+    {
+        std::vector<double> work;
+        work.reserve(order.size());
+        for (int t : order) work.push_back(plans[(size_t)t]->flops);
+        choose_team(net, work, &team, &clusters);
+    }
     const int blocks_max = std::max(1, net->sms);  // (a team has one scratch area)
     const size_t act_bytes = (act_elems * net->elem() + 255) / 256 * 256, slot_bytes = 4 * act_bytes;
     if (net->pq_scratch_bytes < slot_bytes * blocks_max) {
@@ -2112,10 +2136,7 @@ static sgs_status_t persistent_impl(sgs_supernet_t *net, int n_queries, const sg
         qs[(size_t)t].x = din + (size_t)t * in_bytes;
         qs[(size_t)t].logits = reinterpret_cast<float *>(dout + (size_t)t * out_bytes);
     }
-    {   // the longest queries first, so that the last ones to be taken are short
-        std::vector<int> order((size_t)n_queries);
-        for (int t = 0; t < n_queries; t++) order[(size_t)t] = t;
-        std::stable_sort(order.begin(), order.end(), [&](int i, int j) { return plans[(size_t)i]->flops > plans[(size_t)j]->flops; });
+    {
         std::vector<PqQuery> sorted;
         sorted.reserve(qs.size());
         for (int t : order) sorted.push_back(qs[(size_t)t]);
