@@ -479,9 +479,9 @@ sgs_status_t sgs_set_option(sgs_supernet_t *net, const char *name, long long val
  * Per-kernel-class timing.  After sgs_set_option(net, "profile", 2) (2 = on and reset, 1 = on, 0 = off)
  * every kernel the handle launches is bracketed by CUDA events on the launching stream (graphs are
  * bypassed and queries run one at a time meanwhile; a short sleeping kernel ahead of every 8 queries
- * lets the host queue their launches first, so the intervals hold device time, not launch latency).  kernel_class: 0 tensor-core convolution, 1 CUDA-core convolution,
- * 2 depthwise convolution, 3 everything else.  Returns the launches, their summed device time, their
- * summed algorithmic bytes (sliced weights + input + output + residual of each launch) and useful
+ * lets the host queue their launches first, so the intervals hold device time, not launch latency).  kernel_class: 0 tensor-core convolution (the fused
+ * stem among them: sgs_profile_trace tells it by its stored layer), 1 CUDA-core convolution, 2 depthwise convolution, 3 everything else.  Returns the launches, their summed device time, their
+ * summed algorithmic bytes (sliced weights + input + output + residual of each launch, what a launch never writes left out) and useful
  * FLOPs since the last reset.  Synchronises the device.
  */
 sgs_status_t sgs_profile_read(sgs_supernet_t *net, int kernel_class, long long *launches, double *total_ms,

@@ -476,6 +476,7 @@ struct Builder {
             cv.type = OP_STEM; cv.out = out;
             cv.N = N; cv.H = Hin; cv.W = Win; cv.C = 3; cv.K = s.K; cv.act = act;
             if (pool) { H = Hp; W = Wp; }
+            cv.alg_bytes = ((double)s.K * s.C * s.k * s.k + (double)N * Hin * Win * 3 + (double)N * H * W * s.K) * net->elem();  // (the map in front of the pool is never written)
             note((size_t)N * H * W * C);
             return;
         }

@@ -156,6 +156,28 @@ def test_profile_trace_lists_every_launch_of_a_wave():
     assert gnet.profile_trace() == []
 
 
+@pytest.mark.parametrize("family,res,batch", [(wl.RESNET, 64, 1), (wl.RESNET, 75, 2), (wl.MBV3, 64, 1)])
+def test_bytes_of_a_fused_stem_are_its_own(family, res, batch):
+    # weights, image and the map that the launch writes: behind the 7x7 stem that is the pooled one
+    _, _, gnet = gu.nets(family, True)
+    n = 3
+    cfgs = wl.uniform_stream(family, n, seed=12)
+    d_in = gu.to_device(wl.make_inputs(n, batch, res, seed=2, bf16=True).reshape(n * batch, res, res, 3), True)
+    gnet.set_option("profile", 2)
+    try:
+        _run(gnet, cfgs, d_in, batch, res, 1000, wave=n, conc=1)
+        stem = gnet.profile_trace()[0]
+    finally:
+        gnet.set_option("profile", 0)
+    side = (res + 1) // 2
+    k = 3
+    if family == wl.RESNET:
+        side, k = (side + 1) // 2, 7
+    K = [int(gnet.subnet_encode(c)[0][0]) for c in cfgs]
+    assert stem["name"] == "stem" and stem["members"] == n
+    assert stem["alg_bytes"] == 2 * sum(f * 3 * k * k + batch * (res * res * 3 + side * side * f) for f in K)
+
+
 @pytest.mark.parametrize("family,res", [(wl.RESNET, 224), (wl.MBV3, 224), (wl.RESNET, 192)])
 def test_members_sharing_a_tile_at_7x7_maps(family, res):
     # at 224x224 the last stage works on 7x7 maps: two members of a wave then share the 128 rows of a tile
