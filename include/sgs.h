@@ -449,6 +449,14 @@ sgs_status_t sgs_device_status_clear(void);
  * scratch buffer and synchronises. */
 sgs_status_t sgs_measure_fma_peak(double *tflops, void *cuda_stream);
 
+/* Test aid: the map that stored convolution `layer` (index as in sgs_subnet_encode) left for a SubNet, as the next layer reads it.  First
+ * run the SubNet with option "stop_after_layer" = layer (later layers reuse the buffers), by sgs_subnet_run (member = -1) or as
+ * member `member` of the first wave of a stream.  Copies [N][H][W][ld] elements of the handle's dtype to d_out on `cuda_stream` and
+ * sets dims[0..3] to N, H, W, ld: the channels beyond the slice are zeros, the max pool fused behind a 7x7 stem has run.  SGS_EINVAL
+ * where the SubNet does not use the layer, has not run there, or out_bytes is too small. */
+sgs_status_t sgs_debug_layer_map(sgs_supernet_t *net, const sgs_subnet_cfg_t *cfg, int batch, int res, int member, int layer, void *d_out,
+                                 size_t out_bytes, int *dims, void *cuda_stream);
+
 /* Test aid for the time-out path: enqueues a one-block kernel on `cuda_stream` whose only wait can never be
  * satisfied, with a limit of limit_us microseconds (1 .. 1000000).  The kernel gives up after the limit, sets the
  * device status word exactly as the convolution kernels do, and returns normally; nothing faults or hangs. */
@@ -470,7 +478,8 @@ sgs_status_t sgs_debug_expire_team_wait(int team, int block, int thread, unsigne
  * execution spends on the cached SubGraph's first pointwise layers (default 16, 0 = none); "persistent_team" n = SMs that serve a
  * query of persistent execution together (1, 2, 4, 8, 16; default 0 = chosen by the number and size of a call's queries); "nvtx" 1 = an NVTX range named after the stored layer around
  * every launch (for timeline tools); "fail_alloc_after" n = the handle's device allocations fail from
- * the (n+1)-th on with SGS_ENOMEM (fault injection on the host, -1 = off); "drop_plans" forgets every cached plan (measuring what a never-seen config costs); "profile" see
+ * the (n+1)-th on with SGS_ENOMEM (fault injection on the host, -1 = off); "stop_after_layer" n = queries and waves end behind the
+ * convolution of stored layer n (test aid, -1 = off; no logits); "drop_plans" forgets every cached plan (measuring what a never-seen config costs); "profile" see
  * sgs_profile_read; "stage_group" 0..4 is accepted
  * and has no effect (every pipeline stage of the grouped convolution kernel has its own barriers).  Unknown name -> SGS_EINVAL. */
 sgs_status_t sgs_set_option(sgs_supernet_t *net, const char *name, long long value);
@@ -504,7 +513,8 @@ typedef struct {
 int sgs_profile_trace(sgs_supernet_t *net, sgs_launch_record_t *out, int cap);
 int sgs_layer_name(const sgs_supernet_t *net, int layer, char *out, int cap);
 
-/* Counters by name ("kernel_launches", "plan_hits", "plan_misses", "device_bytes", "tc_convs";
+/* Counters by name ("kernel_launches", "plan_hits", "plan_misses", "device_bytes"; convolutions of the cached plans: "tc_convs" on the
+ * tensor cores, "grouped_convs" of single queries that go to the waves' kernel;
  * diagnostics: "host_us_stream", "host_us_query", "host_us_table", "host_us_graph", "host_us_direct" =
  * accumulated host microseconds spent issuing streams / queries / cache-table updates / graph
  * launches / direct launches). */

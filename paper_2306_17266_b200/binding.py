@@ -27,7 +27,7 @@ EXPORTS = [
     "sgs_set_option", "sgs_get_counter", "sgs_last_error", "sgs_supernet_free", "sgs_conv2d_sliced", "sgs_device_status",
     "sgs_profile_read", "sgs_conv2d_sliced_static", "sgs_cache_set_candidates", "sgs_cache_set_policy",
     "sgs_sched_create", "sgs_sched_free", "sgs_sched_dims", "sgs_sched_set_table", "sgs_sched_get_table", "sgs_sched_measure",
-    "sgs_sched_step", "sgs_sched_subnet", "sgs_profile_trace", "sgs_layer_name", "sgs_aux_op", "sgs_device_status_clear", "sgs_debug_expire_wait", "sgs_debug_expire_team_wait", "sgs_measure_fma_peak", "sgs_conv2d_sliced_i8",
+    "sgs_sched_step", "sgs_sched_subnet", "sgs_profile_trace", "sgs_layer_name", "sgs_aux_op", "sgs_device_status_clear", "sgs_debug_expire_wait", "sgs_debug_expire_team_wait", "sgs_debug_layer_map", "sgs_measure_fma_peak", "sgs_conv2d_sliced_i8",
 ]
 
 
@@ -202,6 +202,7 @@ def lib():
         L.sgs_aux_op.argtypes = [ci, vp, vp, ci, vp]
         L.sgs_device_status_clear.argtypes = []
         L.sgs_debug_expire_wait.argtypes = [ctypes.c_uint, vp]
+        L.sgs_debug_layer_map.argtypes = [vp, vp, ci, ci, ci, ci, vp, ctypes.c_size_t, vp, vp]
         L.sgs_debug_expire_team_wait.argtypes = [ci, ci, ci, ctypes.c_uint, vp, vp]
         L.sgs_measure_fma_peak.argtypes = [vp, vp]
         L.sgs_conv2d_sliced_i8.argtypes = [vp] * 9
@@ -367,6 +368,13 @@ class SuperNet:
             out.append({"kernel_class": r.kernel_class, "layer": r.layer, "name": name, "members": r.members, "tiles": r.tiles,
                         "ms": r.ms, "alg_bytes": r.alg_bytes, "flops": r.flops})
         return out
+
+    def debug_layer_map(self, cfg, batch: int, res: int, member: int, layer: int, out_ptr: int, out_bytes: int, stream: int = 0):
+        """Copies the map of a stored convolution (see sgs.h) to device memory; returns (N, H, W, ld)."""
+        dims = (ctypes.c_int * 4)()
+        self._check(lib().sgs_debug_layer_map(self._h, ctypes.byref(cfg), batch, res, member, layer, ctypes.c_void_p(out_ptr), out_bytes, dims,
+                                              ctypes.c_void_p(stream)))
+        return tuple(dims)
 
     def profile_read(self, kernel_class: int):
         n, ms, b, f = ctypes.c_longlong(), ctypes.c_double(), ctypes.c_double(), ctypes.c_double()

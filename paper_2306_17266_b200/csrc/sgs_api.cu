@@ -243,6 +243,7 @@ struct sgs_supernet {
     int persistent_team = 0;  // persistent execution: blocks that serve a query together (0: chosen by the call)
     int persistent_held_kb = 16;  // persistent execution: shared memory per SM for the cached SubGraph's first layers (0: none)
     long long fail_alloc_after = -1;  // < 0: off; else device allocations left before they start failing (test aid)
+    int stop_after_layer = -1;  // >= 0: queries end behind the convolution of this stored layer (test aid, see sgs_debug_layer_map)
     int cache_mech = 0;    // how grouped launches keep the cached SubGraph in L2: 0 per-tile hints, 1 access-policy window of the launch, 2 both
     int pad_channels = 1;  // waves of the ResNet-shaped family keep activation pixels at multiples of 16 channels
     int throughput_mode = 0;  // set by streams that keep many queries in flight; part of the plan key
@@ -918,6 +919,8 @@ sgs_status_t launch_op(sgs_supernet *net, Plan *plan, Op &op, const void *d_inpu
     return SGS_OK;
 }
 
+bool is_conv(const Op &op) { return op.type == OP_CONV || op.type == OP_DW || op.type == OP_STEM; }
+
 template <typename T>
 sgs_status_t run_ops(sgs_supernet *net, Plan *plan, const void *d_input, void *d_logits, cudaStream_t st, size_t first,
                      size_t last) {
@@ -939,11 +942,13 @@ sgs_status_t run_ops(sgs_supernet *net, Plan *plan, const void *d_input, void *d
             LayerRange range(net, op.layer, "two layers");
             CU(tc_conv_launch_pair(*op.tc, a, *next.tc, b, st));
             net->kernel_launches++;
+            if (net->stop_after_layer >= 0 && (op.layer == net->stop_after_layer || next.layer == net->stop_after_layer)) break;
             continue;
         }
         sgs_status_t rc = launch_op<T>(net, plan, op, d_input, d_logits, st);
         if (rc != SGS_OK) return rc;
         if (net->profile) CU(cudaEventRecord(plan->prof_ev[2 * oi + 1], st));
+        if (net->stop_after_layer >= 0 && is_conv(op) && op.layer == net->stop_after_layer) break;
     }
     return SGS_OK;
 }
@@ -1028,7 +1033,7 @@ sgs_status_t run_query(sgs_supernet *net, const sgs_subnet_cfg_t *cfg, const voi
     if (rc != SGS_OK) return rc;
     const size_t n_ops = plan->ops.size();
     if (net->profile) net->prof_used.push_back(plan);
-    if (!use_graph || net->profile || n_ops < 3) {
+    if (!use_graph || net->profile || net->stop_after_layer >= 0 || n_ops < 3) {
         long long before = net->kernel_launches;
         rc = run_plan(net, plan, d_input, d_logits, st, 0, n_ops);
         plan->launches = (int)(net->kernel_launches - before);
@@ -1474,6 +1479,14 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
     const size_t in_bytes = (size_t)batch * res * res * 3 * net->elem();
     const size_t out_bytes = (size_t)batch * net->def.classes * sizeof(float);
     const int n_ranks = (int)net->op_rank.size();
+    int stop_rank = n_ranks;  // of the last launches
+    if (net->stop_after_layer >= 0) {
+        stop_rank = -1;
+        for (const auto &kv : net->op_rank) {
+            const int type = (int)(kv.first >> 32);
+            if ((int)(kv.first & 0xffffffff) == net->stop_after_layer && (type == OP_CONV || type == OP_DW || type == OP_STEM)) stop_rank = std::max(stop_rank, kv.second);
+        }
+    }
     const int n_waves = (n_queries + G - 1) / G;
     std::vector<cudaEvent_t> ev;  // per wave: start and end on the wave's stream
     if (o.record_latency) {
@@ -1775,6 +1788,7 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
         };
         void *dlog = host_buffers ? (void *)cx.stage_out : dout;
         for (const Launch &L : launches) {
+            if (L.rank > stop_rank) break;
             double pb = 0, pf = 0;
             LayerRange range(net, first_layer(L.rank), "layer without weights");
             if (L.group) {
@@ -2664,6 +2678,11 @@ sgs_status_t sgs_set_option(sgs_supernet_t *net, const char *name, long long val
         net->persistent_held_kb = (int)value;
         return SGS_OK;
     }
+    if (n == "stop_after_layer") {
+        if (value < -1 || value >= (long long)net->layers.size() || (value >= 0 && net->layers[(size_t)value].kind == KIND_LINEAR)) return fail(net, SGS_EINVAL, "stop_after_layer names a stored convolution, or is -1");
+        net->stop_after_layer = (int)value;
+        return SGS_OK;
+    }
     if (n == "nvtx") {
         net->nvtx = value != 0;
         return SGS_OK;
@@ -2705,10 +2724,10 @@ long long sgs_get_counter(const sgs_supernet_t *net, const char *name) try {
     if (n == "host_us_stream") return (long long)net->host_us_stream;
     if (n == "host_us_query") return (long long)net->host_us_query;
     if (n == "host_us_table") return (long long)net->host_us_table;
-    if (n == "tc_convs") {
+    if (n == "tc_convs" || n == "grouped_convs") {
         long long c = 0;
         for (auto &kv : net->plans)
-            for (const Op &op : kv.second->ops) c += op.impl == 1;
+            for (const Op &op : kv.second->ops) c += op.impl == 1 && (n == "tc_convs" || tc_conv_grouped(*op.tc));
         return c;
     }
     return -1;
@@ -2858,6 +2877,32 @@ sgs_status_t sgs_measure_fma_peak(double *tflops, void *cuda_stream) {
     if (!tflops) return SGS_EINVAL;
     return measure_fma_rate(tflops, (cudaStream_t)cuda_stream) == cudaSuccess ? SGS_OK : SGS_ECUDA;
 }
+
+sgs_status_t sgs_debug_layer_map(sgs_supernet_t *net, const sgs_subnet_cfg_t *cfg, int batch, int res, int member, int layer, void *d_out,
+                                 size_t out_bytes, int *dims, void *cuda_stream) try {
+    if (!net) return SGS_EINVAL;
+    if (!cfg || !d_out || !dims || batch <= 0 || member < -1) return fail(net, SGS_EINVAL, "bad argument");
+    DeviceGuard guard(net->device);
+    if (!guard.ok) return fail(net, SGS_ECUDA, "cudaSetDevice failed");
+    if (member >= (int)net->slots.size()) return fail(net, SGS_EINVAL, "no such member");
+    Plan *plan = nullptr;
+    net->throughput_mode = member < 0 ? 0 : 2;
+    const sgs_status_t rc = get_plan(net, cfg, batch, res, std::max(0, member), &plan);
+    net->throughput_mode = 0;
+    if (rc != SGS_OK) return rc;
+    if (!plan->prepared) return fail(net, SGS_EINVAL, "this config has not run there");
+    for (const Op &op : plan->ops) {
+        if (!is_conv(op) || op.layer != layer) continue;
+        const ConvArgs &a = op.conv;
+        const bool pooled = op.type == OP_STEM && a.k == 7;
+        dims[0] = a.N; dims[1] = pooled ? (a.Ho - 1) / 2 + 1 : a.Ho; dims[2] = pooled ? (a.Wo - 1) / 2 + 1 : a.Wo; dims[3] = a.ldy ? a.ldy : a.K;
+        const size_t bytes = (size_t)dims[0] * dims[1] * dims[2] * dims[3] * net->elem();
+        if (bytes > out_bytes) return fail(net, SGS_EINVAL, "the layer's map takes " + std::to_string(bytes) + " bytes");
+        CU(cudaMemcpyAsync(d_out, net->slots[plan->slot].act[op.out], bytes, cudaMemcpyDeviceToDevice, (cudaStream_t)cuda_stream));
+        return SGS_OK;
+    }
+    return fail(net, SGS_EINVAL, "this config does not use that convolution");
+} SGS_NO_THROW
 
 sgs_status_t sgs_debug_expire_wait(unsigned limit_us, void *cuda_stream) {
     if (limit_us == 0 || limit_us > 1000000u) return SGS_EINVAL;

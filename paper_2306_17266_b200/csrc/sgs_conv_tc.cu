@@ -823,6 +823,8 @@ static TcParams launch_params(const TcConvPlan &pl, const ConvArgs &a, int dev) 
     return prm;
 }
 
+bool tc_conv_grouped(const TcConvPlan &p) { return p.grouped != 0; }
+
 // One launch instead of two saves a link of a query's chain (some 4 us) as long as the blocks of both layers are on the GPU at the
 // same time.  The tiles have one shape and the reductions one split (a property of the launch).
 bool tc_conv_pairs(const TcConvPlan &a, const TcConvPlan &b) {

@@ -240,6 +240,7 @@ cudaError_t launch_stem(const SmallEntry *h, const SmallEntry *d, int n, cudaStr
 // Returns nullptr when the shape is not handled by the tensor-core kernel (caller falls back).
 std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::string *why);
 cudaError_t tc_conv_launch(const TcConvPlan &p, const ConvArgs &a, cudaStream_t st);
+bool tc_conv_grouped(const TcConvPlan &p);  // a single query's layer on the grouped kernel?
 bool tc_conv_pairs(const TcConvPlan &a, const TcConvPlan &b);  // may two layers that do not depend on each other share a launch?
 cudaError_t tc_conv_launch_pair(const TcConvPlan &pa, const ConvArgs &a, const TcConvPlan &pb, const ConvArgs &b, cudaStream_t st);
 cudaError_t tc_conv_init(int device);  // one-time device set-up; call outside stream capture

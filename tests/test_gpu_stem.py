@@ -1,5 +1,5 @@
 """Stem kernels (7x7 stride 2 with its max pool, 3x3 of both strides) through whole networks at the edges of their tiles: 17 x 7
-convolution outputs around 8 x 3 pooled ones, 16 x 8 without a pool."""
+convolution outputs around 8 x 3 pooled ones, 16 x 8 without a pool.  (The stem's map itself: test_gpu_layer_maps.py.)"""
 import numpy as np
 import pytest
 import torch
@@ -17,7 +17,7 @@ TOL_BF16 = 2e-2  # max|err| / max|ref| per row, as in the other bf16 parity test
 # odd and even images, maps that end inside a tile, at its end and one beyond (resnet pools to 8 a tile across, 3 down: 33 -> 17 -> 9)
 @pytest.mark.parametrize("family,res,batch", [
     ("resnet", 64, 1), ("resnet", 75, 2), ("resnet", 97, 1), ("resnet", 32, 3), ("resnet", 130, 1),
-    ("mbv3", 34, 2), ("mbv3", 64, 1), ("mbv3", 70, 1), ("tiny", 32, 1), ("tiny", 24, 3), ("tiny", 41, 2),
+    ("mbv3", 34, 2), ("mbv3", 64, 1), ("mbv3", 70, 1), ("mbv3", 33, 2), ("mbv3", 71, 1), ("tiny", 32, 1), ("tiny", 24, 3), ("tiny", 41, 2),
 ])
 def test_networks_behind_the_stem(family, res, batch):
     fam = {"resnet": wl.RESNET, "mbv3": wl.MBV3, "tiny": wl.TINY}[family]
