@@ -807,16 +807,12 @@ sgs_status_t get_plan(sgs_supernet *net, const sgs_subnet_cfg_t *cfg, int batch,
     return SGS_OK;
 }
 
-// Argument record of a max pool, global average pool, linear or stem op (bf16 handles).
+// Argument record of a global average pool, linear, squeeze-excite or stem op (bf16 handles).
 SmallEntry small_entry(const sgs_supernet *net, const Plan *plan, const Op &op, const void *d_input, void *d_logits) {
     const sgs_supernet::Slot &sl = net->slots[plan->slot];
     SmallEntry e;
     std::memset(&e, 0, sizeof e);
     switch (op.type) {
-    case OP_MAXPOOL:
-        e.x = op.in < 0 ? d_input : sl.act[op.in]; e.y = sl.act[op.out];
-        e.N = op.N; e.H = op.H; e.W = op.W; e.C = op.C; e.Ho = (op.H - 1) / 2 + 1; e.Wo = (op.W - 1) / 2 + 1;
-        break;
     case OP_GAP:
         e.x = op.in < 0 ? d_input : sl.act[op.in]; e.y = sl.vec[op.vout];
         e.N = op.N; e.H = op.H; e.W = op.W; e.C = op.C;
@@ -1693,7 +1689,7 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
             // member's op has the vectorised form; the remaining ops run member by member
             const Op &op0 = plans[b[0].first]->ops[(size_t)b[0].second];
             const int kind = op0.type;
-            bool grouped = kind == OP_MAXPOOL || kind == OP_GAP || kind == OP_LINEAR || kind == OP_STEM || kind == OP_SCALE || kind == OP_SE_GATE || kind == OP_SE;
+            bool grouped = kind == OP_GAP || kind == OP_LINEAR || kind == OP_STEM || kind == OP_SCALE || kind == OP_SE_GATE || kind == OP_SE;
             if (grouped) {
                 const size_t off0 = off;
                 for (const auto &mo : b) {
@@ -1716,7 +1712,6 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
                 bool ok = true;
                 int total_dw = 0;
                 for (int kk : {3, 5, 7}) {
-                    const size_t offk = off;
                     int cnt = 0;
                     for (const auto &mo : b) {
                         const Op &op = plans[mo.first]->ops[(size_t)mo.second];
@@ -1727,7 +1722,6 @@ static sgs_status_t wave_impl(sgs_supernet_t *net, int n_queries, const sgs_subn
                         off += DW_ENTRY_BYTES;
                         cnt++;
                     }
-                    (void)offk;
                     total_dw += cnt;
                 }
                 // one launch for the layer: blocks pick the kernel body of their member's kernel size

@@ -55,7 +55,7 @@ struct __align__(16) GroupEntry {
     short pix_rows;          // rows of the pixel box (bw * bh * bn)
     short map_y, map_r;      // output and residual views (not of swapped members)
     short can_pair;          // (host) one tile of at most 64 pixels, square kernel: may share a tile, see below
-    unsigned char k, stride, p, act, swap, kw;  // k x kw taps
+    unsigned char k, stride, p, act, swap, pad2_;  // k x k taps
     // Two members with at most 64 output pixels each can share a tile: the first ("pair") owns the tile's
     // geometry, filters and weight map and takes MMA rows 0..63, the entry after it ("second") takes rows
     // 64..127 with its own activation map, outputs and filter count (not larger than the first's).
@@ -223,14 +223,14 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
             const uint32_t w_bytes = uniform((uint32_t)(wrows * CHUNK_C * 2));
             const uint32_t dst0 = uniform(ring + (e.swap ? 0u : (uint32_t)G_X_BYTES));
             const CUtensorMap *map_w = &P.maps[uniform((uint32_t)e.map_w)];
-            const int k = (int)uniform(e.k), kw = (int)uniform(e.kw), cchunks = (int)uniform((uint32_t)e.cchunks), R = (int)uniform((uint32_t)e.R);
+            const int k = (int)uniform(e.k), cchunks = (int)uniform((uint32_t)e.cchunks), R = (int)uniform((uint32_t)e.R);
             // channels below hint_c take a hint: the cached SubGraph's box (keep), or everything (stream)
             const int cacheK = P.cache_tbl ? tblK : (int)uniform((uint32_t)e.cacheK), cacheC = P.cache_tbl ? tblC : (int)uniform((uint32_t)e.cacheC);
             const int hint_c = cacheK < 0 ? 0x7fffffff : f0 < cacheK ? cacheC : 0;
             const uint64_t pol = cacheK < 0 ? pol_stream : pol_keep;
             int tap_row = (int)uniform((uint32_t)e.tap0);
             for (int r = 0; r < k && ok; r++, tap_row += R) {
-                for (int sx = 0; sx < kw && ok; sx++) {
+                for (int sx = 0; sx < k && ok; sx++) {
                     for (int cc = 0, c0 = 0; cc < cchunks; cc++, c0 += CHUNK_C) {
                         if (wrapped && !(ok = __all_sync(0xffffffffu, mbar_wait(&empty_bar[s], phase ^ 1, abort_flag)))) break;
                         const uint32_t sb = dst0 + (uint32_t)(s * stage_bytes), fb = full0 + (uint32_t)(s * 8);
@@ -262,9 +262,9 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
             const uint32_t dst0 = uniform(ring + (e.swap ? (uint32_t)G_X_BYTES : 0u));
             const int dh2 = (int)uniform((uint32_t)(pair ? (&e)[1].slot_h - e.slot_h : 0)), dn2 = (int)uniform((uint32_t)(pair ? (&e)[1].slot_n - e.slot_n : 0));
             const int map_a = (int)uniform((uint32_t)e.map_a), map_a2 = (int)uniform((uint32_t)(pair ? (&e)[1].map_a : e.map_a));
-            const int k = (int)uniform(e.k), kw = (int)uniform(e.kw), cchunks = (int)uniform((uint32_t)e.cchunks), pad = (int)uniform(e.p), stride = (int)uniform(e.stride);
+            const int k = (int)uniform(e.k), cchunks = (int)uniform((uint32_t)e.cchunks), pad = (int)uniform(e.p), stride = (int)uniform(e.stride);
             for (int r = 0; r < k && ok; r++) {
-                for (int sx = 0; sx < kw && ok; sx++) {
+                for (int sx = 0; sx < k && ok; sx++) {
                     const int dh = r - pad, dw = sx - pad;
                     // stride 2: one of the four parity views, at half the offset
                     const int ph = stride == 2 ? (dh & 1) : 0, pw = stride == 2 ? (dw & 1) : 0, view = ph * 2 + pw;
@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
             const int n_mma = e.swap ? e.bn_tile : min((int)e.bn_tile, (e.K - (rec.x >> 8) + 15) & ~15);
             const uint32_t idesc = uniform((1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n_mma >> 3) << 17) | ((uint32_t)(TILE_M >> 4) << 24));
             const int buf = j & 1;
-            const int cchunks = (int)uniform((uint32_t)e.cchunks), iters = (int)uniform((uint32_t)(e.k * e.kw)) * cchunks;
+            const int cchunks = (int)uniform((uint32_t)e.cchunks), iters = (int)uniform((uint32_t)(e.k * e.k)) * cchunks;
             const int last_ksteps = (int)uniform((uint32_t)((e.C - (cchunks - 1) * CHUNK_C + 15) / 16));  // 16-channel steps of a tap's last chunk
             ok = j < 2 || mbar_wait(&acc_empty[buf], ((j >> 1) - 1) & 1, abort_flag);  // epilogue drained this buffer
             ok = __all_sync(0xffffffffu, ok);
@@ -600,7 +600,7 @@ void tc_group_entry(TcConvPlan &pl, const ConvArgs &a) {
     e.pix_rows = (short)(p.bw * p.bh * p.bn);
     e.swap = (unsigned char)pl.swap;
     e.bn_tile = (short)(pl.swap ? (e.pix_rows + 15) / 16 * 16 : pl.bn_tile);
-    e.k = (unsigned char)p.k; e.kw = (unsigned char)pl.kw; e.stride = (unsigned char)p.stride; e.p = (unsigned char)p.p; e.act = (unsigned char)p.act;
+    e.k = (unsigned char)p.k; e.stride = (unsigned char)p.stride; e.p = (unsigned char)p.p; e.act = (unsigned char)p.act;
     e.can_pair = !pl.swap && e.mtiles == 1 && e.pix_rows <= 64;
     std::memcpy(pl.entry, &e, sizeof e);
     pl.g_iters = p.iters;

@@ -653,7 +653,6 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
     std::memset(&p, 0, sizeof(p));
     p.N = a.N; p.Ho = a.Ho; p.Wo = a.Wo; p.K = a.K; p.C = a.C;
     p.k = a.k; p.stride = a.stride; p.R = a.R; p.o = (a.R - a.k) / 2; p.p = (a.k - 1) / 2;
-    plan->kw = a.k;
     p.act = a.act;
     const bool flat = a.k == 1 && a.stride == 1;
     // C = channels per pixel of x as stored (pitch and extent of the activation maps): with padded pixels the
@@ -715,7 +714,7 @@ std::shared_ptr<TcConvPlan> tc_conv_prepare(const ConvArgs &a, int device, std::
     // filter tile: 128 wide unless the layer is narrow or too few CTAs would stream the weights
     const int sms = sm_count();
     p.cchunks = (a.C + (int)CH - 1) / (int)CH;
-    p.iters = a.k * plan->kw * p.cchunks;
+    p.iters = a.k * a.k * p.cchunks;
     // Filter tile: 128 wide where the tiles then still occupy every SM (half the pixel copies per filter), else 64.
     int BN = (a.K > 64 && (long long)mtiles * ((a.K + 127) / 128) >= sms) ? 128 : 64;
     // 8-bit layers whose 64-wide tiles are all resident at two blocks per SM take those: no SM then gets two 128-wide tiles

@@ -129,11 +129,9 @@ __device__ __forceinline__ void tma_store_4d_if(uint32_t on, const CUtensorMap *
         ::"l"(map), "r"(src), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(on)
         : "memory");
 }
-// Groups of bulk stores: commit() closes one, wait_read<N> waits until all but the last N have read their shared memory,
-// wait_all until everything is written.
+// Groups of bulk stores: commit() closes one, wait_read<N> waits until all but the last N have read their shared memory.
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory"); }
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ uint4 lds128(uint32_t addr) {
     uint4 v;
@@ -263,7 +261,6 @@ struct TcConvPlan {
     CUtensorMap tmY, tmR;  // grouped launches, not swapped: output and residual as boxes of 64 filters x the tile's pixels
     int has_res = 0;
     int grouped = 0;     // this layer of a single query runs on the grouped kernel
-    int kw = 1;          // taps along x
 };
 
 }  // namespace sgs
