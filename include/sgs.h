@@ -184,6 +184,8 @@ sgs_status_t sgs_subnet_validate(const sgs_supernet_t *net, const sgs_subnet_cfg
  * Asynchronous on `cuda_stream`.  Invalid config -> SGS_ECONFIG before anything is launched.
  * No sliced copy of any weight is made; the only device memory that may grow is the activation
  * workspace, on the first use of a larger (batch, res).
+ * Can be captured after a first call with the same (cfg, batch, res) outside the capture.  The cached SubGraph's load hints are not part
+ * of a graph: a replay uses those in force, and a choice made under capture reaches the device with the next call outside one.
  */
 sgs_status_t sgs_subnet_run(sgs_supernet_t *net, const sgs_subnet_cfg_t *cfg, const void *d_input, int batch,
                             int res, void *d_logits, void *cuda_stream);

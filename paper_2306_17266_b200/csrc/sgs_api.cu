@@ -987,6 +987,9 @@ sgs_status_t run_plan(sgs_supernet *net, Plan *plan, const void *d_input, void *
 sgs_status_t push_cache_table(sgs_supernet *net, cudaStream_t st) {
     const CacheState &cs = net->cache;
     if (net->cache_tbl_epoch == cs.epoch) return SGS_OK;
+    // Not part of a capture: a replay would bring back the SubGraph of that day, and the ring's events are not the graph's.  The captured
+    // kernels read whatever the table holds; the next call outside a capture brings it up to date.  (The table only holds load hints.)
+    if (being_captured(st)) return SGS_OK;
     const size_t n = 1 + 2 * net->layers.size();
     const int slot = net->tbl_ring_pos;
     net->tbl_ring_pos = (slot + 1) % 16;

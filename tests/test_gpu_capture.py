@@ -66,6 +66,38 @@ def test_captured_calls_replay(make, kind):
     assert sgs.device_status() == 0
 
 
+def test_a_query_is_captured_while_the_cached_subgraph_changes():
+    # window 1: every query is a caching decision, so the capture begins with a table the device has not seen yet, and changes it
+    net = sgs.SuperNet(wl.RESNET, gu.nets(wl.RESNET, True)[0], sgs.SGS_BF16)
+    cfgs, res = wl.cfg_array([wl.extreme_cfg(wl.RESNET, False), wl.extreme_cfg(wl.RESNET, True)]), 64
+    x, y = torch.randn(1, res, res, 3, device="cuda").bfloat16(), torch.zeros(2, 1000, device="cuda")
+    st = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    run = lambda i: net.subnet_run(cfgs[i], x.data_ptr(), 1, res, y[i].data_ptr(), st.cuda_stream)
+    for i in (0, 1):
+        run(i)
+    torch.cuda.synchronize()
+    want = y.clone()
+    net.cache_configure(True, 0, 1)
+    run(0)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=st):
+        run(1)
+        run(0)
+    assert net.cache_stats().decisions == 3
+    y.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(y, want)
+    y.zero_()
+    torch.cuda.synchronize()
+    run(1)
+    run(0)
+    torch.cuda.synchronize()
+    assert torch.equal(y, want)
+    net.close()
+
+
 def test_grouped_layers_refuse_capture():
     x, y, b = torch.randn(3, 512, device="cuda"), torch.zeros(3, 100, device="cuda"), torch.zeros(100, device="cuda")
     w = torch.randn(100, 512, device="cuda").bfloat16()
