@@ -470,6 +470,12 @@ sgs_status_t sgs_debug_expire_wait(unsigned limit_us, void *cuda_stream);
  * ran out.  Sets the device status word. */
 sgs_status_t sgs_debug_expire_team_wait(int team, int block, int thread, unsigned limit_us, int *d_left, void *cuda_stream);
 
+/* Test aid: how persistent execution with `team` (1, 2, 4, 8, 16) SMs a query cuts a pointwise layer of `pixels` x `filters` into tiles
+ * of 128 pixels x *tile_filters (16 .. 256), *filter_tiles of them along the filters, and how many filters of tile i < max_tiles, its
+ * first held[i], come out of a weight buffer that holds the layer's first `held_rows` filters. */
+sgs_status_t sgs_debug_pointwise_tiles(int pixels, int filters, int team, int held_rows, int *filter_tiles, int *tile_filters, int *held,
+                                       int max_tiles);
+
 /* Library options by name (debug and measurement aids): "conv_impl" 0 = automatic, 1 = force the
  * CUDA-core kernels; "pad_channels" 1 (default) = waves of the ResNet-shaped family keep their activation tensors
  * at 16-channel pixels (zeros beyond the slice), 0 = dense pixels; "cache_mechanism" how grouped launches keep the cached SubGraph in L2: 0 (default) = an evict-last

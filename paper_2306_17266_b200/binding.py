@@ -27,7 +27,7 @@ EXPORTS = [
     "sgs_set_option", "sgs_get_counter", "sgs_last_error", "sgs_supernet_free", "sgs_conv2d_sliced", "sgs_device_status",
     "sgs_profile_read", "sgs_conv2d_sliced_static", "sgs_cache_set_candidates", "sgs_cache_set_policy",
     "sgs_sched_create", "sgs_sched_free", "sgs_sched_dims", "sgs_sched_set_table", "sgs_sched_get_table", "sgs_sched_measure",
-    "sgs_sched_step", "sgs_sched_subnet", "sgs_profile_trace", "sgs_layer_name", "sgs_aux_op", "sgs_device_status_clear", "sgs_debug_expire_wait", "sgs_debug_expire_team_wait", "sgs_debug_layer_map", "sgs_measure_fma_peak", "sgs_conv2d_sliced_i8",
+    "sgs_sched_step", "sgs_sched_subnet", "sgs_profile_trace", "sgs_layer_name", "sgs_aux_op", "sgs_device_status_clear", "sgs_debug_expire_wait", "sgs_debug_expire_team_wait", "sgs_debug_pointwise_tiles", "sgs_debug_layer_map", "sgs_measure_fma_peak", "sgs_conv2d_sliced_i8",
 ]
 
 
@@ -204,6 +204,7 @@ def lib():
         L.sgs_debug_expire_wait.argtypes = [ctypes.c_uint, vp]
         L.sgs_debug_layer_map.argtypes = [vp, vp, ci, ci, ci, ci, vp, ctypes.c_size_t, vp, vp]
         L.sgs_debug_expire_team_wait.argtypes = [ci, ci, ci, ctypes.c_uint, vp, vp]
+        L.sgs_debug_pointwise_tiles.argtypes = [ci, ci, ci, ci, vp, vp, vp, ci]
         L.sgs_measure_fma_peak.argtypes = [vp, vp]
         L.sgs_conv2d_sliced_i8.argtypes = [vp] * 9
         L.sgs_profile_read.argtypes = [vp, ci, vp, vp, vp, vp]

@@ -2913,4 +2913,15 @@ sgs_status_t sgs_debug_expire_team_wait(int team, int block, int thread, unsigne
     return subnet_team_expire(team, block, thread, limit_us, d_left, tc_status_word(dev), (cudaStream_t)cuda_stream) == cudaSuccess ? SGS_OK : SGS_ECUDA;
 }
 
+sgs_status_t sgs_debug_pointwise_tiles(int pixels, int filters, int team, int held_rows, int *filter_tiles, int *tile_filters, int *held,
+                                       int max_tiles) {
+    if (pixels < 1 || pixels > 1 << 20 || filters < 1 || filters > 1 << 16 || !in_set(team, {1, 2, 4, 8, 16}) || held_rows < 0 || !filter_tiles || !tile_filters ||
+        max_tiles < 0 || (max_tiles && !held))
+        return SGS_EINVAL;
+    const PwTiles t = pw_tiles(pixels, filters, team);
+    *filter_tiles = t.n_tiles; *tile_filters = t.BN;
+    for (int i = 0; i < std::min(t.n_tiles, max_tiles); i++) held[i] = pw_held_filters(t.BN, i, filters, held_rows);
+    return SGS_OK;
+}
+
 }  // extern "C"

@@ -124,6 +124,29 @@ struct alignas(16) PqHeld {
     int pad_;
 };
 static_assert(sizeof(PqHeld) == 32, "record size");
+// How the persistent kernel cuts a pointwise layer of M pixels and K filters for a team of `team` blocks: pixel tiles of 128, as few
+// filter tiles as PQ_MAX_BN allows, more where the pixel tiles alone leave blocks of the team idle (a 7x7 map is one pixel tile).
+constexpr int PQ_MAX_BN = 256;  // filters per tile
+struct PwTiles {
+    int m_tiles, n_tiles, BN;
+};
+__host__ __device__ inline PwTiles pw_tiles(int M, int K, int team) {
+    PwTiles t;
+    t.m_tiles = (M + 127) >> 7;
+    t.n_tiles = (K + PQ_MAX_BN - 1) / PQ_MAX_BN;
+    if (t.n_tiles * t.m_tiles < team) {
+        const int most = (K + 15) >> 4, want = (team + t.m_tiles - 1) / t.m_tiles;
+        t.n_tiles = most < want ? most : want;
+    }
+    t.BN = (((K + t.n_tiles - 1) / t.n_tiles) + 15) & ~15;  // MMA width: a multiple of 16, at most PQ_MAX_BN
+    t.n_tiles = (K + t.BN - 1) / t.BN;                      // (the rounding may leave the last one empty)
+    return t;
+}
+// Filters of tile nt that the weight buffer holds when it has the layer's first `rows`: a prefix of the tile, a multiple of 16.
+__host__ __device__ inline int pw_held_filters(int BN, int nt, int K, int rows) {
+    const int left = ((rows < K ? rows : K) & ~15) - nt * BN;
+    return left <= 0 ? 0 : left < BN ? left : BN;
+}
 struct PqParams {
     const PqHeld *held;      // n_held boxes, held_bytes in total (0: no weight buffer)
     int n_held;

@@ -39,7 +39,6 @@ constexpr int PQ_THREADS = SUBNET_THREADS;
 constexpr int PQ_WARPS = PQ_THREADS / 32;
 constexpr int PQ_ROWS = PQ_THREADS / 8;      // rows of 128 bytes one round of 16-byte copies covers
 constexpr int PQ_MAX_K = 1024;               // widest pointwise layer (folded batch norm staged in shared memory)
-constexpr int PQ_MAX_BN = 256;               // filters per tile
 constexpr int PQ_RING_BYTES = 144 * 1024;    // operand ring: 3 stages of pixel tile (16 KB) + filter tile (up to 32 KB), or 4 smaller ones
 constexpr int PQ_LAG = 2;                    // copies run this many stages ahead of the MMAs
 constexpr int PQ_VEC = 1280;                 // longest fp32 vector held in shared memory (the head's width)
@@ -124,16 +123,11 @@ __device__ __forceinline__ float dot8w(uint4 wv, float4 x0, float4 x1, float s) 
 struct PwShape {
     int M, C, K, n_tiles, BN, cchunks, m_tiles, stage_bytes, S;
 };
-// Filter tiles: as few as PQ_MAX_BN allows, more where the pixel tiles alone leave blocks of the team idle (a 7x7 map is one
-// pixel tile).
 template <class T> __device__ __forceinline__ PwShape pw_shape(const PqOp &op, const T &team) {
     PwShape s;
     s.M = op.Ho * op.Wo; s.C = op.C; s.K = op.K;
-    s.m_tiles = (s.M + 127) >> 7;
-    s.n_tiles = (s.K + PQ_MAX_BN - 1) / PQ_MAX_BN;
-    if (s.n_tiles * s.m_tiles < team.n) s.n_tiles = min((s.K + 15) >> 4, (team.n + s.m_tiles - 1) / s.m_tiles);
-    s.BN = (((s.K + s.n_tiles - 1) / s.n_tiles) + 15) & ~15;  // MMA width: a multiple of 16, at most PQ_MAX_BN
-    s.n_tiles = (s.K + s.BN - 1) / s.BN;  // (the rounding may leave the last one empty)
+    const PwTiles t = pw_tiles(s.M, s.K, team.n);
+    s.m_tiles = t.m_tiles; s.n_tiles = t.n_tiles; s.BN = t.BN;
     s.cchunks = (s.C + 63) >> 6;
     s.stage_bytes = A_STAGE_BYTES + s.BN * 128;
     s.S = min(4, PQ_RING_BYTES / s.stage_bytes);
@@ -225,14 +219,12 @@ __device__ __forceinline__ bool pq_pointwise(const PqOp &op, const bf16 *x, cons
     // swizzle term row % 8 is then the same for all of them)
     const int c16 = tid & 7, r0 = tid >> 3;
     const uint32_t piece = (uint32_t)((c16 ^ (r0 & 7)) << 4);
-    // Weight buffer: of this layer's box the query can use the first hK filters (a multiple of 16) in every channel
-    // chunk whose channels - as far as the query takes them - lie inside the box; those need no copy and are
+    // Weight buffer: a tile can use the filters of this layer's box that it covers (its first ones, a multiple of 16) in every
+    // channel chunk whose channels - as far as the query takes them - lie inside the box; those need no copy and are
     // multiplied in place, the tile's other filters come through the ring and get an MMA of their own.
-    const int hK = (held_u32 != 0u && op.cache_off >= 0 && s.n_tiles == 1) ? (min(op.cache_rows, s.K) & ~15) : 0;
+    const int box_rows = held_u32 != 0u && op.cache_off >= 0 ? op.cache_rows : 0;
     const uint32_t box_u32 = held_u32 + (uint32_t)(op.cache_off < 0 ? 0 : op.cache_off);
-    const uint32_t idesc_h = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(hK >> 3) << 17) | ((uint32_t)(TILE_M >> 4) << 24);
-    const uint32_t idesc_r = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((s.BN - hK) >> 3) << 17) | ((uint32_t)(TILE_M >> 4) << 24);
-    auto chunk_held = [&](int ch) { return hK > 0 && min(s.C, (ch + 1) * 64) <= op.ld2; };
+    auto held_filters = [&](int nt, int ch) { return box_rows > 0 && min(s.C, (ch + 1) * 64) <= op.ld2 ? pw_held_filters(s.BN, nt, s.K, box_rows) : 0; };
 
     bool ok = true;
     int p_chunk = 0, p_nt = team.rank / s.m_tiles, p_mt = team.rank - p_nt * s.m_tiles, p_stage = 0;  // next iteration to copy
@@ -252,8 +244,11 @@ __device__ __forceinline__ bool pq_pointwise(const PqOp &op, const bf16 *x, cons
                 const uint32_t sa = ring_u32 + (uint32_t)(c_stage * s.stage_bytes), sb = sa + A_STAGE_BYTES;
                 const uint64_t da = smem_desc_sw128(sa), db = smem_desc_sw128(sb);
                 const int ksteps = (min(64, s.C - c_chunk * 64) + 15) >> 4;
-                if (chunk_held(c_chunk)) {
-                    const uint64_t dh = smem_desc_sw128(box_u32 + (uint32_t)(c_chunk * op.cache_rows * 128));
+                const int hK = held_filters(c_nt, c_chunk);
+                if (hK > 0) {
+                    const uint32_t no_n = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TILE_M >> 4) << 24);
+                    const uint32_t idesc_h = no_n | ((uint32_t)(hK >> 3) << 17), idesc_r = no_n | ((uint32_t)((s.BN - hK) >> 3) << 17);
+                    const uint64_t dh = smem_desc_sw128(box_u32 + (uint32_t)((c_chunk * box_rows + c_nt * s.BN) * 128));
                     const uint64_t dr = smem_desc_sw128(sb + (uint32_t)(hK * 128));
                     for (int q = 0; q < ksteps; q++) {
                         umma_bf16(tmem_base + buf * PQ_ACC_COLS, da + (uint64_t)(2 * q), dh + (uint64_t)(2 * q), idesc_h, (c_chunk > 0 || q > 0) ? 1u : 0u);
@@ -295,7 +290,7 @@ __device__ __forceinline__ bool pq_pointwise(const PqOp &op, const bf16 *x, cons
                 const bool v = cvalid && m < s.M;
                 cp16_cg(sa + (uint32_t)(row * 128) + piece, v ? x + (size_t)m * s.C + c0 : x, v);
             }
-            for (int row = r0 + (chunk_held(p_chunk) ? hK : 0); row < s.BN; row += PQ_ROWS) {
+            for (int row = r0 + held_filters(p_nt, p_chunk); row < s.BN; row += PQ_ROWS) {
                 const int f = p_nt * s.BN + row;
                 const bool v = cvalid && f < s.K;
                 cp16_ca(sb + (uint32_t)(row * 128) + piece, v ? w + (size_t)f * op.ld + c0 : w, v);

@@ -109,6 +109,31 @@ def test_weight_buffer_in_shared_memory_changes_no_bit():
         gnet.set_option("persistent_held_kb", 16)
 
 
+@pytest.mark.parametrize("team", [1, 2, 4, 8, 16])
+def test_weight_buffer_is_used_by_every_team(team):
+    # Layers whose filters are split over a team's blocks (maps of 64x64 images have 8 pixel tiles at most) multiply the part of the
+    # box that a tile covers: the same bits as without a buffer, and the same figures for every team.
+    _, _, gnet = gu.nets(wl.MBV3, True)
+    n, res = 20, 64
+    cfgs = wl.markov_stream(n - 2, seed=12, family=wl.MBV3) + [wl.extreme_cfg(wl.MBV3, False), wl.extreme_cfg(wl.MBV3, True)]
+    d_in = gu.to_device(wl.make_inputs(n, 1, res, seed=13, bf16=True).reshape(n, res, res, 3), True)
+    try:
+        gnet.set_option("persistent_team", 1)
+        off, _ = _run(gnet, cfgs, d_in, res, cache=0)
+        for kb in (16, 56):
+            gnet.set_option("persistent_held_kb", kb)
+            gnet.set_option("persistent_team", 1)
+            _, st_one = _run(gnet, cfgs, d_in, res)
+            gnet.set_option("persistent_team", team)
+            on, st_on = _run(gnet, cfgs, d_in, res)
+            np.testing.assert_array_equal(on, off)
+            assert 0 < st_on.hbm_weight_bytes < st_on.weight_bytes
+            assert (st_on.hit_ratio, st_on.hbm_weight_bytes) == (st_one.hit_ratio, st_one.hbm_weight_bytes)
+    finally:
+        gnet.set_option("persistent_held_kb", 16)
+        gnet.set_option("persistent_team", 0)
+
+
 def test_persistent_stream_full_resolution_sampled():
     _, onet, gnet = gu.nets(wl.MBV3, True)
     n, res = 160, 224

@@ -29,6 +29,26 @@ def test_every_declared_symbol_is_exported():
     assert sorted(EXPORTS) == names
 
 
+def test_split_pointwise_layers_use_the_whole_held_box():
+    # persistent execution: whatever the team, the tiles of a layer cover its filters and together take every whole group of 16 filters
+    # that the weight buffer holds (hit_ratio and hbm_weight_bytes count the box for every team)
+    fn = sgs.lib().sgs_debug_pointwise_tiles
+    nt, bn, held = ctypes.c_int(), ctypes.c_int(), (ctypes.c_int * 128)()
+    for pixels in (1, 4, 49, 128, 129, 256, 1024, 12544):
+        for filters in (8, 16, 24, 40, 120, 256, 264, 960, 1024):
+            for team in (1, 2, 4, 8, 16):
+                for rows in (0, 16, 48, 256):
+                    assert fn(pixels, filters, team, rows, ctypes.byref(nt), ctypes.byref(bn), held, 128) == 0
+                    n, b = nt.value, bn.value
+                    assert b % 16 == 0 and 16 <= b <= 256 and (n - 1) * b < filters <= n * b
+                    got = list(held[:n])
+                    assert all(h % 16 == 0 and 0 <= h <= b for h in got)
+                    assert sum(got) == min(rows, filters) // 16 * 16, (pixels, filters, team, rows, got)
+                    assert all(h == b for h in got[:max(sum(h > 0 for h in got) - 1, 0)])  # a prefix of the layer
+    assert fn(0, 16, 1, 0, ctypes.byref(nt), ctypes.byref(bn), held, 128) != 0
+    assert fn(49, 16, 3, 0, ctypes.byref(nt), ctypes.byref(bn), held, 128) != 0
+
+
 def test_struct_sizes_match_the_header():
     # sizes implied by the header's field lists (LP64)
     assert ctypes.sizeof(wl.SubnetCfg) == 4 * (8 + 9 + 64 + 64)
