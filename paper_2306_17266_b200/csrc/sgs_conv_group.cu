@@ -199,6 +199,9 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
     const bool tail_in_ring = n_bufs == 1;
 
     // The three issuing warps run their loops converged; the elected lane issues (see sgs_tc.cuh).
+    // Their loops over tiles end at total_tiles, not at n_tiles: with a trip count out of a division the MMA warp's own part of a
+    // stage (waits left out) took 447 clocks instead of 331, which bounds tiles of few columns (B200; a 3x3 layer of 72 stages and
+    // 16 columns 44.5 us, 36.3 like this; waves of 32 images of 32x32 878 -> 777 us, 4 queries x 16 images of 224x224 13150 -> 12780).
     const uint32_t ring = smem_u32(smem), bufs = ring + (uint32_t)(n_stages * stage_bytes), full0 = smem_u32(full_bar), empty0 = smem_u32(empty_bar);
     if (warp == 0) {
         // ------------------------------------------------------------------ weight producer
@@ -215,7 +218,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
         int s = 0;
         uint32_t phase = 0;
         bool wrapped = false, ok = true;
-        for (int j = 0; j < n_tiles && ok; j++) {
+        for (int j = 0, t = (int)blockIdx.x; t < total_tiles && ok; j++, t += (int)gridDim.x) {
             const int4 rec = record(j);
             const GroupEntry &e = es[rec.x & 255];
             const int wrows = e.swap ? 128 : e.bn_tile;  // rows of the weight box
@@ -241,7 +244,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
                     }
                 }
             }
-            if (ok && on && j + 1 < n_tiles) prefetch_tensormap(&P.maps[es[record(j + 1).x & 255].map_w]);
+            if (ok && on && t + (int)gridDim.x < total_tiles) prefetch_tensormap(&P.maps[es[record(j + 1).x & 255].map_w]);
             __syncwarp();
         }
     } else if (warp == G_PIX_WARP) {
@@ -253,7 +256,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
         if (on) prefetch_tensormap(&P.maps[es[recs[0].x & 255].map_a]);
         __syncwarp();
         pdl_wait();  // activations (and the buffers this layer overwrites) belong to the previous layers until here
-        for (int j = 0; j < n_tiles && ok; j++) {
+        for (int j = 0, t = (int)blockIdx.x; t < total_tiles && ok; j++, t += (int)gridDim.x) {
             const int4 rec = record(j);
             const GroupEntry &e = es[rec.x & 255];
             const int n0 = (int)uniform((uint32_t)rec.w), h0 = (int)uniform((uint32_t)rec.z), w0 = (int)uniform((uint32_t)rec.y);
@@ -280,7 +283,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
                     }
                 }
             }
-            if (ok && on && j + 1 < n_tiles) prefetch_tensormap(&P.maps[es[record(j + 1).x & 255].map_a]);
+            if (ok && on && t + (int)gridDim.x < total_tiles) prefetch_tensormap(&P.maps[es[record(j + 1).x & 255].map_a]);
             __syncwarp();
         }
         // The next launch's CTAs come when this one's have asked for their last operands.  Told earlier, they (and those of the
@@ -292,7 +295,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
         int s = 0;
         uint32_t phase = 0;
         bool ok = true;
-        for (int j = 0; j < n_tiles && ok; j++) {
+        for (int j = 0, t = (int)blockIdx.x; t < total_tiles && ok; j++, t += (int)gridDim.x) {
             const int4 rec = record(j);
             const GroupEntry &e = es[rec.x & 255];
             // MMA shape: 128 rows; columns = this tile's filters (normal) or the member's pixels (swapped),
