@@ -10,7 +10,8 @@
 //
 // What bounds it: the shared-memory pipe (some 2200 clocks a tile of 128 B a clock: the build's 4-byte reads and 16-byte writes
 // are 1000 of them, the MMAs' operand reads 530) and the latency of a block's phases in series (8000 clocks a tile; two blocks
-// share an SM; 512 threads a block were slower, 148 us for the 133 below).  64 images of 224x224, 7x7 with pool: 125 us, against
+// share an SM; a version with 512 threads a block took 148 us where the same one with 256 took 133).  64 images of 224x224, 7x7
+// with pool, as it is now: 125 us, against
 // 188 of three launches (copy to 8-channel pixels 24, convolution over windows of them by the copy unit 137, max pool 27); 32
 // images one by one 71 us against 111.  3x3, 16 filters, 32 images: 31.5 us against 16 + 48.
 #include "sgs_tc.cuh"

@@ -7,7 +7,7 @@
 // next unserved query from a counter and runs all layers of that query's SubNet by itself, image to logits.  With fewer queries
 // than SMs a query is served by a team of 2 to 16 blocks, a cluster: every layer's tiles, rows, pixels or outputs are dealt to
 // them, pooled vectors and gates go to all through distributed shared memory, and a cluster barrier ends a layer (8 queries:
-// 3.45 ms with a block each, 0.87 with 8; the choice is the host's, choose_team in sgs_api.cu).
+// 3.05 ms with a block each, 0.87 with 8; the choice is the host's, choose_team in sgs_api.cu).
 //   * pointwise (1x1) convolutions on the tensor cores: tcgen05.mma with the fp32 accumulator in tensor memory
 //     (two 256-column buffers, so the epilogue of one tile overlaps the MMAs of the next); the operands are
 //     brought into 128-byte-swizzled shared-memory tiles by the block's own threads with 16-byte asynchronous
