@@ -2,7 +2,7 @@
 """Benchmark of the SubNet query stream (ResNet-50-shaped SuperNet, batch 1, 224x224, bf16).
 
     python bench.py --gpus N --steps K --warmup W            # this library
-    python bench.py --impl reference --steps K --warmup W    # the CPU checker on the host cores
+    python bench.py --impl reference --steps K --warmup W    # the CPU oracle on the host cores
 
 A step is one pass of the whole hot path over the query stream: `--queries` SubNet queries, each a
 different uniformly sampled SubNet config, through sgs_stream_run with inputs resident in HBM.
@@ -90,7 +90,7 @@ class ClockSampler:
 
 
 def cpu_oracle_qps(n_queries: int):
-    """Times the CPU checker, as it stands, on the first queries of the same workload."""
+    """Times the CPU oracle, as it stands, on the first queries of the same workload."""
     import oracle
     blob = wl.make_blob(wl.RESNET, seed=0, bf16_weights=True)
     net = oracle.Net(wl.RESNET, blob)

@@ -1,4 +1,4 @@
-"""ctypes front end of the CPU checker (oracle/sgs_oracle.c).
+"""ctypes front end of the CPU oracle (oracle/sgs_oracle.c).
 
 TEST INFRASTRUCTURE ONLY: imported by tests/, by the smoke check and by the CPU-baseline leg of
 the benchmark.  Nothing in the product package may import it.  The C file is compiled on the
@@ -38,7 +38,7 @@ def _cpu_tag() -> str:
 
 
 def build(force: bool = False) -> str:
-    """Compile the checker for this machine and return the path of the shared object."""
+    """Compile the oracle for this machine and return the path of the shared object."""
     out_dir = os.path.join(_HERE, "_build")
     os.makedirs(out_dir, exist_ok=True)
     so = os.path.join(out_dir, f"liboracle_{_cpu_tag()}.so")

@@ -1,5 +1,5 @@
 /*
- * CPU checker for SubNet inference on a weight-shared SuperNet.
+ * CPU oracle for SubNet inference on a weight-shared SuperNet.
  *
  * TEST INFRASTRUCTURE ONLY.  This file is the slow, plain statement of what the GPU library
  * must compute.  It shares no code, header, table or helper with the CUDA path and must never be

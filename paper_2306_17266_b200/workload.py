@@ -1,6 +1,6 @@
 """Seeded synthetic workloads: SuperNet weight blobs, query inputs and SubNet config streams.
 
-This module is the one piece shared by the CUDA library's callers and by the CPU checker.
+This module is the one piece shared by the CUDA library's callers and by the CPU oracle.
 It holds no inference arithmetic and no slicing rule: it only knows the *stored* (maximum)
 shape of every SuperNet tensor, the elastic choice sets a config may draw from, and the
 random recipes.  The paper evaluates on weight-shared ResNet50 / MobileNetV3 SuperNets with

@@ -1,9 +1,9 @@
 """Layer-level GPU parity of the layers that are not convolutions (max pool, global average pool, sliced fully
-connected layer, squeeze-excite gate and scale) against the CPU checker's single-layer functions, through the C
+connected layer, squeeze-excite gate and scale) against the CPU oracle's single-layer functions, through the C
 entry point sgs_aux_op: the kernel a single query uses (grouped = 0) and the kernel a wave uses (grouped = 1), on odd
 map sizes, ragged member mixes and channel counts at and off the kernels' 8-element vector width.
 
-Tolerances: max pool is exact (a maximum of bf16 values); sums are fp32 in a different order than the checker's
+Tolerances: max pool is exact (a maximum of bf16 values); sums are fp32 in a different order than the oracle's
 (<= 2e-5 relative to the largest value); SE scale rounds one product to bf16 (one flip of 2^-8 relative at most).
 """
 import numpy as np

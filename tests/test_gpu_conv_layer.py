@@ -1,5 +1,5 @@
 """Layer-level GPU parity of the sliced convolution (tensor-core and CUDA-core kernels) against the
-CPU checker's single-layer functions, through the C entry point sgs_conv2d_sliced.
+CPU oracle's single-layer functions, through the C entry point sgs_conv2d_sliced.
 
 Tolerance (bf16 operands, fp32 accumulation, bf16 store): max|err| <= 1e-2 * max|ref| over the
 tensor; the only differences are the fp32 summation order and the folded batch norm, i.e. at most a
@@ -17,7 +17,7 @@ pytestmark = pytest.mark.gpu
 
 
 def make_case(N, H, W, Cmax, C, Kmax, K, R, k, stride, act, use_res, seed=0, depthwise=False):
-    """Seeded layer inputs, the checker's result, and the device tensors in the library's layouts."""
+    """Seeded layer inputs, the oracle's result, and the device tensors in the library's layouts."""
     rng = np.random.default_rng(seed)
     cin = K if depthwise else C
     x = wl.round_to_bf16(rng.standard_normal((N, H, W, cin)).astype(np.float32))

@@ -45,7 +45,7 @@ def test_small_and_odd_resolutions(fam, res):
 
 def test_largest_and_smallest_config_full_size():
     # the two extreme SubNets at the benchmark's resolution and at batch 16 (the launch configuration of
-    # the batch-16 suites); the checker computes the first two images of the batch
+    # the batch-16 suites); the oracle computes the first two images of the batch
     _, onet, gnet = gu.nets(wl.RESNET, True)
     for largest in (False, True):
         c = wl.extreme_cfg(wl.RESNET, largest)

@@ -1,4 +1,4 @@
-"""Grouped launches at the edges of their tiles against the CPU checker: maps whose pixels end inside a tile, filter tiles that end
+"""Grouped launches at the edges of their tiles against the CPU oracle: maps whose pixels end inside a tile, filter tiles that end
 inside a block of 64, several output buffers and a single one, tiles shared by two members, maps shared between slots."""
 import numpy as np
 import pytest

@@ -1,5 +1,5 @@
 """GPU parity of the 8-bit sliced convolution layer (sgs_conv2d_sliced_i8: the paper's numeric format on the 8-bit
-tensor cores) against the CPU checker's exact integer layer.  Integer work: the comparison is bit exact."""
+tensor cores) against the CPU oracle's exact integer layer.  Integer work: the comparison is bit exact."""
 import numpy as np
 import pytest
 import torch

@@ -1,10 +1,10 @@
 """The paper's 8-bit format through a whole SubNet trunk: every bottleneck block of a ResNet-shaped SubNet (projection
 shortcut, 1x1, 3x3 with the stage's stride, 1x1 + residual + ReLU) as a chain of sgs_conv2d_sliced_i8 calls on padded
-pixels, against the same chain of the CPU checker's exact integer layer.  Integer work: bit exact, layer after layer.
+pixels, against the same chain of the CPU oracle's exact integer layer.  Integer work: bit exact, layer after layer.
 
 The 8-bit SuperNet is synthetic: seeded int8 weights in the stored shapes of the family, per-filter multipliers from the
 layer's shape alone (no data-dependent calibration: the paper gives no rule), post-ReLU tensors unsigned with zero point
-0, shortcuts signed.  The slices come from the checker's encoding of the config, so slicing by prefix is exercised on
+0, shortcuts signed.  The slices come from the oracle's encoding of the config, so slicing by prefix is exercised on
 every layer.
 """
 import numpy as np

@@ -1,7 +1,7 @@
-"""GPU parity: libsgs (through the C interface) against the CPU checker on the same seeded inputs.
+"""GPU parity: libsgs (through the C interface) against the CPU oracle on the same seeded inputs.
 
 Tolerances: fp32 mode max|err| <= 1e-4 * max|ref| per output row; bf16 mode (fp32 accumulation, every
-stored tensor rounded to bf16) max|err| <= 2e-2 * max|ref| against the checker run with the same
+stored tensor rounded to bf16) max|err| <= 2e-2 * max|ref| against the oracle run with the same
 storage rounding points.
 """
 import numpy as np
@@ -62,7 +62,7 @@ def test_tiny_bf16_all_queries():
 @pytest.mark.parametrize("fam", [wl.RESNET, wl.MBV3])
 @pytest.mark.parametrize("bf16", [False, True])
 def test_small_resolution_configs(fam, bf16):
-    # 64x64 inputs keep the checker fast while every layer type, stride and elastic choice runs;
+    # 64x64 inputs keep the oracle fast while every layer type, stride and elastic choice runs;
     # batch 3 and an odd feature-map size (res 72 -> 9, 5, 3 in the last stages) give ragged tiles
     _, onet, gnet = gu.nets(fam, bf16)
     cfgs = wl.uniform_stream(fam, 4, seed=7) + [wl.extreme_cfg(fam, False), wl.extreme_cfg(fam, True)]
@@ -148,7 +148,7 @@ def test_stream_run_matches_single_queries_and_counts_bytes():
 
 
 def test_cache_accounting_matches_checker_formulas():
-    # hit ratio and missed bytes of a stream, recomputed from the checker's encodings and formulas
+    # hit ratio and missed bytes of a stream, recomputed from the oracle's encodings and formulas
     _, onet, gnet = gu.nets(wl.RESNET, True)
     n, res, q = 16, 64, 4
     cfgs = wl.markov_stream(n, seed=9)
@@ -184,7 +184,7 @@ def test_encoding_matches_checker():
 
 def test_bench_launch_configuration_sampled_against_checker():
     # the benchmark's configuration (224x224, batch 1, graphs, cache on, 16 queries in flight) on the
-    # first 48 queries of its stream; four sampled queries are recomputed by the checker, all logits
+    # first 48 queries of its stream; four sampled queries are recomputed by the oracle, all logits
     # must be finite, and the stream must reproduce itself bit for bit
     _, onet, gnet = gu.nets(wl.RESNET, True)
     n, res = 48, 224
@@ -211,9 +211,9 @@ def test_bench_launch_configuration_sampled_against_checker():
 
 
 def _three_argmax_figures(got, ref_store, ref_f32):
-    """strict agreement with the bf16-store checker, strict and tie-aware agreement with the plain fp32 checker.
-    Tie-aware: the GPU's class counts as agreeing when the checker's own logit at that class is within the error
-    bound (2e-2 * max|ref|) of the checker's maximum."""
+    """strict agreement with the bf16-store oracle, strict and tie-aware agreement with the plain fp32 oracle.
+    Tie-aware: the GPU's class counts as agreeing when the oracle's own logit at that class is within the error
+    bound (2e-2 * max|ref|) of the oracle's maximum."""
     g = got.argmax(-1)
     strict_store = float(np.mean(g == ref_store.argmax(-1)))
     strict_f32 = float(np.mean(g == ref_f32.argmax(-1)))
@@ -225,10 +225,10 @@ def _three_argmax_figures(got, ref_store, ref_f32):
 @pytest.mark.parametrize("fam,n", [(wl.RESNET, 200), (wl.MBV3, 120)])
 def test_stream_against_plain_fp32_checker_and_argmax(fam, n):
     # The first queries of the benchmark streams, executed as the benchmark does (waves of 32, 4 in flight), against
-    # BOTH checker modes: the plain fp32 forward pass on the same bf16-valued weights and inputs (the bar of
+    # BOTH oracle modes: the plain fp32 forward pass on the same bf16-valued weights and inputs (the bar of
     # max|err| <= 2e-2 * max|ref| is meant against this one: it knows nothing about where the GPU rounds), and the
-    # forward pass that rounds every stored tensor to bf16.  Top-1: strict agreement with the bf16-store checker and
-    # tie-aware agreement with the fp32 checker must reach 99.5 %; strict agreement with the fp32 checker is reported
+    # forward pass that rounds every stored tensor to bf16.  Top-1: strict agreement with the bf16-store oracle and
+    # tie-aware agreement with the fp32 oracle must reach 99.5 %; strict agreement with the fp32 oracle is reported
     # and held to the same bar: with random weights a few top-2 margins are below one bf16 step, if it misses the
     # test says so.
     _, onet, gnet = gu.nets(fam, True)
@@ -246,13 +246,13 @@ def test_stream_against_plain_fp32_checker_and_argmax(fam, n):
     ref_f32 = np.stack([onet.forward(cfgs[t], xs[t], oracle.FP32)[0] for t in range(n)])
     worst_store, worst_f32 = gu.rel_err(got, ref_store), gu.rel_err(got, ref_f32)
     strict_store, strict_f32, tie_f32 = _three_argmax_figures(got, ref_store, ref_f32)
-    print(f"family {fam}: worst rel err vs bf16-store checker {worst_store:.2e}, vs fp32 checker {worst_f32:.2e}; "
+    print(f"family {fam}: worst rel err vs bf16-store oracle {worst_store:.2e}, vs fp32 oracle {worst_f32:.2e}; "
           f"argmax strict vs bf16-store {strict_store:.3f}, strict vs fp32 {strict_f32:.3f}, tie-aware vs fp32 {tie_f32:.3f}")
     assert worst_f32 <= TOL_BF16
     assert worst_store <= TOL_BF16
     assert strict_store >= 0.995
     assert tie_f32 >= 0.995
-    assert strict_f32 >= 0.995, "strict top-1 agreement with the plain fp32 checker is below 99.5 %"
+    assert strict_f32 >= 0.995, "strict top-1 agreement with the plain fp32 oracle is below 99.5 %"
 
 
 @pytest.mark.parametrize("fam", [wl.RESNET, wl.MBV3])

@@ -1,7 +1,7 @@
-"""GPU parity of persistent execution (the whole stream as one launch of the SubNet kernel) against the CPU checker.
+"""GPU parity of persistent execution (the whole stream as one launch of the SubNet kernel) against the CPU oracle.
 
-Same tolerance as the other bf16 parity tests: max|err| <= 2e-2 * max|ref| per output row, against the checker run
-with the same storage rounding points and against the plain fp32 checker.
+Same tolerance as the other bf16 parity tests: max|err| <= 2e-2 * max|ref| per output row, against the oracle run
+with the same storage rounding points and against the plain fp32 oracle.
 """
 import numpy as np
 import pytest
@@ -56,8 +56,8 @@ def test_persistent_stream_matches_checker(res, n):
 
 def test_persistent_stream_many_queries_per_block_equals_the_wave_path():
     # 400 queries on 148 blocks: every block serves several queries out of the same scratch area.  The layer-by-layer
-    # wave path (itself checked against the checker elsewhere) computes the same layers with other kernels: the two
-    # agree within the parity bound on every query, and sampled queries are compared with the checker directly.
+    # wave path (itself checked against the oracle elsewhere) computes the same layers with other kernels: the two
+    # agree within the parity bound on every query, and sampled queries are compared with the oracle directly.
     _, onet, gnet = gu.nets(wl.MBV3, True)
     n, res = 400, 64
     cfgs = wl.uniform_stream(wl.MBV3, n, seed=33)

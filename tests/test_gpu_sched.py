@@ -1,4 +1,4 @@
-"""AvgNet cache policy (Algorithm 1's caching decision) through the C ABI against the checker's scheduler:
+"""AvgNet cache policy (Algorithm 1's caching decision) through the C ABI against the oracle's scheduler:
 the choices, the hit ratio of Appendix A.4 and the missed weight bytes must agree exactly."""
 import numpy as np
 import pytest

@@ -1,7 +1,7 @@
-"""GPU parity of the wave execution (grouped launches over many queries in flight) against the CPU checker.
+"""GPU parity of the wave execution (grouped launches over many queries in flight) against the CPU oracle.
 
 Same tolerance as the other bf16 parity tests: max|err| <= 2e-2 * max|ref| per output row against the
-checker run with the same storage rounding points.
+oracle run with the same storage rounding points.
 """
 import numpy as np
 import pytest
@@ -69,7 +69,7 @@ def test_resnet_wave_accounting_equals_the_sequential_stream():
 
 
 def test_resnet_wave_batched_members_224():
-    # members with several images each (4 configs x 4 images), full resolution: sampled against the checker
+    # members with several images each (4 configs x 4 images), full resolution: sampled against the oracle
     _, onet, gnet = gu.nets(wl.RESNET, True)
     groups, batch, res = 4, 4, 224
     cfgs = wl.uniform_stream(wl.RESNET, groups, seed=5)
@@ -98,7 +98,7 @@ def test_wave_mode_on_the_other_families():
 
 def test_bench_wave_configuration_sampled_against_checker():
     # the benchmark's launch configuration (224x224, batch 1, waves of 32, 4 waves in flight, cache on) on the
-    # first 160 queries of its stream: sampled queries recomputed by the checker, every logit finite, the
+    # first 160 queries of its stream: sampled queries recomputed by the oracle, every logit finite, the
     # stream reproduces itself bit for bit, and the top-1 class of the sampled queries agrees
     _, onet, gnet = gu.nets(wl.RESNET, True)
     n, res = 160, 224
@@ -207,7 +207,7 @@ def test_members_sharing_a_tile_at_7x7_maps(family, res):
 @pytest.mark.parametrize("res", [160, 192, 224])
 def test_sweep_launch_shape_16_images_per_member(res):
     # the throughput sweep's launch shape: waves of 4 SubNet configs x 16 images each (one batch of 64 per grouped
-    # launch), two waves in flight; two members per resolution are recomputed by the checker (both modes), and the
+    # launch), two waves in flight; two members per resolution are recomputed by the oracle (both modes), and the
     # result must be the bits of the same queries run one member per wave
     _, onet, gnet = gu.nets(wl.RESNET, True)
     groups, batch = 8, 16
@@ -228,7 +228,7 @@ def test_sweep_launch_shape_16_images_per_member(res):
 def test_mbv3_bench_wave_configuration_sampled_against_checker():
     # the MobileNetV3-shaped stream as the benchmark runs it: 224x224, waves of 32, 4 in flight, the first 128 queries
     # of its stream (depthwise kernels of 3, 5 and 7 mixed inside every wave, so one depthwise launch dispatches all
-    # three bodies); sampled queries against the checker, bit-identical to waves of 5
+    # three bodies); sampled queries against the oracle, bit-identical to waves of 5
     _, onet, gnet = gu.nets(wl.MBV3, True)
     n, res = 128, 224
     cfgs = wl.uniform_stream(wl.MBV3, 1000, seed=3)[:n]
@@ -247,7 +247,7 @@ def test_mbv3_bench_wave_configuration_sampled_against_checker():
 
 @pytest.mark.parametrize("fam", [wl.RESNET, wl.MBV3])
 def test_fp32_mode_at_full_resolution(fam):
-    # fp32 handles at 224x224 (CUDA-core kernels throughout): max|err| <= 1e-4 * max|ref| against the fp32 checker
+    # fp32 handles at 224x224 (CUDA-core kernels throughout): max|err| <= 1e-4 * max|ref| against the fp32 oracle
     _, onet, gnet = gu.nets(fam, False)
     c = wl.uniform_stream(fam, 2, seed=17)[1]
     x = wl.make_inputs(1, 2, 224, seed=6)[0]

@@ -1,4 +1,4 @@
-"""Pins for the CPU checker: what the paper and plain mathematics fix, independent of the checker.
+"""Pins for the CPU oracle: what the paper and plain mathematics fix, independent of it.
 
 Paper facts used (Section 2.1): a SubNet is a selection of SuperNet weights; the largest SubNet is
 the whole SuperNet and the smallest is contained in all others; a SubNet predicts without being
@@ -210,7 +210,7 @@ def _bf16_representable(a):
 
 
 def _stored_tensors(net, fam, cfg, x, mode):
-    """Every tensor the checker stores on the way (one tapped run per stored layer the SubNet uses) and its logits."""
+    """Every tensor the oracle stores on the way (one tapped run per stored layer the SubNet uses) and its logits."""
     names = [r.name for r in wl.supernet_records(fam)]
     out, logits = {}, None
     for i, name in enumerate(names):
@@ -222,7 +222,7 @@ def _stored_tensors(net, fam, cfg, x, mode):
 
 @pytest.mark.parametrize("fam,res", [(wl.TINY, 32), (wl.RESNET, 64), (wl.MBV3, 64)])
 def test_bf16_store_mode_rounds_exactly_the_stored_tensors(fam, res):
-    """Pins where the bf16-store mode rounds.  Layer by layer, each layer fed with the checker's own stored inputs:
+    """Pins where the bf16-store mode rounds.  Layer by layer, each layer fed with the oracle's own stored inputs:
     a tensor the mode stores (layer outputs, SE-scaled maps) holds only bf16 values and equals the fp64 library
     restatement rounded once, up to a few one-step flips from the order of additions; what is not stored (pooled and
     SE vectors, the head's mixing vector, logits) is not rounded, so the logits computed from the last stored tensor
@@ -244,7 +244,7 @@ def test_bf16_store_mode_rounds_exactly_the_stored_tensors(fam, res):
             assert rep["beyond_one_step"] == 0, (name, rep)
             assert rep["unequal"] <= max(2, 0.005 * rep["n"]), (name, rep)
         assert np.abs(logits - ref_logits).max() <= 2e-5 * max(1.0, np.abs(ref_logits).max())
-        # a checker that forgot to round (its fp32 mode) is caught by the same checks
+        # an oracle that forgot to round (its fp32 mode) is caught by the same checks
         plain, _ = _stored_tensors(net, fam, c, x, oracle.FP32)
         assert not any(_bf16_representable(t) for t in plain.values())
 

@@ -1,4 +1,4 @@
-"""CPU pins of the checker's scheduler functions (Algorithm 1's caching decision, Section 3.3): hand-computed
+"""CPU pins of the oracle's scheduler functions (Algorithm 1's caching decision, Section 3.3): hand-computed
 vectors, closed forms and special cases that fix the running average, the distance, tie handling, the
 budget clipping and the timing of the decisions."""
 import numpy as np

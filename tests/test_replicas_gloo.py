@@ -64,7 +64,7 @@ def test_shard_bounds_partition():
 
 
 def _mean_hit_ratio(encs, q=4):
-    """Appendix A.4 hit ratio of a shard served with the intersection policy (window q), from the checker's formulas."""
+    """Appendix A.4 hit ratio of a shard served with the intersection policy (window q), from the oracle's formulas."""
     import numpy as np
     import oracle
     G, hits = None, []

@@ -1,4 +1,4 @@
-"""An fp64 PyTorch restatement of the three synthetic SuperNets, used only to pin the C checker.
+"""An fp64 PyTorch restatement of the three synthetic SuperNets, used only to pin the C oracle.
 
 It is written against library routines (``torch.nn.functional.conv2d`` and friends) on tensors
 that are first cut out of the blob with ordinary Python slices, so a wiring or indexing mistake in
