@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) conv_group_kernel(const __grid_c
 
     // The three issuing warps run their loops converged; the elected lane issues (see sgs_tc.cuh).
     // Their loops over tiles end at total_tiles, not at n_tiles: with a trip count out of a division the MMA warp's own part of a
-    // stage (waits left out) took 447 clocks instead of 331, which bounds tiles of few columns (B200; a 3x3 layer of 72 stages and
+    // stage (waits left out) took 435 clocks instead of 315, which bounds tiles of few columns (B200; a 3x3 layer of 72 stages and
     // 16 columns 44.5 us, 36.3 like this; waves of 32 images of 32x32 878 -> 777 us, 4 queries x 16 images of 224x224 13150 -> 12780).
     const uint32_t ring = smem_u32(smem), bufs = ring + (uint32_t)(n_stages * stage_bytes), full0 = smem_u32(full_bar), empty0 = smem_u32(empty_bar);
     if (warp == 0) {
